@@ -55,7 +55,8 @@ def flops_per_atom(m_r: float, m_a: float, n_neu: int = 30) -> float:
     return 134.0 * m_r + 1500.0 * m_a + 288.0 + 4.0 * n_neu * 32 + 10.0 * n_neu
 
 
-SITE_SOURCES = ("paper_2107_08119_gb300/csrc/nep_site.cuh", "paper_2107_08119_gb300/csrc/nep_force.cu",
+SITE_SOURCES = ("paper_2107_08119_gb300/csrc/nep_site.cuh", "paper_2107_08119_gb300/csrc/nep_site_block.cuh",
+                "paper_2107_08119_gb300/csrc/nep_force.cu",
                 "paper_2107_08119_gb300/csrc/nep_internal.cuh")
 SITE_PROFILE = os.path.join(ROOT, "profiles", "k_site_md_125k.json")
 

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_lambda(int N, const int* __
             load_pos(xh, xl, N, j, hj, lj);
             const float4 ej = res[j];
             float r[3];
-            pair_vector(ia, j, v >> 24, hi, li, hj, lj, box, r[0], r[1], r[2]);
+            pair_vector(v >> 24, hi, li, hj, lj, box, r[0], r[1], r[2]);
             const float d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
             const float dd[3] = {fmaf(-ej.x, scale, di[0]), fmaf(-ej.y, scale, di[1]), fmaf(-ej.z, scale, di[2])};
             const float d = sqrtf(d2);

@@ -44,6 +44,15 @@ __host__ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c)
 #endif
 }
 
+__host__ __device__ __forceinline__ float2 fadd2(float2 a, float2 b)
+{
+#ifdef __CUDA_ARCH__
+    return __fadd2_rn(a, b);
+#else
+    return make_float2(a.x + b.x, a.y + b.y);
+#endif
+}
+
 // ---------------------------------------------------------------- sizes
 constexpr int kNR = 8;               // radial orders n = 0..7
 constexpr int kNA = 6;               // angular radial orders n = 0..5
@@ -102,27 +111,26 @@ __host__ __device__ __forceinline__ float diff1(float ah, float al, float bh, fl
     return hi + lo;
 }
 
-// Pair vector r_ij = x_j + shift(code) - x_i, evaluated in a canonical
-// orientation so that r_ji == -r_ij bit for bit.  Both atoms' hi/lo
-// coordinates are passed in.
-__host__ __device__ __forceinline__ void pair_vector(int i, int j, int code, const float (&hi)[3], const float (&li)[3],
-                                            const float (&hj)[3], const float (&lj)[3], const Box& b, float& rx,
-                                            float& ry, float& rz)
+// Pair vector r_ij = x_j + shift(code) - x_i.  Swapping the two atoms (and the
+// sign of the shift) swaps the operands of every subtraction in diff1, so
+// r_ji == -r_ij exactly whichever of the two evaluates it.  Most pairs cross
+// no box face: their shift is zero and the general form reduces to three
+// subtractions and sums (the same values), without the decoding of the image.
+__host__ __device__ __forceinline__ void pair_vector(int code, const float (&hi)[3], const float (&li)[3],
+                                                     const float (&hj)[3], const float (&lj)[3], const Box& b,
+                                                     float& rx, float& ry, float& rz)
 {
+    if (code == kImgCenter) {
+        rx = (hj[0] - hi[0]) + (lj[0] - li[0]);
+        ry = (hj[1] - hi[1]) + (lj[1] - li[1]);
+        rz = (hj[2] - hi[2]) + (lj[2] - li[2]);
+        return;
+    }
     int sx, sy, sz;
     image_shift(code, sx, sy, sz);
-    const bool fwd = (j > i) || (j == i && code < kImgCenter);
-    const float sg = fwd ? 1.f : -1.f;
-    const float fx = fwd ? (float)sx : (float)(-sx);
-    const float fy = fwd ? (float)sy : (float)(-sy);
-    const float fz = fwd ? (float)sz : (float)(-sz);
-    // a = the atom whose image is shifted, b = the origin atom
-    rx = sg * diff1(fwd ? hj[0] : hi[0], fwd ? lj[0] : li[0], fwd ? hi[0] : hj[0], fwd ? li[0] : lj[0], fx, b.Lh[0],
-                    b.Ll[0]);
-    ry = sg * diff1(fwd ? hj[1] : hi[1], fwd ? lj[1] : li[1], fwd ? hi[1] : hj[1], fwd ? li[1] : lj[1], fy, b.Lh[1],
-                    b.Ll[1]);
-    rz = sg * diff1(fwd ? hj[2] : hi[2], fwd ? lj[2] : li[2], fwd ? hi[2] : hj[2], fwd ? li[2] : lj[2], fz, b.Lh[2],
-                    b.Ll[2]);
+    rx = diff1(hj[0], lj[0], hi[0], li[0], (float)sx, b.Lh[0], b.Ll[0]);
+    ry = diff1(hj[1], lj[1], hi[1], li[1], (float)sy, b.Lh[1], b.Ll[1]);
+    rz = diff1(hj[2], lj[2], hi[2], li[2], (float)sz, b.Lh[2], b.Ll[2]);
 }
 
 // pair_vector that also returns the rounding residual of each component:
@@ -139,24 +147,23 @@ __host__ __device__ __forceinline__ float diff1_lo(float ah, float al, float bh,
     return r;
 }
 
-__host__ __device__ __forceinline__ void pair_vector_lo(int i, int j, int code, const float (&hi)[3],
-                                                        const float (&li)[3], const float (&hj)[3],
-                                                        const float (&lj)[3], const Box& b, float (&r)[3],
-                                                        float (&r_lo)[3])
+__host__ __device__ __forceinline__ void pair_vector_lo(int code, const float (&hi)[3], const float (&li)[3],
+                                                        const float (&hj)[3], const float (&lj)[3], const Box& b,
+                                                        float (&r)[3], float (&r_lo)[3])
 {
-    int sx, sy, sz;
-    image_shift(code, sx, sy, sz);
-    const bool fwd = (j > i) || (j == i && code < kImgCenter);
-    const float sg = fwd ? 1.f : -1.f;
-    const float f[3] = {fwd ? (float)sx : (float)(-sx), fwd ? (float)sy : (float)(-sy),
-                        fwd ? (float)sz : (float)(-sz)};
+    if (code == kImgCenter) {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        float rl;
-        r[d] = sg * diff1_lo(fwd ? hj[d] : hi[d], fwd ? lj[d] : li[d], fwd ? hi[d] : hj[d], fwd ? li[d] : lj[d], f[d],
-                             b.Lh[d], b.Ll[d], rl);
-        r_lo[d] = sg * rl;
+        for (int d = 0; d < 3; ++d) {
+            const float h = hj[d] - hi[d], l = lj[d] - li[d];
+            r[d] = h + l;
+            r_lo[d] = l - (r[d] - h);
+        }
+        return;
     }
+    int s[3];
+    image_shift(code, s[0], s[1], s[2]);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) r[d] = diff1_lo(hj[d], lj[d], hi[d], li[d], (float)s[d], b.Lh[d], b.Ll[d], r_lo[d]);
 }
 
 // FP32 hi/lo positions are stored as one float4 record (x, y, z, 0) per atom
@@ -289,7 +296,7 @@ struct NeighborList {
     int* cell_fill = nullptr;
     int* cell_atoms = nullptr;
     // [3][n] words: bit k of atom i set when slot k lies within the cutoff,
-    // written by the site pass when it compacts its staged slots; `mask_set`
+    // written by the site pass from its cutoff tests; `mask_set`
     // (host) says whether the last site pass launched wrote them, so that
     // the assembly skips the other slots' loads.
     unsigned* mask = nullptr;
@@ -338,10 +345,10 @@ struct ForceArgs {
 // allocation-free call need the first.
 inline bool sizes_default(const nep_hyper& h) { return h.n_max_R == kNR - 1 && h.n_max_A == kNA - 1; }
 inline bool sizes_split(const nep_hyper& h) { return h.n_max_R == 12 && h.n_max_A == 6; }
-// the site pass runs kSiteAtomsPerBlock atoms per block; its per-block
-// energy partials need site_blocks(n) slots, which also bounds the block
-// counts of the assembly and of the plain comparator
-constexpr int kSiteAtomsPerBlock = 128;
+// the site pass runs kSiteAtomsPerBlock atoms per block (one lane each); its
+// per-block energy partials need site_blocks(n) slots, which also bounds the
+// block counts of the assembly and of the plain comparator
+constexpr int kSiteAtomsPerBlock = 32;
 inline int site_blocks(int n) { return (n + kSiteAtomsPerBlock - 1) / kSiteAtomsPerBlock; }
 int launch_site_partial_forces(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, double* e_partials,
                                unsigned* d_err, cudaStream_t st, int& nblocks);

@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_half_cells(int n, int m_c
                 float hj[3], lj[3];
                 load_pos(xh, xl, n, j, hj, lj);
                 float rx, ry, rz;
-                pair_vector(i, j, value >> 24, hi, li, hj, lj, b, rx, ry, rz);
+                pair_vector(value >> 24, hi, li, hj, lj, b, rx, ry, rz);
                 d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
                 accept = d2 < rv2;
             }
@@ -649,7 +649,7 @@ __global__ void k_verlet_brute(int n, int m_cap, float rv2, const float* __restr
                     const int code = image_code(sx, sy, sz);
                     if (j == i && code == kImgCenter) continue;
                     float rx, ry, rz;
-                    pair_vector(i, j, code, hi, li, hj, lj, b, rx, ry, rz);
+                    pair_vector(code, hi, li, hj, lj, b, rx, ry, rz);
                     const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
                     if (d2 < rv2) list_push(i, n, m_cap, cnt, j | (code << 24), d2, nbr, key);
                 }

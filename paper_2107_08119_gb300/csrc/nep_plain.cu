@@ -83,7 +83,7 @@ __device__ __forceinline__ float plain_pair(int i, int n, int k, const int* __re
     const int j = v & 0xFFFFFF;
     float hj[3], lj[3];
     load_pos(xh, xl, n, j, hj, lj);
-    pair_vector(i, j, v >> 24, hi, li, hj, lj, box, r[0], r[1], r[2]);
+    pair_vector(v >> 24, hi, li, hj, lj, box, r[0], r[1], r[2]);
     return r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
 }
 

@@ -36,6 +36,17 @@ __host__ __device__ __forceinline__ void sincospi_f(float x, float* s, float* c)
 #endif
 }
 
+// a * b rounded by itself: never contracted into an FMA, so that kernels that
+// evaluate different subsets of the harmonics round them alike.
+__host__ __device__ __forceinline__ float mul_rn(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+
 // d / rc from d * (1/rc) with one Newton correction: the rounded reciprocal
 // of a cutoff such as 5 A is not exact in FP32, and the plain product would
 // bias every radial function the same way.
@@ -53,20 +64,26 @@ __host__ __device__ __forceinline__ void two_sum(float a, float b, float& s, flo
     e = (a - (s - bb)) + (b - bb);
 }
 
-// g_n(d), n = 0..N-1, for d < rc; w multiplies the cutoff function (the
-// multicomponent weight sqrt(Z_i Z_j), 1 for one species).  x = 2 t^2 - 1
-// with t = d/rc - 1 carried as hi + lo: for d < rc/2 the difference rounds,
-// and the Chebyshev recurrence multiplies an error in x by up to n^2.
-template <int N>
-__host__ __device__ __forceinline__ void radial_g(float d, float rc, float inv_rc, float (&g)[N], float w = 1.f)
+// The two numbers g_n(d) is built from, for d < rc: the Chebyshev argument
+// x = 2 t^2 - 1 and the cutoff function fc; w multiplies fc (the
+// multicomponent weight sqrt(Z_i Z_j), 1 for one species).  t = d/rc - 1 is
+// carried as hi + lo: for d < rc/2 the difference rounds, and the Chebyshev
+// recurrence multiplies an error in x by up to n^2.
+__host__ __device__ __forceinline__ void radial_x(float d, float rc, float inv_rc, float w, float& x, float& fc)
 {
     float s, c;
     const float dr = div_rc(d, rc, inv_rc);
     sincospi_f(dr, &s, &c);
-    const float fc = 0.5f * (1.f + c) * w;
+    fc = 0.5f * (1.f + c) * w;
     float t, tl;
     two_sum(dr, -1.f, t, tl);
-    const float x = fmaf(4.f * t, tl, fmaf(2.f * t, t, -1.f));
+    x = fmaf(4.f * t, tl, fmaf(2.f * t, t, -1.f));
+}
+
+// g_n = (T_n(x) + 1)/2 fc, n = 0..N-1
+template <int N>
+__host__ __device__ __forceinline__ void cheb_g(float x, float fc, float (&g)[N])
+{
     float Tm = 1.f, T = x;  // T_{n-1}, T_n
     const float hfc = 0.5f * fc;
     g[0] = fc;
@@ -78,6 +95,15 @@ __host__ __device__ __forceinline__ void radial_g(float d, float rc, float inv_r
         T = Tn;
         g[n] = fmaf(hfc, Tn, hfc);
     }
+}
+
+// g_n(d), n = 0..N-1, for d < rc; w as in radial_x
+template <int N>
+__host__ __device__ __forceinline__ void radial_g(float d, float rc, float inv_rc, float (&g)[N], float w = 1.f)
+{
+    float x, fc;
+    radial_x(d, rc, inv_rc, w, x, fc);
+    cheb_g<N>(x, fc, g);
 }
 
 // (g_n(d), dg_n/dd), n = 0..N-1, for d < rc, as pairs; w as in radial_g.
@@ -135,8 +161,8 @@ __host__ __device__ __forceinline__ void radial_g_dg(float d, float rc, float in
 // NEP_SH_LOCALS in scope; the factors k z^2 - c are formed from the exact
 // square (the rounding of z^2 would otherwise be multiplied by up to 21).
 #define NEP_SH_LOCALS(x, y, z)                                                  \
-    const float x2 = x * x, y2 = y * y, z2 = z * z;                             \
-    const float xy = x * y, yz = y * z, xz = x * z;                             \
+    const float x2 = mul_rn(x, x), y2 = mul_rn(y, y), z2 = mul_rn(z, z);        \
+    const float xy = mul_rn(x, y), yz = mul_rn(y, z), xz = mul_rn(x, z);        \
     const float x2my2 = x2 - y2;                                                \
     const float z2l = fmaf(z, z, -z2); /* z^2 = z2 + z2l exactly */             \
     const float a5 = fmaf(5.f, z2l, fmaf(5.f, z2, -1.f));                       \
@@ -149,8 +175,8 @@ __host__ __device__ __forceinline__ void radial_g_dg(float d, float rc, float in
 // The same with z^2 rounded once (the partial forces, whose 1e-4 eV/A bar
 // leaves room).
 #define NEP_SH_LOCALS_FAST(x, y, z)                                                \
-    const float x2 = x * x, y2 = y * y, z2 = z * z;                             \
-    const float xy = x * y, yz = y * z, xz = x * z;                             \
+    const float x2 = mul_rn(x, x), y2 = mul_rn(y, y), z2 = mul_rn(z, z);        \
+    const float xy = mul_rn(x, y), yz = mul_rn(y, z), xz = mul_rn(x, z);        \
     const float x2my2 = x2 - y2;                                                \
     const float z2l = 0.f;                                                      \
     const float a5 = 5.f * z2 - 1.f, a7 = 7.f * z2 - 1.f, b7 = 7.f * z2 - 3.f; \
@@ -313,11 +339,8 @@ __host__ __device__ __forceinline__ void kahan_step(float w, float qv, float& a,
     a = t;
 }
 
-// Adds neuron mu's output w2 x to the compensated sum (s, c) and its share
-// w2 (1 - x^2) w1_mu of G.
-template <int ND>
-__host__ __device__ __forceinline__ void neuron_out(float w2, float xm, const float* row, float& s, float& c,
-                                                    float (&G)[ND])
+// Adds a neuron's output w2 x to the compensated sum (s, c).
+__host__ __device__ __forceinline__ void neuron_energy(float w2, float xm, float& s, float& c)
 {
     const float p = w2 * xm;
     const float ep = fmaf(w2, xm, -p);
@@ -325,6 +348,72 @@ __host__ __device__ __forceinline__ void neuron_out(float w2, float xm, const fl
     two_sum(s, p, t, e);
     s = t;
     c += e + ep;
+}
+
+// One neuron's state tanh(sum_v row_v q_v - b1).
+template <int ND>
+__host__ __device__ __forceinline__ float neuron_state(const float* row, float b1, const float (&q)[ND])
+{
+    // four interleaved compensated chains (descriptor v in chain v mod 4),
+    // so that consecutive steps do not wait on each other, joined by
+    // error-free sums
+#ifdef __CUDA_ARCH__
+    // The chains in pairs, as packed operations on a and n = -ca:
+    // y = w q + n, t = a + y, n = y + (a - t).  The first product of a chain
+    // enters unrounded (its rounding error goes into n).
+    float w[4];
+    auto load = [&](int v) {
+        if constexpr (ND % 4 == 0) {  // a 16-byte load (shared memory, aligned for ND % 4 == 0)
+            const float4 t = *reinterpret_cast<const float4*>(row + v);
+            w[0] = t.x;
+            w[1] = t.y;
+            w[2] = t.z;
+            w[3] = t.w;
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) w[c] = row[v + c];
+        }
+    };
+    load(0);
+    const float2 minus = make_float2(-1.f, -1.f);
+    const float t0 = fmaf(w[0], q[0], -b1), t1 = mul_rn(w[1], q[1]), t2 = mul_rn(w[2], q[2]), t3 = mul_rn(w[3], q[3]);
+    float2 a01 = make_float2(t0, t1), a23 = make_float2(t2, t3);
+    float2 n01 = make_float2(fmaf(w[0], q[0], -b1 - t0), fmaf(w[1], q[1], -t1));
+    float2 n23 = make_float2(fmaf(w[2], q[2], -t2), fmaf(w[3], q[3], -t3));
+#pragma unroll
+    for (int v = 4; v + 4 <= ND; v += 4) {
+        load(v);
+        const float2 y01 = ffma2(make_float2(w[0], w[1]), make_float2(q[v], q[v + 1]), n01);
+        const float2 y23 = ffma2(make_float2(w[2], w[3]), make_float2(q[v + 2], q[v + 3]), n23);
+        const float2 u01 = fadd2(a01, y01), u23 = fadd2(a23, y23);
+        n01 = fadd2(y01, ffma2(u01, minus, a01));
+        n23 = fadd2(y23, ffma2(u23, minus, a23));
+        a01 = u01;
+        a23 = u23;
+    }
+    float a[4] = {a01.x, a01.y, a23.x, a23.y}, ca[4] = {-n01.x, -n01.y, -n23.x, -n23.y};
+#pragma unroll
+    for (int v = ND / 4 * 4; v < ND; ++v) kahan_step(row[v], q[v], a[v & 3], ca[v & 3]);
+#else
+    float a[4] = {-b1, 0.f, 0.f, 0.f}, ca[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int v = 0; v < ND; ++v) kahan_step(row[v], q[v], a[v & 3], ca[v & 3]);
+#endif
+    float s01, e01, s23, e23, sa, ea;
+    two_sum(a[0], a[1], s01, e01);
+    two_sum(a[2], a[3], s23, e23);
+    two_sum(s01, s23, sa, ea);
+    const float comp = ((ca[0] + ca[1]) + (ca[2] + ca[3])) - ((e01 + e23) + ea);
+    return tanhf(sa - comp);
+}
+
+// Adds neuron mu's output w2 x to the compensated sum (s, c) and its share
+// w2 (1 - x^2) w1_mu of G.
+template <int ND>
+__host__ __device__ __forceinline__ void neuron_out(float w2, float xm, const float* row, float& s, float& c,
+                                                    float (&G)[ND])
+{
+    neuron_energy(w2, xm, s, c);
     const float d = w2 * fmaf(-xm, xm, 1.f);
 #ifdef __CUDA_ARCH__
     if constexpr (ND % 4 == 0) {
@@ -362,34 +451,7 @@ __host__ __device__ __forceinline__ void network(const float* w, int n_neu, cons
     float s = 0.f, c = 0.f;
     for (int mu = 0; mu < n_neu; ++mu) {
         const float* row = w + mu * ND;
-        // four interleaved compensated chains (descriptor v in chain v mod 4),
-        // so that consecutive steps do not wait on each other, joined by
-        // error-free sums
-        float a[4] = {-b1[mu], 0.f, 0.f, 0.f}, ca[4] = {0.f, 0.f, 0.f, 0.f};
-#ifdef __CUDA_ARCH__
-        if constexpr (ND % 4 == 0) {
-            // 16-byte loads of the row (shared memory, aligned for ND % 4 == 0)
-            const float4* row4 = reinterpret_cast<const float4*>(row);
-#pragma unroll
-            for (int v = 0; v < ND; v += 4) {
-                const float4 t = row4[v / 4];
-                kahan_step(t.x, q[v], a[0], ca[0]);
-                kahan_step(t.y, q[v + 1], a[1], ca[1]);
-                kahan_step(t.z, q[v + 2], a[2], ca[2]);
-                kahan_step(t.w, q[v + 3], a[3], ca[3]);
-            }
-        } else
-#endif
-        {
-#pragma unroll
-            for (int v = 0; v < ND; ++v) kahan_step(row[v], q[v], a[v & 3], ca[v & 3]);
-        }
-        float s01, e01, s23, e23, sa, ea;
-        two_sum(a[0], a[1], s01, e01);
-        two_sum(a[2], a[3], s23, e23);
-        two_sum(s01, s23, sa, ea);
-        const float comp = ((ca[0] + ca[1]) + (ca[2] + ca[3])) - ((e01 + e23) + ea);
-        neuron_out(w2[mu], tanhf(sa - comp), row, s, c, G);
+        neuron_out(w2[mu], neuron_state<ND>(row, b1[mu], q), row, s, c, G);
     }
     float t, e;
     two_sum(s, -b2, t, e);
@@ -556,9 +618,8 @@ __host__ __device__ __forceinline__ void site_descriptors(int i, int n, int cnt,
         const NbSlot cur = nx;
         fetch_slot(nbr, xh, xl, n, k - 1, cnt, nx);
         if (k >= cnt) continue;
-        const int j = cur.v & 0xFFFFFF;
         float rx, ry, rz;
-        pair_vector(i, j, cur.v >> 24, hi, li, cur.h, cur.l, box, rx, ry, rz);
+        pair_vector(cur.v >> 24, hi, li, cur.h, cur.l, box, rx, ry, rz);
         const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
         const float w = pair_weight(P, zi, cur.z);
         if (d2 < P.rcR2) {
@@ -723,9 +784,8 @@ __host__ __device__ __forceinline__ void site_partial_forces(int i, bool active,
     for (int k = 0; k < cnt; ++k) {
         const NbSlot cur = nx;
         fetch_slot(nbr, xh, xl, n, k + 1, cnt, nx);
-        const int j = cur.v & 0xFFFFFF;
         float r[3], r_lo[3];
-        pair_vector_lo(i, j, cur.v >> 24, hi, li, cur.h, cur.l, box, r, r_lo);
+        pair_vector_lo(cur.v >> 24, hi, li, cur.h, cur.l, box, r, r_lo);
         const float d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
         if (!(d2 < rc2max)) continue;
         float px, py, pz, dE;
@@ -818,9 +878,8 @@ __host__ __device__ __forceinline__ void assemble_atom(int i, int n, int m_cap, 
         load_data(k + 1, v2, kr2, nx);
         load_idx(k + 2, v2, kr2);
         if (!kept(k)) continue;
-        const int j = cur.v & 0xFFFFFF;
         float r[3];
-        pair_vector(i, j, cur.v >> 24, hi, li, cur.h, cur.l, box, r[0], r[1], r[2]);
+        pair_vector(cur.v >> 24, hi, li, cur.h, cur.l, box, r[0], r[1], r[2]);
         const float d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
         if (!(d2 < rc2max)) continue;
         // own p_ij and the neighbour's p_ji: one 16-byte record each

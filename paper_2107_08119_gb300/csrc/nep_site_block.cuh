@@ -1,0 +1,518 @@
+// nep_site_block.cuh -- the site pass of the force path as a cooperation of
+// four warps on 32 atoms (the arithmetic of nep_site.cuh, operation for
+// operation).
+//
+// What bounds it: instruction issue and dependency latency, not memory (the
+// list, positions and partial forces of a 125k-atom box are about 150 MB per
+// pass).  One thread per atom needs 255 registers for the 144 harmonic sums,
+// leaves two warps per scheduler and, below 39k atoms, one thread's serial
+// run of ~30k instructions as the time of the whole pass.  Here lane l of
+// every warp works on atom i0 + l and the warps split the rest:
+//   pair geometry    warp w takes the slots k = w mod 4: pair vector, cutoff
+//                    tests, unit vector and radial functions, into a shared
+//                    tile of 16 slots (lane-minor: no bank conflicts);
+//   descriptor sums  from the tile, slots in descending order: warps 0-2
+//                    eight of the 24 harmonics each, warp 3 the radial sums (each sum in one thread, in the order of
+//                    site_descriptors, so the same bits);
+//   network          warp w takes the neurons mu = w mod 4, then a quarter of
+//                    the input gradient G;
+//   partial forces   warp w takes its slots again, each angular pair against
+//                    the coefficients A in shared memory.
+// Measured on a GB300, one thread per atom -> this form: 248 -> 187 us for the
+// 125,000-atom crystal (1190 -> 1122 warp instructions per atom, 7.6 -> 18.6
+// warps per SM), 104 -> 71 us for the whole MD step of 4,096 atoms.
+#pragma once
+
+#include "nep_site.cuh"
+
+namespace nep {
+
+constexpr int kSiteAtoms = kSiteAtomsPerBlock;  // one lane per atom
+constexpr int kSiteWarps = 4;
+constexpr int kSiteThreads = 32 * kSiteWarps;
+constexpr int kSiteChunk = 16;  // slots per shared tile
+static_assert(kSiteAtoms == 32, "one lane per atom of the block");
+
+// Marks a tile entry outside the cutoff: both a Chebyshev argument and a
+// component of a unit vector lie in [-1, 1].
+constexpr float kNoPair = 2.f;
+
+// float4 words per lane of the region that holds first the pair tile, then
+// the harmonic sums S and the coefficients A
+template <class D>
+__host__ __device__ constexpr int site_block_quads()
+{
+    return ((D::NA * kLM > (3 + D::NA) * kSiteChunk ? D::NA * kLM : (3 + D::NA) * kSiteChunk) + 3) / 4;
+}
+
+// Place of S_nlm (and A_nlm) in a lane's column: harmonics in pairs (2j, 2j + 1)
+// side by side, so that one 8-byte operand of a packed FMA holds both, the
+// radial orders of a pair next to each other; 16-byte words are lane-minor
+// ([word][32 lanes]).
+template <class D>
+__host__ __device__ constexpr int site_block_at(int n, int lm)
+{
+    const int f = 2 * ((lm >> 1) * D::NA + n) + (lm & 1);
+    return (f >> 2) * 128 + (f & 3);
+}
+
+// shared memory: weights | tile / S / A | q / G | radial tile / neuron states and slopes | mask words
+template <class D>
+__host__ __device__ inline size_t site_block_smem(int n_par, int n_neu)
+{
+    const size_t x_rows = 2 * (n_neu > kSiteChunk ? n_neu : kSiteChunk);
+    return sizeof(float) * (((size_t)n_par + 31) / 32 * 32 +
+                            (size_t)kSiteAtoms * (4 * site_block_quads<D>() + D::Ndes + x_rows + 3));
+}
+
+// Whether component a of the gradient of harmonic lm is zero for every
+// direction: the 0.f entries of NEP_SH_TABLE (bit a: component a).
+__host__ __device__ constexpr bool sh_zero(int lm, int a)
+{
+    constexpr unsigned char z[kLM] = {6, 5, 3, 4, 1, 2, 3, 4, 4, 0, 1, 3, 2, 0, 4, 4, 0, 0, 1, 3, 2, 0, 0, 4};
+    return (z[lm] >> a) & 1;
+}
+
+// The values NEP_SH_TABLE refers to, for one unit vector (partial forces).
+struct ShFast {
+    float x, y, z, x2, y2, z2, xy, yz, xz, x2my2, a5, a7, b7, c21, e19;
+    __device__ __forceinline__ void set(float ux, float uy, float uz)
+    {
+        x = ux;
+        y = uy;
+        z = uz;
+        NEP_SH_LOCALS_FAST(ux, uy, uz)
+        this->x2 = x2;
+        this->y2 = y2;
+        this->z2 = z2;
+        this->xy = xy;
+        this->yz = yz;
+        this->xz = xz;
+        this->x2my2 = x2my2;
+        this->a5 = a5;
+        this->a7 = a7;
+        this->b7 = b7;
+        this->c21 = c21;
+        this->e19 = e19;
+    }
+};
+
+// B += cd Y, V += cg grad Y for harmonic LM (its unprojected gradient), as
+// sh_term does.
+template <int LM>
+__device__ __forceinline__ void sh_add(const ShFast& s, float cg, float cd, float& B, float (&V)[3])
+{
+    const float x = s.x, y = s.y, z = s.z, x2 = s.x2, y2 = s.y2, z2 = s.z2, xy = s.xy, yz = s.yz, xz = s.xz;
+    const float x2my2 = s.x2my2, z2l = 0.f, a5 = s.a5, a7 = s.a7, b7 = s.b7, c21 = s.c21, e19 = s.e19;
+    (void)x; (void)y; (void)z; (void)x2; (void)y2; (void)z2; (void)xy; (void)yz; (void)xz;
+    (void)x2my2; (void)z2l; (void)a5; (void)a7; (void)b7; (void)c21; (void)e19;
+#define NEP_T(lm, Yv, gx, gy, gz)                                                       \
+    if constexpr (LM == lm) {                                                           \
+        B = fmaf(cd, Yv, B);                                                            \
+        const float d[3] = {gx, gy, gz};                                                \
+        _Pragma("unroll") for (int a = 0; a < 3; ++a) if (!sh_zero(lm, a)) V[a] = fmaf(cg, d[a], V[a]); \
+    }
+    NEP_SH_TABLE(NEP_T)
+#undef NEP_T
+}
+
+// Harmonic sums of lm in [LO, LO + 8) over the tile's slots, last slot first:
+// S[j][n] = (S_n,LO+2j, S_n,LO+2j+1).
+template <class D, int LO>
+__device__ __forceinline__ void site_block_harmonics(const float* tile, float2 (&S)[4][D::NA])
+{
+    constexpr int row = kSiteChunk * 32;
+#pragma unroll 1
+    for (int s = kSiteChunk - 1; s >= 0; --s) {
+        const float* t = tile + s * 32;
+        const float x = t[0];
+        if (x > 1.5f) continue;  // kNoPair
+        const float y = t[row], z = t[2 * row];
+        float2 g[D::NA];
+#pragma unroll
+        for (int n = 0; n < D::NA; ++n) g[n] = bcast2(t[(3 + n) * row]);
+        float Y[8];
+        NEP_SH_LOCALS(x, y, z)
+#define NEP_T(lm, Yv, gx, gy, gz) \
+    if constexpr (lm >= LO && lm < LO + 8) Y[lm - LO] = Yv;
+        NEP_SH_TABLE(NEP_T)
+#undef NEP_T
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int n = 0; n < D::NA; ++n) S[j][n] = ffma2(make_float2(Y[2 * j], Y[2 * j + 1]), g[n], S[j][n]);
+    }
+}
+
+// The descriptors q_nl of order n from the harmonic sums in the lane's column
+// (compensated over m, as in site_descriptors)
+template <class D>
+__device__ __forceinline__ void site_block_descriptors(int n, const float* s_S, float* s_q)
+{
+    float q[kLmax] = {0.f, 0.f, 0.f, 0.f}, qc[kLmax] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int m = 0; m < kLM; ++m) {
+        const int l = sh_l(m);
+        const int f = 2 * ((m >> 1) * D::NA + n) + (m & 1);  // site_block_at
+        const float h = s_S[(f >> 2) * 128 + (f & 3)];
+        const float y = fmaf(sh_c(m) * h, h, -qc[l]);
+        const float t = q[l] + y;
+        qc[l] = (t - q[l]) - y;
+        q[l] = t;
+    }
+#pragma unroll
+    for (int l = 0; l < kLmax; ++l) s_q[(D::NR + n * kLmax + l) * 32] = q[l] - qc[l];
+}
+
+// A_nlm = 2 c_lm G_nl S_nlm in place, order n of the lane's column
+template <class D>
+__device__ __forceinline__ void site_block_coefficients(int n, float* s_A, const float* s_G)
+{
+    float g[kLmax];
+#pragma unroll
+    for (int l = 0; l < kLmax; ++l) g[l] = s_G[(D::NR + n * kLmax + l) * 32];
+#pragma unroll
+    for (int m = 0; m < kLM; ++m) {
+        const int f = 2 * ((m >> 1) * D::NA + n) + (m & 1);  // site_block_at
+        float* a = s_A + (f >> 2) * 128 + (f & 3);
+        *a = *a * (2.f * sh_c(m) * g[sh_l(m)]);
+    }
+}
+
+// What a pair's partial force needs of its geometry: the distance and its
+// square, the unit vector u and 1/|r|, and for the energy correction what
+// rounding left out of d (dd) and of u (du); w the pair's weight.
+struct PairGeom {
+    float u[3], d, d2, inv, dd, du[3], w;
+};
+
+__device__ __forceinline__ void site_pair_geometry(int v, const float* __restrict__ xh, const float* __restrict__ xl,
+                                                   const Box& box, const SiteParams& P, const float (&hi)[3],
+                                                   const float (&li)[3], float zi, PairGeom& g)
+{
+    const int j = v & 0xFFFFFF;
+    float hj[3], lj[3], r[3], r_lo[3], u_res[3], dres;
+    load_pos(xh, xl, 0, j, hj, lj);
+    pair_vector_lo(v >> 24, hi, li, hj, lj, box, r, r_lo);
+    g.d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
+    g.d = sqrtf(g.d2);
+    unit_vector_res(r[0], r[1], r[2], g.d, g.u[0], g.u[1], g.u[2], u_res, dres, g.inv);
+    const float ur = fmaf(g.u[0], r_lo[0], fmaf(g.u[1], r_lo[1], g.u[2] * r_lo[2]));
+    g.dd = dres + ur;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) g.du[a] = fmaf(fmaf(-g.u[a], ur, r_lo[a]), g.inv, u_res[a]);
+    g.w = pair_weight(P, zi, load_z(xh, j));
+}
+
+// radial part of dU/dd (0 beyond the radial cutoff); s_G: the lane's column of G
+template <class D>
+__device__ __forceinline__ float site_pair_radial(const PairGeom& g, const SiteParams& P, const float* s_G)
+{
+    float radial = 0.f;
+    if (g.d2 < P.rcR2) {
+        float2 gd[D::NR];
+        radial_gd<D::NR>(g.d, P.rcR, P.inv_rcR, gd, g.w);
+#pragma unroll
+        for (int a = 0; a < D::NR; ++a) radial = fmaf(s_G[a * 32], gd[a].y, radial);
+    }
+    return radial;
+}
+
+// Angular terms of one pair against the atom's coefficients (the sums of
+// sh_pass2): (cg, cd) = sum_n A_nlm (g_n, g_n'), B += cd Y, V += cg grad_u Y,
+// two harmonics per packed FMA.  Gradient components that are zero for every
+// direction (a third of them) are left out.  gg, gp: (g_n, g_n), (g_n', g_n').
+template <class D, int J>
+__device__ __forceinline__ void site_angular_terms(const float* s_A, const ShFast& sh, const float2 (&gg)[D::NA],
+                                                   const float2 (&gp)[D::NA], float& B, float (&V)[3])
+{
+    if constexpr (J < kLM / 2) {
+        float2 cg = make_float2(0.f, 0.f), cd = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int n = 0; n < D::NA; ++n) {
+            const float2 A = *reinterpret_cast<const float2*>(s_A + site_block_at<D>(n, 2 * J));
+            cg = ffma2(A, gg[n], cg);
+            cd = ffma2(A, gp[n], cd);
+        }
+        sh_add<2 * J>(sh, cg.x, cd.x, B, V);
+        sh_add<2 * J + 1>(sh, cg.y, cd.y, B, V);
+        site_angular_terms<D, J + 1>(s_A, sh, gg, gp, B, V);
+    }
+}
+
+// The site pass of the block's atoms.  z: the parameters; pf: partial-force
+// records [k][n] float4; mask: in-cutoff bits [3][n] of the first 96 slots,
+// or NULL.  Warp 0 returns the site energies (hi + lo).
+template <class D, int WORDS>
+__device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, const int* __restrict__ nbr,
+                                           const float* __restrict__ xh, const float* __restrict__ xl, const Box& box,
+                                           const float* __restrict__ z, int n_par, SiteParams P,
+                                           float* __restrict__ pf, unsigned* __restrict__ mask, float& U_hi,
+                                           float& U_lo)
+{
+    constexpr int NR = D::NR, NA = D::NA, ND = D::Ndes;
+    extern __shared__ __align__(16) float s_site[];
+    __shared__ float s_dU[kSiteWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* s_w = s_site;
+    float* s_A = s_w + (n_par + 31) / 32 * 32;         // [quads][32] float4
+    float* s_q = s_A + 128 * site_block_quads<D>();    // [ND][32]
+    float* s_x = s_q + 32 * ND;                        // radial tile; then x_mu, w2 (1 - x_mu^2): [n_neu][32][2]
+    unsigned* s_mask = reinterpret_cast<unsigned*>(s_x + 64 * (P.n_neu > kSiteChunk ? P.n_neu : kSiteChunk));
+    for (int t = threadIdx.x; t < n_par; t += kSiteThreads) s_w[t] = z[t];
+    if (threadIdx.x < 96) s_mask[threadIdx.x] = 0u;
+    P.w = s_w;
+    const int ia = active ? i : 0;
+    float hi[3], li[3];
+    load_pos(xh, xl, n, ia, hi, li);
+    const float zi = load_z(xh, ia);
+    const int kmax = __reduce_max_sync(0xffffffffu, cnt);  // the same in every warp
+    const int chunks = (kmax + kSiteChunk - 1) / kSiteChunk;
+    const float rc2max = P.rcR2 > P.rcA2 ? P.rcR2 : P.rcA2;
+
+    // own slots k = 4 b + warp: bit b of word b / 32 in kept (within either
+    // cutoff) and ang (within the angular one)
+    unsigned kept[WORDS], ang[WORDS];
+#pragma unroll
+    for (int w = 0; w < WORDS; ++w) kept[w] = ang[w] = 0u;
+
+    // ---- descriptor sums, 16 slots at a time, the farthest first
+    {
+        // this warp's sums: harmonics 8 warp .. 8 warp + 7 (warps 0-2), or the
+        // radial orders in pairs with their negated compensations (warp 3)
+        constexpr int NR2 = (NR + 1) / 2;
+        static_assert(2 * NR2 <= 4 * NA, "the radial sums fit the harmonic sums' registers");
+        float2 S[4][NA];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int a = 0; a < NA; ++a) S[j][a] = make_float2(0.f, 0.f);
+        float* tile = s_A + lane;
+        float2* tileR = reinterpret_cast<float2*>(s_x) + lane;
+        int v_nx = 0;
+        auto load_slot = [&](int k) { return k < cnt ? nbr[(size_t)k * n + ia] : 0; };
+        if (chunks > 0) v_nx = load_slot((chunks - 1) * kSiteChunk + warp);
+#pragma unroll 1
+        for (int c = chunks - 1; c >= 0; --c) {
+#pragma unroll 1
+            for (int t = 0; t < kSiteChunk / kSiteWarps; ++t) {
+                const int s = 4 * t + warp, k = c * kSiteChunk + s;
+                const int v = v_nx;
+                v_nx = t < kSiteChunk / kSiteWarps - 1 ? load_slot(k + 4) : (c > 0 ? load_slot(k - 28) : 0);
+                float x = kNoPair, fc = 0.f, ux = kNoPair;
+                if (k < cnt) {
+                    const int j = v & 0xFFFFFF;
+                    float hj[3], lj[3], rx, ry, rz;
+                    load_pos(xh, xl, n, j, hj, lj);
+                    pair_vector(v >> 24, hi, li, hj, lj, box, rx, ry, rz);
+                    const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+                    if (d2 < rc2max) {
+                        const int b = 4 * c + t;
+                        const float w = pair_weight(P, zi, load_z(xh, j));
+                        const float d = sqrtf(d2);
+#pragma unroll
+                        for (int q = 0; q < WORDS; ++q)
+                            if (WORDS == 1 || (b >> 5) == q) kept[q] |= 1u << (b & 31);
+                        if (d2 < P.rcR2) radial_x(d, P.rcR, P.inv_rcR, w, x, fc);
+                        if (d2 < P.rcA2) {
+#pragma unroll
+                            for (int q = 0; q < WORDS; ++q)
+                                if (WORDS == 1 || (b >> 5) == q) ang[q] |= 1u << (b & 31);
+                            float g[NA], uy, uz;
+                            radial_g<NA>(d, P.rcA, P.inv_rcA, g, w);
+                            unit_vector(rx, ry, rz, ux, uy, uz);
+                            tile[(kSiteChunk + s) * 32] = uy;
+                            tile[(2 * kSiteChunk + s) * 32] = uz;
+#pragma unroll
+                            for (int a = 0; a < NA; ++a) tile[((3 + a) * kSiteChunk + s) * 32] = g[a];
+                        }
+                    }
+                }
+                tile[s * 32] = ux;
+                tileR[s * 32] = make_float2(x, fc);
+            }
+            __syncthreads();
+            if (warp == 0) {
+                site_block_harmonics<D, 0>(tile, S);
+            } else if (warp == 1) {
+                site_block_harmonics<D, 8>(tile, S);
+            } else if (warp == 2) {
+                site_block_harmonics<D, 16>(tile, S);
+            } else {
+                const float2 minus = make_float2(-1.f, -1.f);
+#pragma unroll 1
+                for (int s = kSiteChunk - 1; s >= 0; --s) {
+                    const float2 xf = tileR[s * 32];
+                    if (xf.x > 1.5f) continue;  // kNoPair
+                    float g[NR];
+                    cheb_g<NR>(xf.x, xf.y, g);
+                    // Kahan: y = g - c, t = R + y, c = (t - R) - y with -c kept
+#pragma unroll
+                    for (int p = 0; p < NR2; ++p) {
+                        float2& R = S[(2 * p) / NA][(2 * p) % NA];
+                        float2& nc = S[(2 * p + 1) / NA][(2 * p + 1) % NA];
+                        const float2 y = fadd2(make_float2(g[2 * p], 2 * p + 1 < NR ? g[2 * p + 1] : 0.f), nc);
+                        const float2 t = fadd2(R, y);
+                        nc = fadd2(y, ffma2(t, minus, R));
+                        R = t;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        if (warp < 3) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int a = 0; a < NA; ++a) {
+                    const int f = 2 * (j * NA + a);  // site_block_at<D>(a, 8 warp + 2 j)
+                    *reinterpret_cast<float2*>(s_A + (warp * 2 * NA + (f >> 2)) * 128 + 4 * lane + (f & 3)) = S[j][a];
+                }
+        } else {
+#pragma unroll
+            for (int a = 0; a < NR; ++a) {
+                const float2 R = S[(a & ~1) / NA][(a & ~1) % NA], nc = S[(a | 1) / NA][(a | 1) % NA];
+                s_q[a * 32 + lane] = (a & 1) ? R.y + nc.y : R.x + nc.x;
+            }
+        }
+        if (mask) {
+            // own bits b of word j (slots 32 j + 4 (b - 8 j) + warp)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                unsigned e = (kept[0] >> (8 * j)) & 0xFFu;
+                e = (e | (e << 12)) & 0x000F000Fu;
+                e = (e | (e << 6)) & 0x03030303u;
+                e = (e | (e << 3)) & 0x11111111u;
+                if (e) atomicOr(s_mask + 32 * j + lane, e << warp);
+            }
+        }
+    }
+    __syncthreads();
+    for (int a = warp; a < NA; a += kSiteWarps) site_block_descriptors<D>(a, s_A + 4 * lane, s_q + lane);
+    if (mask && warp < 3 && active) mask[(size_t)warp * n + i] = s_mask[32 * warp + lane];
+    __syncthreads();
+
+    // ---- network: neurons mu = warp mod 4
+    const float* b1 = s_w + P.n_neu * ND;
+    const float* w2 = b1 + P.n_neu;
+    float2* s_xd = reinterpret_cast<float2*>(s_x) + lane;
+    {
+        float q[ND];
+#pragma unroll
+        for (int a = 0; a < ND; ++a) q[a] = s_q[a * 32 + lane];
+#pragma unroll 1
+        for (int mu = warp; mu < P.n_neu; mu += kSiteWarps) {
+            const float x = neuron_state<ND>(s_w + mu * ND, b1[mu], q);
+            s_xd[mu * 32] = make_float2(x, w2[mu] * fmaf(-x, x, 1.f));
+        }
+    }
+    __syncthreads();
+    {
+        // G_v of a quarter of the descriptors, in s_q
+        constexpr int VB = (ND + kSiteWarps - 1) / kSiteWarps;
+        const int v0 = warp * VB;
+        if constexpr (ND % (4 * kSiteWarps) == 0) {  // 16-byte aligned quarters
+            float2 G[VB / 2];
+#pragma unroll
+            for (int v = 0; v < VB / 2; ++v) G[v] = make_float2(0.f, 0.f);
+#pragma unroll 2
+            for (int mu = 0; mu < P.n_neu; ++mu) {
+                const float2 d = bcast2(s_xd[mu * 32].y);
+                const float4* row = reinterpret_cast<const float4*>(s_w + mu * ND + v0);
+#pragma unroll
+                for (int v = 0; v < VB / 4; ++v) {
+                    const float4 t = row[v];
+                    G[2 * v] = ffma2(d, make_float2(t.x, t.y), G[2 * v]);
+                    G[2 * v + 1] = ffma2(d, make_float2(t.z, t.w), G[2 * v + 1]);
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < VB / 2; ++v) {
+                s_q[(v0 + 2 * v) * 32 + lane] = G[v].x;
+                s_q[(v0 + 2 * v + 1) * 32 + lane] = G[v].y;
+            }
+        } else {
+            float G[VB];
+#pragma unroll
+            for (int v = 0; v < VB; ++v) G[v] = 0.f;
+#pragma unroll 1
+            for (int mu = 0; mu < P.n_neu; ++mu) {
+                const float d = s_xd[mu * 32].y;
+                const float* row = s_w + mu * ND + v0;
+#pragma unroll
+                for (int v = 0; v < VB; ++v)
+                    if (v0 + v < ND) G[v] = fmaf(d, row[v], G[v]);
+            }
+#pragma unroll
+            for (int v = 0; v < VB; ++v)
+                if (v0 + v < ND) s_q[(v0 + v) * 32 + lane] = G[v];
+        }
+    }
+    __syncthreads();
+
+    // ---- coefficients A (warps 1-3) and the compensated output sum (warp 0)
+    if (warp == 0) {
+        float s = 0.f, c = 0.f;
+        for (int mu = 0; mu < P.n_neu; ++mu) neuron_energy(w2[mu], s_xd[mu * 32].x, s, c);
+        float t, e;
+        two_sum(s, -w2[P.n_neu], t, e);
+        U_hi = t;
+        U_lo = c + e;
+    } else {
+        for (int a = warp - 1; a < NA; a += kSiteWarps - 1) site_block_coefficients<D>(a, s_A + 4 * lane, s_q + lane);
+    }
+    __syncthreads();
+
+    // ---- partial forces of the own slots, and the first-order energy
+    // correction of the pair geometry's roundings (nep_site.cuh)
+    float dU = 0.f;
+    const float* sA = s_A + 4 * lane;
+    const float* sG = s_q + lane;
+    float4* out = reinterpret_cast<float4*>(pf) + ia;
+#pragma unroll
+    for (int w = 0; w < WORDS; ++w) {
+        unsigned rest = kept[w];
+#pragma unroll 1
+        while (rest) {
+            // the angular pairs first, then those beyond the angular cutoff
+            const bool angular = ang[w] != 0u;
+            const int b = __ffs((int)(angular ? ang[w] : rest)) - 1;
+            ang[w] &= ~(1u << b);
+            rest &= ~(1u << b);
+            const int k = 4 * (32 * w + b) + warp;
+            PairGeom g;
+            site_pair_geometry(nbr[(size_t)k * n + ia], xh, xl, box, P, hi, li, zi, g);
+            float radial = site_pair_radial<D>(g, P, sG);
+            float V[3] = {0.f, 0.f, 0.f};
+            float eu = 0.f;
+            if (angular) {
+                float2 gg[NA], gp[NA];
+                {
+                    float2 gd[NA];
+                    radial_gd<NA>(g.d, P.rcA, P.inv_rcA, gd, g.w);
+#pragma unroll
+                    for (int a = 0; a < NA; ++a) {
+                        gg[a] = bcast2(gd[a].x);
+                        gp[a] = bcast2(gd[a].y);
+                    }
+                }
+                ShFast sh;
+                sh.set(g.u[0], g.u[1], g.u[2]);
+                site_angular_terms<D, 0>(sA, sh, gg, gp, radial, V);
+                eu = fmaf(V[0], g.du[0], fmaf(V[1], g.du[1], V[2] * g.du[2]));
+                // tangential projection of V, divided by r
+                const float uv = fmaf(g.u[0], V[0], fmaf(g.u[1], V[1], g.u[2] * V[2]));
+#pragma unroll
+                for (int a = 0; a < 3; ++a) V[a] = (V[a] - uv * g.u[a]) * g.inv;
+            }
+            dU += fmaf(radial, g.dd, eu);
+            out[(size_t)k * n] = make_float4(fmaf(radial, g.u[0], V[0]), fmaf(radial, g.u[1], V[1]),
+                                             fmaf(radial, g.u[2], V[2]), 0.f);
+        }
+    }
+    s_dU[warp][lane] = dU;
+    __syncthreads();
+    if (warp == 0) U_lo += (s_dU[0][lane] + s_dU[1][lane]) + (s_dU[2][lane] + s_dU[3][lane]);
+}
+
+}  // namespace nep

@@ -99,7 +99,7 @@ __global__ void k_ds_list(int N, const int* __restrict__ sid, const int* __restr
                     const int code = image_code(sx, sy, sz);
                     if (j == i && code == kImgCenter) continue;
                     float rx, ry, rz;
-                    pair_vector(i, j, code, hi, li, hj, lj, b, rx, ry, rz);
+                    pair_vector(code, hi, li, hj, lj, b, rx, ry, rz);
                     const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
                     if (d2 < rc2) {
                         if (c < kDsCap) tmp[(size_t)i * kDsCap + c] = j | (code << 24);
@@ -135,7 +135,7 @@ __global__ void k_ds_sort(int N, const int* __restrict__ sid, const Box* __restr
         float hj[3], lj[3];
         load_pos(xh, xl, N, j, hj, lj);
         float rx, ry, rz;
-        pair_vector(i, j, v >> 24, hi, li, hj, lj, b, rx, ry, rz);
+        pair_vector(v >> 24, hi, li, hj, lj, b, rx, ry, rz);
         key[t] = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
     }
     // insertion sort (stable): only entries with a strictly larger key move
@@ -172,7 +172,7 @@ __global__ void k_ds_compact(int N, const int* __restrict__ tmp, const long long
         float hj[3], lj[3];
         load_pos(xh, xl, N, j, hj, lj);
         float rx, ry, rz;
-        pair_vector(i, j, v >> 24, hi, li, hj, lj, b, rx, ry, rz);
+        pair_vector(v >> 24, hi, li, hj, lj, b, rx, ry, rz);
         const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
         aidx[p] = d2 < rcA2 ? a++ : -1;
     }
@@ -230,7 +230,7 @@ __global__ void k_ds_site(int N, const int* __restrict__ sid, const Box* __restr
         float hj[3], lj[3];
         load_pos(xh, xl, N, j, hj, lj);
         float rx, ry, rz;
-        pair_vector(i, j, v >> 24, hi, li, hj, lj, b, rx, ry, rz);
+        pair_vector(v >> 24, hi, li, hj, lj, b, rx, ry, rz);
         const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
         const float d = sqrtf(d2);
         const float wz = typed ? sqrtf(zi * load_z(xh, j)) : 1.f;
@@ -273,7 +273,7 @@ __global__ void k_ds_site(int N, const int* __restrict__ sid, const Box* __restr
         float hj[3], lj[3];
         load_pos(xh, xl, N, j, hj, lj);
         float r[3];
-        pair_vector(i, j, v >> 24, hi, li, hj, lj, b, r[0], r[1], r[2]);
+        pair_vector(v >> 24, hi, li, hj, lj, b, r[0], r[1], r[2]);
         const float d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
         const float d = sqrtf(d2);
         const float inv = 1.f / d;

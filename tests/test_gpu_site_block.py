@@ -1,0 +1,38 @@
+"""The site pass works on 32 atoms per block, 16 list slots per shared tile
+and 32 own slots per word and thread: atom counts around the block, slot
+counts around the tile and every capacity class against the oracle, at the
+bars of the force path (1e-6 eV, 1e-4 eV/A)."""
+import numpy as np
+import pytest
+
+from gpu_util import aos, f32_exact, soa, virial_aos
+from paper_2107_08119_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,edge,capacity,n_neu", [
+    (1, 5.43, 96, 30),      # no neighbour: no tile at all
+    (31, 5.43, 96, 30),
+    (32, 5.43, 16, 30),     # clusters of few neighbours
+    (33, 5.43, 96, 1),      # fewer neurons than warps
+    (65, 4.6, 96, 7),
+    (512, 4.3, 128, 30),    # 60 neighbours; the last capacity of one word per thread
+    (512, 4.3, 129, 30),    # three words, no in-cutoff masks
+    (500, 4.0, 384, 64),
+])
+def test_block_edges(orc, n, edge, capacity, n_neu):
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(n + capacity)
+    pos, box = inputs.diamond(4, 4, 4, edge)
+    pos = inputs.displace(pos, 0.1, rng)[:n]
+    hyper = nep.Hyper(max_neighbors=capacity, n_neu=n_neu)
+    z = inputs.random_z(hyper.n_par, rng)
+    model = nep.NEP(z, hyper)
+    out = model.compute(soa(pos), box)
+    U, F, W = orc.efv(orc.NepHyper(n_neu=n_neu), f32_exact(z), pos, box)
+    assert np.abs(out["e_atom"].cpu().numpy() - U).max() <= 1e-6 * max(1.0, n_neu / 30)
+    assert np.abs(aos(out["force"]) - F).max() <= 1e-4
+    assert np.abs(virial_aos(out["virial_atom"]) - W).max() <= 1e-4
+    assert abs(out["e_total"].item() - U.sum()) <= 1e-6 * n * max(1.0, n_neu / 30)
+    model.close()
