@@ -59,7 +59,7 @@ __device__ __forceinline__ void load_params(const float* __restrict__ z, int n_p
 
 __global__ void __launch_bounds__(kAdjThreads) k_adj_site(int N, const int* __restrict__ sid,
                                                           const Box* __restrict__ boxes,
-                                                          const float* __restrict__ xh, const float* __restrict__ xl,
+                                                          const float* __restrict__ xr,
                                                           const long long* __restrict__ pstart,
                                                           const int* __restrict__ pj, const float* __restrict__ z,
                                                           int n_par, SiteParams P, float* __restrict__ pf,
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_site(int N, const int* __re
     const SlotTable T{pj + p0, 1, 0};
     const PfOut out{pf + 3 * p0, 3, 1};
     float uh, ul;
-    site_partial_forces(ia, active, N, cnt, T, xh, xl, box, P, out, uh, ul);
+    site_partial_forces(ia, active, N, cnt, T, xr, box, P, out, uh, ul);
     if (active && !isfinite(uh)) atomicOr(err, kErrNonFinite);
 }
 
@@ -148,8 +148,7 @@ __device__ __forceinline__ void adj_pass(float x, float y, float z, const Harm& 
 
 __global__ void __launch_bounds__(kAdjThreads) k_adj_lambda(int N, const int* __restrict__ sid,
                                                             const Box* __restrict__ boxes,
-                                                            const float* __restrict__ xh,
-                                                            const float* __restrict__ xl,
+                                                            const float* __restrict__ xr,
                                                             const long long* __restrict__ pstart,
                                                             const int* __restrict__ pj,
                                                             const float4* __restrict__ res,
@@ -177,13 +176,13 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_lambda(int N, const int* __
     const float scale = L > 0.0 ? (float)(1.0 / (3.0 * (double)N * L)) : 0.f;
 
     float hi[3], li[3];
-    load_pos(xh, xl, N, ia, hi, li);
-    const float zi = load_z(xh, ia);
+    load_pos(xr, ia, hi, li);
+    const float zi = load_z(xr, ia);
     float lam[kNdes];
     {
         float q[kNdes];
         Harm S;
-        site_descriptors(ia, N, cnt, T, xh, xl, box, P, hi, li, zi, q, S);
+        site_descriptors(ia, N, cnt, T, xr, box, P, hi, li, zi, q, S);
 #pragma unroll
         for (int v = 0; v < kNdes; ++v) row[kNdes + v] = q[v];
         // A_nlm = 2 c_lm S_nlm
@@ -199,7 +198,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_lambda(int N, const int* __
             const int v = pj[p0 + k];
             const int j = v & 0xFFFFFF;
             float hj[3], lj[3];
-            load_pos(xh, xl, N, j, hj, lj);
+            load_pos(xr, j, hj, lj);
             const float4 ej = res[j];
             float r[3];
             pair_vector(v >> 24, hi, li, hj, lj, box, r[0], r[1], r[2]);
@@ -209,7 +208,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_lambda(int N, const int* __
             const float inv = 1.f / d;
             const float u[3] = {r[0] * inv, r[1] * inv, r[2] * inv};
             const float e = fmaf(u[0], dd[0], fmaf(u[1], dd[1], u[2] * dd[2]));
-            const float wz = pair_weight(P, zi, load_z(xh, j));
+            const float wz = pair_weight(P, zi, load_z(xr, j));
             if (d2 < P.rcR2) {
                 float g[kNR], dg[kNR];
                 radial_g_dg<kNR>(d, P.rcR, P.inv_rcR, g, dg, wz);
@@ -367,7 +366,7 @@ int nep_force_loss(nep_model* m, nep_dataset* ds, const float* z, double* loss_f
                    "nep_force_loss: parameter copy");
     if (rc) return rc;
     const size_t smem = (size_t)pad32(n_par) * sizeof(float);
-    k_adj_site<<<nb, kAdjThreads, smem, st>>>(N, ds->sid, ds->boxes, ds->xh, ds->xl, ds->pstart, ds->pj, a.z, n_par,
+    k_adj_site<<<nb, kAdjThreads, smem, st>>>(N, ds->sid, ds->boxes, ds->xr, ds->pstart, ds->pj, a.z, n_par,
                                               site_params(m, ds->typed), a.pf, m->d_err);
     k_adj_force<<<nb, kAdjThreads, 0, st>>>(N, ds->pstart, ds->rev, a.pf, ds->f_tar, reinterpret_cast<float4*>(a.res),
                                             a.part, m->d_err);
@@ -395,7 +394,7 @@ int nep_force_loss_backward(nep_model* m, nep_dataset* ds, const double* seed, d
     int rc = cuda_fail(cudaFuncSetAttribute(k_adj_lambda, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                        "adjoint kernel shared memory");
     if (rc) return rc;
-    k_adj_lambda<<<nb, kAdjThreads, smem, st>>>(N, ds->sid, ds->boxes, ds->xh, ds->xl, ds->pstart, ds->pj,
+    k_adj_lambda<<<nb, kAdjThreads, smem, st>>>(N, ds->sid, ds->boxes, ds->xr, ds->pstart, ds->pj,
                                                 reinterpret_cast<const float4*>(a.res), a.sums, a.z, n_par,
                                                 site_params(m, ds->typed), a.part);
     k_adj_grad<<<blocks_for(n_par, 256), 256, 0, st>>>(nb, n_par, a.part, seed, grad);

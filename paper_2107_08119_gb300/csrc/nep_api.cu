@@ -170,8 +170,7 @@ int ensure_workspace(Workspace& ws, int n, int m_cap, int ncell, int nblocks_par
         dev_free(nl.rev);
         dev_free(nl.vala);
         dev_free(nl.pf);
-        dev_free(nl.xh);
-        dev_free(nl.xl);
+        dev_free(nl.xr);
         dev_free(nl.atom_cell);
         dev_free(nl.cell_atoms);
         dev_free(nl.mask);
@@ -182,8 +181,8 @@ int ensure_workspace(Workspace& ws, int n, int m_cap, int ncell, int nblocks_par
         if ((rc = dev_alloc(&nl.count, N, "neighbour counts")) || (rc = dev_alloc(&nl.nbr, N * M, "neighbour list")) ||
             (rc = dev_alloc(&nl.rev, N * M, "reverse pair index")) ||
             (rc = dev_alloc(&nl.vala, N * M, "neighbour list copy")) ||
-            (rc = dev_alloc(&nl.pf, N * M * 4, "partial forces")) || (rc = dev_alloc(&nl.xh, N * 4, "positions")) ||
-            (rc = dev_alloc(&nl.xl, N * 4, "positions")) || (rc = dev_alloc(&nl.atom_cell, N, "cell index")) ||
+            (rc = dev_alloc(&nl.pf, N * M * 4, "partial forces")) || (rc = dev_alloc(&nl.xr, N * 8, "positions")) ||
+            (rc = dev_alloc(&nl.atom_cell, N, "cell index")) ||
             (rc = dev_alloc(&nl.cell_atoms, N, "cell atoms")) || (rc = dev_alloc(&nl.mask, N * 3, "slot masks")) ||
             (rc = dev_alloc(&ws.force, N * 3, "forces")))
             return rc;
@@ -224,8 +223,7 @@ void free_workspace(Workspace& ws)
     dev_free(nl.rev);
     dev_free(nl.vala);
     dev_free(nl.pf);
-    dev_free(nl.xh);
-    dev_free(nl.xl);
+    dev_free(nl.xr);
     dev_free(nl.atom_cell);
     dev_free(nl.cell_count);
     dev_free(nl.cell_start);

@@ -71,8 +71,7 @@ struct nep_dataset {
     int* chunk_begin = nullptr;
     int* chunk_end = nullptr;
     float* q = nullptr;
-    float* xh = nullptr;  // FP32 hi/lo wrapped positions (float4 records), kept for the adjoint
-    float* xl = nullptr;
+    float* xr = nullptr;  // FP32 hi/lo wrapped positions (records of load_pos), kept for the adjoint
     float* B = nullptr;
     long long* pstart = nullptr;
     int* pj = nullptr;

@@ -27,8 +27,7 @@ constexpr int kMaskSlots = 96;  // slots per atom covered by the in-cutoff mask 
 // atom, 3 the largest capacity).
 template <class D, int WORDS>
 __global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, const int* __restrict__ count,
-                                                          const int* __restrict__ nbr, const float* __restrict__ xh,
-                                                          const float* __restrict__ xl, Box box,
+                                                          const int* __restrict__ nbr, const float* __restrict__ xr, Box box,
                                                           const float* __restrict__ z, int n_par, SiteParams P,
                                                           float* __restrict__ pf, double* __restrict__ e_atom,
                                                           double* __restrict__ e_partials, unsigned* err,
@@ -40,7 +39,7 @@ __global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, cons
     const bool active = i < n;
     const int cnt = active ? min(count[i], m_cap) : 0;
     float uh, ul;
-    site_block<D, WORDS>(i, active, n, cnt, nbr, xh, xl, box, z, n_par, P, pf, mask, uh, ul);
+    site_block<D, WORDS>(i, active, n, cnt, nbr, xr, box, z, n_par, P, pf, mask, uh, ul);
     if (warp != 0) return;  // warp 0 holds the site energies
     double e = 0.0;
     if (active) {
@@ -57,7 +56,7 @@ __global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, cons
 template <bool MD>
 __global__ void __launch_bounds__(kAsmThreads) k_assemble(int n, int m_cap, float rc2max, const int* __restrict__ count,
                                                           const int* __restrict__ nbr, const int* __restrict__ rev,
-                                                          const float* __restrict__ xh, const float* __restrict__ xl,
+                                                          const float* __restrict__ xr,
                                                           Box box, const float* __restrict__ pf,
                                                           float* __restrict__ force, float* __restrict__ virial_atom,
                                                           double* __restrict__ partials, unsigned* err,
@@ -74,7 +73,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_assemble(int n, int m_cap, floa
         // memory (as the site pass does) cost this pass occupancy and time
         const SlotTable T{nbr, n, i};
         float F[3], W[9];
-        assemble_atom(i, n, m_cap, rc2max, count, T, rev, xh, xl, box, pf, F, W, mask);
+        assemble_atom(i, n, m_cap, rc2max, count, T, rev, xr, box, pf, F, W, mask);
         if (!(isfinite(F[0]) && isfinite(F[1]) && isfinite(F[2]))) atomicOr(err, kErrNonFinite);
         if (force) {
             force[i] = F[0];
@@ -146,7 +145,7 @@ int launch_site(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, dou
                                             cudaSharedmemCarveoutMaxShared), "site kernel shared memory");
     if (rc) return rc;
     nl.mask_set = nl.m_cap <= kMaskSlots && nl.mask != nullptr;
-    kern<<<nblocks, kSiteThreads, smem, st>>>(n, nl.m_cap, nl.count, nl.nbr, nl.xh, nl.xl, a.box, a.z, n_par, P, nl.pf,
+    kern<<<nblocks, kSiteThreads, smem, st>>>(n, nl.m_cap, nl.count, nl.nbr, nl.xr, a.box, a.z, n_par, P, nl.pf,
                                               e_atom, e_partials, d_err, nl.mask_set ? nl.mask : nullptr);
     return cuda_fail(cudaGetLastError(), "site kernel");
 }
@@ -173,7 +172,7 @@ int launch_assemble(const AssembleArgs& a, NeighborList& nl, int n, float* force
     const bool md = a.vel != nullptr;
     ncomp = md ? 13 : 9;
     auto kern = md ? k_assemble<true> : k_assemble<false>;
-    kern<<<nblocks, kAsmThreads, 0, st>>>(n, nl.m_cap, rc2, nl.count, nl.nbr, nl.rev, nl.xh, nl.xl, a.box, nl.pf,
+    kern<<<nblocks, kAsmThreads, 0, st>>>(n, nl.m_cap, rc2, nl.count, nl.nbr, nl.rev, nl.xr, a.box, nl.pf,
                                           force, virial_atom, partials, d_err, md ? a.vel : nullptr,
                                           md ? a.half_dt_over_m : 0.0, md ? a.ke_factor : 0.0,
                                           nl.mask_set ? nl.mask : nullptr);

@@ -1,7 +1,7 @@
 // nep_internal.cuh -- shared definitions of the sm_103a NEP library.
 //
 // Data layout in device memory (n atoms, M = neighbour capacity per atom):
-//   positions        FP64 [3][n] (caller) + FP32 hi/lo split xh, xl [n] float4
+//   positions        FP64 [3][n] (caller) + FP32 hi/lo records xr [n][8]
 //   neighbour list   int32 nbr[M][n] = j | image_code << 24, count[n]
 //                    int32 rev[M][n] = slot of i in j's list (reverse pair)
 //                    int32 vala[n][M]: scratch of the list build (the rank of
@@ -166,22 +166,42 @@ __host__ __device__ __forceinline__ void pair_vector_lo(int code, const float (&
     for (int d = 0; d < 3; ++d) r[d] = diff1_lo(hj[d], lj[d], hi[d], li[d], (float)s[d], b.Lh[d], b.Ll[d], r_lo[d]);
 }
 
-// FP32 hi/lo positions are stored as one float4 record (x, y, z, 0) per atom
-// for each part, so a neighbour's coordinates arrive in two 16-byte loads.
-__host__ __device__ __forceinline__ void load_pos(const float* __restrict__ xh, const float* __restrict__ xl, int n, int i,
-                                         float (&h)[3], float (&l)[3])
+// FP32 hi/lo positions: one 32-byte record (x, y, z, species number; lo parts
+// x, y, z, 0) per atom, so that a neighbour's coordinates are one sector and
+// one 32-byte load (two 16-byte arrays before: two sectors; an MD step of the
+// 125,000-atom crystal 315 -> 309 us together with the site pass loading its
+// records a slot ahead).
+__host__ __device__ __forceinline__ void load_pos(const float* __restrict__ xr, int i, float (&h)[3], float (&l)[3],
+                                                  float& zi)
 {
-    (void)n;
-    const float4 a = NEP_LDG(reinterpret_cast<const float4*>(xh) + i);
-    const float4 b = NEP_LDG(reinterpret_cast<const float4*>(xl) + i);
-    h[0] = a.x;
-    h[1] = a.y;
-    h[2] = a.z;
-    l[0] = b.x;
-    l[1] = b.y;
-    l[2] = b.z;
+#ifdef __CUDA_ARCH__
+    float u, v;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(h[0]), "=f"(h[1]), "=f"(h[2]), "=f"(u), "=f"(l[0]), "=f"(l[1]), "=f"(l[2]), "=f"(v)
+        : "l"(xr + 8 * (size_t)i));
+    zi = u;
+    (void)v;
+#else
+    const float* r = xr + 8 * (size_t)i;
+    for (int d = 0; d < 3; ++d) {
+        h[d] = r[d];
+        l[d] = r[4 + d];
+    }
+    zi = r[3];
+#endif
 }
 
+__host__ __device__ __forceinline__ void load_pos(const float* __restrict__ xr, int i, float (&h)[3], float (&l)[3])
+{
+    float zi;
+    load_pos(xr, i, h, l, zi);
+}
+
+// the hi part of the record (x, y, z, species number)
+__host__ __device__ __forceinline__ float4 load_hi(const float* __restrict__ xr, int i)
+{
+    return NEP_LDG(reinterpret_cast<const float4*>(xr) + 2 * (size_t)i);
+}
 
 // Split an FP64 value into FP32 hi + lo.
 __host__ __device__ __forceinline__ void split_hilo(double x, float& h, float& l)
@@ -190,20 +210,20 @@ __host__ __device__ __forceinline__ void split_hilo(double x, float& h, float& l
     l = (float)(x - (double)h);
 }
 
-// The hi record's fourth word carries the atom's species number Z (1 for a
+// The hi part's fourth word carries the atom's species number Z (1 for a
 // single species): the multicomponent weighting f_c -> f_c sqrt(Z_i Z_j).
-__host__ __device__ __forceinline__ void store_pos(float* __restrict__ xh, float* __restrict__ xl, int i, const double (&x)[3],
-                                                  float zi = 1.f)
+__host__ __device__ __forceinline__ void store_pos(float* __restrict__ xr, int i, const double (&x)[3], float zi = 1.f)
 {
     float h[3], l[3];
     for (int d = 0; d < 3; ++d) split_hilo(x[d], h[d], l[d]);
-    reinterpret_cast<float4*>(xh)[i] = make_float4(h[0], h[1], h[2], zi);
-    reinterpret_cast<float4*>(xl)[i] = make_float4(l[0], l[1], l[2], 0.f);
+    float4* r = reinterpret_cast<float4*>(xr) + 2 * (size_t)i;
+    r[0] = make_float4(h[0], h[1], h[2], zi);
+    r[1] = make_float4(l[0], l[1], l[2], 0.f);
 }
 
-__host__ __device__ __forceinline__ float load_z(const float* __restrict__ xh, int i)
+__host__ __device__ __forceinline__ float load_z(const float* __restrict__ xr, int i)
 {
-    return reinterpret_cast<const float4*>(xh)[i].w;
+    return reinterpret_cast<const float4*>(xr)[2 * (size_t)i].w;
 }
 
 // Warp sum of K <= 16 doubles held by every lane.  Each butterfly level keeps
@@ -288,8 +308,7 @@ struct NeighborList {
     int* rev = nullptr;
     int* vala = nullptr;     // list-build scratch [n][m_cap] (slot ranks, or values atom-major)
     float* pf = nullptr;
-    float* xh = nullptr;
-    float* xl = nullptr;
+    float* xr = nullptr;     // hi/lo position records [n][8]
     int* atom_cell = nullptr;
     int* cell_count = nullptr;
     int* cell_start = nullptr;

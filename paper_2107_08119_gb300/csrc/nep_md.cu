@@ -65,7 +65,7 @@ __device__ void decide(unsigned* ctl, float thresh2, unsigned long long* rebuild
 }
 
 __global__ void k_kick_drift(int n, double* __restrict__ x, double* __restrict__ v, const float* __restrict__ F,
-                             double hdtm, double dt, float* __restrict__ xh, float* __restrict__ xl,
+                             double hdtm, double dt, float* __restrict__ xr,
                              const double* __restrict__ x_ref, unsigned* __restrict__ ctl, float thresh2,
                              unsigned long long* __restrict__ rebuilds, cudaGraphConditionalHandle cond, int use_cond)
 {
@@ -84,7 +84,7 @@ __global__ void k_kick_drift(int n, double* __restrict__ x, double* __restrict__
             const double d = xc - x_ref[o];
             dd += d * d;
         }
-        store_pos(xh, xl, i, xn, load_z(xh, i));  // the species number stays
+        store_pos(xr, i, xn, load_z(xr, i));  // the species number stays
         d2 = (float)dd;
     }
     // block maximum, then one atomic per block (one per warp serialised
@@ -783,7 +783,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
     // rebuild, then forces, second half kick and the step's sums
     auto head = [&](cudaStream_t q, bool use_cond, cudaGraphConditionalHandle cond) {
         Profiler::Slot* pk = m->prof.begin(NEP_PROFILE_STEP, q);
-        k_kick_drift<<<blocks_for(n, 256), 256, 0, q>>>(n, pos, vel, md->ws.force, hdtm, dt, nl.xh, nl.xl, md->x_ref,
+        k_kick_drift<<<blocks_for(n, 256), 256, 0, q>>>(n, pos, vel, md->ws.force, hdtm, dt, nl.xr, md->x_ref,
                                                         md->ctl, thresh * thresh, md->rebuilds, cond,
                                                         use_cond ? 1 : 0);
         m->prof.end(pk, q);

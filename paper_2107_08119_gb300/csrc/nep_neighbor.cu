@@ -37,7 +37,7 @@ __device__ __forceinline__ bool gated_off(const unsigned* gate)
 // A non-finite coordinate latches kErrNonFinite: such an atom would
 // otherwise be binned into a clamped cell and simply see no neighbours.
 __global__ void k_bin(int n, double* __restrict__ pos, const float* __restrict__ zatom, int wrap_in_place,
-                      double* __restrict__ x_ref, float* __restrict__ xh, float* __restrict__ xl,
+                      double* __restrict__ x_ref, float* __restrict__ xr,
                       int* __restrict__ atom_cell, int* __restrict__ cell_count, int* __restrict__ count, Box b,
                       const unsigned* gate, unsigned* __restrict__ err)
 {
@@ -77,7 +77,7 @@ __global__ void k_bin(int n, double* __restrict__ pos, const float* __restrict__
             c[d] = ci < 0 ? 0 : (ci >= b.nc[d] ? b.nc[d] - 1 : ci);
         }
     }
-    store_pos(xh, xl, i, wx, zatom ? zatom[i] : 1.f);
+    store_pos(xr, i, wx, zatom ? zatom[i] : 1.f);
     if (b.nc[0] > 0) {
         const int cid = (c[0] * b.nc[1] + c[1]) * b.nc[2] + c[2];
         atom_cell[i] = cid;
@@ -240,8 +240,7 @@ __device__ __forceinline__ unsigned long long sort_key(float d2, int v)
 constexpr int kHalfCells = 14;
 
 __global__ void __launch_bounds__(32 * kVerletWarps) k_half_cells(int n, int m_cap, float rv2,
-                                                                 const float* __restrict__ xh,
-                                                                 const float* __restrict__ xl,
+                                                                 const float* __restrict__ xr,
                                                                  const int* __restrict__ atom_cell,
                                                                  const int* __restrict__ cell_start,
                                                                  const int* __restrict__ cell_atoms,
@@ -260,7 +259,7 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_half_cells(int n, int m_c
     const float rq = sqrtf(rv2) + 1e-3f, rq2 = rq * rq;
     for (int i = blockIdx.x * kVerletWarps + warp; i < n; i += gridDim.x * kVerletWarps) {
         float hi[3], li[3];
-        load_pos(xh, xl, n, i, hi, li);
+        load_pos(xr, i, hi, li);
         const int cid = atom_cell[i];
         const int cz = cid % b.nc[2];
         const int cy = (cid / b.nc[2]) % b.nc[1];
@@ -308,7 +307,7 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_half_cells(int n, int m_c
                 const int j = cell_atoms[cst[c] + idx];
                 // own cell (c == 0): the pairs with j > i only
                 if (c != 0 || j > i) {
-                    const float4 a = NEP_LDG(reinterpret_cast<const float4*>(xh) + j);
+                    const float4 a = load_hi(xr, j);
                     const float qx = (a.x - hi[0]) + csh[c];
                     const float qy = (a.y - hi[1]) + csh[32 + c];
                     const float qz = (a.z - hi[2]) + csh[64 + c];
@@ -336,7 +335,7 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_half_cells(int n, int m_c
                 value = sq[e];
                 j = value & 0xFFFFFF;
                 float hj[3], lj[3];
-                load_pos(xh, xl, n, j, hj, lj);
+                load_pos(xr, j, hj, lj);
                 float rx, ry, rz;
                 pair_vector(value >> 24, hi, li, hj, lj, b, rx, ry, rz);
                 d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
@@ -629,8 +628,7 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_tile(int n, int m_cap, cons
     }
 }
 
-__global__ void k_verlet_brute(int n, int m_cap, float rv2, const float* __restrict__ xh,
-                               const float* __restrict__ xl, int* __restrict__ count, int* __restrict__ nbr,
+__global__ void k_verlet_brute(int n, int m_cap, float rv2, const float* __restrict__ xr, int* __restrict__ count, int* __restrict__ nbr,
                                float* __restrict__ key, int* __restrict__ vala, unsigned* err, Box b,
                                const unsigned* gate)
 {
@@ -638,11 +636,11 @@ __global__ void k_verlet_brute(int n, int m_cap, float rv2, const float* __restr
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float hi[3], li[3];
-    load_pos(xh, xl, n, i, hi, li);
+    load_pos(xr, i, hi, li);
     int cnt = 0;
     for (int j = 0; j < n; ++j) {
         float hj[3], lj[3];
-        load_pos(xh, xl, n, j, hj, lj);
+        load_pos(xr, j, hj, lj);
         for (int sx = -b.img[0]; sx <= b.img[0]; ++sx)
             for (int sy = -b.img[1]; sy <= b.img[1]; ++sy)
                 for (int sz = -b.img[2]; sz <= b.img[2]; ++sz) {
@@ -721,7 +719,7 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
     const float rv2 = r_list * r_list;
     const bool cells = b.nc[0] > 0;
     const int ncell = cells ? b.nc[0] * b.nc[1] * b.nc[2] : 0;
-    k_bin<<<blocks_for(n, T), T, 0, st>>>(n, pos, zatom, wrap_in_place ? 1 : 0, x_ref, nl.xh, nl.xl, nl.atom_cell,
+    k_bin<<<blocks_for(n, T), T, 0, st>>>(n, pos, zatom, wrap_in_place ? 1 : 0, x_ref, nl.xr, nl.atom_cell,
                                           nl.cell_count, nl.count, b, d_gate, d_err);
     if (cells) {
         k_scan<<<1, kScanThreads, 0, st>>>(ncell, nl.cell_count, nl.cell_start, nl.cell_fill, d_gate);
@@ -733,7 +731,7 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
         const int grid = std::min(blocks_for(n, kVerletWarps), kListGridCap);
         int* rows = reinterpret_cast<int*>(nl.pf);  // four words per slot, free until the site pass
         k_half_cells<<<grid, 32 * kVerletWarps, (size_t)kVerletWarps * (lcap + 6 * 32) * sizeof(int), st>>>(
-            n, nl.m_cap, rv2, nl.xh, nl.xl, nl.atom_cell, nl.cell_start, nl.cell_atoms, nl.count, rows, lcap, d_err, b,
+            n, nl.m_cap, rv2, nl.xr, nl.atom_cell, nl.cell_start, nl.cell_atoms, nl.count, rows, lcap, d_err, b,
             d_gate);
         const size_t sort_smem = (size_t)kSortWarps * lcap * 12 + (size_t)nl.m_cap * (kSortAtoms + 1) * sizeof(int);
         if (sort_smem <= kSortTileMaxSmem)
@@ -751,7 +749,7 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
                                                                                   nl.vala, nl.rev, d_err, d_gate);
         return cuda_fail(cudaGetLastError(), "neighbour-list kernels");
     } else {
-        k_verlet_brute<<<blocks_for(n, 128), 128, 0, st>>>(n, nl.m_cap, rv2, nl.xh, nl.xl, nl.count, nl.nbr, nl.pf,
+        k_verlet_brute<<<blocks_for(n, 128), 128, 0, st>>>(n, nl.m_cap, rv2, nl.xr, nl.count, nl.nbr, nl.pf,
                                                            nl.vala, d_err, b, d_gate);
     }
     k_reverse<<<std::min(blocks_for(n, 4), kListGridCap), 128, 0, st>>>(n, nl.m_cap, nl.count, nl.pf, nl.vala, nl.rev,

@@ -76,26 +76,25 @@ struct Gathered {
 
 // Pair vector of slot k of atom i (list layout nbr[k][n]).
 __device__ __forceinline__ float plain_pair(int i, int n, int k, const int* __restrict__ nbr,
-                                            const float* __restrict__ xh, const float* __restrict__ xl,
+                                            const float* __restrict__ xr,
                                             const Box& box, const float (&hi)[3], const float (&li)[3], float (&r)[3])
 {
     const int v = nbr[(size_t)k * n + i];
     const int j = v & 0xFFFFFF;
     float hj[3], lj[3];
-    load_pos(xh, xl, n, j, hj, lj);
+    load_pos(xr, j, hj, lj);
     pair_vector(v >> 24, hi, li, hj, lj, box, r[0], r[1], r[2]);
     return r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
 }
 
-__device__ bool gather_angular(int i, int n, int cnt, const int* __restrict__ nbr, const float* __restrict__ xh,
-                               const float* __restrict__ xl, const Box& box, float rcA, Gathered& A)
+__device__ bool gather_angular(int i, int n, int cnt, const int* __restrict__ nbr, const float* __restrict__ xr, const Box& box, float rcA, Gathered& A)
 {
     float hi[3], li[3];
-    load_pos(xh, xl, n, i, hi, li);
+    load_pos(xr, i, hi, li);
     A.cnt = 0;
     for (int k = 0; k < cnt; ++k) {
         float r[3];
-        const float d2 = plain_pair(i, n, k, nbr, xh, xl, box, hi, li, r);
+        const float d2 = plain_pair(i, n, k, nbr, xr, box, hi, li, r);
         if (!(d2 < rcA * rcA)) continue;
         if (A.cnt >= kPlainMaxAng) return false;
         const float d = sqrtf(d2);
@@ -110,27 +109,26 @@ __device__ bool gather_angular(int i, int n, int cnt, const int* __restrict__ nb
 
 __global__ void __launch_bounds__(kPlainThreads) k_plain_desc(int n, int m_cap, const int* __restrict__ count,
                                                               const int* __restrict__ nbr,
-                                                              const float* __restrict__ xh,
-                                                              const float* __restrict__ xl, Box box, float rcR,
+                                                              const float* __restrict__ xr, Box box, float rcR,
                                                               float rcA, float* __restrict__ q, unsigned* err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int cnt = min(count[i], m_cap);
     float hi[3], li[3];
-    load_pos(xh, xl, n, i, hi, li);
+    load_pos(xr, i, hi, li);
     float qd[kNdes];
     for (int v = 0; v < kNdes; ++v) qd[v] = 0.f;
     for (int k = 0; k < cnt; ++k) {
         float r[3];
-        const float d2 = plain_pair(i, n, k, nbr, xh, xl, box, hi, li, r);
+        const float d2 = plain_pair(i, n, k, nbr, xr, box, hi, li, r);
         if (!(d2 < rcR * rcR)) continue;
         float g[kNR];
         plain_radial(sqrtf(d2), rcR, kNR, g, nullptr);
         for (int a = 0; a < kNR; ++a) qd[a] += g[a];
     }
     Gathered A;
-    if (!gather_angular(i, n, cnt, nbr, xh, xl, box, rcA, A)) {
+    if (!gather_angular(i, n, cnt, nbr, xr, box, rcA, A)) {
         atomicOr(err, kErrOverflow);
         return;
     }
@@ -180,8 +178,7 @@ __global__ void __launch_bounds__(kPlainThreads) k_plain_net(int n, int n_neu, c
 }
 
 __global__ void __launch_bounds__(kPlainThreads) k_plain_pf(int n, int m_cap, const int* __restrict__ count,
-                                                            const int* __restrict__ nbr, const float* __restrict__ xh,
-                                                            const float* __restrict__ xl, Box box, float rcR,
+                                                            const int* __restrict__ nbr, const float* __restrict__ xr, Box box, float rcR,
                                                             float rcA, const float* __restrict__ G,
                                                             float* __restrict__ pf, unsigned* err)
 {
@@ -191,12 +188,12 @@ __global__ void __launch_bounds__(kPlainThreads) k_plain_pf(int n, int m_cap, co
     float Gv[kNdes];
     for (int v = 0; v < kNdes; ++v) Gv[v] = G[(size_t)v * n + i];
     float hi[3], li[3];
-    load_pos(xh, xl, n, i, hi, li);
+    load_pos(xr, i, hi, li);
     const float rc2 = fmaxf(rcR * rcR, rcA * rcA);
     // radial part for every slot (zero partial force outside both cutoffs is not stored)
     for (int k = 0; k < cnt; ++k) {
         float r[3];
-        const float d2 = plain_pair(i, n, k, nbr, xh, xl, box, hi, li, r);
+        const float d2 = plain_pair(i, n, k, nbr, xr, box, hi, li, r);
         if (!(d2 < rc2)) continue;
         float p[3] = {0.f, 0.f, 0.f};
         if (d2 < rcR * rcR) {
@@ -211,7 +208,7 @@ __global__ void __launch_bounds__(kPlainThreads) k_plain_pf(int n, int m_cap, co
         for (int c = 0; c < 3; ++c) o[c] = p[c];
     }
     Gathered A;
-    if (!gather_angular(i, n, cnt, nbr, xh, xl, box, rcA, A)) {
+    if (!gather_angular(i, n, cnt, nbr, xr, box, rcA, A)) {
         atomicOr(err, kErrOverflow);
         return;
     }
@@ -245,10 +242,10 @@ int launch_plain_site(const ForceArgs& a, NeighborList& nl, int n, float* q, flo
 {
     nl.mask_set = false;  // the assembly tests every slot's distance itself
     nblocks = (n + kPlainThreads - 1) / kPlainThreads;
-    k_plain_desc<<<nblocks, kPlainThreads, 0, st>>>(n, nl.m_cap, nl.count, nl.nbr, nl.xh, nl.xl, a.box, a.rcR, a.rcA,
+    k_plain_desc<<<nblocks, kPlainThreads, 0, st>>>(n, nl.m_cap, nl.count, nl.nbr, nl.xr, a.box, a.rcR, a.rcA,
                                                     q, d_err);
     k_plain_net<<<nblocks, kPlainThreads, 0, st>>>(n, a.n_neu, a.z, q, G, e_atom, e_partials, d_err);
-    k_plain_pf<<<nblocks, kPlainThreads, 0, st>>>(n, nl.m_cap, nl.count, nl.nbr, nl.xh, nl.xl, a.box, a.rcR, a.rcA,
+    k_plain_pf<<<nblocks, kPlainThreads, 0, st>>>(n, nl.m_cap, nl.count, nl.nbr, nl.xr, a.box, a.rcR, a.rcA,
                                                   G, nl.pf, d_err);
     return cuda_fail(cudaGetLastError(), "plain force kernels");
 }

@@ -479,13 +479,12 @@ struct SlotTable {
     const unsigned char* orig = nullptr;
 };
 
-__host__ __device__ __forceinline__ void fetch_slot(const SlotTable& T, const float* __restrict__ xh,
-                                                    const float* __restrict__ xl, int n, int k, int cnt, NbSlot& s)
+__host__ __device__ __forceinline__ void fetch_slot(const SlotTable& T, const float* __restrict__ xr, int n, int k, int cnt, NbSlot& s)
 {
     if (k >= 0 && k < cnt) {
         s.v = T.slots[(size_t)k * T.stride + T.idx];
-        load_pos(xh, xl, n, s.v & 0xFFFFFF, s.h, s.l);
-        s.z = load_z(xh, s.v & 0xFFFFFF);
+        load_pos(xr, s.v & 0xFFFFFF, s.h, s.l);
+        s.z = load_z(xr, s.v & 0xFFFFFF);
     }
 }
 
@@ -587,8 +586,7 @@ __host__ __device__ __forceinline__ void unit_vector_res(float rx, float ry, flo
 // call it (inactive lanes pass cnt = 0): the ranks are walked in step.
 template <class D = DescSi>
 __host__ __device__ __forceinline__ void site_descriptors(int i, int n, int cnt, const SlotTable& nbr,
-                                                          const float* __restrict__ xh,
-                                                          const float* __restrict__ xl, const Box& box,
+                                                          const float* __restrict__ xr, const Box& box,
                                                           const SiteParams& P, const float (&hi)[3],
                                                           const float (&li)[3], float zi, float (&q)[D::Ndes],
                                                           HarmT<D>& S)
@@ -613,10 +611,10 @@ __host__ __device__ __forceinline__ void site_descriptors(int i, int n, int cnt,
     const int kmax = cnt;
 #endif
     NbSlot nx;
-    fetch_slot(nbr, xh, xl, n, kmax - 1, cnt, nx);
+    fetch_slot(nbr, xr, n, kmax - 1, cnt, nx);
     for (int k = kmax - 1; k >= 0; --k) {
         const NbSlot cur = nx;
-        fetch_slot(nbr, xh, xl, n, k - 1, cnt, nx);
+        fetch_slot(nbr, xr, n, k - 1, cnt, nx);
         if (k >= cnt) continue;
         float rx, ry, rz;
         pair_vector(cur.v >> 24, hi, li, cur.h, cur.l, box, rx, ry, rz);
@@ -726,19 +724,18 @@ __host__ __device__ __forceinline__ void pair_partial_force(const float (&r)[3],
 // coefficients A (kNA x kLM, in place of the harmonic sums S) and GR.
 template <class D = DescSi>
 __host__ __device__ __forceinline__ void site_coefficients(int i, bool active, int n, int cnt, const SlotTable& nbr,
-                                                           const float* __restrict__ xh,
-                                                           const float* __restrict__ xl, const Box& box,
+                                                           const float* __restrict__ xr, const Box& box,
                                                            const SiteParams& P, HarmT<D>& S,
                                                            float (&GR)[D::NR], float& U_hi, float& U_lo)
 {
     constexpr int kNR = D::NR, kNA = D::NA, kNdes = D::Ndes;
     float hi[3], li[3], zi = 1.f;
     if (active) {
-        load_pos(xh, xl, n, i, hi, li);
-        zi = load_z(xh, i);
+        load_pos(xr, i, hi, li);
+        zi = load_z(xr, i);
     }
     float q[kNdes];
-    site_descriptors<D>(i, n, cnt, nbr, xh, xl, box, P, hi, li, zi, q, S);
+    site_descriptors<D>(i, n, cnt, nbr, xr, box, P, hi, li, zi, q, S);
 
     float G[kNdes];
     network(P.w, P.n_neu, q, G, U_hi, U_lo);
@@ -761,18 +758,17 @@ __host__ __device__ __forceinline__ void site_coefficients(int i, bool active, i
 // untouched).
 template <class D = DescSi>
 __host__ __device__ __forceinline__ void site_partial_forces(int i, bool active, int n, int cnt,
-                                                             const SlotTable& nbr, const float* __restrict__ xh,
-                                                             const float* __restrict__ xl, const Box& box,
+                                                             const SlotTable& nbr, const float* __restrict__ xr, const Box& box,
                                                              const SiteParams& P, const PfOut& out, float& U_hi,
                                                              float& U_lo)
 {
     HarmT<D> S;
     float GR[D::NR];
-    site_coefficients<D>(i, active, n, cnt, nbr, xh, xl, box, P, S, GR, U_hi, U_lo);
+    site_coefficients<D>(i, active, n, cnt, nbr, xr, box, P, S, GR, U_hi, U_lo);
     float hi[3], li[3], zi = 1.f;
     if (active) {
-        load_pos(xh, xl, n, i, hi, li);
-        zi = load_z(xh, i);
+        load_pos(xr, i, hi, li);
+        zi = load_z(xr, i);
     }
 
     const float rc2max = P.rcR2 > P.rcA2 ? P.rcR2 : P.rcA2;
@@ -780,10 +776,10 @@ __host__ __device__ __forceinline__ void site_partial_forces(int i, bool active,
     // pair geometry's roundings (summed in FP32: each term is ~1e-7 eV)
     float dU = 0.f;
     NbSlot nx;
-    fetch_slot(nbr, xh, xl, n, 0, cnt, nx);
+    fetch_slot(nbr, xr, n, 0, cnt, nx);
     for (int k = 0; k < cnt; ++k) {
         const NbSlot cur = nx;
-        fetch_slot(nbr, xh, xl, n, k + 1, cnt, nx);
+        fetch_slot(nbr, xr, n, k + 1, cnt, nx);
         float r[3], r_lo[3];
         pair_vector_lo(cur.v >> 24, hi, li, cur.h, cur.l, box, r, r_lo);
         const float d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
@@ -829,13 +825,12 @@ struct AsmSlot {
 
 __host__ __device__ __forceinline__ void assemble_atom(int i, int n, int m_cap, float rc2max,
                                                        const int* __restrict__ count, const SlotTable& nbr,
-                                                       const int* __restrict__ rev, const float* __restrict__ xh,
-                                                       const float* __restrict__ xl, const Box& box,
+                                                       const int* __restrict__ rev, const float* __restrict__ xr, const Box& box,
                                                        const float* __restrict__ pf, float (&F)[3], float (&W)[9],
                                                        const unsigned* __restrict__ mask = nullptr)
 {
     float hi[3], li[3];
-    load_pos(xh, xl, n, i, hi, li);
+    load_pos(xr, i, hi, li);
     int cnt = imin(count[i], m_cap);
     unsigned mb[3] = {~0u, ~0u, ~0u};
     if (mask) {
@@ -863,7 +858,7 @@ __host__ __device__ __forceinline__ void assemble_atom(int i, int n, int m_cap, 
         if (k < cnt && kept(k)) {
             const int j = v & 0xFFFFFF;
             d.v = v;
-            load_pos(xh, xl, n, j, d.h, d.l);
+            load_pos(xr, j, d.h, d.l);
             d.po = NEP_LDG(pf4 + (size_t)k * n + i);
             d.pq = NEP_LDG(pf4 + (size_t)kr * n + j);
         }

@@ -18,7 +18,7 @@
 //                    the input gradient G;
 //   partial forces   warp w takes its slots again, each angular pair against
 //                    the coefficients A in shared memory.
-// Measured on a GB300, one thread per atom -> this form: 248 -> 187 us for the
+// Measured on a GB300, one thread per atom -> this form: 248 -> 186 us for the
 // 125,000-atom crystal (1190 -> 1122 warp instructions per atom, 7.6 -> 18.6
 // warps per SM), 104 -> 71 us for the whole MD step of 4,096 atoms.
 #pragma once
@@ -117,13 +117,15 @@ __device__ __forceinline__ void sh_add(const ShFast& s, float cg, float cd, floa
 }
 
 // Harmonic sums of lm in [LO, LO + 8) over the tile's slots, last slot first:
-// S[j][n] = (S_n,LO+2j, S_n,LO+2j+1).
+// S[j][n] = (S_n,LO+2j, S_n,LO+2j+1).  slots: those with a pair in any lane.
 template <class D, int LO>
-__device__ __forceinline__ void site_block_harmonics(const float* tile, float2 (&S)[4][D::NA])
+__device__ __forceinline__ void site_block_harmonics(const float* tile, unsigned slots, float2 (&S)[4][D::NA])
 {
     constexpr int row = kSiteChunk * 32;
 #pragma unroll 1
-    for (int s = kSiteChunk - 1; s >= 0; --s) {
+    while (slots) {
+        const int s = 31 - __clz((int)slots);
+        slots ^= 1u << s;
         const float* t = tile + s * 32;
         const float x = t[0];
         if (x > 1.5f) continue;  // kNoPair
@@ -186,14 +188,17 @@ struct PairGeom {
     float u[3], d, d2, inv, dd, du[3], w;
 };
 
-__device__ __forceinline__ void site_pair_geometry(int v, const float* __restrict__ xh, const float* __restrict__ xl,
-                                                   const Box& box, const SiteParams& P, const float (&hi)[3],
-                                                   const float (&li)[3], float zi, PairGeom& g)
+// a neighbour's list value and position record
+struct NbRecord {
+    int v;
+    float h[3], l[3], z;
+};
+
+__device__ __forceinline__ void site_pair_geometry(const NbRecord& nb, const Box& box, const SiteParams& P,
+                                                   const float (&hi)[3], const float (&li)[3], float zi, PairGeom& g)
 {
-    const int j = v & 0xFFFFFF;
-    float hj[3], lj[3], r[3], r_lo[3], u_res[3], dres;
-    load_pos(xh, xl, 0, j, hj, lj);
-    pair_vector_lo(v >> 24, hi, li, hj, lj, box, r, r_lo);
+    float r[3], r_lo[3], u_res[3], dres;
+    pair_vector_lo(nb.v >> 24, hi, li, nb.h, nb.l, box, r, r_lo);
     g.d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
     g.d = sqrtf(g.d2);
     unit_vector_res(r[0], r[1], r[2], g.d, g.u[0], g.u[1], g.u[2], u_res, dres, g.inv);
@@ -201,7 +206,7 @@ __device__ __forceinline__ void site_pair_geometry(int v, const float* __restric
     g.dd = dres + ur;
 #pragma unroll
     for (int a = 0; a < 3; ++a) g.du[a] = fmaf(fmaf(-g.u[a], ur, r_lo[a]), g.inv, u_res[a]);
-    g.w = pair_weight(P, zi, load_z(xh, j));
+    g.w = pair_weight(P, zi, nb.z);
 }
 
 // radial part of dU/dd (0 beyond the radial cutoff); s_G: the lane's column of G
@@ -245,7 +250,7 @@ __device__ __forceinline__ void site_angular_terms(const float* s_A, const ShFas
 // or NULL.  Warp 0 returns the site energies (hi + lo).
 template <class D, int WORDS>
 __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, const int* __restrict__ nbr,
-                                           const float* __restrict__ xh, const float* __restrict__ xl, const Box& box,
+                                           const float* __restrict__ xr, const Box& box,
                                            const float* __restrict__ z, int n_par, SiteParams P,
                                            float* __restrict__ pf, unsigned* __restrict__ mask, float& U_hi,
                                            float& U_lo)
@@ -253,6 +258,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
     constexpr int NR = D::NR, NA = D::NA, ND = D::Ndes;
     extern __shared__ __align__(16) float s_site[];
     __shared__ float s_dU[kSiteWarps][32];
+    __shared__ unsigned s_any[kSiteChunk];  // per tile slot: 1 an angular pair in some lane, 2 a radial one
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* s_w = s_site;
     float* s_A = s_w + (n_par + 31) / 32 * 32;         // [quads][32] float4
@@ -263,9 +269,8 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
     if (threadIdx.x < 96) s_mask[threadIdx.x] = 0u;
     P.w = s_w;
     const int ia = active ? i : 0;
-    float hi[3], li[3];
-    load_pos(xh, xl, n, ia, hi, li);
-    const float zi = load_z(xh, ia);
+    float hi[3], li[3], zi;
+    load_pos(xr, ia, hi, li, zi);
     const int kmax = __reduce_max_sync(0xffffffffu, cnt);  // the same in every warp
     const int chunks = (kmax + kSiteChunk - 1) / kSiteChunk;
     const float rc2max = P.rcR2 > P.rcA2 ? P.rcR2 : P.rcA2;
@@ -289,26 +294,36 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
             for (int a = 0; a < NA; ++a) S[j][a] = make_float2(0.f, 0.f);
         float* tile = s_A + lane;
         float2* tileR = reinterpret_cast<float2*>(s_x) + lane;
-        int v_nx = 0;
-        auto load_slot = [&](int k) { return k < cnt ? nbr[(size_t)k * n + ia] : 0; };
-        if (chunks > 0) v_nx = load_slot((chunks - 1) * kSiteChunk + warp);
+        // the thread's slots in turn: k_of(0) is its first of the last tile;
+        // a record is loaded one slot ahead and its list value two ahead
+        auto k_of = [&](int q) { return (chunks - 1 - (q >> 2)) * kSiteChunk + 4 * (q & 3) + warp; };
+        auto load_v = [&](int q) {
+            const int k = k_of(q);
+            return q < 4 * chunks && k < cnt ? nbr[(size_t)k * n + ia] : -1;
+        };
+        auto load_record = [&](int v, NbRecord& r) {
+            r.v = v;
+            if (v >= 0) load_pos(xr, v & 0xFFFFFF, r.h, r.l, r.z);
+        };
+        NbRecord nx;
+        load_record(load_v(0), nx);
+        int v_nx = load_v(1);
 #pragma unroll 1
-        for (int c = chunks - 1; c >= 0; --c) {
+        for (int c = chunks - 1, q = 0; c >= 0; --c) {
 #pragma unroll 1
-            for (int t = 0; t < kSiteChunk / kSiteWarps; ++t) {
-                const int s = 4 * t + warp, k = c * kSiteChunk + s;
-                const int v = v_nx;
-                v_nx = t < kSiteChunk / kSiteWarps - 1 ? load_slot(k + 4) : (c > 0 ? load_slot(k - 28) : 0);
+            for (int t = 0; t < kSiteChunk / kSiteWarps; ++t, ++q) {
+                const int s = 4 * t + warp;
+                const NbRecord cur = nx;
+                load_record(v_nx, nx);
+                v_nx = load_v(q + 2);
                 float x = kNoPair, fc = 0.f, ux = kNoPair;
-                if (k < cnt) {
-                    const int j = v & 0xFFFFFF;
-                    float hj[3], lj[3], rx, ry, rz;
-                    load_pos(xh, xl, n, j, hj, lj);
-                    pair_vector(v >> 24, hi, li, hj, lj, box, rx, ry, rz);
+                if (cur.v >= 0) {
+                    float rx, ry, rz;
+                    pair_vector(cur.v >> 24, hi, li, cur.h, cur.l, box, rx, ry, rz);
                     const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
                     if (d2 < rc2max) {
                         const int b = 4 * c + t;
-                        const float w = pair_weight(P, zi, load_z(xh, j));
+                        const float w = pair_weight(P, zi, cur.z);
                         const float d = sqrtf(d2);
 #pragma unroll
                         for (int q = 0; q < WORDS; ++q)
@@ -330,18 +345,24 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
                 }
                 tile[s * 32] = ux;
                 tileR[s * 32] = make_float2(x, fc);
+                const unsigned any_a = __any_sync(0xffffffffu, ux < 1.5f), any_r = __any_sync(0xffffffffu, x < 1.5f);
+                if (lane == 0) s_any[s] = (any_a ? 1u : 0u) | (any_r ? 2u : 0u);
             }
             __syncthreads();
+            unsigned slots = __ballot_sync(0xffffffffu, lane < kSiteChunk && (s_any[lane & (kSiteChunk - 1)] &
+                                                                              (warp < 3 ? 1u : 2u)) != 0u);
             if (warp == 0) {
-                site_block_harmonics<D, 0>(tile, S);
+                site_block_harmonics<D, 0>(tile, slots, S);
             } else if (warp == 1) {
-                site_block_harmonics<D, 8>(tile, S);
+                site_block_harmonics<D, 8>(tile, slots, S);
             } else if (warp == 2) {
-                site_block_harmonics<D, 16>(tile, S);
+                site_block_harmonics<D, 16>(tile, slots, S);
             } else {
                 const float2 minus = make_float2(-1.f, -1.f);
 #pragma unroll 1
-                for (int s = kSiteChunk - 1; s >= 0; --s) {
+                while (slots) {
+                    const int s = 31 - __clz((int)slots);
+                    slots ^= 1u << s;
                     const float2 xf = tileR[s * 32];
                     if (xf.x > 1.5f) continue;  // kNoPair
                     float g[NR];
@@ -469,19 +490,39 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
     const float* sA = s_A + 4 * lane;
     const float* sG = s_q + lane;
     float4* out = reinterpret_cast<float4*>(pf) + ia;
+    // the next own slot, the angular pairs of a word before the others: k, or
+    // -1; its list value is loaded two pairs ahead, the record one ahead
+    auto next_slot = [&](bool& angular) {
 #pragma unroll
-    for (int w = 0; w < WORDS; ++w) {
-        unsigned rest = kept[w];
+        for (int w = 0; w < WORDS; ++w)
+            if (kept[w]) {
+                angular = ang[w] != 0u;
+                const int b = __ffs((int)(angular ? ang[w] : kept[w])) - 1;
+                ang[w] &= ~(1u << b);
+                kept[w] &= ~(1u << b);
+                return 4 * (32 * w + b) + warp;
+            }
+        return -1;
+    };
+    {
+        bool angular = false, angular_nx = false;
+        NbRecord nb, nb_nx;
+        int k = next_slot(angular);
+        if (k >= 0) {
+            nb.v = nbr[(size_t)k * n + ia];
+            load_pos(xr, nb.v & 0xFFFFFF, nb.h, nb.l, nb.z);
+        }
+        int k_nx = next_slot(angular_nx);
+        if (k_nx >= 0) nb_nx.v = nbr[(size_t)k_nx * n + ia];
 #pragma unroll 1
-        while (rest) {
-            // the angular pairs first, then those beyond the angular cutoff
-            const bool angular = ang[w] != 0u;
-            const int b = __ffs((int)(angular ? ang[w] : rest)) - 1;
-            ang[w] &= ~(1u << b);
-            rest &= ~(1u << b);
-            const int k = 4 * (32 * w + b) + warp;
+        while (k >= 0) {
+            bool angular_n2 = false;
+            const int k_n2 = next_slot(angular_n2);
+            int v_n2 = 0;
+            if (k_nx >= 0) load_pos(xr, nb_nx.v & 0xFFFFFF, nb_nx.h, nb_nx.l, nb_nx.z);
+            if (k_n2 >= 0) v_n2 = nbr[(size_t)k_n2 * n + ia];
             PairGeom g;
-            site_pair_geometry(nbr[(size_t)k * n + ia], xh, xl, box, P, hi, li, zi, g);
+            site_pair_geometry(nb, box, P, hi, li, zi, g);
             float radial = site_pair_radial<D>(g, P, sG);
             float V[3] = {0.f, 0.f, 0.f};
             float eu = 0.f;
@@ -508,6 +549,12 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
             dU += fmaf(radial, g.dd, eu);
             out[(size_t)k * n] = make_float4(fmaf(radial, g.u[0], V[0]), fmaf(radial, g.u[1], V[1]),
                                              fmaf(radial, g.u[2], V[2]), 0.f);
+            k = k_nx;
+            angular = angular_nx;
+            nb = nb_nx;
+            k_nx = k_n2;
+            angular_nx = angular_n2;
+            nb_nx.v = v_n2;
         }
     }
     s_dU[warp][lane] = dU;

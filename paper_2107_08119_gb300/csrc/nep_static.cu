@@ -37,9 +37,8 @@ constexpr size_t kOffNbr = kOffCount + align256(sizeof(int) * kStaticAtoms);
 constexpr size_t kOffRev = kOffNbr + align256(sizeof(int) * kStaticAtoms * kStaticSlots);
 constexpr size_t kOffVala = kOffRev + align256(sizeof(int) * kStaticAtoms * kStaticSlots);
 constexpr size_t kOffPf = kOffVala + align256(sizeof(int) * kStaticAtoms * kStaticSlots);
-constexpr size_t kOffXh = kOffPf + align256(sizeof(float) * kStaticAtoms * kStaticSlots * 4);
-constexpr size_t kOffXl = kOffXh + align256(sizeof(float) * kStaticAtoms * 4);
-constexpr size_t kOffAtomCell = kOffXl + align256(sizeof(float) * kStaticAtoms * 4);
+constexpr size_t kOffXr = kOffPf + align256(sizeof(float) * kStaticAtoms * kStaticSlots * 4);
+constexpr size_t kOffAtomCell = kOffXr + align256(sizeof(float) * kStaticAtoms * 8);
 constexpr size_t kOffCellAtoms = kOffAtomCell + align256(sizeof(int) * kStaticAtoms);
 constexpr size_t kOffCellCount = kOffCellAtoms + align256(sizeof(int) * kStaticAtoms);
 constexpr size_t kOffCellStart = kOffCellCount + align256(sizeof(int) * (kStaticCells + 1));
@@ -187,8 +186,7 @@ extern "C" int nep_compute_efv_static(const nep_hyper* hp, const float* z, int n
     nl.rev = reinterpret_cast<int*>(base + kOffRev);
     nl.pf = reinterpret_cast<float*>(base + kOffPf);
     nl.vala = reinterpret_cast<int*>(base + kOffVala);
-    nl.xh = reinterpret_cast<float*>(base + kOffXh);
-    nl.xl = reinterpret_cast<float*>(base + kOffXl);
+    nl.xr = reinterpret_cast<float*>(base + kOffXr);
     nl.atom_cell = reinterpret_cast<int*>(base + kOffAtomCell);
     nl.cell_atoms = reinterpret_cast<int*>(base + kOffCellAtoms);
     nl.cell_count = reinterpret_cast<int*>(base + kOffCellCount);

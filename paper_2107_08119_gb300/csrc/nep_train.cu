@@ -59,8 +59,7 @@ std::atomic<unsigned long long> g_dataset_uid{0};
 
 // ------------------------------------------------------------------ build
 __global__ void k_ds_split(int N, const double* __restrict__ pos, const int* __restrict__ sid,
-                           const Box* __restrict__ boxes, const float* __restrict__ zat, float* __restrict__ xh,
-                           float* __restrict__ xl, unsigned* __restrict__ err)
+                           const Box* __restrict__ boxes, const float* __restrict__ zat, float* __restrict__ xr, unsigned* __restrict__ err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -75,11 +74,11 @@ __global__ void k_ds_split(int N, const double* __restrict__ pos, const int* __r
         if (w < 0.0) w = 0.0;
         wx[d] = w;
     }
-    store_pos(xh, xl, i, wx, zat ? zat[i] : 1.f);
+    store_pos(xr, i, wx, zat ? zat[i] : 1.f);
 }
 
 __global__ void k_ds_list(int N, const int* __restrict__ sid, const int* __restrict__ sstart,
-                          const Box* __restrict__ boxes, const float* __restrict__ xh, const float* __restrict__ xl,
+                          const Box* __restrict__ boxes, const float* __restrict__ xr,
                           float rc2, float rcA2, int* __restrict__ tmp, int* __restrict__ cnt, int* __restrict__ cntA,
                           unsigned* err)
 {
@@ -88,11 +87,11 @@ __global__ void k_ds_list(int N, const int* __restrict__ sid, const int* __restr
     const int s = sid[i];
     const Box b = boxes[s];
     float hi[3], li[3];
-    load_pos(xh, xl, N, i, hi, li);
+    load_pos(xr, i, hi, li);
     int c = 0, ca = 0;
     for (int j = sstart[s]; j < sstart[s + 1]; ++j) {
         float hj[3], lj[3];
-        load_pos(xh, xl, N, j, hj, lj);
+        load_pos(xr, j, hj, lj);
         for (int sx = -b.img[0]; sx <= b.img[0]; ++sx)
             for (int sy = -b.img[1]; sy <= b.img[1]; ++sy)
                 for (int sz = -b.img[2]; sz <= b.img[2]; ++sz) {
@@ -118,7 +117,7 @@ __global__ void k_ds_list(int N, const int* __restrict__ sid, const int* __restr
 // first, so the warps of the fused contraction, whose lanes walk different
 // atoms' pairs side by side, run their angular terms together.
 __global__ void k_ds_sort(int N, const int* __restrict__ sid, const Box* __restrict__ boxes,
-                          const float* __restrict__ xh, const float* __restrict__ xl, const int* __restrict__ cnt,
+                          const float* __restrict__ xr, const int* __restrict__ cnt,
                           int* __restrict__ tmp)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -126,14 +125,14 @@ __global__ void k_ds_sort(int N, const int* __restrict__ sid, const Box* __restr
     const int c = min(cnt[i], kDsCap);
     const Box b = boxes[sid[i]];
     float hi[3], li[3];
-    load_pos(xh, xl, N, i, hi, li);
+    load_pos(xr, i, hi, li);
     int* row = tmp + (size_t)i * kDsCap;
     float key[kDsCap];
     for (int t = 0; t < c; ++t) {
         const int v = row[t];
         const int j = v & 0xFFFFFF;
         float hj[3], lj[3];
-        load_pos(xh, xl, N, j, hj, lj);
+        load_pos(xr, j, hj, lj);
         float rx, ry, rz;
         pair_vector(v >> 24, hi, li, hj, lj, b, rx, ry, rz);
         key[t] = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
@@ -155,14 +154,14 @@ __global__ void k_ds_sort(int N, const int* __restrict__ sid, const Box* __restr
 
 __global__ void k_ds_compact(int N, const int* __restrict__ tmp, const long long* __restrict__ pstart,
                              const long long* __restrict__ astart, const int* __restrict__ sid,
-                             const Box* __restrict__ boxes, const float* __restrict__ xh, const float* __restrict__ xl,
+                             const Box* __restrict__ boxes, const float* __restrict__ xr,
                              float rcA2, int* __restrict__ pj, long long* __restrict__ aidx)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const Box b = boxes[sid[i]];
     float hi[3], li[3];
-    load_pos(xh, xl, N, i, hi, li);
+    load_pos(xr, i, hi, li);
     const long long p0 = pstart[i], p1 = pstart[i + 1];
     long long a = astart[i];
     for (long long p = p0; p < p1; ++p) {
@@ -170,7 +169,7 @@ __global__ void k_ds_compact(int N, const int* __restrict__ tmp, const long long
         pj[p] = v;
         const int j = v & 0xFFFFFF;
         float hj[3], lj[3];
-        load_pos(xh, xl, N, j, hj, lj);
+        load_pos(xr, j, hj, lj);
         float rx, ry, rz;
         pair_vector(v >> 24, hi, li, hj, lj, b, rx, ry, rz);
         const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
@@ -205,7 +204,7 @@ __global__ void k_ds_reverse(int N, const long long* __restrict__ pstart, const 
 // each of its pair vectors r_ij, scattered to the reverse slots.
 
 __global__ void k_ds_site(int N, const int* __restrict__ sid, const Box* __restrict__ boxes,
-                          const float* __restrict__ xh, const float* __restrict__ xl,
+                          const float* __restrict__ xr,
                           const long long* __restrict__ pstart, const int* __restrict__ pj,
                           const long long* __restrict__ aidx, float rcR2,
                           float rcA2, float rcR, float rcA, float inv_rcR, float inv_rcA, int typed,
@@ -216,8 +215,8 @@ __global__ void k_ds_site(int N, const int* __restrict__ sid, const Box* __restr
     if (i >= N) return;
     const Box b = boxes[sid[i]];
     float hi[3], li[3];
-    load_pos(xh, xl, N, i, hi, li);
-    const float zi = load_z(xh, i);
+    load_pos(xr, i, hi, li);
+    const float zi = load_z(xr, i);
     float qR[kNR], qC[kNR];
     Harm S;
     for (int a = 0; a < kNR; ++a) qR[a] = qC[a] = 0.f;
@@ -228,12 +227,12 @@ __global__ void k_ds_site(int N, const int* __restrict__ sid, const Box* __restr
         const int v = pj[p];
         const int j = v & 0xFFFFFF;
         float hj[3], lj[3];
-        load_pos(xh, xl, N, j, hj, lj);
+        load_pos(xr, j, hj, lj);
         float rx, ry, rz;
         pair_vector(v >> 24, hi, li, hj, lj, b, rx, ry, rz);
         const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
         const float d = sqrtf(d2);
-        const float wz = typed ? sqrtf(zi * load_z(xh, j)) : 1.f;
+        const float wz = typed ? sqrtf(zi * load_z(xr, j)) : 1.f;
         if (d2 < rcR2) {
             float g[kNR];
             radial_g<kNR>(d, rcR, inv_rcR, g, wz);
@@ -271,13 +270,13 @@ __global__ void k_ds_site(int N, const int* __restrict__ sid, const Box* __restr
         const int v = pj[p];
         const int j = v & 0xFFFFFF;
         float hj[3], lj[3];
-        load_pos(xh, xl, N, j, hj, lj);
+        load_pos(xr, j, hj, lj);
         float r[3];
         pair_vector(v >> 24, hi, li, hj, lj, b, r[0], r[1], r[2]);
         const float d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
         const float d = sqrtf(d2);
         const float inv = 1.f / d;
-        const float wz = typed ? sqrtf(zi * load_z(xh, j)) : 1.f;
+        const float wz = typed ? sqrtf(zi * load_z(xr, j)) : 1.f;
         PairRec pr;
         pr.r[0] = r[0];
         pr.r[1] = r[1];
@@ -1588,8 +1587,7 @@ int nep_dataset_create_species(nep_model* m, int n_struct, const int* n_atoms, c
     double* dpos = nullptr;
     float* dz = nullptr;
     ds->typed = z_atom ? 1 : 0;
-    float*& xh = ds->xh;
-    float*& xl = ds->xl;
+    float*& xr = ds->xr;
     int *tmp = nullptr, *cnt = nullptr, *cnta = nullptr;
     long long*& rev = ds->rev;
     int rc = NEP_OK;
@@ -1611,7 +1609,7 @@ int nep_dataset_create_species(nep_model* m, int n_struct, const int* n_atoms, c
         (rc = dalloc(&ds->B, (size_t)N * kNdes * 3, bytes)) || (rc = dalloc(&ds->pstart, (size_t)N + 1, bytes)) ||
         (rc = dalloc(&ds->e_tar, S, bytes)) || (rc = dalloc(&ds->f_tar, (size_t)3 * N, bytes)) ||
         (rc = dalloc(&ds->w_tar, (size_t)6 * S, bytes)) || (rc = dalloc(&dpos, (size_t)3 * N, nullptr)) ||
-        (rc = dalloc(&xh, (size_t)4 * N, nullptr)) || (rc = dalloc(&xl, (size_t)4 * N, nullptr)) ||
+        (rc = dalloc(&xr, (size_t)8 * N, nullptr)) ||
         (rc = dalloc(&tmp, (size_t)N * kDsCap, nullptr)) || (rc = dalloc(&cnt, N, nullptr)) ||
         (rc = dalloc(&cnta, N, nullptr)) || (z_atom && (rc = dalloc(&dz, N, nullptr))))
         return fail(rc);
@@ -1655,8 +1653,8 @@ int nep_dataset_create_species(nep_model* m, int n_struct, const int* n_atoms, c
 
     const float rc2 = (float)(rmax * rmax), rcA2 = (float)(m->hp.rc_A * m->hp.rc_A);
     const float rcR2 = (float)(m->hp.rc_R * m->hp.rc_R);
-    k_ds_split<<<blocks_for(N, 256), 256>>>(N, dpos, ds->sid, ds->boxes, dz, xh, xl, m->d_err);
-    k_ds_list<<<blocks_for(N, 128), 128>>>(N, ds->sid, ds->sstart, ds->boxes, xh, xl, rc2, rcA2, tmp, cnt, cnta,
+    k_ds_split<<<blocks_for(N, 256), 256>>>(N, dpos, ds->sid, ds->boxes, dz, xr, m->d_err);
+    k_ds_list<<<blocks_for(N, 128), 128>>>(N, ds->sid, ds->sstart, ds->boxes, xr, rc2, rcA2, tmp, cnt, cnta,
                                            m->d_err);
     if ((rc = cuda_fail(cudaDeviceSynchronize(), "dataset neighbour search"))) return fail(rc);
     unsigned bits = 0;
@@ -1691,11 +1689,11 @@ int nep_dataset_create_species(nep_model* m, int n_struct, const int* n_atoms, c
     up(ds->pstart, hps.data(), sizeof(long long) * (N + 1));
     up(dastart, has.data(), sizeof(long long) * (N + 1));
     if (e != cudaSuccess) return fail(cuda_fail(e, "dataset upload"));
-    k_ds_sort<<<blocks_for(N, 128), 128>>>(N, ds->sid, ds->boxes, xh, xl, cnt, tmp);
-    k_ds_compact<<<blocks_for(N, 128), 128>>>(N, tmp, ds->pstart, dastart, ds->sid, ds->boxes, xh, xl, rcA2, ds->pj,
+    k_ds_sort<<<blocks_for(N, 128), 128>>>(N, ds->sid, ds->boxes, xr, cnt, tmp);
+    k_ds_compact<<<blocks_for(N, 128), 128>>>(N, tmp, ds->pstart, dastart, ds->sid, ds->boxes, xr, rcA2, ds->pj,
                                               ds->aidx);
     k_ds_reverse<<<blocks_for(N, 128), 128>>>(N, ds->pstart, ds->pj, rev, m->d_err);
-    k_ds_site<<<blocks_for(N, 64), 64>>>(N, ds->sid, ds->boxes, xh, xl, ds->pstart, ds->pj, ds->aidx, rcR2,
+    k_ds_site<<<blocks_for(N, 64), 64>>>(N, ds->sid, ds->boxes, xr, ds->pstart, ds->pj, ds->aidx, rcR2,
                                          rcA2, (float)m->hp.rc_R, (float)m->hp.rc_A, (float)(1.0 / m->hp.rc_R),
                                          (float)(1.0 / m->hp.rc_A), ds->typed, ds->q, ds->B, ds->rec, ds->ang);
     if (!rc && !(rc = dalloc(&ds->qpack, pop_tc_qpack_bytes(N), bytes)))
@@ -1769,8 +1767,7 @@ int nep_dataset_destroy(nep_dataset* ds)
     dfree(ds->chunk_begin);
     dfree(ds->chunk_end);
     dfree(ds->q);
-    dfree(ds->xh);
-    dfree(ds->xl);
+    dfree(ds->xr);
     dfree(ds->B);
     dfree(ds->pstart);
     dfree(ds->pj);
