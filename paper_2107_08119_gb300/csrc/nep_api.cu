@@ -14,12 +14,6 @@ namespace nep {
 namespace {
 thread_local char g_err[512] = "";
 
-__global__ void k_finish_efv(const double* __restrict__ red, double* e_total, double* virial_total)
-{
-    if (threadIdx.x == 0 && e_total) *e_total = red[0];
-    if (threadIdx.x < 9 && virial_total) virial_total[threadIdx.x] = red[1 + threadIdx.x];
-}
-
 // J^a = sum_i sum_b W_i^{ab} v_i^b per block, FP32 products, FP64 sums.
 __global__ void k_heat(int n, const float* __restrict__ W, const double* __restrict__ v, double* __restrict__ part)
 {
@@ -328,8 +322,8 @@ int nep_create(const nep_hyper* hp, const float* z, int n_par, nep_model** out)
     m->hp = *hp;
     m->n_des = n_des;
     m->n_par = n_par;
-    if ((rc = dev_alloc(&m->d_z, (size_t)n_par, "parameters")) || (rc = dev_alloc(&m->d_err, 1, "error word")) ||
-        (rc = dev_alloc(&m->d_red, 32, "reduction"))) {
+    if ((rc = dev_alloc(&m->d_z, (size_t)n_par, "parameters")) ||
+        (rc = dev_alloc(&m->d_err, 1, "error word"))) {
         nep_destroy(m);
         return rc;
     }
@@ -360,7 +354,6 @@ int nep_destroy(nep_model* m)
     free_workspace(m->ws);
     dev_free(m->d_z);
     dev_free(m->d_err);
-    dev_free(m->d_red);
     dev_free(m->zatom);
     delete m;
     return NEP_OK;
@@ -486,10 +479,9 @@ int compute_efv(nep_model* m, int n, const double* box9, const double* pos, doub
     if ((rc = launch_assemble(aa, nl, n, force, virial_atom, part_v, m->d_err, st, nb2, nc2))) return rc;
     m->prof.end(ps, st);
     if (e_total || virial_total) {
-        if ((rc = launch_reduce(part_e, nb1, 1, m->d_red, st))) return rc;
-        if ((rc = launch_reduce(part_v, nb2, nc2, m->d_red + 1, st))) return rc;
-        k_finish_efv<<<1, 32, 0, st>>>(m->d_red, e_total, virial_total);
-        if ((rc = cuda_fail(cudaGetLastError(), "finish kernel"))) return rc;
+        // the energy and virial totals, straight to the caller
+        const SumSet e{part_e, nb1, 1, 1, 0, e_total}, w{part_v, nb2, 1, nc2, (size_t)nb2, virial_total};
+        if ((rc = launch_sum(e, w, st))) return rc;
     }
     return NEP_OK;
 }
@@ -581,7 +573,7 @@ int nep_heat_current(nep_model* m, int n, const float* virial_atom, const double
         return rc;
     k_heat<<<nb, 256, 0, st>>>(n, virial_atom, vel, m->ws.partials);
     if ((rc = cuda_fail(cudaGetLastError(), "heat-current kernel"))) return rc;
-    return launch_reduce(m->ws.partials, nb, 3, J, st);
+    return launch_sum(SumSet{m->ws.partials, nb, 3, 3, 1, J}, SumSet{}, st);
 }
 
 }  // extern "C"

@@ -166,6 +166,7 @@ __host__ __device__ __forceinline__ void pair_vector_lo(int code, const float (&
     for (int d = 0; d < 3; ++d) r[d] = diff1_lo(hj[d], lj[d], hi[d], li[d], (float)s[d], b.Lh[d], b.Ll[d], r_lo[d]);
 }
 
+#pragma nv_diag_suppress 550  // the record's last word is loaded and not used
 // FP32 hi/lo positions: one 32-byte record (x, y, z, species number; lo parts
 // x, y, z, 0) per atom, so that a neighbour's coordinates are one sector and
 // one 32-byte load (two 16-byte arrays before: two sectors; an MD step of the
@@ -175,12 +176,12 @@ __host__ __device__ __forceinline__ void load_pos(const float* __restrict__ xr, 
                                                   float& zi)
 {
 #ifdef __CUDA_ARCH__
-    float u, v;
+    float u, pad;
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(h[0]), "=f"(h[1]), "=f"(h[2]), "=f"(u), "=f"(l[0]), "=f"(l[1]), "=f"(l[2]), "=f"(v)
+        : "=f"(h[0]), "=f"(h[1]), "=f"(h[2]), "=f"(u), "=f"(l[0]), "=f"(l[1]), "=f"(l[2]), "=f"(pad)
         : "l"(xr + 8 * (size_t)i));
     zi = u;
-    (void)v;
+    (void)pad;
 #else
     const float* r = xr + 8 * (size_t)i;
     for (int d = 0; d < 3; ++d) {
@@ -191,6 +192,7 @@ __host__ __device__ __forceinline__ void load_pos(const float* __restrict__ xr, 
 #endif
 }
 
+#pragma nv_diag_default 550
 __host__ __device__ __forceinline__ void load_pos(const float* __restrict__ xr, int i, float (&h)[3], float (&l)[3])
 {
     float zi;
@@ -257,10 +259,10 @@ __device__ __forceinline__ double warp_sum_multi(const double (&v)[K])
     return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
 }
 
-// Block-wide sum of K doubles; thread 0 writes out[k].  blockDim.x must be a
+// Block-wide sum of K doubles; writes out[k * stride].  blockDim.x must be a
 // multiple of 32 and at most 1024.
 template <int K>
-__device__ __forceinline__ void block_sum_store(double (&v)[K], double* __restrict__ out)
+__device__ __forceinline__ void block_sum_store(double (&v)[K], double* __restrict__ out, size_t stride = 1)
 {
     __shared__ double red[32][K];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -275,7 +277,7 @@ __device__ __forceinline__ void block_sum_store(double (&v)[K], double* __restri
 #pragma unroll
             for (int k = 0; k < K; ++k) w[k] = lane < nw ? red[lane][k] : 0.0;
             const double t = warp_sum_multi<K>(w);
-            if ((lane & 1) == 0 && c < K) out[c] = t;
+            if ((lane & 1) == 0 && c < K) out[c * stride] = t;
         }
     } else {
 #pragma unroll
@@ -292,10 +294,32 @@ __device__ __forceinline__ void block_sum_store(double (&v)[K], double* __restri
                 double s = lane < nw ? red[lane][k] : 0.0;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) out[k] = s;
+                if (lane == 0) out[k * stride] = s;
             }
         }
     }
+}
+
+// Sum over b < nb of src[b stride] by the THREADS threads of a block, in a
+// fixed order: each thread a fixed stride of the values (eight loads in flight
+// ahead of the ordered adds), a shuffle tree, the warps in order.  Thread 0
+// returns it.
+template <int THREADS>
+__device__ __forceinline__ double sum_partials(const double* __restrict__ src, int nb, int stride)
+{
+    __shared__ double wsum[THREADS / 32];
+    double v = 0.0;
+#pragma unroll 8
+    for (int b = threadIdx.x; b < nb; b += THREADS) v += src[(size_t)b * stride];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int q = 0; q < THREADS / 32; ++q) t += wsum[q];
+    return t;
 }
 
 // ---------------------------------------------------------------- workspace
@@ -364,11 +388,17 @@ struct ForceArgs {
 // allocation-free call need the first.
 inline bool sizes_default(const nep_hyper& h) { return h.n_max_R == kNR - 1 && h.n_max_A == kNA - 1; }
 inline bool sizes_split(const nep_hyper& h) { return h.n_max_R == 12 && h.n_max_A == 6; }
-// the site pass runs kSiteAtomsPerBlock atoms per block (one lane each); its
-// per-block energy partials need site_blocks(n) slots, which also bounds the
-// block counts of the assembly and of the plain comparator
-constexpr int kSiteAtomsPerBlock = 32;
-inline int site_blocks(int n) { return (n + kSiteAtomsPerBlock - 1) / kSiteAtomsPerBlock; }
+// Atoms per 128-thread block of the site pass and the assembly: 8 or 16 while
+// one wave of blocks (152 SMs x 5) holds them all, else 32.  More threads per
+// atom shorten a block's run, fewer waste less (harmonics evaluated by every
+// lane of an atom, narrower rows).  Site pass with 8 / 16 / 32 atoms per block:
+// 512 atoms 10.7 / 13.8 / 20.4 us, 5832 atoms 17.3 / 18.2 / 24.0, 8000 atoms
+// 25.8 / 21.5 / 24.3, 13824 atoms 37.9 / 33.5 / 28.9, 32768 atoms 79 / 62 / 57.
+constexpr int kSiteWave = 152 * 5;
+constexpr int site_atoms_per_block(int n) { return n <= 8 * kSiteWave ? 8 : n <= 16 * kSiteWave ? 16 : 32; }
+// blocks of the site pass (its per-block energy partials), which also bounds
+// the block counts of the assembly and of the plain comparator
+constexpr int site_blocks(int n) { return (n + site_atoms_per_block(n) - 1) / site_atoms_per_block(n); }
 int launch_site_partial_forces(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, double* e_partials,
                                unsigned* d_err, cudaStream_t st, int& nblocks);
 struct AssembleArgs {
@@ -382,7 +412,15 @@ struct AssembleArgs {
 };
 int launch_assemble(const AssembleArgs& a, NeighborList& nl, int n, float* force, float* virial_atom,
                     double* partials, unsigned* d_err, cudaStream_t st, int& nblocks, int& ncomp);
-int launch_reduce(const double* partials, int nblocks, int ncomp, double* out, cudaStream_t st);
+// ncomp totals: out[w] = the sum over b < nb of src[w cstride + b bstride]
+// (out NULL: none)
+struct SumSet {
+    const double* src = nullptr;
+    int nb = 0, bstride = 1, ncomp = 0;
+    size_t cstride = 0;
+    double* out = nullptr;
+};
+int launch_sum(const SumSet& a, const SumSet& b, cudaStream_t st);
 // the plain FP32 comparator (nep_plain.cu): descriptors, network and partial
 // forces by the literal formulas, q and G [32][n] scratch
 int launch_plain_site(const ForceArgs& a, NeighborList& nl, int n, float* q, float* G, double* e_atom,
@@ -473,7 +511,6 @@ struct nep_model {
     int n_par = 0;
     float* d_z = nullptr;
     unsigned* d_err = nullptr;   // latched device error bits
-    double* d_red = nullptr;     // reduction outputs (32 doubles)
     nep::Workspace ws;
     float* zatom = nullptr;      // species numbers of the atoms (nep_set_species), or NULL
     int zatom_n = 0;

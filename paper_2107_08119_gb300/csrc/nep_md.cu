@@ -311,30 +311,18 @@ constexpr int kFinishThreads = 128;
 
 __global__ void __launch_bounds__(kFinishThreads) k_md_finish(const double* __restrict__ part_e, int nb_e,
                                                               const double* __restrict__ part_x, int nb_x,
-                                                              int ncomp_x, int off_x, double* __restrict__ red,
+                                                              int bstride_x, size_t cstride_x, int off_x,
+                                                              double* __restrict__ red,
                                                               double* __restrict__ thermo, double* __restrict__ heat,
                                                               unsigned* __restrict__ ctl, double t0, double tau,
                                                               double dt, double dof_kb)
 {
     // red: [0] E_pot, [1..9] W (row-major), [10] E_kin, [11..13] J, [14] lambda
-    const int w = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const double* src = w == 0 ? part_e : part_x + (w - 1);
-    const int nb = w == 0 ? nb_e : nb_x;
-    const int stride = w == 0 ? 1 : ncomp_x;
-    double v = 0.0;
-    // unrolled so that eight loads are in flight ahead of the (ordered) adds
-#pragma unroll 8
-    for (int b = threadIdx.x; b < nb; b += kFinishThreads) v += src[(size_t)b * stride];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __shared__ double wsum[kFinishThreads / 32];
+    const int w = blockIdx.x;
+    const double t = w == 0 ? sum_partials<kFinishThreads>(part_e, nb_e, 1)
+                            : sum_partials<kFinishThreads>(part_x + (w - 1) * cstride_x, nb_x, bstride_x);
     __shared__ int last;
-    if (lane == 0) wsum[warp] = v;
-    __syncthreads();
     if (threadIdx.x == 0) {
-        double t = 0.0;
-#pragma unroll
-        for (int q = 0; q < kFinishThreads / 32; ++q) t += wsum[q];
         red[w == 0 ? 0 : off_x + w - 1] = t;
         __threadfence();  // this sum before the count
         last = atomicAdd(ctl + kCtlFinish, 1u) == gridDim.x - 1;
@@ -721,7 +709,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
     const int nb = site_blocks(n);
     double* part_e = md->ws.partials;
     double* part_a = md->ws.partials + ((nb + 7) / 8) * 8;
-    double* part_h = part_a + 13 * (size_t)blocks_for(n, 128);  // HNEMD kick partials
+    double* part_h = part_a + 13 * (size_t)nb;  // HNEMD kick partials
     const bool drive = md->drive;
     const int nbk = blocks_for(n, 256);
     const double kef = 0.5 * md->mass * kAmuA2Fs2InEv;
@@ -765,7 +753,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             return rc;
         if (drive) {
             // the starting forces include the driving force (no kick: hdt/m = 0)
-            if ((rc = launch_reduce(part_a, b2, c2, md->red + 1, st))) return rc;
+            if ((rc = launch_sum(SumSet{part_a, b2, 1, c2, (size_t)b2, md->red + 1}, SumSet{}, st))) return rc;
             k_hnemd_kick<<<nbk, 256, 0, st>>>(n, md->ws.force, md->w_atom, vel, md->fe[0], md->fe[1], md->fe[2],
                                               md->red + 1, 1.0 / n, 0.0, kef, part_h, m->d_err);
         }
@@ -816,13 +804,13 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         Profiler::Slot* pk = m->prof.begin(NEP_PROFILE_STEP, q);
         if (drive) {
             // the kick needs the total virial first
-            if ((r = launch_reduce(part_a, b2, c2, md->red + 1, q))) return r;
+            if ((r = launch_sum(SumSet{part_a, b2, 1, c2, (size_t)b2, md->red + 1}, SumSet{}, q))) return r;
             k_hnemd_kick<<<nbk, 256, 0, q>>>(n, md->ws.force, w_out, vel, md->fe[0], md->fe[1], md->fe[2],
                                              md->red + 1, 1.0 / n, hdtm, kef, part_h, m->d_err);
-            k_md_finish<<<5, kFinishThreads, 0, q>>>(part_e, b1, part_h, nbk, 4, 10, md->red, thermo, heat, md->ctl,
+            k_md_finish<<<5, kFinishThreads, 0, q>>>(part_e, b1, part_h, nbk, 4, 1, 10, md->red, thermo, heat, md->ctl,
                                                      md->t0, md->tau, dt, dof_kb);
         } else {
-            k_md_finish<<<1 + c2, kFinishThreads, 0, q>>>(part_e, b1, part_a, b2, c2, 1, md->red, thermo, heat,
+            k_md_finish<<<1 + c2, kFinishThreads, 0, q>>>(part_e, b1, part_a, b2, 1, (size_t)b2, 1, md->red, thermo, heat,
                                                           md->ctl, md->t0, md->tau, dt, dof_kb);
         }
         if (sample) {  // v is that of J: after the second half kick, before the thermostat

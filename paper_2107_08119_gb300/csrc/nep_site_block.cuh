@@ -27,17 +27,26 @@
 
 namespace nep {
 
-constexpr int kSiteAtoms = kSiteAtomsPerBlock;  // one lane per atom
 constexpr int kSiteWarps = 4;
 constexpr int kSiteThreads = 32 * kSiteWarps;
 constexpr int kSiteChunk = 16;  // slots per shared tile
-static_assert(kSiteAtoms == 32, "one lane per atom of the block");
+
+// A block takes AT = 32, 16 or 8 atoms: lane l works on atom l mod AT, and the
+// 32 / AT lanes of an atom in a warp ("subs") split what the warps split once
+// more (slots, neurons, quarters of G; within a harmonic or radial role the
+// radial orders).
+template <int AT>
+struct SiteSplit {
+    static constexpr int SUB = 32 / AT;
+    static constexpr int WAYS = kSiteWarps * SUB;  // threads per atom
+    static_assert(kSiteChunk % WAYS == 0, "every thread takes the same number of slots of a tile");
+};
 
 // Marks a tile entry outside the cutoff: both a Chebyshev argument and a
 // component of a unit vector lie in [-1, 1].
 constexpr float kNoPair = 2.f;
 
-// float4 words per lane of the region that holds first the pair tile, then
+// float4 words per atom of the region that holds first the pair tile, then
 // the harmonic sums S and the coefficients A
 template <class D>
 __host__ __device__ constexpr int site_block_quads()
@@ -47,22 +56,22 @@ __host__ __device__ constexpr int site_block_quads()
 
 // Place of S_nlm (and A_nlm) in a lane's column: harmonics in pairs (2j, 2j + 1)
 // side by side, so that one 8-byte operand of a packed FMA holds both, the
-// radial orders of a pair next to each other; 16-byte words are lane-minor
-// ([word][32 lanes]).
-template <class D>
+// radial orders of a pair next to each other; 16-byte words are atom-minor
+// ([word][AT atoms]).
+template <class D, int AT>
 __host__ __device__ constexpr int site_block_at(int n, int lm)
 {
     const int f = 2 * ((lm >> 1) * D::NA + n) + (lm & 1);
-    return (f >> 2) * 128 + (f & 3);
+    return (f >> 2) * 4 * AT + (f & 3);
 }
 
 // shared memory: weights | tile / S / A | q / G | radial tile / neuron states and slopes | mask words
-template <class D>
+template <class D, int AT>
 __host__ __device__ inline size_t site_block_smem(int n_par, int n_neu)
 {
     const size_t x_rows = 2 * (n_neu > kSiteChunk ? n_neu : kSiteChunk);
     return sizeof(float) * (((size_t)n_par + 31) / 32 * 32 +
-                            (size_t)kSiteAtoms * (4 * site_block_quads<D>() + D::Ndes + x_rows + 3));
+                            (size_t)AT * (4 * site_block_quads<D>() + D::Ndes + x_rows + 3));
 }
 
 // Whether component a of the gradient of harmonic lm is zero for every
@@ -117,22 +126,27 @@ __device__ __forceinline__ void sh_add(const ShFast& s, float cg, float cd, floa
 }
 
 // Harmonic sums of lm in [LO, LO + 8) over the tile's slots, last slot first:
-// S[j][n] = (S_n,LO+2j, S_n,LO+2j+1).  slots: those with a pair in any lane.
-template <class D, int LO>
-__device__ __forceinline__ void site_block_harmonics(const float* tile, unsigned slots, float2 (&S)[4][D::NA])
+// S[j][o] = (S_n,LO+2j, S_n,LO+2j+1) for the orders n = sub + SUB o (an order
+// past the last repeats it and is not stored).  slots: those with a pair in
+// any lane.
+template <class D, int AT, int LO, int NO>
+__device__ __forceinline__ void site_block_harmonics(const float* tile, int sub, unsigned slots, float2 (&S)[4][NO])
 {
-    constexpr int row = kSiteChunk * 32;
+    constexpr int row = kSiteChunk * AT;
 #pragma unroll 1
     while (slots) {
         const int s = 31 - __clz((int)slots);
         slots ^= 1u << s;
-        const float* t = tile + s * 32;
+        const float* t = tile + s * AT;
         const float x = t[0];
         if (x > 1.5f) continue;  // kNoPair
         const float y = t[row], z = t[2 * row];
-        float2 g[D::NA];
+        float2 g[NO];
 #pragma unroll
-        for (int n = 0; n < D::NA; ++n) g[n] = bcast2(t[(3 + n) * row]);
+        for (int o = 0; o < NO; ++o) {
+            const int n = sub + SiteSplit<AT>::SUB * o;
+            g[o] = bcast2(t[(3 + (n < D::NA ? n : D::NA - 1)) * row]);
+        }
         float Y[8];
         NEP_SH_LOCALS(x, y, z)
 #define NEP_T(lm, Yv, gx, gy, gz) \
@@ -142,41 +156,39 @@ __device__ __forceinline__ void site_block_harmonics(const float* tile, unsigned
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int n = 0; n < D::NA; ++n) S[j][n] = ffma2(make_float2(Y[2 * j], Y[2 * j + 1]), g[n], S[j][n]);
+            for (int o = 0; o < NO; ++o) S[j][o] = ffma2(make_float2(Y[2 * j], Y[2 * j + 1]), g[o], S[j][o]);
     }
 }
 
-// The descriptors q_nl of order n from the harmonic sums in the lane's column
+// The descriptors q_nl of order n from the harmonic sums in the atom's column
 // (compensated over m, as in site_descriptors)
-template <class D>
+template <class D, int AT>
 __device__ __forceinline__ void site_block_descriptors(int n, const float* s_S, float* s_q)
 {
     float q[kLmax] = {0.f, 0.f, 0.f, 0.f}, qc[kLmax] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int m = 0; m < kLM; ++m) {
         const int l = sh_l(m);
-        const int f = 2 * ((m >> 1) * D::NA + n) + (m & 1);  // site_block_at
-        const float h = s_S[(f >> 2) * 128 + (f & 3)];
+        const float h = s_S[site_block_at<D, AT>(n, m)];
         const float y = fmaf(sh_c(m) * h, h, -qc[l]);
         const float t = q[l] + y;
         qc[l] = (t - q[l]) - y;
         q[l] = t;
     }
 #pragma unroll
-    for (int l = 0; l < kLmax; ++l) s_q[(D::NR + n * kLmax + l) * 32] = q[l] - qc[l];
+    for (int l = 0; l < kLmax; ++l) s_q[(D::NR + n * kLmax + l) * AT] = q[l] - qc[l];
 }
 
-// A_nlm = 2 c_lm G_nl S_nlm in place, order n of the lane's column
-template <class D>
+// A_nlm = 2 c_lm G_nl S_nlm in place, order n of the atom's column
+template <class D, int AT>
 __device__ __forceinline__ void site_block_coefficients(int n, float* s_A, const float* s_G)
 {
     float g[kLmax];
 #pragma unroll
-    for (int l = 0; l < kLmax; ++l) g[l] = s_G[(D::NR + n * kLmax + l) * 32];
+    for (int l = 0; l < kLmax; ++l) g[l] = s_G[(D::NR + n * kLmax + l) * AT];
 #pragma unroll
     for (int m = 0; m < kLM; ++m) {
-        const int f = 2 * ((m >> 1) * D::NA + n) + (m & 1);  // site_block_at
-        float* a = s_A + (f >> 2) * 128 + (f & 3);
+        float* a = s_A + site_block_at<D, AT>(n, m);
         *a = *a * (2.f * sh_c(m) * g[sh_l(m)]);
     }
 }
@@ -209,8 +221,8 @@ __device__ __forceinline__ void site_pair_geometry(const NbRecord& nb, const Box
     g.w = pair_weight(P, zi, nb.z);
 }
 
-// radial part of dU/dd (0 beyond the radial cutoff); s_G: the lane's column of G
-template <class D>
+// radial part of dU/dd (0 beyond the radial cutoff); s_G: the atom's column of G
+template <class D, int AT>
 __device__ __forceinline__ float site_pair_radial(const PairGeom& g, const SiteParams& P, const float* s_G)
 {
     float radial = 0.f;
@@ -218,7 +230,7 @@ __device__ __forceinline__ float site_pair_radial(const PairGeom& g, const SiteP
         float2 gd[D::NR];
         radial_gd<D::NR>(g.d, P.rcR, P.inv_rcR, gd, g.w);
 #pragma unroll
-        for (int a = 0; a < D::NR; ++a) radial = fmaf(s_G[a * 32], gd[a].y, radial);
+        for (int a = 0; a < D::NR; ++a) radial = fmaf(s_G[a * AT], gd[a].y, radial);
     }
     return radial;
 }
@@ -227,7 +239,7 @@ __device__ __forceinline__ float site_pair_radial(const PairGeom& g, const SiteP
 // sh_pass2): (cg, cd) = sum_n A_nlm (g_n, g_n'), B += cd Y, V += cg grad_u Y,
 // two harmonics per packed FMA.  Gradient components that are zero for every
 // direction (a third of them) are left out.  gg, gp: (g_n, g_n), (g_n', g_n').
-template <class D, int J>
+template <class D, int AT, int J>
 __device__ __forceinline__ void site_angular_terms(const float* s_A, const ShFast& sh, const float2 (&gg)[D::NA],
                                                    const float2 (&gp)[D::NA], float& B, float (&V)[3])
 {
@@ -235,20 +247,21 @@ __device__ __forceinline__ void site_angular_terms(const float* s_A, const ShFas
         float2 cg = make_float2(0.f, 0.f), cd = make_float2(0.f, 0.f);
 #pragma unroll
         for (int n = 0; n < D::NA; ++n) {
-            const float2 A = *reinterpret_cast<const float2*>(s_A + site_block_at<D>(n, 2 * J));
+            const float2 A = *reinterpret_cast<const float2*>(s_A + site_block_at<D, AT>(n, 2 * J));
             cg = ffma2(A, gg[n], cg);
             cd = ffma2(A, gp[n], cd);
         }
         sh_add<2 * J>(sh, cg.x, cd.x, B, V);
         sh_add<2 * J + 1>(sh, cg.y, cd.y, B, V);
-        site_angular_terms<D, J + 1>(s_A, sh, gg, gp, B, V);
+        site_angular_terms<D, AT, J + 1>(s_A, sh, gg, gp, B, V);
     }
 }
 
 // The site pass of the block's atoms.  z: the parameters; pf: partial-force
 // records [k][n] float4; mask: in-cutoff bits [3][n] of the first 96 slots,
-// or NULL.  Warp 0 returns the site energies (hi + lo).
-template <class D, int WORDS>
+// or NULL.  WORDS: 32-bit words of own-slot bits per thread.  The first AT
+// lanes of warp 0 return the site energies (hi + lo).
+template <class D, int AT, int WORDS>
 __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, const int* __restrict__ nbr,
                                            const float* __restrict__ xr, const Box& box,
                                            const float* __restrict__ z, int n_par, SiteParams P,
@@ -256,17 +269,22 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
                                            float& U_lo)
 {
     constexpr int NR = D::NR, NA = D::NA, ND = D::Ndes;
+    constexpr int SUB = SiteSplit<AT>::SUB, WAYS = SiteSplit<AT>::WAYS;
+    constexpr int OWN = kSiteChunk / WAYS;  // slots of a tile per thread
     extern __shared__ __align__(16) float s_site[];
-    __shared__ float s_dU[kSiteWarps][32];
+    __shared__ float s_dU[WAYS][AT];
     __shared__ unsigned s_any[kSiteChunk];  // per tile slot: 1 an angular pair in some lane, 2 a radial one
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int at = lane % AT, sub = lane / AT;
+    const int way = SUB * warp + sub;  // this thread's share of the atom's work
     float* s_w = s_site;
-    float* s_A = s_w + (n_par + 31) / 32 * 32;         // [quads][32] float4
-    float* s_q = s_A + 128 * site_block_quads<D>();    // [ND][32]
-    float* s_x = s_q + 32 * ND;                        // radial tile; then x_mu, w2 (1 - x_mu^2): [n_neu][32][2]
-    unsigned* s_mask = reinterpret_cast<unsigned*>(s_x + 64 * (P.n_neu > kSiteChunk ? P.n_neu : kSiteChunk));
+    float* s_A = s_w + (n_par + 31) / 32 * 32;         // [quads][AT] float4
+    float* s_q = s_A + 4 * AT * site_block_quads<D>();  // [ND][AT]
+    float* s_x = s_q + AT * ND;                        // radial tile; then x_mu, w2 (1 - x_mu^2): [n_neu][AT][2]
+    unsigned* s_mask = reinterpret_cast<unsigned*>(s_x + 2 * AT * (P.n_neu > kSiteChunk ? P.n_neu : kSiteChunk));
     for (int t = threadIdx.x; t < n_par; t += kSiteThreads) s_w[t] = z[t];
-    if (threadIdx.x < 96) s_mask[threadIdx.x] = 0u;
+    if (threadIdx.x < 3 * AT) s_mask[threadIdx.x] = 0u;
+    if (threadIdx.x < kSiteChunk) s_any[threadIdx.x] = 0u;
     P.w = s_w;
     const int ia = active ? i : 0;
     float hi[3], li[3], zi;
@@ -275,7 +293,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
     const int chunks = (kmax + kSiteChunk - 1) / kSiteChunk;
     const float rc2max = P.rcR2 > P.rcA2 ? P.rcR2 : P.rcA2;
 
-    // own slots k = 4 b + warp: bit b of word b / 32 in kept (within either
+    // own slots k = WAYS b + way: bit b of word b / 32 in kept (within either
     // cutoff) and ang (within the angular one)
     unsigned kept[WORDS], ang[WORDS];
 #pragma unroll
@@ -285,21 +303,22 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
     {
         // this warp's sums: harmonics 8 warp .. 8 warp + 7 (warps 0-2), or the
         // radial orders in pairs with their negated compensations (warp 3)
-        constexpr int NR2 = (NR + 1) / 2;
-        static_assert(2 * NR2 <= 4 * NA, "the radial sums fit the harmonic sums' registers");
-        float2 S[4][NA];
+        constexpr int NO = (NA + SUB - 1) / SUB;             // angular orders per thread
+        constexpr int NP = ((NR + 1) / 2 + SUB - 1) / SUB;   // pairs of radial orders per thread
+        static_assert(2 * NP <= 4 * NO, "the radial sums fit the harmonic sums' registers");
+        float2 S[4][NO];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int a = 0; a < NA; ++a) S[j][a] = make_float2(0.f, 0.f);
-        float* tile = s_A + lane;
-        float2* tileR = reinterpret_cast<float2*>(s_x) + lane;
+            for (int o = 0; o < NO; ++o) S[j][o] = make_float2(0.f, 0.f);
+        float* tile = s_A + at;
+        float2* tileR = reinterpret_cast<float2*>(s_x) + at;
         // the thread's slots in turn: k_of(0) is its first of the last tile;
         // a record is loaded one slot ahead and its list value two ahead
-        auto k_of = [&](int q) { return (chunks - 1 - (q >> 2)) * kSiteChunk + 4 * (q & 3) + warp; };
+        auto k_of = [&](int q) { return (chunks - 1 - q / OWN) * kSiteChunk + WAYS * (q % OWN) + way; };
         auto load_v = [&](int q) {
             const int k = k_of(q);
-            return q < 4 * chunks && k < cnt ? nbr[(size_t)k * n + ia] : -1;
+            return q < OWN * chunks && k < cnt ? nbr[(size_t)k * n + ia] : -1;
         };
         auto load_record = [&](int v, NbRecord& r) {
             r.v = v;
@@ -308,11 +327,12 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
         NbRecord nx;
         load_record(load_v(0), nx);
         int v_nx = load_v(1);
+        __syncthreads();  // s_any and s_mask are zero, the weights loaded
 #pragma unroll 1
         for (int c = chunks - 1, q = 0; c >= 0; --c) {
 #pragma unroll 1
-            for (int t = 0; t < kSiteChunk / kSiteWarps; ++t, ++q) {
-                const int s = 4 * t + warp;
+            for (int t = 0; t < OWN; ++t, ++q) {
+                const int s = WAYS * t + way;
                 const NbRecord cur = nx;
                 load_record(v_nx, nx);
                 v_nx = load_v(q + 2);
@@ -322,57 +342,69 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
                     pair_vector(cur.v >> 24, hi, li, cur.h, cur.l, box, rx, ry, rz);
                     const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
                     if (d2 < rc2max) {
-                        const int b = 4 * c + t;
+                        const int b = OWN * c + t;
                         const float w = pair_weight(P, zi, cur.z);
                         const float d = sqrtf(d2);
 #pragma unroll
-                        for (int q = 0; q < WORDS; ++q)
-                            if (WORDS == 1 || (b >> 5) == q) kept[q] |= 1u << (b & 31);
+                        for (int w32 = 0; w32 < WORDS; ++w32)
+                            if (WORDS == 1 || (b >> 5) == w32) kept[w32] |= 1u << (b & 31);
                         if (d2 < P.rcR2) radial_x(d, P.rcR, P.inv_rcR, w, x, fc);
                         if (d2 < P.rcA2) {
 #pragma unroll
-                            for (int q = 0; q < WORDS; ++q)
-                                if (WORDS == 1 || (b >> 5) == q) ang[q] |= 1u << (b & 31);
+                            for (int w32 = 0; w32 < WORDS; ++w32)
+                                if (WORDS == 1 || (b >> 5) == w32) ang[w32] |= 1u << (b & 31);
                             float g[NA], uy, uz;
                             radial_g<NA>(d, P.rcA, P.inv_rcA, g, w);
                             unit_vector(rx, ry, rz, ux, uy, uz);
-                            tile[(kSiteChunk + s) * 32] = uy;
-                            tile[(2 * kSiteChunk + s) * 32] = uz;
+                            tile[(kSiteChunk + s) * AT] = uy;
+                            tile[(2 * kSiteChunk + s) * AT] = uz;
 #pragma unroll
-                            for (int a = 0; a < NA; ++a) tile[((3 + a) * kSiteChunk + s) * 32] = g[a];
+                            for (int a = 0; a < NA; ++a) tile[((3 + a) * kSiteChunk + s) * AT] = g[a];
                         }
                     }
                 }
-                tile[s * 32] = ux;
-                tileR[s * 32] = make_float2(x, fc);
-                const unsigned any_a = __any_sync(0xffffffffu, ux < 1.5f), any_r = __any_sync(0xffffffffu, x < 1.5f);
-                if (lane == 0) s_any[s] = (any_a ? 1u : 0u) | (any_r ? 2u : 0u);
+                tile[s * AT] = ux;
+                tileR[s * AT] = make_float2(x, fc);
+                // a slot's lanes lie in one warp: its first lane keeps the flags
+                const unsigned any_a = __ballot_sync(0xffffffffu, ux < 1.5f);
+                const unsigned any_r = __ballot_sync(0xffffffffu, x < 1.5f);
+                if (at == 0) {
+                    const unsigned m = AT == 32 ? 0xffffffffu : (1u << (AT & 31)) - 1u;
+                    s_any[s] = ((any_a >> (sub * AT % 32)) & m ? 1u : 0u) | ((any_r >> (sub * AT % 32)) & m ? 2u : 0u);
+                }
             }
             __syncthreads();
             unsigned slots = __ballot_sync(0xffffffffu, lane < kSiteChunk && (s_any[lane & (kSiteChunk - 1)] &
                                                                               (warp < 3 ? 1u : 2u)) != 0u);
             if (warp == 0) {
-                site_block_harmonics<D, 0>(tile, slots, S);
+                site_block_harmonics<D, AT, 0>(tile, sub, slots, S);
             } else if (warp == 1) {
-                site_block_harmonics<D, 8>(tile, slots, S);
+                site_block_harmonics<D, AT, 8>(tile, sub, slots, S);
             } else if (warp == 2) {
-                site_block_harmonics<D, 16>(tile, slots, S);
+                site_block_harmonics<D, AT, 16>(tile, sub, slots, S);
             } else {
                 const float2 minus = make_float2(-1.f, -1.f);
 #pragma unroll 1
                 while (slots) {
                     const int s = 31 - __clz((int)slots);
                     slots ^= 1u << s;
-                    const float2 xf = tileR[s * 32];
+                    const float2 xf = tileR[s * AT];
                     if (xf.x > 1.5f) continue;  // kNoPair
-                    float g[NR];
-                    cheb_g<NR>(xf.x, xf.y, g);
+                    float g[NR + 1];
+                    float(&gn)[NR] = reinterpret_cast<float(&)[NR]>(g);
+                    cheb_g<NR>(xf.x, xf.y, gn);
+                    g[NR] = 0.f;
                     // Kahan: y = g - c, t = R + y, c = (t - R) - y with -c kept
 #pragma unroll
-                    for (int p = 0; p < NR2; ++p) {
-                        float2& R = S[(2 * p) / NA][(2 * p) % NA];
-                        float2& nc = S[(2 * p + 1) / NA][(2 * p + 1) % NA];
-                        const float2 y = fadd2(make_float2(g[2 * p], 2 * p + 1 < NR ? g[2 * p + 1] : 0.f), nc);
+                    for (int o = 0; o < NP; ++o) {
+                        float2 gp = make_float2(g[2 * o * SUB], g[2 * o * SUB + 1]);
+#pragma unroll
+                        for (int u = 1; u < SUB; ++u)
+                            if (2 * (o * SUB + u) < NR && sub == u)
+                                gp = make_float2(g[2 * (o * SUB + u)], g[2 * (o * SUB + u) + 1]);
+                        float2& R = S[(2 * o) / NO][(2 * o) % NO];
+                        float2& nc = S[(2 * o + 1) / NO][(2 * o + 1) % NO];
+                        const float2 y = fadd2(gp, nc);
                         const float2 t = fadd2(R, y);
                         nc = fadd2(y, ffma2(t, minus, R));
                         R = t;
@@ -385,60 +417,71 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    const int f = 2 * (j * NA + a);  // site_block_at<D>(a, 8 warp + 2 j)
-                    *reinterpret_cast<float2*>(s_A + (warp * 2 * NA + (f >> 2)) * 128 + 4 * lane + (f & 3)) = S[j][a];
+                for (int o = 0; o < NO; ++o) {
+                    const int a = sub + SUB * o;
+                    const int f = 2 * ((4 * warp + j) * NA + a);  // site_block_at(a, 8 warp + 2 j)
+                    if (a < NA)
+                        *reinterpret_cast<float2*>(s_A + (f >> 2) * 4 * AT + 4 * at + (f & 3)) = S[j][o];
                 }
         } else {
 #pragma unroll
-            for (int a = 0; a < NR; ++a) {
-                const float2 R = S[(a & ~1) / NA][(a & ~1) % NA], nc = S[(a | 1) / NA][(a | 1) % NA];
-                s_q[a * 32 + lane] = (a & 1) ? R.y + nc.y : R.x + nc.x;
+            for (int o = 0; o < NP; ++o) {
+                const int a = 2 * (o * SUB + sub);
+                const float2 R = S[(2 * o) / NO][(2 * o) % NO], nc = S[(2 * o + 1) / NO][(2 * o + 1) % NO];
+                if (a < NR) s_q[a * AT + at] = R.x + nc.x;
+                if (a + 1 < NR) s_q[(a + 1) * AT + at] = R.y + nc.y;
             }
         }
         if (mask) {
-            // own bits b of word j (slots 32 j + 4 (b - 8 j) + warp)
+            // slot k = WAYS b + way is bit k mod 32 of word k / 32
+            if constexpr (WAYS == 4) {
 #pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                unsigned e = (kept[0] >> (8 * j)) & 0xFFu;
-                e = (e | (e << 12)) & 0x000F000Fu;
-                e = (e | (e << 6)) & 0x03030303u;
-                e = (e | (e << 3)) & 0x11111111u;
-                if (e) atomicOr(s_mask + 32 * j + lane, e << warp);
+                for (int j = 0; j < 3; ++j) {  // own bits 8 j .. 8 j + 7, spread to every fourth
+                    unsigned e = (kept[0] >> (8 * j)) & 0xFFu;
+                    e = (e | (e << 12)) & 0x000F000Fu;
+                    e = (e | (e << 6)) & 0x03030303u;
+                    e = (e | (e << 3)) & 0x11111111u;
+                    if (e) atomicOr(s_mask + j * AT + at, e << way);
+                }
+            } else {
+                for (unsigned m = kept[0]; m; m &= m - 1) {
+                    const int k = WAYS * (__ffs((int)m) - 1) + way;
+                    atomicOr(s_mask + (k >> 5) * AT + at, 1u << (k & 31));
+                }
             }
         }
     }
     __syncthreads();
-    for (int a = warp; a < NA; a += kSiteWarps) site_block_descriptors<D>(a, s_A + 4 * lane, s_q + lane);
-    if (mask && warp < 3 && active) mask[(size_t)warp * n + i] = s_mask[32 * warp + lane];
+    for (int a = way; a < NA; a += WAYS) site_block_descriptors<D, AT>(a, s_A + 4 * at, s_q + at);
+    if (mask && warp < 3 && lane < AT && active) mask[(size_t)warp * n + i] = s_mask[warp * AT + lane];
     __syncthreads();
 
-    // ---- network: neurons mu = warp mod 4
+    // ---- network: neurons mu = way mod WAYS
     const float* b1 = s_w + P.n_neu * ND;
     const float* w2 = b1 + P.n_neu;
-    float2* s_xd = reinterpret_cast<float2*>(s_x) + lane;
+    float2* s_xd = reinterpret_cast<float2*>(s_x) + at;
     {
         float q[ND];
 #pragma unroll
-        for (int a = 0; a < ND; ++a) q[a] = s_q[a * 32 + lane];
+        for (int a = 0; a < ND; ++a) q[a] = s_q[a * AT + at];
 #pragma unroll 1
-        for (int mu = warp; mu < P.n_neu; mu += kSiteWarps) {
+        for (int mu = way; mu < P.n_neu; mu += WAYS) {
             const float x = neuron_state<ND>(s_w + mu * ND, b1[mu], q);
-            s_xd[mu * 32] = make_float2(x, w2[mu] * fmaf(-x, x, 1.f));
+            s_xd[mu * AT] = make_float2(x, w2[mu] * fmaf(-x, x, 1.f));
         }
     }
     __syncthreads();
     {
-        // G_v of a quarter of the descriptors, in s_q
-        constexpr int VB = (ND + kSiteWarps - 1) / kSiteWarps;
-        const int v0 = warp * VB;
-        if constexpr (ND % (4 * kSiteWarps) == 0) {  // 16-byte aligned quarters
+        // G_v of this thread's share of the descriptors, in s_q
+        constexpr int VB = (ND + WAYS - 1) / WAYS;
+        const int v0 = way * VB;
+        if constexpr (ND % (4 * WAYS) == 0) {  // 16-byte aligned shares
             float2 G[VB / 2];
 #pragma unroll
             for (int v = 0; v < VB / 2; ++v) G[v] = make_float2(0.f, 0.f);
 #pragma unroll 2
             for (int mu = 0; mu < P.n_neu; ++mu) {
-                const float2 d = bcast2(s_xd[mu * 32].y);
+                const float2 d = bcast2(s_xd[mu * AT].y);
                 const float4* row = reinterpret_cast<const float4*>(s_w + mu * ND + v0);
 #pragma unroll
                 for (int v = 0; v < VB / 4; ++v) {
@@ -449,16 +492,16 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
             }
 #pragma unroll
             for (int v = 0; v < VB / 2; ++v) {
-                s_q[(v0 + 2 * v) * 32 + lane] = G[v].x;
-                s_q[(v0 + 2 * v + 1) * 32 + lane] = G[v].y;
+                s_q[(v0 + 2 * v) * AT + at] = G[v].x;
+                s_q[(v0 + 2 * v + 1) * AT + at] = G[v].y;
             }
         } else {
             float G[VB];
 #pragma unroll
             for (int v = 0; v < VB; ++v) G[v] = 0.f;
-#pragma unroll 1
+#pragma unroll 2
             for (int mu = 0; mu < P.n_neu; ++mu) {
-                const float d = s_xd[mu * 32].y;
+                const float d = s_xd[mu * AT].y;
                 const float* row = s_w + mu * ND + v0;
 #pragma unroll
                 for (int v = 0; v < VB; ++v)
@@ -466,7 +509,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
             }
 #pragma unroll
             for (int v = 0; v < VB; ++v)
-                if (v0 + v < ND) s_q[(v0 + v) * 32 + lane] = G[v];
+                if (v0 + v < ND) s_q[(v0 + v) * AT + at] = G[v];
         }
     }
     __syncthreads();
@@ -474,21 +517,22 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
     // ---- coefficients A (warps 1-3) and the compensated output sum (warp 0)
     if (warp == 0) {
         float s = 0.f, c = 0.f;
-        for (int mu = 0; mu < P.n_neu; ++mu) neuron_energy(w2[mu], s_xd[mu * 32].x, s, c);
+        for (int mu = 0; mu < P.n_neu; ++mu) neuron_energy(w2[mu], s_xd[mu * AT].x, s, c);
         float t, e;
         two_sum(s, -w2[P.n_neu], t, e);
         U_hi = t;
         U_lo = c + e;
     } else {
-        for (int a = warp - 1; a < NA; a += kSiteWarps - 1) site_block_coefficients<D>(a, s_A + 4 * lane, s_q + lane);
+        for (int a = way - SUB; a < NA; a += WAYS - SUB)
+            site_block_coefficients<D, AT>(a, s_A + 4 * at, s_q + at);
     }
     __syncthreads();
 
     // ---- partial forces of the own slots, and the first-order energy
     // correction of the pair geometry's roundings (nep_site.cuh)
     float dU = 0.f;
-    const float* sA = s_A + 4 * lane;
-    const float* sG = s_q + lane;
+    const float* sA = s_A + 4 * at;
+    const float* sG = s_q + at;
     float4* out = reinterpret_cast<float4*>(pf) + ia;
     // the next own slot, the angular pairs of a word before the others: k, or
     // -1; its list value is loaded two pairs ahead, the record one ahead
@@ -500,7 +544,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
                 const int b = __ffs((int)(angular ? ang[w] : kept[w])) - 1;
                 ang[w] &= ~(1u << b);
                 kept[w] &= ~(1u << b);
-                return 4 * (32 * w + b) + warp;
+                return WAYS * (32 * w + b) + way;
             }
         return -1;
     };
@@ -523,7 +567,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
             if (k_n2 >= 0) v_n2 = nbr[(size_t)k_n2 * n + ia];
             PairGeom g;
             site_pair_geometry(nb, box, P, hi, li, zi, g);
-            float radial = site_pair_radial<D>(g, P, sG);
+            float radial = site_pair_radial<D, AT>(g, P, sG);
             float V[3] = {0.f, 0.f, 0.f};
             float eu = 0.f;
             if (angular) {
@@ -539,7 +583,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
                 }
                 ShFast sh;
                 sh.set(g.u[0], g.u[1], g.u[2]);
-                site_angular_terms<D, 0>(sA, sh, gg, gp, radial, V);
+                site_angular_terms<D, AT, 0>(sA, sh, gg, gp, radial, V);
                 eu = fmaf(V[0], g.du[0], fmaf(V[1], g.du[1], V[2] * g.du[2]));
                 // tangential projection of V, divided by r
                 const float uv = fmaf(g.u[0], V[0], fmaf(g.u[1], V[1], g.u[2] * V[2]));
@@ -557,9 +601,18 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
             nb_nx.v = v_n2;
         }
     }
-    s_dU[warp][lane] = dU;
+    s_dU[way][at] = dU;
     __syncthreads();
-    if (warp == 0) U_lo += (s_dU[0][lane] + s_dU[1][lane]) + (s_dU[2][lane] + s_dU[3][lane]);
+    if (warp == 0) {
+        float t[WAYS];
+#pragma unroll
+        for (int w = 0; w < WAYS; ++w) t[w] = s_dU[w][at];
+#pragma unroll
+        for (int h = WAYS / 2; h >= 1; h >>= 1)
+#pragma unroll
+            for (int w = 0; w < h; ++w) t[w] += t[w + h];
+        U_lo += t[0];
+    }
 }
 
 }  // namespace nep

@@ -27,7 +27,7 @@ namespace {
 constexpr int kStaticAtoms = NEP_STATIC_MAX_ATOMS;
 constexpr int kStaticSlots = NEP_STATIC_MAX_NEIGHBORS;
 constexpr int kStaticCells = NEP_STATIC_MAX_CELLS;
-constexpr int kStaticBlocks = (kStaticAtoms + kSiteAtomsPerBlock - 1) / kSiteAtomsPerBlock;
+constexpr int kStaticBlocks = (kStaticAtoms + 7) / 8;  // the most blocks a site pass of that many atoms has
 
 constexpr size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
@@ -43,9 +43,9 @@ constexpr size_t kOffCellAtoms = kOffAtomCell + align256(sizeof(int) * kStaticAt
 constexpr size_t kOffCellCount = kOffCellAtoms + align256(sizeof(int) * kStaticAtoms);
 constexpr size_t kOffCellStart = kOffCellCount + align256(sizeof(int) * (kStaticCells + 1));
 constexpr size_t kOffCellFill = kOffCellStart + align256(sizeof(int) * (kStaticCells + 1));
-constexpr size_t kOffPartials = kOffCellFill + align256(sizeof(int) * (kStaticCells + 1));
-constexpr size_t kOffRed = kOffPartials + align256(sizeof(double) * 16 * (kStaticBlocks + 8));
-constexpr size_t kOffErr = kOffRed + align256(sizeof(double) * 32);
+constexpr size_t kOffMask = kOffCellFill + align256(sizeof(int) * (kStaticCells + 1));
+constexpr size_t kOffPartials = kOffMask + align256(sizeof(unsigned) * 3 * kStaticAtoms);
+constexpr size_t kOffErr = kOffPartials + align256(sizeof(double) * 16 * (kStaticBlocks + 8));
 constexpr size_t kStaticBytes = kOffErr + align256(sizeof(unsigned));
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
@@ -123,14 +123,6 @@ int scratch_address(unsigned char** out)
     return NEP_OK;
 }
 
-__global__ void k_static_finish(const double* __restrict__ red, double* e_total, double* virial_total,
-                                const unsigned* __restrict__ err, unsigned* err_out)
-{
-    if (threadIdx.x == 0 && e_total) *e_total = red[0];
-    if (threadIdx.x < 9 && virial_total) virial_total[threadIdx.x] = red[1 + threadIdx.x];
-    if (threadIdx.x == 0 && err_out) *err_out = *err;
-}
-
 }  // namespace
 }  // namespace nep
 
@@ -192,8 +184,8 @@ extern "C" int nep_compute_efv_static(const nep_hyper* hp, const float* z, int n
     nl.cell_count = reinterpret_cast<int*>(base + kOffCellCount);
     nl.cell_start = reinterpret_cast<int*>(base + kOffCellStart);
     nl.cell_fill = reinterpret_cast<int*>(base + kOffCellFill);
+    nl.mask = reinterpret_cast<unsigned*>(base + kOffMask);
     double* partials = reinterpret_cast<double*>(base + kOffPartials);
-    double* red = reinterpret_cast<double*>(base + kOffRed);
     unsigned* err = reinterpret_cast<unsigned*>(base + kOffErr);
 
     // the cell counters and the error word must start at zero; the array
@@ -217,8 +209,9 @@ extern "C" int nep_compute_efv_static(const nep_hyper* hp, const float* z, int n
     aa.box = box;
     aa.vel = nullptr;
     if ((rc = launch_assemble(aa, nl, n, force, virial_atom, part_v, err, st, nb2, nc2))) return rc;
-    if ((rc = launch_reduce(part_e, nb1, 1, red, st))) return rc;
-    if ((rc = launch_reduce(part_v, nb2, nc2, red + 1, st))) return rc;
-    k_static_finish<<<1, 32, 0, st>>>(red, e_total, virial_total, err, err_out);
-    return cuda_fail(cudaGetLastError(), "nep_compute_efv_static kernels");
+    const SumSet e{part_e, nb1, 1, 1, 0, e_total}, w{part_v, nb2, 1, nc2, (size_t)nb2, virial_total};
+    if ((e_total || virial_total) && (rc = launch_sum(e, w, st))) return rc;
+    return err_out ? cuda_fail(cudaMemcpyAsync(err_out, err, sizeof(unsigned), cudaMemcpyDeviceToDevice, st),
+                               "nep_compute_efv_static error word")
+                   : NEP_OK;
 }

@@ -36,3 +36,26 @@ def test_block_edges(orc, n, edge, capacity, n_neu):
     assert np.abs(virial_aos(out["virial_atom"]) - W).max() <= 1e-4
     assert abs(out["e_total"].item() - U.sum()) <= 1e-6 * n * max(1.0, n_neu / 30)
     model.close()
+
+
+@pytest.mark.parametrize("n", [6080, 6081, 12160, 12161, 12193])
+def test_atoms_per_block(orc, n):
+    """The last size of 8 atoms per block, the range of 16, and 32 with ragged
+    tails: the first and last atoms and a sample, on a cut-open crystal."""
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(n)
+    pos, box = inputs.diamond(12, 12, 12)
+    pos = inputs.displace(pos, 0.1, rng)[:n]
+    z = inputs.random_z(1021, rng)
+    model = nep.NEP(z)
+    out = model.compute(soa(pos), box)
+    idx = np.unique(np.concatenate([np.arange(40), np.arange(n - 40, n), rng.integers(0, n, 100)]))
+    U, F, W = orc.efv_sample(orc.NepHyper(), f32_exact(z), pos, box, idx)
+    assert np.abs(out["e_atom"].cpu().numpy()[idx] - U).max() <= 1e-6
+    assert np.abs(aos(out["force"])[idx] - F).max() <= 1e-4
+    assert np.abs(virial_aos(out["virial_atom"])[idx] - W).max() <= 1e-4
+    # the totals are the sums of the per-atom outputs (FP64 sums, so 1e-9 of the largest terms' sum)
+    e, w = out["e_atom"].sum().item(), out["virial_atom"].double().sum(dim=1)
+    assert abs(out["e_total"].item() - e) <= 1e-9 * n
+    assert (out["virial_total"] - w).abs().max().item() <= 1e-9 * n * 10
+    model.close()
