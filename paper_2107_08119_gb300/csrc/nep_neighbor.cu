@@ -13,10 +13,10 @@
 //      increasing distance, and the reverse-pair index (for slot k of atom
 //      i, the slot of i in j's list) follows from the partners' ranks
 //      (k_half_cells, k_sort_tile, k_rev_tile below);
-// Boxes with fewer than 3 cells in a direction (small training cells) use a
-// brute-force scan over all atoms and images, the rows sorted in place
-// (keys atom-major in the partial-force buffer, the values in vala), and
-// the reverse index by binary search over j's keys (k_reverse).
+// Boxes with fewer than 3 cells in a direction (small training cells) and
+// small atom counts test every pair instead (k_list_direct: the sorted keys
+// atom-major in the partial-force buffer, the values in vala), with the
+// reverse index by binary search over j's keys (k_reverse).
 // Every kernel takes an optional device gate word: when it is zero the kernel
 // returns at once, which lets the MD step skip the rebuild without a host
 // round trip.
@@ -168,37 +168,6 @@ __global__ void k_scatter(int n, const int* __restrict__ atom_cell, const int* _
     const int c = atom_cell[i];
     const int slot = atomicAdd(cell_fill + c, 1);
     cell_atoms[cell_start[c] + slot] = i;
-}
-
-__device__ __forceinline__ void list_push(int i, int n, int m_cap, int& cnt, int value, float d2, int* __restrict__ nbr,
-                                          float* __restrict__ key)
-{
-    if (cnt < m_cap) {
-        nbr[(size_t)cnt * n + i] = value;
-        key[(size_t)i * m_cap + cnt] = d2;
-    }
-    ++cnt;
-}
-
-// Order atom i's slots by increasing distance (insertion sort, stable).  Slot
-// k then holds roughly the k-th nearest neighbour of every atom, so the lanes
-// of a warp agree on which slots need the (long) angular work, and the force
-// pass can add the nearest (largest) terms last by walking ranks downwards.
-__device__ void sort_near_first(int i, int n, int m_cap, int cnt, int* __restrict__ nbr, float* __restrict__ key)
-{
-    float* ki = key + (size_t)i * m_cap;
-    for (int a = 1; a < cnt; ++a) {
-        const float kd = ki[a];
-        const int kv = nbr[(size_t)a * n + i];
-        int b = a - 1;
-        while (b >= 0 && ki[b] > kd) {
-            ki[b + 1] = ki[b];
-            nbr[(size_t)(b + 1) * n + i] = nbr[(size_t)b * n + i];
-            --b;
-        }
-        ki[b + 1] = kd;
-        nbr[(size_t)(b + 1) * n + i] = kv;
-    }
 }
 
 // Warps per block of the warp-per-atom list kernels.
@@ -628,35 +597,117 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_tile(int n, int m_cap, cons
     }
 }
 
-__global__ void k_verlet_brute(int n, int m_cap, float rv2, const float* __restrict__ xr, int* __restrict__ count, int* __restrict__ nbr,
-                               float* __restrict__ key, int* __restrict__ vala, unsigned* err, Box b,
-                               const unsigned* gate)
+// The list by testing every atom, for boxes too small for a cell grid (all
+// images) and for small atom counts (the nearest image): one launch instead of
+// the cells path's scan, scatter, search and sort, each a few microseconds of
+// latency.  A block takes two consecutive atoms; its threads walk all atoms j,
+// test the hi parts against both (the 1e-3 A margin of k_half_cells
+// never drops a pair that the exact test keeps), test survivors exactly and
+// append (squared distance, tie-break) keys to the atoms' shared rows.  The
+// rows are then rank-sorted, 64 threads per row.
+// IMAGES: every shift up to b.img, ties ordered by (j, image); else the
+// nearest image (unique: the edges are at least three list radii), ties
+// ordered by the packed value, as the cells path orders them.
+// A cell of 96 atoms: 400 -> 8 us against one thread per atom with an insertion
+// sort in global memory.  Eight atoms per block instead of two: 18 us there,
+// 14.8 against 7.6 us for 1728 atoms.
+constexpr int kDirectThreads = 128;
+constexpr int kDirectAtoms = 2;
+
+template <bool IMAGES>
+__global__ void __launch_bounds__(kDirectThreads) k_list_direct(int n, int m_cap, float rv2,
+                                                               const float* __restrict__ xr, int* __restrict__ count,
+                                                               int* __restrict__ nbr, float* __restrict__ key,
+                                                               int* __restrict__ vala, unsigned* err, Box b,
+                                                               const unsigned* gate)
 {
     if (gated_off(gate)) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float hi[3], li[3];
-    load_pos(xr, i, hi, li);
-    int cnt = 0;
-    for (int j = 0; j < n; ++j) {
-        float hj[3], lj[3];
+    constexpr int AT = kDirectAtoms;
+    extern __shared__ unsigned long long s_rows[];  // [AT][m_cap]
+    __shared__ int s_cnt[AT];
+    constexpr int PER = kDirectThreads / AT;  // threads that sort one row
+    const int i0 = blockIdx.x * AT;
+    if (threadIdx.x < AT) s_cnt[threadIdx.x] = 0;
+    float hi[AT][3];
+#pragma unroll
+    for (int a = 0; a < AT; ++a) {
+        const float4 h = load_hi(xr, min(i0 + a, n - 1));
+        hi[a][0] = h.x;
+        hi[a][1] = h.y;
+        hi[a][2] = h.z;
+    }
+    __syncthreads();
+    const float rq = sqrtf(rv2) + 1e-3f, rq2 = rq * rq;
+    // the exact test of a survivor, and its key
+    auto exact = [&](int a, int j, int code) {
+        float h0[3], l0[3], hj[3], lj[3], rx, ry, rz;
+        load_pos(xr, i0 + a, h0, l0);
         load_pos(xr, j, hj, lj);
+        pair_vector(code, h0, l0, hj, lj, b, rx, ry, rz);
+        const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+        if (!(d2 < rv2)) return;
+        const int at = atomicAdd(s_cnt + a, 1);
+        if (at < m_cap) s_rows[a * m_cap + at] = sort_key(d2, IMAGES ? (j << 7) | code : j | (code << 24));
+    };
+    if (IMAGES) {
         for (int sx = -b.img[0]; sx <= b.img[0]; ++sx)
             for (int sy = -b.img[1]; sy <= b.img[1]; ++sy)
                 for (int sz = -b.img[2]; sz <= b.img[2]; ++sz) {
                     const int code = image_code(sx, sy, sz);
-                    if (j == i && code == kImgCenter) continue;
-                    float rx, ry, rz;
-                    pair_vector(code, hi, li, hj, lj, b, rx, ry, rz);
-                    const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-                    if (d2 < rv2) list_push(i, n, m_cap, cnt, j | (code << 24), d2, nbr, key);
+                    const float tx = (float)sx * b.Lh[0], ty = (float)sy * b.Lh[1], tz = (float)sz * b.Lh[2];
+                    for (int j = threadIdx.x; j < n; j += kDirectThreads) {
+                        const float4 h = load_hi(xr, j);
+#pragma unroll
+                        for (int a = 0; a < AT; ++a) {
+                            const float qx = (h.x - hi[a][0]) + tx, qy = (h.y - hi[a][1]) + ty,
+                                        qz = (h.z - hi[a][2]) + tz;
+                            if (fmaf(qx, qx, fmaf(qy, qy, qz * qz)) < rq2 && i0 + a < n &&
+                                !(j == i0 + a && code == kImgCenter))
+                                exact(a, j, code);
+                        }
+                    }
                 }
+    } else {
+        const float hx = 0.5f * b.Lh[0], hy = 0.5f * b.Lh[1], hz = 0.5f * b.Lh[2];
+        // shift of the nearest image of a difference d (0 but across a face)
+        auto nearest = [](float d, float half, float L, float& s) {
+            s = d > half ? -1.f : d < -half ? 1.f : 0.f;
+            return fmaf(s, L, d);
+        };
+        for (int j = threadIdx.x; j < n; j += kDirectThreads) {
+            const float4 h = load_hi(xr, j);
+#pragma unroll
+            for (int a = 0; a < AT; ++a) {
+                float sx, sy, sz;
+                const float qx = nearest(h.x - hi[a][0], hx, b.Lh[0], sx);
+                const float qy = nearest(h.y - hi[a][1], hy, b.Lh[1], sy);
+                const float qz = nearest(h.z - hi[a][2], hz, b.Lh[2], sz);
+                if (fmaf(qx, qx, fmaf(qy, qy, qz * qz)) < rq2 && i0 + a < n && j != i0 + a)
+                    exact(a, j, image_code((int)sx, (int)sy, (int)sz));
+            }
+        }
     }
-    count[i] = cnt;
-    if (cnt > m_cap) atomicOr(err, kErrOverflow);
-    const int m = cnt < m_cap ? cnt : m_cap;
-    sort_near_first(i, n, m_cap, m, nbr, key);
-    for (int k = 0; k < m; ++k) vala[(size_t)i * m_cap + k] = nbr[(size_t)k * n + i];
+    __syncthreads();
+    const int a = threadIdx.x / PER, t0 = threadIdx.x % PER, i = i0 + a;
+    if (i >= n) return;
+    const int cnt = s_cnt[a];
+    if (t0 == 0) {
+        count[i] = cnt;
+        if (cnt > m_cap) atomicOr(err, kErrOverflow);
+    }
+    const int ns = min(cnt, m_cap);
+    const unsigned long long* row = s_rows + a * m_cap;
+    for (int e = t0; e < ns; e += PER) {
+        const unsigned long long k = row[e];
+        int rank = 0;
+#pragma unroll 4
+        for (int f = 0; f < ns; ++f) rank += k > row[f] ? 1 : 0;
+        const unsigned low = (unsigned)k;
+        const int v = IMAGES ? (int)((low >> 7) | ((low & 127u) << 24)) : (int)low;
+        nbr[(size_t)rank * n + i] = v;
+        vala[(size_t)i * m_cap + rank] = v;
+        key[(size_t)i * m_cap + rank] = __uint_as_float((unsigned)(k >> 32));
+    }
 }
 
 // rev[k][i] = slot of (i, -image) in j's list.  The pair vectors are exactly
@@ -711,16 +762,25 @@ constexpr int kListGridCap = 152 * 16;
 
 }  // namespace
 
+// Largest atom count of the direct list in a box with a cell grid.  The whole
+// list build, cells path -> direct: 512 atoms 24.0 -> 12.0 us, 1728 25.2 ->
+// 15.6, 4096 26.5 -> 35.8; split model 1728 43 -> 24, 5832 50 -> 71 (and three
+// launches instead of six).
+constexpr int kDirectMax = 2500;
+
 int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, const float* zatom, bool wrap_in_place,
                         double* x_ref,
                         float r_list, unsigned* d_err, const unsigned* d_gate, cudaStream_t st)
 {
     const int T = 256;
     const float rv2 = r_list * r_list;
-    const bool cells = b.nc[0] > 0;
+    const bool grid_box = b.nc[0] > 0;
+    const bool cells = grid_box && n > kDirectMax;
     const int ncell = cells ? b.nc[0] * b.nc[1] * b.nc[2] : 0;
+    Box bb = b;
+    if (!cells) bb.nc[0] = 0;  // no cell counts
     k_bin<<<blocks_for(n, T), T, 0, st>>>(n, pos, zatom, wrap_in_place ? 1 : 0, x_ref, nl.xr, nl.atom_cell,
-                                          nl.cell_count, nl.count, b, d_gate, d_err);
+                                          nl.cell_count, nl.count, bb, d_gate, d_err);
     if (cells) {
         k_scan<<<1, kScanThreads, 0, st>>>(ncell, nl.cell_count, nl.cell_start, nl.cell_fill, d_gate);
         k_scatter<<<blocks_for(n, T), T, 0, st>>>(n, nl.atom_cell, nl.cell_start, nl.cell_fill, nl.cell_atoms,
@@ -748,10 +808,11 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
             k_rev_perm<<<std::min(blocks_for(n, 4), kListGridCap), 128, 0, st>>>(n, nl.m_cap, nl.count, rows,
                                                                                   nl.vala, nl.rev, d_err, d_gate);
         return cuda_fail(cudaGetLastError(), "neighbour-list kernels");
-    } else {
-        k_verlet_brute<<<blocks_for(n, 128), 128, 0, st>>>(n, nl.m_cap, rv2, nl.xr, nl.count, nl.nbr, nl.pf,
-                                                           nl.vala, d_err, b, d_gate);
     }
+    const size_t rows_bytes = (size_t)kDirectAtoms * nl.m_cap * sizeof(unsigned long long);
+    (grid_box ? k_list_direct<false> : k_list_direct<true>)<<<blocks_for(n, kDirectAtoms), kDirectThreads, rows_bytes,
+                                                             st>>>(n, nl.m_cap, rv2, nl.xr, nl.count, nl.nbr, nl.pf,
+                                                                   nl.vala, d_err, b, d_gate);
     k_reverse<<<std::min(blocks_for(n, 4), kListGridCap), 128, 0, st>>>(n, nl.m_cap, nl.count, nl.pf, nl.vala, nl.rev,
                                                                          d_err, d_gate);
     return cuda_fail(cudaGetLastError(), "neighbour-list kernels");

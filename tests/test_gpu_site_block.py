@@ -59,3 +59,39 @@ def test_atoms_per_block(orc, n):
     assert abs(out["e_total"].item() - e) <= 1e-9 * n
     assert (out["virial_total"] - w).abs().max().item() <= 1e-9 * n * 10
     model.close()
+
+
+@pytest.mark.parametrize("cells,n", [
+    ((1, 1, 1), 8),      # every pair through several images
+    ((2, 2, 2), 63),     # no cell grid, odd count
+    ((2, 3, 5), 240),    # no cell grid in one direction only
+    ((4, 4, 4), 511),    # grid box, nearest images
+    ((7, 7, 7), 2500),   # the last count of the direct list
+    ((7, 7, 7), 2501),   # the first of the cells path
+])
+def test_list_by_direct_tests(orc, cells, n):
+    """The list built by testing every atom: the same neighbours, distances
+    ascending, as the oracle's brute-force list, and the forces from it."""
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(n)
+    pos, box = inputs.diamond(*cells)
+    pos = inputs.displace(pos, 0.1, rng)[:n]
+    z = inputs.random_z(1021, rng)
+    model = nep.NEP(z)
+    out = model.compute(soa(pos), box)
+    cnt, nbr = (t.cpu().numpy() for t in model.neighbors(n))
+    _, F, _ = orc.efv_sample(orc.NepHyper(), f32_exact(z), pos, box, np.arange(min(n, 200)))
+    assert np.abs(aos(out["force"])[:200] - F).max() <= 1e-4
+    L = np.diag(box)
+    x = pos - L * np.floor(pos / L)
+    for i in range(0, n, max(1, n // 50)):
+        v = nbr[:cnt[i], i]
+        code = v >> 24
+        shift = np.stack([code // 25 - 2, code // 5 % 5 - 2, code % 5 - 2], 1)
+        r = np.linalg.norm(x[v & 0xFFFFFF] + shift * L - x[i], axis=1)
+        assert np.all(np.diff(r) >= -1e-5) and r.max() < 5.0 + 1e-5
+        assert len(set(v.tolist())) == len(v)
+        img = np.stack(np.meshgrid(*[np.arange(-2, 3)] * 3, indexing="ij"), -1).reshape(-1, 1, 3) * L
+        d = np.linalg.norm(x[None] + img - x[i], axis=2)
+        assert abs(int(np.sum((d < 5.0) & (d > 1e-9))) - len(v)) <= int(np.sum(np.abs(d - 5.0) < 1e-5))
+    model.close()
