@@ -85,10 +85,6 @@ struct nep_dataset {
     double* w_tar = nullptr;
     // evaluation scratch (grown on demand)
     int pop_cap = 0;
-    float* W1t = nullptr;
-    float* b1t = nullptr;
-    float* w2t = nullptr;
-    float* b2t = nullptr;
     float* G = nullptr;
     double* U = nullptr;
     double* partials = nullptr;  // loss records (ChunkRec, 64 B) [chunk][member]

@@ -16,10 +16,9 @@
 //   F_ki = G_ki . B_i - sum_j p_kji                                (Eqs. 4-5)
 //   W_k  = sum_i sum_j r_ij (x) p_kji                              (Eq. 6)
 // and the RMSEs of Eqs. 29-34.  Kernels per evaluation:
-//   k_pack      z_pop -> member-innermost weight layout (FP32 network; the
-//               tensor-core records are packed from z_pop by k_pack_tc)
-//   k_mlp_f32   FP32 network per (atom pair, member): U [N][P] and
-//               G [N][32][Pst] (member innermost, Pst = P rounded up to 4)
+//   k_mlp_f32   FP32 network, a member per warp and four atoms per lane:
+//               U [N][P] and G [N][32][Pst] (member innermost, Pst = P
+//               rounded up to 4)
 //   k_pop_tc    the same network as BF16 tensor-core GEMMs (nep_pop_tc.cu)
 //   k_contract_owner  warp per atom j, two members per lane: p_kji for j's
 //               pairs from G_j held in registers, stored at the reverse slot
@@ -325,78 +324,189 @@ __global__ void k_ds_site(int N, const int* __restrict__ sid, const Box* __restr
 }
 
 // ------------------------------------------------------------------ evaluation
-// z_pop [P][n_par] -> W1t [n_neu][32][P], b1t [n_neu][P], w2t [n_neu][P], b2t [P]
-__global__ void k_pack(int P, int n_neu, const float* __restrict__ z, float* __restrict__ W1t,
-                       float* __restrict__ b1t, float* __restrict__ w2t, float* __restrict__ b2t)
+// FP32 network of M members (one per warp) on 128 atoms (four per lane), in
+// two passes over the neurons: the pre-activations, states, site energies and
+// the slopes d_mu = w2 (1 - x_mu^2), which go to shared memory, and then the
+// input gradients.  The members' parameters sit in shared memory, where a warp
+// reads its neuron's weights as uniform 16-byte words.  G goes out through
+// shared memory as one 4 M-byte piece per (atom, descriptor): members are
+// innermost in G.
+//
+// What bounds it: the shared-memory return path and issue.  A uniform read
+// still returns 128 bytes per clock and SM, so a neuron's 32 weights cost the
+// four schedulers' warps 128 clocks; four atoms per lane make 128 FMAs per
+// scheduler of them in each pass (q or G fill 128 registers).  One atom per
+// lane with both passes on one read: 206 us; two atoms: spills, 299 us.  The
+// blocks stay resident (eight warps per SM) and copy the next item's inputs
+// while they work: 188 -> 177 us.  One thread per (atom pair, member) that
+// read every weight from global memory, coalesced over members: 276 us for
+// 20,840 atoms x 50 members.
+constexpr int kMlpPer = 4;                  // atoms per lane
+constexpr int kMlpAtoms = 32 * kMlpPer;
+
+__host__ __device__ inline size_t mlp_f32_d_floats(int n_neu)  // per warp: slopes, later 32 atoms' G
 {
-    const int n_par = (kNdes + 2) * n_neu + 1;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= P * n_par) return;
-    const int k = e / n_par, t = e % n_par;
-    const float v = z[e];
-    if (t < n_neu * kNdes)
-        W1t[(size_t)t * P + k] = v;
-    else if (t < n_neu * kNdes + n_neu)
-        b1t[(size_t)(t - n_neu * kNdes) * P + k] = v;
-    else if (t < n_neu * kNdes + 2 * n_neu)
-        w2t[(size_t)(t - n_neu * kNdes - n_neu) * P + k] = v;
-    else
-        b2t[k] = v;
+    const size_t d = (size_t)n_neu * kMlpAtoms, g = (size_t)kNdes * 32;
+    return d > g ? d : g;
 }
 
-// FP32 network, two atoms per thread (each weight load feeds two FMAs):
-// thread t -> atom pair a = t / P, member k = t % P.
-__global__ void __launch_bounds__(256) k_mlp_f32(int N, int P, int Pst, int n_neu, const float* __restrict__ q,
-                                                 const float* __restrict__ W1t, const float* __restrict__ b1t,
-                                                 const float* __restrict__ w2t, const float* __restrict__ b2t,
-                                                 float* __restrict__ G, double* __restrict__ U)
+template <int M>
+__global__ void __launch_bounds__(32 * M, 8 / M) k_mlp_f32(int N, int P, int Pst, int n_neu,
+                                                           const float* __restrict__ q, const float* __restrict__ z,
+                                                           float* __restrict__ G, double* __restrict__ U)
 {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long a = t / P;
-    const int k = (int)(t % P);
-    const long long i0 = 2 * a;
-    if (i0 >= N) return;
-    const bool two = i0 + 1 < N;
-    const long long i1 = two ? i0 + 1 : i0;
-    // the two atoms side by side: (atom i0, atom i1) pairs for the f32x2 FMAs
-    float2 q2[kNdes], G2[kNdes];
+    // a tile's descriptors [128 atoms][8 words of 16 bytes], M parameter vectors
+    // twice, then the slopes, over them [32 v][M][32 atoms] of G
+    extern __shared__ __align__(16) float s_mlp[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_par = (kNdes + 2) * n_neu + 1, stride = (n_par + 3) / 4 * 4;
+    float4* s_q = reinterpret_cast<float4*>(s_mlp);
+    float* s_w = s_mlp + kMlpAtoms * kNdes;
+    float* s_out = s_w + 2 * M * stride;
+    float* s_d = s_out + warp * mlp_f32_d_floats(n_neu) + lane;  // [n_neu][kMlpPer][32]
+    // work items (tile of atoms, member group), the groups of a tile in
+    // neighbouring blocks at the same time: their 4 M-byte pieces of G share
+    // sectors, which then merge in L2 (a block that kept its group or its tile
+    // over consecutive items cost 500-580 MB of DRAM traffic instead of 107)
+    const int groups = (P + M - 1) / M, items = groups * ((N + kMlpAtoms - 1) / kMlpAtoms);
+    // asynchronous copies for item `it`: the warp's parameters, and
+    // the tile's descriptors, word c of atom a at place c ^ (a & 7), so that a
+    // warp's reads of one word have no bank conflicts
+    auto fetch = [&](int it, int buf) {
+        const int k = it % groups * M + warp;
+        if (k < P) {
+            const float* src = z + (size_t)k * n_par;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(s_w + (buf * M + warp) * stride);
+#pragma unroll 8
+            for (int t = lane; t < n_par; t += 32)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * t), "l"(src + t) : "memory");
+        }
+        const int a0 = it / groups * kMlpAtoms;
+#pragma unroll 4
+        for (int t = threadIdx.x; t < kMlpAtoms * (kNdes / 4); t += 32 * M) {
+            const int a = t / (kNdes / 4), c = t % (kNdes / 4);
+            const float* src = q + (size_t)min(a0 + a, N - 1) * kNdes + 4 * c;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(s_q + a * (kNdes / 4) + (c ^ (a & 7)));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int buf = 0;
+    if (blockIdx.x < items) fetch(blockIdx.x, 0);
+#pragma unroll 1
+    for (int it = blockIdx.x; it < items; it += gridDim.x, buf ^= 1) {
+        const int k0 = it % groups * M, k = k0 + warp, i0 = it / groups * kMlpAtoms;
+        const bool on = k < P;
+        const float* w = s_w + (buf * M + warp) * stride;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();  // the copies are here, and the previous item's G is read
+        float qv[kMlpPer][kNdes];
 #pragma unroll
-    for (int v = 0; v < kNdes; ++v) {
-        q2[v] = make_float2(q[i0 * kNdes + v], q[i1 * kNdes + v]);
-        G2[v] = make_float2(0.f, 0.f);
-    }
-    float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
-    for (int mu = 0; mu < n_neu; ++mu) {
-        const float* w = W1t + (size_t)mu * kNdes * P + k;
-        float2 a = make_float2(0.f, 0.f);
+        for (int h = 0; h < kMlpPer; ++h)
 #pragma unroll
-        for (int v = 0; v < kNdes; ++v) a = __ffma2_rn(bcast2(w[(size_t)v * P]), q2[v], a);
-        const float bb = b1t[(size_t)mu * P + k], ww = w2t[(size_t)mu * P + k];
-        const float x0 = tanhf(a.x - bb), x1 = tanhf(a.y - bb);
-        float tt, e;
-        float p = ww * x0, ep = fmaf(ww, x0, -p);
-        two_sum(s0, p, tt, e);
-        s0 = tt;
-        c0 += e + ep;
-        p = ww * x1;
-        ep = fmaf(ww, x1, -p);
-        two_sum(s1, p, tt, e);
-        s1 = tt;
-        c1 += e + ep;
-        const float2 d = make_float2(ww * fmaf(-x0, x0, 1.f), ww * fmaf(-x1, x1, 1.f));
+            for (int c = 0; c < kNdes / 4; ++c) {
+                const float4 t = s_q[(32 * h + lane) * (kNdes / 4) + (c ^ (lane & 7))];
+                qv[h][4 * c] = t.x;
+                qv[h][4 * c + 1] = t.y;
+                qv[h][4 * c + 2] = t.z;
+                qv[h][4 * c + 3] = t.w;
+            }
+        __syncthreads();
+        if (it + (int)gridDim.x < items) fetch(it + gridDim.x, buf ^ 1);
+        if (on) {
+            const float* b1 = w + n_neu * kNdes;
+            const float* w2 = b1 + n_neu;
+            float s[kMlpPer], c[kMlpPer];
 #pragma unroll
-        for (int v = 0; v < kNdes; ++v) G2[v] = __ffma2_rn(d, bcast2(w[(size_t)v * P]), G2[v]);
-    }
-    const double b2 = (double)b2t[k];
-    U[i0 * P + k] = (double)s0 + (double)c0 - b2;
+            for (int h = 0; h < kMlpPer; ++h) s[h] = c[h] = 0.f;
+#pragma unroll 1
+            for (int mu = 0; mu < n_neu; ++mu) {
+                const float4* row4 = reinterpret_cast<const float4*>(w + mu * kNdes);
+                const float ww = w2[mu], bb = b1[mu];
+                float a[kMlpPer];
 #pragma unroll
-    for (int v = 0; v < kNdes; ++v) G[(i0 * kNdes + v) * Pst + k] = G2[v].x;
-    if (two) {
-        U[i1 * P + k] = (double)s1 + (double)c1 - b2;
+                for (int h = 0; h < kMlpPer; ++h) a[h] = 0.f;
 #pragma unroll
-        for (int v = 0; v < kNdes; ++v) G[(i1 * kNdes + v) * Pst + k] = G2[v].y;
+                for (int v = 0; v < kNdes / 4; ++v) {
+                    const float4 r = row4[v];
+#pragma unroll
+                    for (int h = 0; h < kMlpPer; ++h) {
+                        a[h] = fmaf(r.x, qv[h][4 * v], a[h]);
+                        a[h] = fmaf(r.y, qv[h][4 * v + 1], a[h]);
+                        a[h] = fmaf(r.z, qv[h][4 * v + 2], a[h]);
+                        a[h] = fmaf(r.w, qv[h][4 * v + 3], a[h]);
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < kMlpPer; ++h) {
+                    const float x = tanhf(a[h] - bb);
+                    neuron_energy(ww, x, s[h], c[h]);
+                    s_d[(mu * kMlpPer + h) * 32] = ww * fmaf(-x, x, 1.f);
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < kMlpPer; ++h) {
+                const int i = i0 + 32 * h + lane;
+                if (i < N) U[(size_t)i * P + k] = (double)s[h] + (double)c[h] - (double)w2[n_neu];
+            }
+        }
+        float2 Gv[kMlpPer][kNdes / 2];
+#pragma unroll
+        for (int h = 0; h < kMlpPer; ++h)
+#pragma unroll
+            for (int v = 0; v < kNdes / 2; ++v) Gv[h][v] = make_float2(0.f, 0.f);
+        if (on)
+#pragma unroll 1
+            for (int mu = 0; mu < n_neu; ++mu) {
+                const float4* row4 = reinterpret_cast<const float4*>(w + mu * kNdes);
+                float2 d[kMlpPer];
+#pragma unroll
+                for (int h = 0; h < kMlpPer; ++h) d[h] = bcast2(s_d[(mu * kMlpPer + h) * 32]);
+#pragma unroll
+                for (int v = 0; v < kNdes / 4; ++v) {
+                    const float4 r = row4[v];
+#pragma unroll
+                    for (int h = 0; h < kMlpPer; ++h) {
+                        Gv[h][2 * v] = ffma2(d[h], make_float2(r.x, r.y), Gv[h][2 * v]);
+                        Gv[h][2 * v + 1] = ffma2(d[h], make_float2(r.z, r.w), Gv[h][2 * v + 1]);
+                    }
+                }
+            }
+#pragma unroll
+        for (int h = 0; h < kMlpPer; ++h) {
+            __syncthreads();  // the slopes, or the previous 32 atoms, are read
+#pragma unroll
+            for (int v = 0; v < kNdes; ++v)
+                s_out[(v * M + warp) * 32 + lane] = (v & 1) ? Gv[h][v / 2].y : Gv[h][v / 2].x;
+            __syncthreads();
+            // lanes on atoms, a warp per descriptor
+            const int i = i0 + 32 * h + lane;
+            if (i < N)
+                for (int v = warp; v < kNdes; v += M)
+#pragma unroll
+                    for (int m = 0; m < M; m += 4)
+                        if (k0 + m < Pst) {
+                            const float* t = s_out + (v * M + m) * 32 + lane;
+                            *reinterpret_cast<float4*>(G + ((size_t)i * kNdes + v) * Pst + k0 + m) =
+                                make_float4(t[0], t[32], t[64], t[96]);
+                        }
+        }
     }
 }
+
+size_t mlp_f32_smem(int M, int n_par, int n_neu)
+{
+    return sizeof(float) *
+           (kMlpAtoms * kNdes + M * (2 * ((size_t)(n_par + 3) / 4 * 4) + mlp_f32_d_floats(n_neu)));
+}
+
+// members per block: mlp_threads / 32, or four where the slopes of eight do
+// not fit in shared memory
+int mlp_f32_members(int threads, int n_par, int n_neu)
+{
+    return threads == 256 && mlp_f32_smem(8, n_par, n_neu) <= 220 * 1024 ? 8 : 4;
+}
+
 
 // Contraction, pass 1 (owner side): one warp per atom j, lane l holding
 // members 2l and 2l + 1.  The lane loads its members' G_j once (registers).
@@ -1243,10 +1353,6 @@ inline int member_stride(int P) { return (P + 3) / 4 * 4; }
 int ensure_pop(nep_dataset* ds, int P)
 {
     if (P <= ds->pop_cap) return NEP_OK;
-    dfree(ds->W1t);
-    dfree(ds->b1t);
-    dfree(ds->w2t);
-    dfree(ds->b2t);
     dfree(ds->G);
     dfree(ds->U);
     dfree(ds->partials);
@@ -1255,11 +1361,8 @@ int ensure_pop(nep_dataset* ds, int P)
     dfree(ds->w6);
     dfree(ds->fown);
     ds->pop_cap = 0;
-    const int nn = ds->m->hp.n_neu;
     int rc;
-    if ((rc = dalloc(&ds->W1t, (size_t)nn * kNdes * P, nullptr)) || (rc = dalloc(&ds->b1t, (size_t)nn * P, nullptr)) ||
-        (rc = dalloc(&ds->w2t, (size_t)nn * P, nullptr)) || (rc = dalloc(&ds->b2t, (size_t)P, nullptr)) ||
-        (rc = dalloc(&ds->G, (size_t)ds->N * kNdes * member_stride(P), nullptr)) ||
+    if ((rc = dalloc(&ds->G, (size_t)ds->N * kNdes * member_stride(P), nullptr)) ||
         (rc = dalloc(&ds->U, (size_t)ds->N * P, nullptr)) ||
         (rc = dalloc(&ds->partials, (size_t)ds->n_chunks * P * 8, nullptr)) ||
         (rc = dalloc(&ds->packed, pop_tc_packed_bytes(P), nullptr)) ||
@@ -1307,6 +1410,15 @@ int prepare_evaluation(nep_dataset* ds, int P)
         (rc = cuda_fail(cudaFuncSetAttribute(k_contract_bulk<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)sizeof(BulkSmem)), "contraction shared memory")))
         return rc;
+    for (int t = 128; t <= 256; t += 128) {
+        const int n_neu = ds->m->hp.n_neu, M = mlp_f32_members(t, ds->m->n_par, n_neu);
+        auto kern = M == 4 ? k_mlp_f32<4> : k_mlp_f32<8>;
+        if ((rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)mlp_f32_smem(M, ds->m->n_par, n_neu)), "network shared memory")) ||
+            (rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                 cudaSharedmemCarveoutMaxShared), "network shared memory")))
+            return rc;
+    }
     for (int gm = 4; gm <= 16; gm *= 2) {
         if (!fused_fits(ds, gm)) continue;
         const int smem = (int)fused_smem_bytes(ds->amax, gm);
@@ -1402,12 +1514,11 @@ int enqueue_evaluation(nep_model* m, nep_dataset* ds, const float* z_pop, int P,
                                 ds->U, m->d_err, sh.pop_pipe != 0, st)))
             return rc;
     } else {
-        k_pack<<<blocks_for((long long)P * n_par, 256), 256, 0, st>>>(P, nn, z_pop, ds->W1t, ds->b1t, ds->w2t,
-                                                                      ds->b2t);
-        const long long pairs = (ds->N + 1) / 2;
-        const int mt = sh.mlp_threads == 128 ? 128 : 256;
-        k_mlp_f32<<<blocks_for(pairs * P, mt), mt, 0, st>>>(ds->N, P, Pst, nn, ds->q, ds->W1t, ds->b1t, ds->w2t,
-                                                            ds->b2t, ds->G, ds->U);
+        const int M = mlp_f32_members(sh.mlp_threads, n_par, nn);
+        const long long items = (long long)blocks_for(ds->N, kMlpAtoms) * ((P + M - 1) / M);
+        const int grid = (int)std::min<long long>(items, 152 * (8 / M));  // eight warps per SM
+        (M == 4 ? k_mlp_f32<4> : k_mlp_f32<8>)<<<grid, 32 * M, mlp_f32_smem(M, n_par, nn), st>>>(
+            ds->N, P, Pst, nn, ds->q, z_pop, reinterpret_cast<float*>(ds->G), ds->U);
     }
     const double lam[5] = {lambdas ? lambdas[0] : 1.0, lambdas ? lambdas[1] : 1.0, lambdas ? lambdas[2] : 1.0,
                            lambdas ? lambdas[3] : 0.05, lambdas ? lambdas[4] : 0.05};
@@ -1778,10 +1889,6 @@ int nep_dataset_destroy(nep_dataset* ds)
     dfree(ds->e_tar);
     dfree(ds->f_tar);
     dfree(ds->w_tar);
-    dfree(ds->W1t);
-    dfree(ds->b1t);
-    dfree(ds->w2t);
-    dfree(ds->b2t);
     dfree(ds->G);
     dfree(ds->U);
     dfree(ds->partials);

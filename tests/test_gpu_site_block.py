@@ -95,3 +95,34 @@ def test_list_by_direct_tests(orc, cells, n):
         d = np.linalg.norm(x[None] + img - x[i], axis=2)
         assert abs(int(np.sum((d < 5.0) & (d > 1e-9))) - len(v)) <= int(np.sum(np.abs(d - 5.0) < 1e-5))
     model.close()
+
+
+@pytest.mark.parametrize("n_struct,n_pop,n_neu,threads", [
+    (1, 1, 30, 128),     # one member, one ragged tile of atoms
+    (1, 2, 1, 256),
+    (3, 5, 30, 128),     # a partial member group
+    (3, 9, 30, 256),
+    (2, 64, 64, 256),    # the largest network and population: four members per block
+])
+def test_population_network_shapes(orc, n_struct, n_pop, n_neu, threads):
+    """The FP32 population network around its tiles (128 atoms, 4 or 8
+    members): every loss term of every member against the oracle.  FP32 sums of
+    ~100 terms per force: 3e-4, the bar of the population tests."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(n_pop)
+    hyper = nep.Hyper(n_neu=n_neu)
+    structures = inputs.training_structures(n_struct, seed_stream=n_pop)
+    n = sum(len(s["pos"]) for s in structures)
+    e = rng.normal(-3.0, 0.1, n_struct) * [len(s["pos"]) for s in structures]
+    f, w = rng.normal(0.0, 1.0, (n, 3)), rng.normal(0.0, 1.0, (n_struct, 6))
+    pop = rng.normal(0.0, 0.1, (n_pop, hyper.n_par)).astype(np.float32)
+    model = nep.NEP(pop[0], hyper)
+    ds = nep.Dataset(model, structures, e, f, w)
+    ds.set_shape(fused=0, mlp_threads=threads)
+    got = ds.evaluate(torch.tensor(pop, device="cuda")).cpu().numpy()
+    for k in {0, n_pop // 2, n_pop - 1}:
+        want = orc.loss(orc.NepHyper(n_neu=n_neu), f32_exact(pop[k]), structures, e, f, w)
+        assert np.abs(got[k] - want).max() <= 3e-4, (k, got[k], want)
+    ds.close()
+    model.close()
