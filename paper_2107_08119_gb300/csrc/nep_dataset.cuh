@@ -22,13 +22,15 @@ struct PairRec {
     float pad;
 };
 
+constexpr int kDsCap = 192;  // pairs per atom within the cutoffs that a training set can hold
+
 // Scratch of the force-loss adjoint.
 struct AdjointScratch {
     int n_blocks = 0;          // per-atom kernel blocks the partial buffers hold
     float* pf = nullptr;       // [n_pairs][3] dU_i/dr_ij of the last forward
     float* res = nullptr;      // [N] float4: F_i - F_tar_i of the last forward
     float* z = nullptr;        // [n_par] parameters of the last forward
-    double* part = nullptr;    // [n_blocks][n_par] per-block FP64 partial sums
+    double* part = nullptr;    // per-block partial sums: FP64 [n_blocks], or FP32 [n_blocks][n_par]
     double* sums = nullptr;    // [2]: sum |F - F_tar|^2, L_f
     bool ready = false;        // a forward has run since the scratch was made
 };

@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, cons
     const bool active = i < n;
     const int cnt = active ? min(count[i], m_cap) : 0;
     float uh, ul;
-    site_block<D, AT, WORDS>(i, active, n, cnt, nbr, xr, box, z, n_par, P, pf, mask, uh, ul);
+    const SlotMajorPairs pairs{nbr, reinterpret_cast<float4*>(pf), (size_t)n, active ? i : 0};
+    site_block<D, AT, WORDS>(pairs, i, active, n, cnt, xr, box, z, n_par, P, mask, uh, ul);
     if (threadIdx.x >= 32) return;  // the first AT lanes hold the site energies
     double e = 0.0;
     if (active && lane < AT) {
@@ -323,12 +324,13 @@ int launch_site(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, dou
     const size_t smem = site_block_smem<D, AT>(n_par, a.n_neu);
     constexpr int kWide = (384 / SiteSplit<AT>::WAYS + 31) / 32;  // words that hold any capacity
     auto kern = nl.m_cap <= 32 * SiteSplit<AT>::WAYS ? k_site<D, AT, 1> : k_site<D, AT, kWide>;
-    int rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                       "site kernel shared memory");
-    if (!rc)
-        rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                            cudaSharedmemCarveoutMaxShared), "site kernel shared memory");
-    if (rc) return rc;
+    // only large networks of the split model need more than the default 48 KB:
+    // an attribute call costs as much host time as a launch
+    if (smem > 48 * 1024) {
+        const int rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                                 "site kernel shared memory");
+        if (rc) return rc;
+    }
     nl.mask_set = nl.m_cap <= kMaskSlots && nl.mask != nullptr;
     kern<<<nblocks, kSiteThreads, smem, st>>>(n, nl.m_cap, nl.count, nl.nbr, nl.xr, a.box, a.z, n_par, P, nl.pf,
                                               e_atom, e_partials, d_err, nl.mask_set ? nl.mask : nullptr);

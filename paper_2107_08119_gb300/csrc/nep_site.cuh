@@ -16,8 +16,9 @@
 //     grad(g Z(rhat)) = g' Z rhat + g (grad_u Z - rhat (rhat . grad_u Z)) / r.
 // Chebyshev T_n and U_n come from the recurrences of App. A (Eqs. A1-A3).
 //
-// The functions are __host__ __device__ so the same code can be exercised
-// on the CPU; on the device the weights pointer refers to shared memory.
+// The site pass (nep_site_block.cuh) spreads this arithmetic over the threads
+// of a block.  The functions are __host__ __device__ so the same code can be
+// exercised on the CPU.
 #pragma once
 
 #include <math.h>
@@ -290,31 +291,6 @@ __host__ __device__ __forceinline__ void sh_pass1(float x, float y, float z, con
 #undef NEP_T
 }
 
-// One harmonic's contribution to the angular partial force:
-//   (cg, cd) = sum_n A[n][lm] (g_n, g_n')   (one packed FMA per order)
-//   B += cd Y, V += cg grad_u Y             ((Vx, Vy) packed).
-template <int NA, int N2>
-__host__ __device__ __forceinline__ void sh_term(const float2 (&A)[N2][kLM], const float2 (&gd)[NA], int lm, float Y,
-                                                 float gx, float gy, float gz, float& B, float2& Vxy, float& Vz)
-{
-    float2 c = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int n = 0; n < NA; ++n) c = ffma2(bcast2(harm(A, n, lm)), gd[n], c);
-    B = fmaf(c.y, Y, B);
-    Vxy = ffma2(bcast2(c.x), make_float2(gx, gy), Vxy);
-    Vz = fmaf(c.x, gz, Vz);
-}
-
-template <int NA, int N2>
-__host__ __device__ __forceinline__ void sh_pass2(float x, float y, float z, const float2 (&A)[N2][kLM],
-                                                  const float2 (&gd)[NA], float& B, float2& Vxy, float& Vz)
-{
-    NEP_SH_LOCALS_FAST(x, y, z)
-#define NEP_T(lm, Yv, gx, gy, gz) sh_term(A, gd, lm, Yv, gx, gy, gz, B, Vxy, Vz);
-    NEP_SH_TABLE(NEP_T)
-#undef NEP_T
-}
-
 // All 24 harmonics and their (unprojected) gradients.
 __host__ __device__ __forceinline__ void sh_eval(float x, float y, float z, float (&Y)[kLM], float (&dY)[kLM][3])
 {
@@ -407,86 +383,12 @@ __host__ __device__ __forceinline__ float neuron_state(const float* row, float b
     return tanhf(sa - comp);
 }
 
-// Adds neuron mu's output w2 x to the compensated sum (s, c) and its share
-// w2 (1 - x^2) w1_mu of G.
-template <int ND>
-__host__ __device__ __forceinline__ void neuron_out(float w2, float xm, const float* row, float& s, float& c,
-                                                    float (&G)[ND])
-{
-    neuron_energy(w2, xm, s, c);
-    const float d = w2 * fmaf(-xm, xm, 1.f);
-#ifdef __CUDA_ARCH__
-    if constexpr (ND % 4 == 0) {
-        // the row is 16-byte aligned (shared memory, ND floats per row)
-        const float4* row4 = reinterpret_cast<const float4*>(row);
-#pragma unroll
-        for (int v = 0; v < ND; v += 4) {
-            const float4 t = row4[v / 4];
-            G[v] = fmaf(d, t.x, G[v]);
-            G[v + 1] = fmaf(d, t.y, G[v + 1]);
-            G[v + 2] = fmaf(d, t.z, G[v + 2]);
-            G[v + 3] = fmaf(d, t.w, G[v + 3]);
-        }
-    } else
-#endif
-    {
-#pragma unroll
-        for (int v = 0; v < ND; ++v) G[v] = fmaf(d, row[v], G[v]);
-    }
-}
-
-// Network of Eqs. 21-22 and its input gradient.  w points at the parameter
-// vector [w1 (n_neu x N_des), b1, w2, b2].  The pre-activations and the output
-// sum are compensated (rounding errors carried along) because the site energy
-// must hold ~1e-7 relative accuracy.  Returns U as hi + lo.
-template <int ND>
-__host__ __device__ __forceinline__ void network(const float* w, int n_neu, const float (&q)[ND], float (&G)[ND],
-                                                 float& U_hi, float& U_lo)
-{
-    const float* b1 = w + n_neu * ND;
-    const float* w2 = b1 + n_neu;
-    const float b2 = w2[n_neu];
-#pragma unroll
-    for (int v = 0; v < ND; ++v) G[v] = 0.f;
-    float s = 0.f, c = 0.f;
-    for (int mu = 0; mu < n_neu; ++mu) {
-        const float* row = w + mu * ND;
-        neuron_out(w2[mu], neuron_state<ND>(row, b1[mu], q), row, s, c, G);
-    }
-    float t, e;
-    two_sum(s, -b2, t, e);
-    U_hi = t;
-    U_lo = c + e;
-}
-
-// One neighbour slot: packed index and the neighbour's hi/lo position.  The
-// loops below fetch slot k+1 (or k-1) before working on slot k so the loads
-// overlap the arithmetic of the current slot.
-struct NbSlot {
-    int v;
-    float h[3], l[3];
-    float z;  // the neighbour's species number
-};
-
-// Slot k of the atom is slots[k * stride + idx]: the global list (stride n,
-// idx i) or a block's staged copy in shared memory (stride blockDim, idx tid).
+// Slot k of the atom is slots[k * stride + idx].
 struct SlotTable {
     const int* slots;
     int stride;
     int idx;
-    // for a compacted table (only the slots within the cutoff, in their
-    // order): the original slot of entry k at orig[k * stride + idx]
-    const unsigned char* orig = nullptr;
 };
-
-__host__ __device__ __forceinline__ void fetch_slot(const SlotTable& T, const float* __restrict__ xr, int n, int k, int cnt, NbSlot& s)
-{
-    if (k >= 0 && k < cnt) {
-        s.v = T.slots[(size_t)k * T.stride + T.idx];
-        load_pos(xr, s.v & 0xFFFFFF, s.h, s.l);
-        s.z = load_z(xr, s.v & 0xFFFFFF);
-    }
-}
 
 // Parameters of the per-atom site functions.
 struct SiteParams {
@@ -501,15 +403,6 @@ __host__ __device__ __forceinline__ float pair_weight(const SiteParams& P, float
 {
     return P.typed ? sqrtf(zi * zj) : 1.f;
 }
-
-// Where the partial force of slot k goes: base[k * slot_stride + c * comp_stride].
-// The MD list stores pf[k][c][i] (base = pf + i, strides 3n and n); a
-// training-set CSR list stores pf[p][c] (base = pf + 3 p0, strides 3 and 1).
-struct PfOut {
-    float* base;
-    size_t slot_stride;
-    size_t comp_stride;
-};
 
 // Unit vector r / |r| with each component rounded once from a near-exact
 // value.  The solid harmonics of degree l scale as |u|^l, so an error delta
@@ -579,221 +472,6 @@ __host__ __device__ __forceinline__ void unit_vector_res(float rx, float ry, flo
     const float ll = fmaf(sh, yh, -lh) + fmaf(sh, yl, sl * yh);
     dres = (lh - d) + ll;
     inv = yh;
-}
-
-// Pass 1 of atom i: the descriptor vector q (Eqs. 12-13 through the harmonic
-// sums) and the harmonic sums S_nlm themselves.  Every lane of a warp must
-// call it (inactive lanes pass cnt = 0): the ranks are walked in step.
-template <class D = DescSi>
-__host__ __device__ __forceinline__ void site_descriptors(int i, int n, int cnt, const SlotTable& nbr,
-                                                          const float* __restrict__ xr, const Box& box,
-                                                          const SiteParams& P, const float (&hi)[3],
-                                                          const float (&li)[3], float zi, float (&q)[D::Ndes],
-                                                          HarmT<D>& S)
-{
-    constexpr int kNR = D::NR, kNA = D::NA, kNA2 = D::NA2;
-    // radial sums are compensated (Kahan): q_0 ~ 4 accumulates ~28 terms and
-    // its plain FP32 rounding dominates the site-energy error budget
-    float qR[kNR], qC[kNR];
-#pragma unroll
-    for (int a = 0; a < kNR; ++a) qR[a] = qC[a] = 0.f;
-#pragma unroll
-    for (int a = 0; a < kNA2; ++a)
-#pragma unroll
-        for (int b = 0; b < kLM; ++b) S[a][b] = make_float2(0.f, 0.f);
-
-    // Slots are sorted by increasing distance (MD lists); walk the ranks
-    // downwards so the largest (nearest) terms are added last, with all lanes
-    // of a warp at the same rank.
-#ifdef __CUDA_ARCH__
-    const int kmax = __reduce_max_sync(0xffffffffu, cnt);
-#else
-    const int kmax = cnt;
-#endif
-    NbSlot nx;
-    fetch_slot(nbr, xr, n, kmax - 1, cnt, nx);
-    for (int k = kmax - 1; k >= 0; --k) {
-        const NbSlot cur = nx;
-        fetch_slot(nbr, xr, n, k - 1, cnt, nx);
-        if (k >= cnt) continue;
-        float rx, ry, rz;
-        pair_vector(cur.v >> 24, hi, li, cur.h, cur.l, box, rx, ry, rz);
-        const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-        const float w = pair_weight(P, zi, cur.z);
-        if (d2 < P.rcR2) {
-            const float d = sqrtf(d2);
-            float g[kNR];
-            radial_g<kNR>(d, P.rcR, P.inv_rcR, g, w);
-#pragma unroll
-            for (int a = 0; a < kNR; ++a) {
-                const float y = g[a] - qC[a];
-                const float t = qR[a] + y;
-                qC[a] = (t - qR[a]) - y;
-                qR[a] = t;
-            }
-        }
-        if (d2 < P.rcA2) {
-            const float d = sqrtf(d2);
-            float g[kNA];
-            radial_g<kNA>(d, P.rcA, P.inv_rcA, g, w);
-            float2 g2[kNA2];
-            pair_orders(g, g2);
-            float ux, uy, uz;
-            unit_vector(rx, ry, rz, ux, uy, uz);
-            sh_pass1(ux, uy, uz, g2, S);
-        }
-    }
-
-    // descriptor vector: q_nl = sum_m c_lm S_nlm^2 (compensated), n outer, l inner
-#pragma unroll
-    for (int a = 0; a < kNR; ++a) q[a] = qR[a] - qC[a];
-#pragma unroll
-    for (int a = 0; a < kNA; ++a) {
-#pragma unroll
-        for (int l = 0; l < kLmax; ++l) q[kNR + a * kLmax + l] = 0.f;
-        float qc[kLmax] = {0.f, 0.f, 0.f, 0.f};  // Kahan compensation per l
-#pragma unroll
-        for (int m = 0; m < kLM; ++m) {
-            const int v = kNR + a * kLmax + sh_l(m);
-            const float y = fmaf(sh_c(m) * harm(S, a, m), harm(S, a, m), -qc[sh_l(m)]);
-            const float t = q[v] + y;
-            qc[sh_l(m)] = (t - q[v]) - y;
-            q[v] = t;
-        }
-#pragma unroll
-        for (int l = 0; l < kLmax; ++l) q[kNR + a * kLmax + l] -= qc[l];
-    }
-}
-
-// Partial force dU_i/dr_ij of one pair r = r_ij (d2 = |r|^2 < max cutoff^2)
-// from the atom's coefficients A_nlm = 2 c_lm G_nl S_nlm and G_n (Eqs.
-// 23-25): radial G_n g_n' rhat, angular sum_nlm A_nlm grad(g_n Z_lm).
-//
-// It also returns dE, the first-order correction of the site energy for the
-// roundings of this pair's geometry in the descriptor pass: there the
-// descriptors were evaluated at the FP32 distance d = sqrtf(d2) and unit
-// vector u (each rounded), from the pair vector r rounded from the exact
-// r + r_lo.  With dU/dd (the radial coefficient below) and dU/du (the
-// unprojected harmonic gradient V, Z_lm being polynomials in u),
-//   dE = dU/dd (|r + r_lo| - d) + dU/du . ((r + r_lo)/|r + r_lo| - u),
-// which removes those roundings from U_i to second order (~1e-14 relative).
-template <class D, class ArrA, class ArrR>
-__host__ __device__ __forceinline__ void pair_partial_force(const float (&r)[3], const float (&r_lo)[3], float d2,
-                                                            float w, const SiteParams& P, const ArrA& A,
-                                                            const ArrR& GR, float& px, float& py, float& pz,
-                                                            float& dE)
-{
-    constexpr int kNR = D::NR, kNA = D::NA;
-    const float d = sqrtf(d2);
-    float ux, uy, uz, u_res[3], dres, inv;
-    unit_vector_res(r[0], r[1], r[2], d, ux, uy, uz, u_res, dres, inv);
-    float radial = 0.f;  // coefficient of rhat (dU/dd)
-    float Vx = 0.f, Vy = 0.f, Vz = 0.f;
-    // geometry residuals: r_lo along and across u
-    const float ur = fmaf(ux, r_lo[0], fmaf(uy, r_lo[1], uz * r_lo[2]));
-    const float dd = dres + ur;
-    if (d2 < P.rcR2) {
-        float2 gd[kNR];
-        radial_gd<kNR>(d, P.rcR, P.inv_rcR, gd, w);
-#pragma unroll
-        for (int a = 0; a < kNR; ++a) radial = fmaf(GR[a], gd[a].y, radial);
-    }
-    float eu = 0.f;
-    if (d2 < P.rcA2) {
-        float2 gd[kNA];
-        radial_gd<kNA>(d, P.rcA, P.inv_rcA, gd, w);
-        float2 Vxy = make_float2(0.f, 0.f);
-        sh_pass2(ux, uy, uz, A, gd, radial, Vxy, Vz);
-        const float dux = fmaf(fmaf(-ux, ur, r_lo[0]), inv, u_res[0]);
-        const float duy = fmaf(fmaf(-uy, ur, r_lo[1]), inv, u_res[1]);
-        const float duz = fmaf(fmaf(-uz, ur, r_lo[2]), inv, u_res[2]);
-        eu = fmaf(Vxy.x, dux, fmaf(Vxy.y, duy, Vz * duz));
-        // tangential projection of V, divided by r
-        const float uv = fmaf(ux, Vxy.x, fmaf(uy, Vxy.y, uz * Vz));
-        Vx = (Vxy.x - uv * ux) * inv;
-        Vy = (Vxy.y - uv * uy) * inv;
-        Vz = (Vz - uv * uz) * inv;
-    }
-    dE = fmaf(radial, dd, eu);
-    px = fmaf(radial, ux, Vx);
-    py = fmaf(radial, uy, Vy);
-    pz = fmaf(radial, uz, Vz);
-}
-
-// Pass 1 and the network of atom i: site energy (hi + lo) and the
-// coefficients A (kNA x kLM, in place of the harmonic sums S) and GR.
-template <class D = DescSi>
-__host__ __device__ __forceinline__ void site_coefficients(int i, bool active, int n, int cnt, const SlotTable& nbr,
-                                                           const float* __restrict__ xr, const Box& box,
-                                                           const SiteParams& P, HarmT<D>& S,
-                                                           float (&GR)[D::NR], float& U_hi, float& U_lo)
-{
-    constexpr int kNR = D::NR, kNA = D::NA, kNdes = D::Ndes;
-    float hi[3], li[3], zi = 1.f;
-    if (active) {
-        load_pos(xr, i, hi, li);
-        zi = load_z(xr, i);
-    }
-    float q[kNdes];
-    site_descriptors<D>(i, n, cnt, nbr, xr, box, P, hi, li, zi, q, S);
-
-    float G[kNdes];
-    network(P.w, P.n_neu, q, G, U_hi, U_lo);
-
-    // A_nlm = 2 c_lm G_nl S_nlm (reuses S)
-#pragma unroll
-    for (int a = 0; a < kNA; ++a) {
-#pragma unroll
-        for (int m = 0; m < kLM; ++m) {
-            harm(S, a, m) *= 2.f * sh_c(m) * G[kNR + a * kLmax + sh_l(m)];
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < kNR; ++a) GR[a] = G[a];
-}
-
-// Everything atom i contributes in the first force pass, in one thread: site
-// energy and the partial forces dU_i/dr_ij of its first cnt slots (written
-// through `out` for slots within max(rc_R, rc_A); other slots are left
-// untouched).
-template <class D = DescSi>
-__host__ __device__ __forceinline__ void site_partial_forces(int i, bool active, int n, int cnt,
-                                                             const SlotTable& nbr, const float* __restrict__ xr, const Box& box,
-                                                             const SiteParams& P, const PfOut& out, float& U_hi,
-                                                             float& U_lo)
-{
-    HarmT<D> S;
-    float GR[D::NR];
-    site_coefficients<D>(i, active, n, cnt, nbr, xr, box, P, S, GR, U_hi, U_lo);
-    float hi[3], li[3], zi = 1.f;
-    if (active) {
-        load_pos(xr, i, hi, li);
-        zi = load_z(xr, i);
-    }
-
-    const float rc2max = P.rcR2 > P.rcA2 ? P.rcR2 : P.rcA2;
-    // pass 2: partial forces, and the first-order energy correction of the
-    // pair geometry's roundings (summed in FP32: each term is ~1e-7 eV)
-    float dU = 0.f;
-    NbSlot nx;
-    fetch_slot(nbr, xr, n, 0, cnt, nx);
-    for (int k = 0; k < cnt; ++k) {
-        const NbSlot cur = nx;
-        fetch_slot(nbr, xr, n, k + 1, cnt, nx);
-        float r[3], r_lo[3];
-        pair_vector_lo(cur.v >> 24, hi, li, cur.h, cur.l, box, r, r_lo);
-        const float d2 = fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2]));
-        if (!(d2 < rc2max)) continue;
-        float px, py, pz, dE;
-        pair_partial_force<D>(r, r_lo, d2, pair_weight(P, zi, cur.z), P, S, GR, px, py, pz, dE);
-        dU += dE;
-        const int ko = nbr.orig ? (int)nbr.orig[(size_t)k * nbr.stride + nbr.idx] : k;
-        float* p = out.base + (size_t)ko * out.slot_stride;
-        p[0] = px;
-        p[out.comp_stride] = py;
-        p[2 * out.comp_stride] = pz;
-    }
-    U_lo += dU;
 }
 
 // Force and per-atom virial of atom i from the stored partial forces

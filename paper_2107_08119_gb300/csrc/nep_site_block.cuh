@@ -1,6 +1,5 @@
 // nep_site_block.cuh -- the site pass of the force path as a cooperation of
-// four warps on 32 atoms (the arithmetic of nep_site.cuh, operation for
-// operation).
+// four warps on 32 (or 16 or 8) atoms.
 //
 // What bounds it: instruction issue and dependency latency, not memory (the
 // list, positions and partial forces of a 125k-atom box are about 150 MB per
@@ -106,8 +105,7 @@ struct ShFast {
     }
 };
 
-// B += cd Y, V += cg grad Y for harmonic LM (its unprojected gradient), as
-// sh_term does.
+// B += cd Y, V += cg grad Y for harmonic LM (its unprojected gradient).
 template <int LM>
 __device__ __forceinline__ void sh_add(const ShFast& s, float cg, float cd, float& B, float (&V)[3])
 {
@@ -161,7 +159,7 @@ __device__ __forceinline__ void site_block_harmonics(const float* tile, int sub,
 }
 
 // The descriptors q_nl of order n from the harmonic sums in the atom's column
-// (compensated over m, as in site_descriptors)
+// (compensated over m): q_nl = sum_m c_lm S_nlm^2
 template <class D, int AT>
 __device__ __forceinline__ void site_block_descriptors(int n, const float* s_S, float* s_q)
 {
@@ -235,8 +233,8 @@ __device__ __forceinline__ float site_pair_radial(const PairGeom& g, const SiteP
     return radial;
 }
 
-// Angular terms of one pair against the atom's coefficients (the sums of
-// sh_pass2): (cg, cd) = sum_n A_nlm (g_n, g_n'), B += cd Y, V += cg grad_u Y,
+// Angular terms of one pair against the atom's coefficients:
+// (cg, cd) = sum_n A_nlm (g_n, g_n'), B += cd Y, V += cg grad_u Y,
 // two harmonics per packed FMA.  Gradient components that are zero for every
 // direction (a third of them) are left out.  gg, gp: (g_n, g_n), (g_n', g_n').
 template <class D, int AT, int J>
@@ -257,45 +255,77 @@ __device__ __forceinline__ void site_angular_terms(const float* s_A, const ShFas
     }
 }
 
-// The site pass of the block's atoms.  z: the parameters; pf: partial-force
-// records [k][n] float4; mask: in-cutoff bits [3][n] of the first 96 slots,
-// or NULL.  WORDS: 32-bit words of own-slot bits per thread.  The first AT
-// lanes of warp 0 return the site energies (hi + lo).
-template <class D, int AT, int WORDS>
-__device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, const int* __restrict__ nbr,
-                                           const float* __restrict__ xr, const Box& box,
-                                           const float* __restrict__ z, int n_par, SiteParams P,
-                                           float* __restrict__ pf, unsigned* __restrict__ mask, float& U_hi,
-                                           float& U_lo)
+// One lane's atom and its pairs: the MD list (slot-major nbr[k][n], partial
+// forces pf[k][n] float4), or a training set's CSR pairs (pj[p0 + k], partial
+// forces of three floats each).
+struct SlotMajorPairs {
+    const int* nbr;
+    float4* pf;
+    size_t n;
+    int ia;
+    __device__ __forceinline__ int value(int k) const { return nbr[(size_t)k * n + ia]; }
+    __device__ __forceinline__ void store(int k, float x, float y, float z) const
+    {
+        pf[(size_t)k * n + ia] = make_float4(x, y, z, 0.f);
+    }
+};
+
+struct CsrPairs {
+    const int* pj;  // of the atom's first pair
+    float* pf;
+    __device__ __forceinline__ int value(int k) const { return pj[k]; }
+    __device__ __forceinline__ void store(int k, float x, float y, float z) const
+    {
+        pf[3 * (size_t)k] = x;
+        pf[3 * (size_t)k + 1] = y;
+        pf[3 * (size_t)k + 2] = z;
+    }
+};
+
+// Shared memory of a block of AT atoms.
+template <class D, int AT>
+struct SiteShared {
+    float* w;        // parameters
+    float* A;        // [quads][AT] float4: pair tile, then S, then A
+    float* q;        // [ND][AT]: q, then G
+    float* x;        // radial tile; then x_mu, w2 (1 - x_mu^2): [n_neu][AT][2]
+    unsigned* mask;  // [3][AT]
+    __device__ __forceinline__ SiteShared(float* base, int n_par, int n_neu)
+    {
+        w = base;
+        A = w + (n_par + 31) / 32 * 32;
+        q = A + 4 * AT * site_block_quads<D>();
+        x = q + AT * D::Ndes;
+        mask = reinterpret_cast<unsigned*>(x + 2 * AT * (n_neu > kSiteChunk ? n_neu : kSiteChunk));
+    }
+};
+
+// Descriptor sums of the block's atoms: q in sh.q, the harmonic sums S in
+// sh.A, and the own-slot bits of the thread (slot k = WAYS b + way is bit
+// b mod 32 of word b / 32): kept (within either cutoff) and ang (within the
+// angular one).  Also zeroes sh.mask and loads the parameters z.  Ends with a
+// barrier.
+template <class D, int AT, int WORDS, class Pairs>
+__device__ __forceinline__ void site_block_sums(const Pairs& pairs, int cnt, const float* __restrict__ xr,
+                                                const Box& box, const float* __restrict__ z, int n_par,
+                                                const SiteParams& P, const SiteShared<D, AT>& sh,
+                                                const float (&hi)[3], const float (&li)[3], float zi,
+                                                unsigned (&kept)[WORDS], unsigned (&ang)[WORDS])
 {
-    constexpr int NR = D::NR, NA = D::NA, ND = D::Ndes;
+    constexpr int NR = D::NR, NA = D::NA;
     constexpr int SUB = SiteSplit<AT>::SUB, WAYS = SiteSplit<AT>::WAYS;
     constexpr int OWN = kSiteChunk / WAYS;  // slots of a tile per thread
-    extern __shared__ __align__(16) float s_site[];
-    __shared__ float s_dU[WAYS][AT];
     __shared__ unsigned s_any[kSiteChunk];  // per tile slot: 1 an angular pair in some lane, 2 a radial one
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int at = lane % AT, sub = lane / AT;
     const int way = SUB * warp + sub;  // this thread's share of the atom's work
-    float* s_w = s_site;
-    float* s_A = s_w + (n_par + 31) / 32 * 32;         // [quads][AT] float4
-    float* s_q = s_A + 4 * AT * site_block_quads<D>();  // [ND][AT]
-    float* s_x = s_q + AT * ND;                        // radial tile; then x_mu, w2 (1 - x_mu^2): [n_neu][AT][2]
-    unsigned* s_mask = reinterpret_cast<unsigned*>(s_x + 2 * AT * (P.n_neu > kSiteChunk ? P.n_neu : kSiteChunk));
-    for (int t = threadIdx.x; t < n_par; t += kSiteThreads) s_w[t] = z[t];
-    if (threadIdx.x < 3 * AT) s_mask[threadIdx.x] = 0u;
+    float *s_A = sh.A, *s_q = sh.q, *s_x = sh.x;
+    for (int t = threadIdx.x; t < n_par; t += kSiteThreads) sh.w[t] = z[t];
+    if (threadIdx.x < 3 * AT) sh.mask[threadIdx.x] = 0u;
     if (threadIdx.x < kSiteChunk) s_any[threadIdx.x] = 0u;
-    P.w = s_w;
-    const int ia = active ? i : 0;
-    float hi[3], li[3], zi;
-    load_pos(xr, ia, hi, li, zi);
     const int kmax = __reduce_max_sync(0xffffffffu, cnt);  // the same in every warp
     const int chunks = (kmax + kSiteChunk - 1) / kSiteChunk;
     const float rc2max = P.rcR2 > P.rcA2 ? P.rcR2 : P.rcA2;
-
-    // own slots k = WAYS b + way: bit b of word b / 32 in kept (within either
-    // cutoff) and ang (within the angular one)
-    unsigned kept[WORDS], ang[WORDS];
 #pragma unroll
     for (int w = 0; w < WORDS; ++w) kept[w] = ang[w] = 0u;
 
@@ -318,7 +348,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
         auto k_of = [&](int q) { return (chunks - 1 - q / OWN) * kSiteChunk + WAYS * (q % OWN) + way; };
         auto load_v = [&](int q) {
             const int k = k_of(q);
-            return q < OWN * chunks && k < cnt ? nbr[(size_t)k * n + ia] : -1;
+            return q < OWN * chunks && k < cnt ? pairs.value(k) : -1;
         };
         auto load_record = [&](int v, NbRecord& r) {
             r.v = v;
@@ -432,29 +462,56 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
                 if (a + 1 < NR) s_q[(a + 1) * AT + at] = R.y + nc.y;
             }
         }
-        if (mask) {
-            // slot k = WAYS b + way is bit k mod 32 of word k / 32
-            if constexpr (WAYS == 4) {
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {  // own bits 8 j .. 8 j + 7, spread to every fourth
-                    unsigned e = (kept[0] >> (8 * j)) & 0xFFu;
-                    e = (e | (e << 12)) & 0x000F000Fu;
-                    e = (e | (e << 6)) & 0x03030303u;
-                    e = (e | (e << 3)) & 0x11111111u;
-                    if (e) atomicOr(s_mask + j * AT + at, e << way);
-                }
-            } else {
-                for (unsigned m = kept[0]; m; m &= m - 1) {
-                    const int k = WAYS * (__ffs((int)m) - 1) + way;
-                    atomicOr(s_mask + (k >> 5) * AT + at, 1u << (k & 31));
-                }
-            }
-        }
     }
     __syncthreads();
     for (int a = way; a < NA; a += WAYS) site_block_descriptors<D, AT>(a, s_A + 4 * at, s_q + at);
-    if (mask && warp < 3 && lane < AT && active) mask[(size_t)warp * n + i] = s_mask[warp * AT + lane];
     __syncthreads();
+}
+
+// The site pass of the block's atoms.  z: the parameters; mask: in-cutoff
+// bits [3][n] of the first 96 slots, or NULL (i, n: the lane's atom and the
+// number of atoms).  WORDS: 32-bit words of own-slot bits per thread.  The
+// first AT lanes of warp 0 return the site energies (hi + lo).
+template <class D, int AT, int WORDS, class Pairs>
+__device__ __forceinline__ void site_block(const Pairs& pairs, int i, bool active, int n, int cnt,
+                                           const float* __restrict__ xr, const Box& box,
+                                           const float* __restrict__ z, int n_par, SiteParams P,
+                                           unsigned* __restrict__ mask, float& U_hi, float& U_lo)
+{
+    constexpr int NA = D::NA, ND = D::Ndes;
+    constexpr int SUB = SiteSplit<AT>::SUB, WAYS = SiteSplit<AT>::WAYS;
+    extern __shared__ __align__(16) float s_site[];
+    __shared__ float s_dU[WAYS][AT];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int at = lane % AT, sub = lane / AT;
+    const int way = SUB * warp + sub;  // this thread's share of the atom's work
+    const SiteShared<D, AT> sh(s_site, n_par, P.n_neu);
+    float *s_w = sh.w, *s_A = sh.A, *s_q = sh.q, *s_x = sh.x;
+    unsigned* s_mask = sh.mask;
+    P.w = s_w;
+    const int ia = active ? i : 0;
+    float hi[3], li[3], zi;
+    load_pos(xr, ia, hi, li, zi);
+    unsigned kept[WORDS], ang[WORDS];
+    site_block_sums<D, AT, WORDS>(pairs, cnt, xr, box, z, n_par, P, sh, hi, li, zi, kept, ang);
+    if (mask) {
+        // slot k = WAYS b + way is bit k mod 32 of word k / 32
+        if constexpr (WAYS == 4) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {  // own bits 8 j .. 8 j + 7, spread to every fourth
+                unsigned e = (kept[0] >> (8 * j)) & 0xFFu;
+                e = (e | (e << 12)) & 0x000F000Fu;
+                e = (e | (e << 6)) & 0x03030303u;
+                e = (e | (e << 3)) & 0x11111111u;
+                if (e) atomicOr(s_mask + j * AT + at, e << way);
+            }
+        } else {
+            for (unsigned m = kept[0]; m; m &= m - 1) {
+                const int k = WAYS * (__ffs((int)m) - 1) + way;
+                atomicOr(s_mask + (k >> 5) * AT + at, 1u << (k & 31));
+            }
+        }
+    }
 
     // ---- network: neurons mu = way mod WAYS
     const float* b1 = s_w + P.n_neu * ND;
@@ -471,6 +528,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
         }
     }
     __syncthreads();
+    if (mask && warp < 3 && lane < AT && active) mask[(size_t)warp * n + i] = s_mask[warp * AT + lane];
     {
         // G_v of this thread's share of the descriptors, in s_q
         constexpr int VB = (ND + WAYS - 1) / WAYS;
@@ -528,12 +586,19 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
     }
     __syncthreads();
 
-    // ---- partial forces of the own slots, and the first-order energy
-    // correction of the pair geometry's roundings (nep_site.cuh)
+    // ---- partial forces dU_i/dr_ij of the own slots (Eqs. 23-25): radial
+    // G_n g_n' rhat, angular sum_nlm A_nlm grad(g_n Z_lm); and the first-order
+    // correction of the site energy for the roundings of the pair's geometry
+    // in the descriptor sums.  There the descriptors were evaluated at the FP32
+    // distance d and unit vector u (each rounded), from the pair vector r
+    // rounded from the exact r + r_lo; with dU/dd (the radial coefficient) and
+    // dU/du (the unprojected harmonic gradient V, Z_lm being polynomials in u)
+    //   dE = dU/dd (|r + r_lo| - d) + dU/du . ((r + r_lo)/|r + r_lo| - u)
+    // removes those roundings from U_i to second order (~1e-14 relative; the
+    // terms are ~1e-7 eV, summed in FP32).
     float dU = 0.f;
     const float* sA = s_A + 4 * at;
     const float* sG = s_q + at;
-    float4* out = reinterpret_cast<float4*>(pf) + ia;
     // the next own slot, the angular pairs of a word before the others: k, or
     // -1; its list value is loaded two pairs ahead, the record one ahead
     auto next_slot = [&](bool& angular) {
@@ -553,18 +618,18 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
         NbRecord nb, nb_nx;
         int k = next_slot(angular);
         if (k >= 0) {
-            nb.v = nbr[(size_t)k * n + ia];
+            nb.v = pairs.value(k);
             load_pos(xr, nb.v & 0xFFFFFF, nb.h, nb.l, nb.z);
         }
         int k_nx = next_slot(angular_nx);
-        if (k_nx >= 0) nb_nx.v = nbr[(size_t)k_nx * n + ia];
+        if (k_nx >= 0) nb_nx.v = pairs.value(k_nx);
 #pragma unroll 1
         while (k >= 0) {
             bool angular_n2 = false;
             const int k_n2 = next_slot(angular_n2);
             int v_n2 = 0;
             if (k_nx >= 0) load_pos(xr, nb_nx.v & 0xFFFFFF, nb_nx.h, nb_nx.l, nb_nx.z);
-            if (k_n2 >= 0) v_n2 = nbr[(size_t)k_n2 * n + ia];
+            if (k_n2 >= 0) v_n2 = pairs.value(k_n2);
             PairGeom g;
             site_pair_geometry(nb, box, P, hi, li, zi, g);
             float radial = site_pair_radial<D, AT>(g, P, sG);
@@ -591,8 +656,7 @@ __device__ __forceinline__ void site_block(int i, bool active, int n, int cnt, c
                 for (int a = 0; a < 3; ++a) V[a] = (V[a] - uv * g.u[a]) * g.inv;
             }
             dU += fmaf(radial, g.dd, eu);
-            out[(size_t)k * n] = make_float4(fmaf(radial, g.u[0], V[0]), fmaf(radial, g.u[1], V[1]),
-                                             fmaf(radial, g.u[2], V[2]), 0.f);
+            pairs.store(k, fmaf(radial, g.u[0], V[0]), fmaf(radial, g.u[1], V[1]), fmaf(radial, g.u[2], V[2]));
             k = k_nx;
             angular = angular_nx;
             nb = nb_nx;

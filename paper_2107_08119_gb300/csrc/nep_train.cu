@@ -48,7 +48,6 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kDsCap = 192;      // neighbour capacity per atom while building (within r_c)
 constexpr int kChunkAtoms = 32;       // atoms per contraction block (chunks never span structures)
 constexpr int kOwnerMaxThreads = 256;  // owner pass: 4 or 8 warps per block, one atom per warp at a time
 

@@ -126,3 +126,36 @@ def test_population_network_shapes(orc, n_struct, n_pop, n_neu, threads):
         assert np.abs(got[k] - want).max() <= 3e-4, (k, got[k], want)
     ds.close()
     model.close()
+
+
+@pytest.mark.parametrize("n_struct", [1, 40, 110, 140])
+def test_adjoint_by_atoms_per_block(orc, n_struct):
+    """The force loss and its gradient with 8 atoms per block (1 and 40
+    structures), 16 and 32, and ragged tails: against the oracle for the small
+    set, and by a central difference of the loss along the gradient for all
+    (the loss is smooth: step 1e-3 |z| leaves ~1e-6 relative, FP32 forces
+    ~1e-4 of the difference)."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(n_struct)
+    structures = inputs.training_structures(n_struct, seed_stream=77)
+    n = sum(len(s["pos"]) for s in structures)
+    f = rng.normal(0.0, 1.0, (n, 3))
+    z = inputs.random_z(1021, rng).astype(np.float32)
+    model = nep.NEP(z)
+    ds = nep.Dataset(model, structures, np.zeros(n_struct), f, np.zeros((n_struct, 6)))
+    t = torch.tensor(z, device="cuda", requires_grad=True)
+    loss = nep.force_loss(t, ds)
+    loss.backward()
+    g = t.grad.double()
+    if n_struct == 1:
+        want, lf = orc.force_loss_grad(orc.NepHyper(), f32_exact(z), structures, f)
+        assert abs(loss.item() - lf) <= 1e-6 * lf
+        assert np.abs(g.cpu().numpy() - want).max() <= 1e-5 * np.abs(want).max()
+    d = g / g.norm()
+    h = 1e-3 * float(t.detach().norm())
+    up, dn = ((t.detach().double() + s * h * d).float() for s in (1.0, -1.0))
+    fd = (ds.force_loss(up) - ds.force_loss(dn)).item() / float(((up - dn).double() * d).sum())
+    assert abs(fd - float(g.norm())) <= 2e-3 * float(g.norm()), (fd, float(g.norm()))
+    ds.close()
+    model.close()
