@@ -371,6 +371,9 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
                         double* x_ref,
                         float r_list, unsigned* d_err, const unsigned* d_gate, cudaStream_t st);
 
+// whether the list of n atoms in a box with a cell grid is built by direct tests
+bool list_is_direct(int n);
+
 // force path (nep_force.cu)
 struct ForceArgs {
     const float* z;          // parameters on the device

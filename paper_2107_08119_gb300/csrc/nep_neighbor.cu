@@ -768,6 +768,8 @@ constexpr int kListGridCap = 152 * 16;
 // launches instead of six).
 constexpr int kDirectMax = 2500;
 
+bool list_is_direct(int n) { return n <= kDirectMax; }
+
 int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, const float* zatom, bool wrap_in_place,
                         double* x_ref,
                         float r_list, unsigned* d_err, const unsigned* d_gate, cudaStream_t st)

@@ -188,11 +188,12 @@ extern "C" int nep_compute_efv_static(const nep_hyper* hp, const float* z, int n
     double* partials = reinterpret_cast<double*>(base + kOffPartials);
     unsigned* err = reinterpret_cast<unsigned*>(base + kOffErr);
 
-    // the cell counters and the error word must start at zero; the array
-    // keeps whatever the previous call left
-    if ((rc = cuda_fail(cudaMemsetAsync(nl.cell_count, 0, sizeof(int) * (ncell + 1), st), "cudaMemsetAsync")) ||
-        (rc = cuda_fail(cudaMemsetAsync(nl.cell_fill, 0, sizeof(int) * (ncell + 1), st), "cudaMemsetAsync")) ||
-        (rc = cuda_fail(cudaMemsetAsync(err, 0, sizeof(unsigned), st), "cudaMemsetAsync")))
+    // the error word must start at zero, and for the cells path its counters
+    // (the build leaves them zero, but not when a call failed between launches)
+    if ((rc = cuda_fail(cudaMemsetAsync(err, 0, sizeof(unsigned), st), "cudaMemsetAsync"))) return rc;
+    if (ncell > 0 && !list_is_direct(n) &&
+        ((rc = cuda_fail(cudaMemsetAsync(nl.cell_count, 0, sizeof(int) * (ncell + 1), st), "cudaMemsetAsync")) ||
+         (rc = cuda_fail(cudaMemsetAsync(nl.cell_fill, 0, sizeof(int) * (ncell + 1), st), "cudaMemsetAsync"))))
         return rc;
 
     if ((rc = build_neighbor_list(nl, box, n, const_cast<double*>(pos), nullptr, false, nullptr, (float)rmax, err, nullptr,

@@ -122,8 +122,11 @@ def _ptr(t):
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return _vp(s.cuda_stream)
+    # the raw handle of the current stream of the current device: building the
+    # torch.cuda.Stream object takes about 3 us per call
+    if stream is None:
+        return _vp(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return _vp(stream.cuda_stream)
 
 
 def _box9(box):
@@ -501,7 +504,7 @@ class Dataset:
         """seed * dL_f/dz at the z of the last force_loss (CUDA float64 (n_par,));
         seed: CUDA float64 scalar tensor or None for 1."""
         grad = torch.empty(self.model.hyper.n_par, dtype=torch.float64, device="cuda")
-        if seed is not None:
+        if seed is not None and not (seed.is_cuda and seed.dtype == torch.float64 and seed.numel() == 1):
             seed = seed.detach().to(device="cuda", dtype=torch.float64).reshape(1).contiguous()
         _check(_lib.nep_force_loss_backward(self.model._h, self._h, None if seed is None else _ptr(seed), _ptr(grad),
                                             _stream(stream)), "nep_force_loss_backward")
