@@ -166,7 +166,7 @@ int ensure_workspace(Workspace& ws, int n, int m_cap, int ncell, int nblocks_par
         dev_free(nl.pf);
         dev_free(nl.xr);
         dev_free(nl.atom_cell);
-        dev_free(nl.cell_atoms);
+        dev_free(nl.xs);
         dev_free(nl.mask);
         dev_free(ws.force);
         nl.n_cap = nl.m_cap = 0;
@@ -177,7 +177,7 @@ int ensure_workspace(Workspace& ws, int n, int m_cap, int ncell, int nblocks_par
             (rc = dev_alloc(&nl.vala, N * M, "neighbour list copy")) ||
             (rc = dev_alloc(&nl.pf, N * M * 4, "partial forces")) || (rc = dev_alloc(&nl.xr, N * 8, "positions")) ||
             (rc = dev_alloc(&nl.atom_cell, N, "cell index")) ||
-            (rc = dev_alloc(&nl.cell_atoms, N, "cell atoms")) || (rc = dev_alloc(&nl.mask, N * 3, "slot masks")) ||
+            (rc = dev_alloc(&nl.xs, N, "cell atoms")) || (rc = dev_alloc(&nl.mask, N * 3, "slot masks")) ||
             (rc = dev_alloc(&ws.force, N * 3, "forces")))
             return rc;
         nl.n_cap = n;
@@ -222,7 +222,7 @@ void free_workspace(Workspace& ws)
     dev_free(nl.cell_count);
     dev_free(nl.cell_start);
     dev_free(nl.cell_fill);
-    dev_free(nl.cell_atoms);
+    dev_free(nl.xs);
     dev_free(nl.mask);
     dev_free(ws.partials);
     dev_free(ws.force);

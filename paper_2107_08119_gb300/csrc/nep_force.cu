@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_assemble_atoms(int n, int m_cap
 
 // One total per block, the totals of `a` and then those of `b`: several SMs
 // share the FP64 adds, which are slow on this part.
-constexpr int kSumThreads = 128;
+constexpr int kSumThreads = 512;
 __global__ void __launch_bounds__(kSumThreads) k_sum(SumSet a, SumSet b)
 {
     const bool first = blockIdx.x < a.ncomp;

@@ -4,9 +4,7 @@
 //   positions        FP64 [3][n] (caller) + FP32 hi/lo records xr [n][8]
 //   neighbour list   int32 nbr[M][n] = j | image_code << 24, count[n]
 //                    int32 rev[M][n] = slot of i in j's list (reverse pair)
-//                    int32 vala[n][M]: scratch of the list build (the rank of
-//                    each unsorted slot; the values atom-major in the brute
-//                    search)
+//                    int32 vala[n][M]: the list values atom-major
 //   partial forces   FP32 pf[M][n] float4 (x, y, z, unused) = dU_i/dr_ij
 //                    (Eq. 23), slot-major: one 16-byte gather per reverse pair
 //   forces           FP32 [3][n], per-atom virials FP32 [9][n]
@@ -330,14 +328,14 @@ struct NeighborList {
     int* count = nullptr;
     int* nbr = nullptr;
     int* rev = nullptr;
-    int* vala = nullptr;     // list-build scratch [n][m_cap] (slot ranks, or values atom-major)
+    int* vala = nullptr;     // list values atom-major [n][m_cap]
     float* pf = nullptr;
     float* xr = nullptr;     // hi/lo position records [n][8]
     int* atom_cell = nullptr;
     int* cell_count = nullptr;
     int* cell_start = nullptr;
     int* cell_fill = nullptr;
-    int* cell_atoms = nullptr;
+    float4* xs = nullptr;    // hi parts and indices in cell order [n]
     // [3][n] words: bit k of atom i set when slot k lies within the cutoff,
     // written by the site pass from its cutoff tests; `mask_set`
     // (host) says whether the last site pass launched wrote them, so that

@@ -307,7 +307,7 @@ __global__ void k_scale_v(int n, double* __restrict__ vel, const double* __restr
 // order, then a fixed tree: deterministic).  Several SMs share the FP64 adds
 // (slow on this part).  The last block to finish (a count in ctl, which it
 // clears) writes the thermo row and J and the Berendsen factor.
-constexpr int kFinishThreads = 128;
+constexpr int kFinishThreads = 512;
 
 __global__ void __launch_bounds__(kFinishThreads) k_md_finish(const double* __restrict__ part_e, int nb_e,
                                                               const double* __restrict__ part_x, int nb_x,

@@ -51,20 +51,22 @@ __global__ void k_bin(int n, double* __restrict__ pos, const float* __restrict__
     for (int d = 0; d < 3; ++d) {
         const double L = b.L[d];
         const double x = pos[(size_t)d * n + i];
-        if (!isfinite(x)) atomicOr(err, kErrNonFinite);
-        // FP64 division is slow here: atoms within one box length of the box
-        // (all of them between MD rebuilds) wrap by one exact subtraction
-        double w;
-        if (x >= 0.0 && x < L)
-            w = x;
-        else if (x >= L && x < 2.0 * L)
-            w = x - L;
-        else if (x < 0.0 && x >= -L)
-            w = x + L;
-        else
-            w = x - L * floor(x / L);
-        if (w >= L) w -= L;
-        if (w < 0.0) w = 0.0;
+        // FP64 operations are slow here (comparisons and division among them):
+        // 0 <= x < L, nearly every atom, is one integer comparison of the bits
+        // (a negative or non-finite x compares above), and atoms within one box
+        // length of the box wrap by one exact subtraction
+        double w = x;
+        if ((unsigned long long)__double_as_longlong(x) >= (unsigned long long)__double_as_longlong(L)) {
+            if (!isfinite(x)) atomicOr(err, kErrNonFinite);
+            if (x >= L && x < 2.0 * L)
+                w = x - L;
+            else if (x < 0.0 && x >= -L)
+                w = x + L;
+            else if (!(x == 0.0))
+                w = x - L * floor(x / L);
+            if (w >= L) w -= L;
+            if (w < 0.0) w = 0.0;
+        }
         if (wrap_in_place) {
             pos[(size_t)d * n + i] = w;
             if (x_ref) x_ref[(size_t)d * n + i] = w;
@@ -91,7 +93,7 @@ __global__ void k_bin(int n, double* __restrict__ pos, const float* __restrict__
 // reads and writes; padded so that a thread's run of kScanPer consecutive
 // cells is conflict-free); warp shuffles and the warp totals give the prefix.
 constexpr int kScanThreads = 1024;
-constexpr int kScanPer = 8;
+constexpr int kScanPer = 8;  // 32 cells per thread and a third of the rounds took the same time
 constexpr int kScanRound = kScanThreads * kScanPer;
 
 __device__ __forceinline__ int scan_pad(int x) { return x + (x >> 5); }
@@ -159,15 +161,19 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(int ncell, int* __restric
     if (t == 0) start[ncell] = carry;
 }
 
+// Atoms in cell order: their hi parts with the index in the fourth word, so
+// that a cell's candidates are contiguous 16-byte reads.
 __global__ void k_scatter(int n, const int* __restrict__ atom_cell, const int* __restrict__ cell_start,
-                          int* __restrict__ cell_fill, int* __restrict__ cell_atoms, const unsigned* gate)
+                          int* __restrict__ cell_fill, const float* __restrict__ xr, float4* __restrict__ xs,
+                          const unsigned* gate)
 {
     if (gated_off(gate)) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int c = atom_cell[i];
     const int slot = atomicAdd(cell_fill + c, 1);
-    cell_atoms[cell_start[c] + slot] = i;
+    const float4 h = load_hi(xr, i);
+    xs[cell_start[c] + slot] = make_float4(h.x, h.y, h.z, __int_as_float(i));
 }
 
 // Warps per block of the warp-per-atom list kernels.
@@ -181,11 +187,12 @@ __device__ __forceinline__ unsigned long long sort_key(float d2, int v)
 }
 
 // The list in three steps, each pair's distance tested once (the cells path):
-//   k_half_cells  one warp per atom i scans the 14 cells of its half shell
-//                 (cell offsets after (0, 0, 0) in x-slowest order, and its
-//                 own cell for j > i), so that every pair within the list
-//                 radius is met by exactly one of its two atoms; the
-//                 quick hi-part test and the exact hi/lo test as before, and
+//   k_half_cells  one block per cell gathers the 14 cells of its half shell
+//                 (cell offsets after (0, 0, 0) in x-slowest order, and the
+//                 cell itself for j > i) into shared memory, and a warp per
+//                 atom i of the cell tests them, so that every pair within the
+//                 list radius is met by exactly one of its two atoms: a quick
+//                 hi-part test, the exact hi/lo test on the survivors, and
 //                 each accepted pair goes into both rows unsorted at slots
 //                 taken with atomics: (value, distance word, the partner
 //                 entry's slot).  The rows live in the partial-force buffer,
@@ -206,133 +213,180 @@ __device__ __forceinline__ unsigned long long sort_key(float d2, int v)
 // the rows and the reverse index are the same as those of the full-shell
 // search (the order of the unsorted slots, which the atomics decide, does
 // not reach the results).  The counts are cleared by k_bin.
-constexpr int kHalfCells = 14;
+// What bounds the search: issue.  A warp per atom that looked up its own cells,
+// prefix sums and candidate indices spent most of its instructions on those;
+// per cell they are done once for ~6 to 16 atoms, and the candidates are
+// contiguous reads: 105 -> 75 us for 125,000 atoms at 5 A, 92 -> 70 us for
+// 64,000 of the split model at 8 A.  WARPS warps share a cell's atoms: eight
+// while the cells are few (343 cells of 17 atoms: 17 us, with four 26), two for
+// small cells (6.4 atoms: 75 us, with four 86, with eight 131), else four (16
+// atoms: 70 us, with two 78, with eight 79).
+constexpr int kHalfQuick = 96;  // survivors of the quick test waiting for the exact one, per warp
+constexpr int kHalfRanges = 10;
 
-__global__ void __launch_bounds__(32 * kVerletWarps) k_half_cells(int n, int m_cap, float rv2,
-                                                                 const float* __restrict__ xr,
-                                                                 const int* __restrict__ atom_cell,
-                                                                 const int* __restrict__ cell_start,
-                                                                 const int* __restrict__ cell_atoms,
-                                                                 int* __restrict__ count, int* __restrict__ rows,
-                                                                 int lcap, unsigned* err, Box b, const unsigned* gate)
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) k_half_cells(int m_cap, float rv2, int cap,
+                                                          const float* __restrict__ xr,
+                                                          const float4* __restrict__ xs,
+                                                          const int* __restrict__ cell_start,
+                                                          int* __restrict__ count, int* __restrict__ rows, Box b,
+                                                          const unsigned* gate)
 {
     if (gated_off(gate)) return;
-    extern __shared__ int s_half[];
+    extern __shared__ __align__(16) float4 s_cand[];  // [cap]: x, y, z from the cell's corner, packed value
+    __shared__ int s_sq[WARPS][kHalfQuick];
+    __shared__ int s_r0[kHalfRanges], s_at[kHalfRanges + 1], s_code[kHalfRanges];
+    __shared__ float s_shift[kHalfRanges][3];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // per warp: lcap quick-test survivors, 15 prefix sums, 14 starts, codes, shifts
-    int* sq = s_half + (size_t)warp * (lcap + 6 * 32);
-    int* pre = sq + lcap;
-    int* cst = pre + 32;
-    int* ccode = cst + 32;
-    float* csh = reinterpret_cast<float*>(ccode + 32);
-    const float rq = sqrtf(rv2) + 1e-3f, rq2 = rq * rq;
-    for (int i = blockIdx.x * kVerletWarps + warp; i < n; i += gridDim.x * kVerletWarps) {
-        float hi[3], li[3];
-        load_pos(xr, i, hi, li);
-        const int cid = atom_cell[i];
-        const int cz = cid % b.nc[2];
-        const int cy = (cid / b.nc[2]) % b.nc[1];
-        const int cx = cid / (b.nc[2] * b.nc[1]);
-        // lane c < 14 describes half-shell cell c: offset index 13 + c of the
-        // 27 in x-slowest order (13 is the atom's own cell)
-        int ccount = 0;
-        if (lane < kHalfCells) {
-            const int o = 13 + lane;
-            int x2 = cx + o / 9 - 1, y2 = cy + (o / 3) % 3 - 1, z2 = cz + o % 3 - 1;
-            int sx = 0, sy = 0, sz = 0;
-            if (x2 < 0) { x2 += b.nc[0]; sx = -1; } else if (x2 >= b.nc[0]) { x2 -= b.nc[0]; sx = 1; }
-            if (y2 < 0) { y2 += b.nc[1]; sy = -1; } else if (y2 >= b.nc[1]) { y2 -= b.nc[1]; sy = 1; }
-            if (z2 < 0) { z2 += b.nc[2]; sz = -1; } else if (z2 >= b.nc[2]) { z2 -= b.nc[2]; sz = 1; }
-            const int c2 = (x2 * b.nc[1] + y2) * b.nc[2] + z2;
-            const int c2s = cell_start[c2];
-            ccount = cell_start[c2 + 1] - c2s;
-            cst[lane] = c2s;
-            ccode[lane] = image_code(sx, sy, sz);
-            csh[lane] = (float)sx * b.Lh[0];  // exact: s in {-1, 0, 1}
-            csh[32 + lane] = (float)sy * b.Lh[1];
-            csh[64 + lane] = (float)sz * b.Lh[2];
+    const int cell = blockIdx.x;
+    const int c0 = cell_start[cell], c1 = cell_start[cell + 1];
+    if (c0 == c1) return;
+    const int cz = cell % b.nc[2];
+    const int cy = (cell / b.nc[2]) % b.nc[1];
+    const int cx = cell / (b.nc[2] * b.nc[1]);
+    const float ox = (float)cx * (b.Lh[0] / (float)b.nc[0]), oy = (float)cy * (b.Lh[1] / (float)b.nc[1]),
+                oz = (float)cz * (b.Lh[2] / (float)b.nc[2]);
+    if (warp == 0) {
+        // lane r < 10: range r of candidates.  0: the cell itself; 1: the next
+        // along z; 2 + 2 c + part: column c of (dx, dy) = (0, 1), (1, -1),
+        // (1, 0), (1, 1), contiguous in z, part 1 what wraps across a z face
+        int r0 = 0, rn = 0, sx = 0, sy = 0, sz = 0;
+        if (lane < kHalfRanges) {
+            int x2 = cx, y2 = cy, z0 = cz, z1 = cz;
+            if (lane == 1) {
+                z0 = z1 = cz + 1;
+                if (z0 == b.nc[2]) {
+                    z0 = z1 = 0;
+                    sz = 1;
+                }
+            } else if (lane >= 2) {
+                const int col = (lane - 2) >> 1;
+                x2 += col == 0 ? 0 : 1;
+                y2 += col == 0 ? 1 : col - 2;
+                if (x2 >= b.nc[0]) { x2 -= b.nc[0]; sx = 1; }
+                if (y2 < 0) { y2 += b.nc[1]; sy = -1; } else if (y2 >= b.nc[1]) { y2 -= b.nc[1]; sy = 1; }
+                z0 = max(cz - 1, 0);
+                z1 = min(cz + 1, b.nc[2] - 1);
+                if (lane & 1) {
+                    z1 = z0 - 1;  // nothing
+                    if (cz == 0) {
+                        z0 = z1 = b.nc[2] - 1;
+                        sz = -1;
+                    } else if (cz == b.nc[2] - 1) {
+                        z0 = z1 = 0;
+                        sz = 1;
+                    }
+                }
+            }
+            if (z0 <= z1) {
+                const int base = (x2 * b.nc[1] + y2) * b.nc[2];
+                r0 = cell_start[base + z0];
+                rn = cell_start[base + z1 + 1] - r0;
+            }
         }
-        int incl = ccount;
+        int incl = rn;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += t;
         }
-        if (lane <= kHalfCells) pre[lane] = incl - ccount;
-        if (lane < kHalfCells) cst[lane] -= incl - ccount;
-        __syncwarp();
-        const int total = pre[kHalfCells];
-        // pass 1, quick rejection with the hi parts only: their pair vector is
-        // within 1e-4 A of the hi/lo one, so the 1e-3 A margin never drops a
-        // pair that the exact test keeps; survivors are compacted into sq
-        int nq = 0, c0 = 0;
-        for (int base = 0; base < total; base += 32) {
-            const int idx = base + lane;
-            bool pass = false;
-            int value = 0;
-            int c = c0;
-            if (idx < total) {
-                while (pre[c + 1] <= idx) ++c;
-                const int j = cell_atoms[cst[c] + idx];
-                // own cell (c == 0): the pairs with j > i only
-                if (c != 0 || j > i) {
-                    const float4 a = load_hi(xr, j);
-                    const float qx = (a.x - hi[0]) + csh[c];
-                    const float qy = (a.y - hi[1]) + csh[32 + c];
-                    const float qz = (a.z - hi[2]) + csh[64 + c];
-                    pass = j != i && fmaf(qx, qx, fmaf(qy, qy, qz * qz)) < rq2;
-                    value = j | (ccode[c] << 24);
-                }
-            }
-            c0 = __shfl_sync(0xffffffffu, c, 31);
-            const unsigned mask = __ballot_sync(0xffffffffu, pass);
-            const int pos = nq + __popc(mask & ((1u << lane) - 1u));
-            if (pass && pos < lcap) sq[pos] = value;
-            nq += __popc(mask);
+        if (lane < kHalfRanges) {
+            s_r0[lane] = r0 - (incl - rn);  // candidate e of the concatenation is xs[e + s_r0] in its range
+            s_at[lane + 1] = incl;
+            s_code[lane] = image_code(sx, sy, sz) << 24;
+            s_shift[lane][0] = (float)sx * b.Lh[0];  // exact: s in {-1, 0, 1}
+            s_shift[lane][1] = (float)sy * b.Lh[1];
+            s_shift[lane][2] = (float)sz * b.Lh[2];
         }
-        __syncwarp();
-        if (nq > lcap && lane == 0) atomicOr(err, kErrOverflow);
-        // pass 2: the exact test; an accepted pair takes a slot in i's row
-        // (one atomic per warp round) and one in j's row
-        const int nqs = nq < lcap ? nq : lcap;
-        for (int base = 0; base < nqs; base += 32) {
-            const int e = base + lane;
-            bool accept = false;
-            int value = 0, j = 0;
-            float d2 = 0.f;
-            if (e < nqs) {
-                value = sq[e];
-                j = value & 0xFFFFFF;
-                float hj[3], lj[3];
-                load_pos(xr, j, hj, lj);
-                float rx, ry, rz;
-                pair_vector(value >> 24, hi, li, hj, lj, b, rx, ry, rz);
-                d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-                accept = d2 < rv2;
-            }
-            const unsigned mask = __ballot_sync(0xffffffffu, accept);
-            int si0 = 0;
-            if (lane == 0 && mask) si0 = atomicAdd(count + i, __popc(mask));
-            si0 = __shfl_sync(0xffffffffu, si0, 0);
-            if (accept) {
-                const int si = si0 + __popc(mask & ((1u << lane) - 1u));
-                const int sj = atomicAdd(count + j, 1);
-                const int vj = i | ((124 - (value >> 24)) << 24);  // the reverse image
-                if (si < m_cap) {
-                    int* ri = rows + ((size_t)i * m_cap + si) * 4;
-                    ri[0] = value;
-                    ri[1] = (int)__float_as_uint(d2);
-                    ri[2] = sj;
-                }
-                if (sj < m_cap) {
-                    int* rj = rows + ((size_t)j * m_cap + sj) * 4;
-                    rj[0] = vj;
-                    rj[1] = (int)__float_as_uint(d2);
-                    rj[2] = si;
-                }
-            }
+        if (lane == 0) s_at[0] = 0;
+    }
+    __syncthreads();
+    const int own = s_at[1], total = s_at[kHalfRanges];
+    // the hi parts alone are within half an ulp of the edge of the positions:
+    // the margin never drops a pair that the exact test keeps
+    const float rq = sqrtf(rv2) + 1e-3f + 1e-6f * fmaxf(b.Lh[0], fmaxf(b.Lh[1], b.Lh[2])), rq2 = rq * rq;
+    int* sq = s_sq[warp];
+    // a dense spot in a coarse grid can hold more candidates than the buffer
+    for (int f0 = 0; f0 < total; f0 += cap) {
+        if (f0) __syncthreads();  // the previous piece is read
+        const int m = min(cap, total - f0);
+        for (int e = threadIdx.x; e < m; e += 32 * WARPS) {
+            int r = 0;
+            while (s_at[r + 1] <= f0 + e) ++r;
+            const float4 h = NEP_LDG(xs + s_r0[r] + f0 + e);
+            s_cand[e] = make_float4((h.x - ox) + s_shift[r][0], (h.y - oy) + s_shift[r][1], (h.z - oz) + s_shift[r][2],
+                                    __int_as_float(__float_as_int(h.w) | s_code[r]));
         }
-        __syncwarp();  // the warp's buffers are reused by its next atom
+        __syncthreads();
+        for (int c = c0 + warp; c < c1; c += WARPS) {
+            const float4 me = NEP_LDG(xs + c);
+            const int i = __float_as_int(me.w);
+            const float hx = me.x - ox, hy = me.y - oy, hz = me.z - oz;
+            float hi[3], li[3];
+            load_pos(xr, i, hi, li);
+            int nq = 0;
+            // the exact test of the waiting survivors; an accepted pair takes a
+            // slot in i's row (one atomic per warp round) and one in j's row
+            auto flush = [&]() {
+                __syncwarp();
+                for (int e0 = 0; e0 < nq; e0 += 32) {
+                    const int e = e0 + lane;
+                    bool accept = false;
+                    int v = 0, j = 0;
+                    float d2 = 0.f;
+                    if (e < nq) {
+                        v = sq[e];
+                        j = v & 0xFFFFFF;
+                        float hj[3], lj[3], rx, ry, rz;
+                        load_pos(xr, j, hj, lj);
+                        pair_vector(v >> 24, hi, li, hj, lj, b, rx, ry, rz);
+                        d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+                        accept = d2 < rv2;
+                    }
+                    const unsigned mask = __ballot_sync(0xffffffffu, accept);
+                    int si0 = 0;
+                    if (lane == 0 && mask) si0 = atomicAdd(count + i, __popc(mask));
+                    si0 = __shfl_sync(0xffffffffu, si0, 0);
+                    if (accept) {
+                        const int si = si0 + __popc(mask & ((1u << lane) - 1u));
+                        const int sj = atomicAdd(count + j, 1);
+                        const int vj = i | ((124 - (v >> 24)) << 24);  // the reverse image
+                        // the fourth word is written by the partner's sort
+                        if (si < m_cap) {
+                            int* ri = rows + ((size_t)i * m_cap + si) * 4;
+                            *reinterpret_cast<int2*>(ri) = make_int2(v, (int)__float_as_uint(d2));
+                            ri[2] = sj;
+                        }
+                        if (sj < m_cap) {
+                            int* rj = rows + ((size_t)j * m_cap + sj) * 4;
+                            *reinterpret_cast<int2*>(rj) = make_int2(vj, (int)__float_as_uint(d2));
+                            rj[2] = si;
+                        }
+                    }
+                }
+                nq = 0;
+                __syncwarp();
+            };
+#pragma unroll 2
+            for (int e0 = 0; e0 < m; e0 += 32) {
+                const int e = e0 + lane;
+                bool pass = false;
+                int v = 0;
+                if (e < m) {
+                    const float4 q = s_cand[e];
+                    const float qx = q.x - hx, qy = q.y - hy, qz = q.z - hz;
+                    v = __float_as_int(q.w);
+                    // the cell itself: the pairs with j > i only
+                    pass = fmaf(qx, qx, fmaf(qy, qy, qz * qz)) < rq2 && (f0 + e >= own || (v & 0xFFFFFF) > i);
+                }
+                const unsigned mask = __ballot_sync(0xffffffffu, pass);
+                const int pos = nq + __popc(mask & ((1u << lane) - 1u));
+                if (pass) sq[pos] = v;
+                nq += __popc(mask);
+                if (nq > kHalfQuick - 32) flush();
+            }
+            flush();
+        }
     }
 }
 
@@ -354,10 +408,26 @@ __device__ __forceinline__ void rank_rows_write(int c0, int ns, int m, int lane,
         ke[t] = e < ns ? sk[e] : ~0ull;
         rk[t] = 0;
     }
+    // by the distance words alone; equal distances (the ranks then miss some
+    // value, and their sum is short) are ranked again by the whole keys
+    const unsigned* hi = reinterpret_cast<const unsigned*>(sk) + 1;
+    int sum = 0;
+#pragma unroll 4
     for (int f = 0; f < ns; ++f) {
-        const unsigned long long kf = sk[f];
+        const unsigned kf = hi[2 * f];
 #pragma unroll
-        for (int t = 0; t < EPL; ++t) rk[t] += ke[t] > kf ? 1 : 0;
+        for (int t = 0; t < EPL; ++t) rk[t] += (unsigned)(ke[t] >> 32) > kf ? 1 : 0;
+    }
+#pragma unroll
+    for (int t = 0; t < EPL; ++t) sum += c0 + lane + 32 * t < ns ? rk[t] : 0;
+    if (ns > 32 * EPL || __reduce_add_sync(0xffffffffu, sum) != ns * (ns - 1) / 2) {
+#pragma unroll
+        for (int t = 0; t < EPL; ++t) rk[t] = 0;
+        for (int f = 0; f < ns; ++f) {
+            const unsigned long long kf = sk[f];
+#pragma unroll
+            for (int t = 0; t < EPL; ++t) rk[t] += ke[t] > kf ? 1 : 0;
+        }
     }
 #pragma unroll
     for (int t = 0; t < EPL; ++t) {
@@ -601,8 +671,7 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_tile(int n, int m_cap, cons
 // images) and for small atom counts (the nearest image): one launch instead of
 // the cells path's scan, scatter, search and sort, each a few microseconds of
 // latency.  A block takes two consecutive atoms; its threads walk all atoms j,
-// test the hi parts against both (the 1e-3 A margin of k_half_cells
-// never drops a pair that the exact test keeps), test survivors exactly and
+// test the hi parts against both (with a margin, as k_half_cells), test survivors exactly and
 // append (squared distance, tie-break) keys to the atoms' shared rows.  The
 // rows are then rank-sorted, 64 threads per row.
 // IMAGES: every shift up to b.img, ties ordered by (j, image); else the
@@ -637,7 +706,7 @@ __global__ void __launch_bounds__(kDirectThreads) k_list_direct(int n, int m_cap
         hi[a][2] = h.z;
     }
     __syncthreads();
-    const float rq = sqrtf(rv2) + 1e-3f, rq2 = rq * rq;
+    const float rq = sqrtf(rv2) + 1e-3f + 1e-6f * fmaxf(b.Lh[0], fmaxf(b.Lh[1], b.Lh[2])), rq2 = rq * rq;
     // the exact test of a survivor, and its key
     auto exact = [&](int a, int j, int code) {
         float h0[3], l0[3], hj[3], lj[3], rx, ry, rz;
@@ -785,16 +854,18 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
                                           nl.cell_count, nl.count, bb, d_gate, d_err);
     if (cells) {
         k_scan<<<1, kScanThreads, 0, st>>>(ncell, nl.cell_count, nl.cell_start, nl.cell_fill, d_gate);
-        k_scatter<<<blocks_for(n, T), T, 0, st>>>(n, nl.atom_cell, nl.cell_start, nl.cell_fill, nl.cell_atoms,
-                                                  d_gate);
-        // per-warp buffers: a power of two >= m_cap entries
+        k_scatter<<<blocks_for(n, T), T, 0, st>>>(n, nl.atom_cell, nl.cell_start, nl.cell_fill, nl.xr, nl.xs, d_gate);
+        // per-warp buffers of the row sort: a power of two >= m_cap entries
         int lcap = 32;
         while (lcap < nl.m_cap) lcap <<= 1;
         const int grid = std::min(blocks_for(n, kVerletWarps), kListGridCap);
         int* rows = reinterpret_cast<int*>(nl.pf);  // four words per slot, free until the site pass
-        k_half_cells<<<grid, 32 * kVerletWarps, (size_t)kVerletWarps * (lcap + 6 * 32) * sizeof(int), st>>>(
-            n, nl.m_cap, rv2, nl.xr, nl.atom_cell, nl.cell_start, nl.cell_atoms, nl.count, rows, lcap, d_err, b,
-            d_gate);
+        // candidates per cell: 14 mean cells and half as many again
+        const int cap = std::min(std::max(128, (int)(1.5 * 14.0 * n / ncell) / 32 * 32), 1024);
+        const int warps = ncell <= 608 ? 8 : n < 8 * (long long)ncell ? 2 : 4;
+        (warps == 8 ? k_half_cells<8> : warps == 2 ? k_half_cells<2> : k_half_cells<4>)<<<
+            ncell, 32 * warps, (size_t)cap * sizeof(float4), st>>>(nl.m_cap, rv2, cap, nl.xr, nl.xs, nl.cell_start,
+                                                                   nl.count, rows, b, d_gate);
         const size_t sort_smem = (size_t)kSortWarps * lcap * 12 + (size_t)nl.m_cap * (kSortAtoms + 1) * sizeof(int);
         if (sort_smem <= kSortTileMaxSmem)
             k_sort_tile<<<std::min(blocks_for(n, kSortAtoms), kSortGridCap), 32 * kSortWarps, sort_smem, st>>>(

@@ -40,7 +40,7 @@ constexpr size_t kOffPf = kOffVala + align256(sizeof(int) * kStaticAtoms * kStat
 constexpr size_t kOffXr = kOffPf + align256(sizeof(float) * kStaticAtoms * kStaticSlots * 4);
 constexpr size_t kOffAtomCell = kOffXr + align256(sizeof(float) * kStaticAtoms * 8);
 constexpr size_t kOffCellAtoms = kOffAtomCell + align256(sizeof(int) * kStaticAtoms);
-constexpr size_t kOffCellCount = kOffCellAtoms + align256(sizeof(int) * kStaticAtoms);
+constexpr size_t kOffCellCount = kOffCellAtoms + align256(sizeof(float4) * kStaticAtoms);
 constexpr size_t kOffCellStart = kOffCellCount + align256(sizeof(int) * (kStaticCells + 1));
 constexpr size_t kOffCellFill = kOffCellStart + align256(sizeof(int) * (kStaticCells + 1));
 constexpr size_t kOffMask = kOffCellFill + align256(sizeof(int) * (kStaticCells + 1));
@@ -180,7 +180,7 @@ extern "C" int nep_compute_efv_static(const nep_hyper* hp, const float* z, int n
     nl.vala = reinterpret_cast<int*>(base + kOffVala);
     nl.xr = reinterpret_cast<float*>(base + kOffXr);
     nl.atom_cell = reinterpret_cast<int*>(base + kOffAtomCell);
-    nl.cell_atoms = reinterpret_cast<int*>(base + kOffCellAtoms);
+    nl.xs = reinterpret_cast<float4*>(base + kOffCellAtoms);
     nl.cell_count = reinterpret_cast<int*>(base + kOffCellCount);
     nl.cell_start = reinterpret_cast<int*>(base + kOffCellStart);
     nl.cell_fill = reinterpret_cast<int*>(base + kOffCellFill);

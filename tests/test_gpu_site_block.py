@@ -159,3 +159,44 @@ def test_adjoint_by_atoms_per_block(orc, n_struct):
     assert abs(fd - float(g.norm())) <= 2e-3 * float(g.norm()), (fd, float(g.norm()))
     ds.close()
     model.close()
+
+
+@pytest.mark.parametrize("kind", ["dense spot", "thin grid", "few large cells", "split model"])
+def test_cells_path_search(orc, kind):
+    """The half-shell search per cell: a cell with more candidates than its
+    shared buffer (a dense cluster in a large box), a grid of three cells in one
+    direction, eight warps per cell, and the 8 A cells of the split model.
+    Counts and forces of a sample against the oracle."""
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(len(kind))
+    hyper, oh = nep.Hyper(max_neighbors=384), orc.NepHyper()
+    if kind == "dense spot":      # 3000 atoms at 2.4 A spacing in one corner of a 400 A box
+        g = np.stack(np.meshgrid(*[np.arange(15)] * 3, indexing="ij"), -1).reshape(-1, 3)[:3000] * 2.4
+        pos, box = g + rng.normal(0.0, 0.1, (3000, 3)), np.diag([400.0] * 3)
+    elif kind == "thin grid":
+        pos, box = inputs.diamond(3, 12, 11)
+        pos = inputs.displace(pos, 0.1, rng)
+    elif kind == "few large cells":
+        pos, box = inputs.diamond(7, 7, 8)
+        pos = inputs.displace(pos, 0.1, rng)
+    else:
+        pos, _, box, z, _ = inputs.config_pbte((7, 7, 8))
+        hyper = nep.Hyper(**inputs.PBTE_HYPER)
+        oh = orc.NepHyper(12, 6, 4, 40, 8.0, 4.0)
+    assert len(pos) > 2500
+    if kind != "split model":
+        z = inputs.random_z(hyper.n_par, rng)
+    model = nep.NEP(z, hyper)
+    out = model.compute(soa(pos), box)
+    cnt, _ = model.neighbors(len(pos))
+    idx = np.unique(rng.integers(0, len(pos), 150))
+    U, F, _ = orc.efv_sample(oh, f32_exact(z), pos, box, idx)
+    assert np.abs(out["e_atom"].cpu().numpy()[idx] - U).max() <= 1e-6
+    assert np.abs(aos(out["force"])[idx] - F).max() <= 1e-4
+    rc, L = hyper.rc_R, np.diag(box)
+    for i in idx[:40]:
+        d = pos - pos[i]
+        r = np.linalg.norm(d - L * np.round(d / L), axis=1)
+        near = int(np.sum(np.abs(r - rc) < 1e-5))
+        assert abs(int(cnt[i]) - int(np.sum((r < rc) & (r > 0)))) <= near
+    model.close()
