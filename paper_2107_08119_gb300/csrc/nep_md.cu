@@ -367,6 +367,11 @@ inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
 
 using namespace nep;
 
+// Steps per graph launch where a call has that many left: the gap between two
+// graphs costs more than the one between their kernels (4,096 atoms 49.4 -> 46.1
+// us per step; 10 steps per graph 45.5).
+constexpr int kGraphSteps = 5;
+
 struct nep_md {
     nep_model* m = nullptr;
     int n = 0;
@@ -395,7 +400,7 @@ struct nep_md {
     // one step captured as a CUDA graph (the list rebuild behind a conditional
     // node), kept while everything it bakes in is unchanged
     cudaStream_t gcap = nullptr, gcap2 = nullptr;
-    cudaGraphExec_t gexec = nullptr;
+    cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // one step, kGraphSteps steps
     struct GraphKey {
         const double *pos, *vel;
         double *thermo, *heat;
@@ -490,7 +495,8 @@ int nep_md_destroy(nep_md* md)
     if (md->red) cudaFree(md->red);
     if (md->w_atom) cudaFree(md->w_atom);
     free_shc(md);
-    if (md->gexec) cudaGraphExecDestroy(md->gexec);
+    for (auto e : md->gexec)
+        if (e) cudaGraphExecDestroy(e);
     if (md->gcap) cudaStreamDestroy(md->gcap);
     if (md->gcap2) cudaStreamDestroy(md->gcap2);
     delete md;
@@ -829,71 +835,87 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
     };
 
     // Without phase timing and without the per-step host logic of the
-    // spectral heat current, a step runs from a CUDA graph captured once: the
-    // list rebuild is the body of a conditional node that the last block of
-    // k_kick_drift switches,
+    // spectral heat current, the steps run from CUDA graphs of one and of
+    // kGraphSteps steps, captured when first needed: the list rebuild is the
+    // body of a conditional node that the last block of k_kick_drift switches,
     // so a step without a rebuild launches none of the list kernels.
     if (!m->prof.on && md->shc_lags == 0) {
+        auto drop = [&]() {
+            for (auto& e : md->gexec) {
+                if (e) cudaGraphExecDestroy(e);
+                e = nullptr;
+            }
+        };
+        // `steps` steps as one graph
+        auto capture = [&](int steps, cudaGraphExec_t* exec) {
+            cudaGraph_t g = nullptr;
+            int r = cuda_fail(cudaGraphCreate(&g, 0), "graph create");
+            if (!r) r = cuda_fail(cudaStreamBeginCaptureToGraph(md->gcap, g, nullptr, nullptr, 0,
+                                                                cudaStreamCaptureModeRelaxed), "begin capture");
+            if (r) {
+                if (g) cudaGraphDestroy(g);
+                return r;
+            }
+            for (int s = 0; s < steps && !r; ++s) {
+                cudaGraphConditionalHandle cond;
+                r = cuda_fail(cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault), "handle");
+                if (r) break;
+                head(md->gcap, true, cond);
+                cudaStreamCaptureStatus cs;
+                const cudaGraphNode_t* deps = nullptr;
+                size_t nd = 0;
+                r = cuda_fail(cudaStreamGetCaptureInfo(md->gcap, &cs, nullptr, nullptr, &deps, nullptr, &nd),
+                              "capture info");
+                cudaGraphNodeParams cp = {};
+                cp.type = cudaGraphNodeTypeConditional;
+                cp.conditional.handle = cond;
+                cp.conditional.type = cudaGraphCondTypeIf;
+                cp.conditional.size = 1;
+                cudaGraphNode_t cnode = nullptr;
+                if (!r) r = cuda_fail(cudaGraphAddNode(&cnode, g, deps, nullptr, nd, &cp), "conditional node");
+                if (!r)
+                    r = cuda_fail(cudaStreamUpdateCaptureDependencies(md->gcap, &cnode, nullptr, 1,
+                                                                      cudaStreamSetCaptureDependencies),
+                                  "capture dependencies");
+                if (!r) {
+                    cudaGraph_t body = cp.conditional.phGraph_out[0];
+                    r = cuda_fail(cudaStreamBeginCaptureToGraph(md->gcap2, body, nullptr, nullptr, 0,
+                                                                cudaStreamCaptureModeRelaxed), "begin body capture");
+                    if (!r) {
+                        r = rebuild(md->gcap2, nullptr);
+                        cudaGraph_t b2 = nullptr;
+                        const cudaError_t e = cudaStreamEndCapture(md->gcap2, &b2);
+                        if (!r && e != cudaSuccess) r = cuda_fail(e, "end body capture");
+                    }
+                }
+                if (!r) r = tail(md->gcap);
+            }
+            cudaGraph_t g2 = nullptr;
+            const cudaError_t e = cudaStreamEndCapture(md->gcap, &g2);
+            if (!r && e != cudaSuccess) r = cuda_fail(e, "end capture");
+            if (!r) r = cuda_fail(cudaGraphInstantiate(exec, g, 0), "instantiate step graph");
+            cudaGraphDestroy(g);
+            return r;
+        };
         nep_md::GraphKey key{pos, vel, thermo, heat, dt, md->t0, md->tau, {md->fe[0], md->fe[1], md->fe[2]}, drive,
                              md_zatom(md), md->plain};
-        if (!md->gexec || !(key == md->gkey)) {
-            if (md->gexec) cudaGraphExecDestroy(md->gexec);
-            md->gexec = nullptr;
+        if (!(key == md->gkey) || !(md->gexec[0] || md->gexec[1])) {
+            drop();
             if (!md->gcap && (rc = cuda_fail(cudaStreamCreateWithFlags(&md->gcap, cudaStreamNonBlocking), "stream")))
                 return rc;
             if (!md->gcap2 && (rc = cuda_fail(cudaStreamCreateWithFlags(&md->gcap2, cudaStreamNonBlocking), "stream")))
                 return rc;
-            cudaGraph_t g = nullptr;
-            cudaGraphConditionalHandle cond;
-            rc = cuda_fail(cudaGraphCreate(&g, 0), "graph create");
-            if (!rc) rc = cuda_fail(cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault), "handle");
-            if (!rc) rc = cuda_fail(cudaStreamBeginCaptureToGraph(md->gcap, g, nullptr, nullptr, 0,
-                                                                  cudaStreamCaptureModeRelaxed), "begin capture");
-            if (rc) {
-                if (g) cudaGraphDestroy(g);
-                return rc;
-            }
-            head(md->gcap, true, cond);
-            cudaStreamCaptureStatus cs;
-            const cudaGraphNode_t* deps = nullptr;
-            size_t nd = 0;
-            rc = cuda_fail(cudaStreamGetCaptureInfo(md->gcap, &cs, nullptr, nullptr, &deps, nullptr, &nd), "capture info");
-            cudaGraphNodeParams cp = {};
-            cp.type = cudaGraphNodeTypeConditional;
-            cp.conditional.handle = cond;
-            cp.conditional.type = cudaGraphCondTypeIf;
-            cp.conditional.size = 1;
-            cudaGraphNode_t cnode = nullptr;
-            if (!rc) rc = cuda_fail(cudaGraphAddNode(&cnode, g, deps, nullptr, nd, &cp), "conditional node");
-            if (!rc)
-                rc = cuda_fail(cudaStreamUpdateCaptureDependencies(md->gcap, &cnode, nullptr, 1,
-                                                                   cudaStreamSetCaptureDependencies),
-                               "capture dependencies");
-            if (!rc) {
-                cudaGraph_t body = cp.conditional.phGraph_out[0];
-                rc = cuda_fail(cudaStreamBeginCaptureToGraph(md->gcap2, body, nullptr, nullptr, 0,
-                                                             cudaStreamCaptureModeRelaxed), "begin body capture");
-                if (!rc) {
-                    rc = rebuild(md->gcap2, nullptr);
-                    cudaGraph_t b2 = nullptr;
-                    const cudaError_t e = cudaStreamEndCapture(md->gcap2, &b2);
-                    if (!rc && e != cudaSuccess) rc = cuda_fail(e, "end body capture");
-                }
-            }
-            if (!rc) rc = tail(md->gcap);
-            cudaGraph_t g2 = nullptr;
-            const cudaError_t e = cudaStreamEndCapture(md->gcap, &g2);
-            if (!rc && e != cudaSuccess) rc = cuda_fail(e, "end capture");
-            if (!rc) rc = cuda_fail(cudaGraphInstantiate(&md->gexec, g, 0), "instantiate step graph");
-            cudaGraphDestroy(g);
-            if (rc) {
-                md->gexec = nullptr;
-                return rc;
-            }
             md->gkey = key;
         }
-        for (int s = 0; s < n_steps; ++s)
-            if ((rc = cuda_fail(cudaGraphLaunch(md->gexec, st), "launch step graph"))) return rc;
+        for (int s = 0; s < n_steps;) {
+            const int u = n_steps - s >= kGraphSteps ? 1 : 0;
+            if (!md->gexec[u] && (rc = capture(u ? kGraphSteps : 1, &md->gexec[u]))) {
+                md->gexec[u] = nullptr;
+                return rc;
+            }
+            if ((rc = cuda_fail(cudaGraphLaunch(md->gexec[u], st), "launch step graph"))) return rc;
+            s += u ? kGraphSteps : 1;
+        }
         return NEP_OK;
     }
 
