@@ -468,7 +468,7 @@ int compute_efv(nep_model* m, int n, const double* box9, const double* pos, doub
         if ((rc = launch_plain_site(fa, nl, n, ws.plain, ws.plain + (size_t)kNdes * n, e_atom, part_e, m->d_err, st,
                                     nb1)))
             return rc;
-    } else if ((rc = launch_site_partial_forces(fa, nl, n, e_atom, part_e, m->d_err, st, nb1))) {
+    } else if ((rc = launch_site_partial_forces(fa, nl, n, e_atom, part_e, m->d_err, st, nb1, true))) {
         return rc;
     }
     m->prof.end(ps, st);
@@ -483,7 +483,7 @@ int compute_efv(nep_model* m, int n, const double* box9, const double* pos, doub
     if (e_total || virial_total) {
         // the energy and virial totals, straight to the caller
         const SumSet e{part_e, nb1, 1, 1, 0, e_total}, w{part_v, nb2, 1, nc2, (size_t)nb2, virial_total};
-        if ((rc = launch_sum(e, w, st))) return rc;
+        if ((rc = launch_sum(e, w, st, true))) return rc;
     }
     return NEP_OK;
 }

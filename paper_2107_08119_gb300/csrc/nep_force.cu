@@ -35,8 +35,9 @@ __global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, cons
                                                           double* __restrict__ e_partials, unsigned* err,
                                                           unsigned* __restrict__ mask)
 {
+    const int block = block_after();
     const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * AT + lane % AT;
+    const int i = block * AT + lane % AT;
     const bool active = i < n;
     const int cnt = active ? min(count[i], m_cap) : 0;
     float uh, ul;
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, cons
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    if (lane == 0) e_partials[blockIdx.x] = e;
+    if (lane == 0) e_partials[block] = e;
 }
 
 // Totals of block b, [component][gridDim.x]: components 0..8 the virial, and
@@ -86,8 +87,9 @@ __global__ void __launch_bounds__(kAsmThreads, 8) k_assemble(int n, int m_cap, f
     __shared__ float s_t[ROWS][CH][AT];
     __shared__ float s_sum[12][AT];
     __shared__ float s_v[3][AT];
+    const int block = block_after();
     const int at = threadIdx.x % AT, way = threadIdx.x / AT;
-    const int i = blockIdx.x * AT + at;
+    const int i = block * AT + at;
     const bool active = i < n;
     const int ia = active ? i : 0;
     float hi[3], li[3];
@@ -234,7 +236,7 @@ __global__ void __launch_bounds__(kAsmThreads, 8) k_assemble(int n, int m_cap, f
     const int c = 2 * (b1 ? 1 : 0) + (b0 ? 1 : 0);
     if (at % (AT / 4) == 0) {
         const int k = row == 0 ? (MD && c == 0 ? 9 : -1) : c < 3 ? 3 * (row - 1) + c : MD ? 9 + row : -1;
-        if (k >= 0) partials[(size_t)k * gridDim.x + blockIdx.x] = sum;
+        if (k >= 0) partials[(size_t)k * gridDim.x + block] = sum;
     }
 }
 
@@ -251,7 +253,8 @@ __global__ void __launch_bounds__(kAsmThreads) k_assemble_atoms(int n, int m_cap
                                                           const unsigned* __restrict__ mask)
 {
     constexpr int K = MD ? 13 : 9;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int block = block_after();
+    const int i = block * blockDim.x + threadIdx.x;
     double acc[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) acc[k] = 0.0;
@@ -287,7 +290,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_assemble_atoms(int n, int m_cap
                               (double)(W[3 * a + 2] * (float)v[2]);
         }
     }
-    block_sum_store<K>(acc, partials + blockIdx.x, gridDim.x);
+    block_sum_store<K>(acc, partials + block, gridDim.x);
 }
 
 // One total per block, the totals of `a` and then those of `b`: several SMs
@@ -295,9 +298,10 @@ __global__ void __launch_bounds__(kAsmThreads) k_assemble_atoms(int n, int m_cap
 constexpr int kSumThreads = 512;
 __global__ void __launch_bounds__(kSumThreads) k_sum(SumSet a, SumSet b)
 {
-    const bool first = blockIdx.x < a.ncomp;
+    const int block = block_after();
+    const bool first = block < a.ncomp;
     const SumSet s = first ? a : b;
-    const int w = first ? blockIdx.x : blockIdx.x - a.ncomp;
+    const int w = first ? block : block - a.ncomp;
     if (!s.out) return;
     const double t = sum_partials<kSumThreads>(s.src + (size_t)w * s.cstride, s.nb, s.bstride);
     if (threadIdx.x == 0) s.out[w] = t;
@@ -307,7 +311,7 @@ inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
 
 template <class D, int AT>
 int launch_site(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, double* e_partials, unsigned* d_err,
-                cudaStream_t st, int& nblocks)
+                cudaStream_t st, int& nblocks, bool after)
 {
     SiteParams P;
     P.w = nullptr;
@@ -332,26 +336,26 @@ int launch_site(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, dou
         if (rc) return rc;
     }
     nl.mask_set = nl.m_cap <= kMaskSlots && nl.mask != nullptr;
-    kern<<<nblocks, kSiteThreads, smem, st>>>(n, nl.m_cap, nl.count, nl.nbr, nl.xr, a.box, a.z, n_par, P, nl.pf,
-                                              e_atom, e_partials, d_err, nl.mask_set ? nl.mask : nullptr);
-    return cuda_fail(cudaGetLastError(), "site kernel");
+    return cuda_fail(launch_after(after, kern, nblocks, kSiteThreads, smem, st, n, nl.m_cap, nl.count,
+                                  nl.nbr, nl.xr, a.box, a.z, n_par, P, nl.pf, e_atom, e_partials, d_err,
+                                  nl.mask_set ? nl.mask : nullptr), "site kernel");
 }
 
 }  // namespace
 
 int launch_site_partial_forces(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, double* e_partials,
-                               unsigned* d_err, cudaStream_t st, int& nblocks)
+                               unsigned* d_err, cudaStream_t st, int& nblocks, bool after)
 {
     const int at = site_atoms_per_block(n);
     if (a.nr == DescPbTe::NR && a.na == DescPbTe::NA)
         return (at == 8 ? launch_site<DescPbTe, 8> : at == 16 ? launch_site<DescPbTe, 16> : launch_site<DescPbTe, 32>)(
-            a, nl, n, e_atom, e_partials, d_err, st, nblocks);
+            a, nl, n, e_atom, e_partials, d_err, st, nblocks, after);
     if (a.nr != DescSi::NR || a.na != DescSi::NA) {
         set_error("no site kernel for %d radial and %d angular orders", a.nr, a.na);
         return NEP_ERR_UNSUPPORTED;
     }
     return (at == 8 ? launch_site<DescSi, 8> : at == 16 ? launch_site<DescSi, 16> : launch_site<DescSi, 32>)(
-        a, nl, n, e_atom, e_partials, d_err, st, nblocks);
+        a, nl, n, e_atom, e_partials, d_err, st, nblocks, after);
 }
 
 // One thread per atom in the assembly, by the number of atoms and the mean
@@ -378,18 +382,16 @@ int launch_assemble(const AssembleArgs& a, NeighborList& nl, int n, float* force
                 : at == 8  ? (md ? k_assemble<true, 8> : k_assemble<false, 8>)
                 : at == 16 ? (md ? k_assemble<true, 16> : k_assemble<false, 16>)
                            : (md ? k_assemble<true, 32> : k_assemble<false, 32>);
-    kern<<<nblocks, kAsmThreads, 0, st>>>(n, nl.m_cap, rc2, nl.count, nl.nbr, nl.rev, nl.xr, a.box, nl.pf, force,
-                                          virial_atom, partials, d_err, md ? a.vel : nullptr,
-                                          md ? a.half_dt_over_m : 0.0, md ? a.ke_factor : 0.0,
-                                          nl.mask_set ? nl.mask : nullptr);
-    return cuda_fail(cudaGetLastError(), "assemble kernel");
+    return cuda_fail(launch_after(true, kern, nblocks, kAsmThreads, 0, st, n, nl.m_cap, rc2,
+                                  nl.count, nl.nbr, nl.rev, nl.xr, a.box, nl.pf, force, virial_atom, partials, d_err,
+                                  md ? a.vel : nullptr, md ? a.half_dt_over_m : 0.0, md ? a.ke_factor : 0.0,
+                                  nl.mask_set ? nl.mask : nullptr), "assemble kernel");
 }
 
-int launch_sum(const SumSet& a, const SumSet& b, cudaStream_t st)
+int launch_sum(const SumSet& a, const SumSet& b, cudaStream_t st, bool after)
 {
     if (a.ncomp + b.ncomp == 0) return NEP_OK;
-    k_sum<<<a.ncomp + b.ncomp, kSumThreads, 0, st>>>(a, b);
-    return cuda_fail(cudaGetLastError(), "sum kernel");
+    return cuda_fail(launch_after(after, k_sum, a.ncomp + b.ncomp, kSumThreads, 0, st, a, b), "sum kernel");
 }
 
 }  // namespace nep

@@ -69,7 +69,7 @@ __global__ void k_kick_drift(int n, double* __restrict__ x, double* __restrict__
                              const double* __restrict__ x_ref, unsigned* __restrict__ ctl, float thresh2,
                              unsigned long long* __restrict__ rebuilds, cudaGraphConditionalHandle cond, int use_cond)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = block_after() * blockDim.x + threadIdx.x;
     float d2 = 0.f;
     if (i < n) {
         double dd = 0.0, xn[3];
@@ -121,10 +121,11 @@ __global__ void k_hnemd_kick(int n, float* __restrict__ F, const float* __restri
                              double fe0, double fe1, double fe2, const double* __restrict__ wtot, double inv_n,
                              double hdtm, double kef, double* __restrict__ partials, unsigned* err)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = block_after() * blockDim.x + threadIdx.x;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     if (i < n) {
         const double fe[3] = {fe0, fe1, fe2};
+        wtot = reread(wtot);
         float w[9];
 #pragma unroll
         for (int c = 0; c < 9; ++c) w[c] = W[(size_t)c * n + i];
@@ -294,9 +295,9 @@ __global__ void __launch_bounds__(kKappaThreads) k_hnemd_kappa(int n, const doub
 // v *= lambda (the Berendsen factor k_md_finish left in red[14])
 __global__ void k_scale_v(int n, double* __restrict__ vel, const double* __restrict__ red)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = block_after() * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double lam = red[14];
+    const double lam = reread(red)[14];
 #pragma unroll
     for (int c = 0; c < 3; ++c) vel[(size_t)c * n + i] *= lam;
 }
@@ -318,7 +319,7 @@ __global__ void __launch_bounds__(kFinishThreads) k_md_finish(const double* __re
                                                               double dt, double dof_kb)
 {
     // red: [0] E_pot, [1..9] W (row-major), [10] E_kin, [11..13] J, [14] lambda
-    const int w = blockIdx.x;
+    const int w = block_after();
     const double t = w == 0 ? sum_partials<kFinishThreads>(part_e, nb_e, 1)
                             : sum_partials<kFinishThreads>(part_x + (w - 1) * cstride_x, nb_x, bstride_x);
     __shared__ int last;
@@ -738,18 +739,18 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
     // site energies and partial forces: the optimised pass, or the plain FP32
     // comparator (literal Eq. 13, unfused) when selected
     Workspace& wsp = md->ws;
-    auto site_pass = [&](cudaStream_t q, int& b1) {
+    auto site_pass = [&](cudaStream_t q, int& b1, bool after) {
         if (md->plain)
             return launch_plain_site(fa, nl, n, wsp.plain, wsp.plain + (size_t)kNdes * n, nullptr, part_e, m->d_err, q,
                                      b1);
-        return launch_site_partial_forces(fa, nl, n, nullptr, part_e, m->d_err, q, b1);
+        return launch_site_partial_forces(fa, nl, n, nullptr, part_e, m->d_err, q, b1, after);
     };
     if (md->need_init) {
         // forces of the starting configuration (list built unconditionally)
         if ((rc = build_neighbor_list(nl, md->box, n, pos, md_zatom(md), true, md->x_ref, md->r_list, m->d_err, nullptr, st)))
             return rc;
         int b1 = 0, b2 = 0, c2 = 0;
-        if ((rc = site_pass(st, b1))) return rc;
+        if ((rc = site_pass(st, b1, true))) return rc;
         AssembleArgs aa{};
         aa.rc_max = (float)rmax;
         aa.box = md->box;
@@ -775,11 +776,11 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
 
     // one step in three parts: kick-drift and the rebuild decision, the list
     // rebuild, then forces, second half kick and the step's sums
-    auto head = [&](cudaStream_t q, bool use_cond, cudaGraphConditionalHandle cond) {
+    // (follows: another step comes before it in the stream)
+    auto head = [&](cudaStream_t q, bool use_cond, cudaGraphConditionalHandle cond, bool follows) {
         Profiler::Slot* pk = m->prof.begin(NEP_PROFILE_STEP, q);
-        k_kick_drift<<<blocks_for(n, 256), 256, 0, q>>>(n, pos, vel, md->ws.force, hdtm, dt, nl.xr, md->x_ref,
-                                                        md->ctl, thresh * thresh, md->rebuilds, cond,
-                                                        use_cond ? 1 : 0);
+        launch_after(follows, k_kick_drift, blocks_for(n, 256), 256, 0, q, n, pos, vel, md->ws.force, hdtm, dt,
+                     nl.xr, md->x_ref, md->ctl, thresh * thresh, md->rebuilds, cond, use_cond ? 1 : 0);
         m->prof.end(pk, q);
     };
     auto rebuild = [&](cudaStream_t q, const unsigned* g) {
@@ -795,7 +796,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         const int slot = sample ? (int)(md->shc_samples % md->shc_lags) : 0;
         float* w_out = sample ? md->shc_ring + (size_t)slot * 9 * n : (drive ? md->w_atom : nullptr);
         Profiler::Slot* ps = m->prof.begin(NEP_PROFILE_SITE, q);
-        if ((r = site_pass(q, b1))) return r;
+        if ((r = site_pass(q, b1, false))) return r;  // after the conditional node
         m->prof.end(ps, q);
         AssembleArgs aa{};
         aa.rc_max = (float)rmax;
@@ -810,14 +811,14 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         Profiler::Slot* pk = m->prof.begin(NEP_PROFILE_STEP, q);
         if (drive) {
             // the kick needs the total virial first
-            if ((r = launch_sum(SumSet{part_a, b2, 1, c2, (size_t)b2, md->red + 1}, SumSet{}, q))) return r;
-            k_hnemd_kick<<<nbk, 256, 0, q>>>(n, md->ws.force, w_out, vel, md->fe[0], md->fe[1], md->fe[2],
-                                             md->red + 1, 1.0 / n, hdtm, kef, part_h, m->d_err);
-            k_md_finish<<<5, kFinishThreads, 0, q>>>(part_e, b1, part_h, nbk, 4, 1, 10, md->red, thermo, heat, md->ctl,
-                                                     md->t0, md->tau, dt, dof_kb);
+            if ((r = launch_sum(SumSet{part_a, b2, 1, c2, (size_t)b2, md->red + 1}, SumSet{}, q, true))) return r;
+            launch_after(true, k_hnemd_kick, nbk, 256, 0, q, n, md->ws.force, w_out, vel, md->fe[0], md->fe[1],
+                         md->fe[2], md->red + 1, 1.0 / n, hdtm, kef, part_h, m->d_err);
+            launch_after(true, k_md_finish, 5, kFinishThreads, 0, q, part_e, b1, part_h, nbk, 4, 1, 10, md->red, thermo,
+                         heat, md->ctl, md->t0, md->tau, dt, dof_kb);
         } else {
-            k_md_finish<<<1 + c2, kFinishThreads, 0, q>>>(part_e, b1, part_a, b2, 1, (size_t)b2, 1, md->red, thermo, heat,
-                                                          md->ctl, md->t0, md->tau, dt, dof_kb);
+            launch_after(true, k_md_finish, 1 + c2, kFinishThreads, 0, q, part_e, b1, part_a, b2, 1, (size_t)b2, 1,
+                         md->red, thermo, heat, md->ctl, md->t0, md->tau, dt, dof_kb);
         }
         if (sample) {  // v is that of J: after the second half kick, before the thermostat
             const int avail = (int)(md->shc_samples + 1 < md->shc_lags ? md->shc_samples + 1 : md->shc_lags);
@@ -829,7 +830,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             ++md->shc_samples;
         }
         if (md->shc_lags > 0) ++md->shc_step;
-        if (md->tau > 0.0 && n > 1) k_scale_v<<<nbk, 256, 0, q>>>(n, vel, md->red);
+        if (md->tau > 0.0 && n > 1) launch_after(!sample, k_scale_v, nbk, 256, 0, q, n, vel, md->red);
         m->prof.end(pk, q);
         return cuda_fail(cudaGetLastError(), "md step kernels");
     };
@@ -860,7 +861,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
                 cudaGraphConditionalHandle cond;
                 r = cuda_fail(cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault), "handle");
                 if (r) break;
-                head(md->gcap, true, cond);
+                head(md->gcap, true, cond, s > 0);
                 cudaStreamCaptureStatus cs;
                 const cudaGraphNode_t* deps = nullptr;
                 size_t nd = 0;
@@ -921,7 +922,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
 
     const unsigned* gate = md->ctl + kCtlGate;
     for (int s = 0; s < n_steps; ++s) {
-        head(st, false, cudaGraphConditionalHandle{});
+        head(st, false, cudaGraphConditionalHandle{}, s > 0);
         if ((rc = rebuild(st, gate))) return rc;
         if ((rc = tail(st))) return rc;
     }

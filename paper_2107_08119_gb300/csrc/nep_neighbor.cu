@@ -101,6 +101,8 @@ __device__ __forceinline__ int scan_pad(int x) { return x + (x >> 5); }
 __global__ void __launch_bounds__(kScanThreads) k_scan(int ncell, int* __restrict__ count, int* __restrict__ start,
                                                        int* __restrict__ fill, const unsigned* gate)
 {
+    block_after();
+    count = reread(count);
     if (gated_off(gate)) return;
     __shared__ int sc[kScanRound + kScanRound / 32];
     __shared__ int wsum[kScanThreads / 32];
@@ -167,8 +169,9 @@ __global__ void k_scatter(int n, const int* __restrict__ atom_cell, const int* _
                           int* __restrict__ cell_fill, const float* __restrict__ xr, float4* __restrict__ xs,
                           const unsigned* gate)
 {
+    const int block = block_after();
     if (gated_off(gate)) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = block * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int c = atom_cell[i];
     const int slot = atomicAdd(cell_fill + c, 1);
@@ -232,13 +235,14 @@ __global__ void __launch_bounds__(32 * WARPS) k_half_cells(int m_cap, float rv2,
                                                           int* __restrict__ count, int* __restrict__ rows, Box b,
                                                           const unsigned* gate)
 {
+    const int block = block_after();
     if (gated_off(gate)) return;
     extern __shared__ __align__(16) float4 s_cand[];  // [cap]: x, y, z from the cell's corner, packed value
     __shared__ int s_sq[WARPS][kHalfQuick];
     __shared__ int s_r0[kHalfRanges], s_at[kHalfRanges + 1], s_code[kHalfRanges];
     __shared__ float s_shift[kHalfRanges][3];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cell = blockIdx.x;
+    const int cell = block;
     const int c0 = cell_start[cell], c1 = cell_start[cell + 1];
     if (c0 == c1) return;
     const int cz = cell % b.nc[2];
@@ -447,6 +451,7 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_sort_rows(int n, int m_ca
                                                                 int* __restrict__ inv, unsigned* err,
                                                                 const unsigned* gate)
 {
+    const int block = block_after();
     if (gated_off(gate)) return;
     extern __shared__ unsigned long long s_sort[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -467,8 +472,8 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_sort_rows(int n, int m_ca
             if (e < ns_a) pre[t] = *reinterpret_cast<const int4*>(rows + ((size_t)a * m_cap + e) * 4);
         }
     };
-    fetch(blockIdx.x * kVerletWarps + warp);
-    for (int i = blockIdx.x * kVerletWarps + warp; i < n; i += stride) {
+    fetch(block * kVerletWarps + warp);
+    for (int i = block * kVerletWarps + warp; i < n; i += stride) {
         const int cnt = pre_cnt;
         if (cnt > m_cap && lane == 0) atomicOr(err, kErrOverflow);
         const int m = cnt < m_cap ? cnt : m_cap;
@@ -517,6 +522,7 @@ __global__ void __launch_bounds__(32 * kSortWarps) k_sort_tile(int n, int m_cap,
                                                               int* __restrict__ inv, unsigned* err,
                                                               const unsigned* gate)
 {
+    const int block = block_after();
     if (gated_off(gate)) return;
     extern __shared__ unsigned long long s_sort[];
     __shared__ int s_cnt[kSortAtoms];
@@ -526,9 +532,9 @@ __global__ void __launch_bounds__(32 * kSortWarps) k_sort_tile(int n, int m_cap,
     int* s_tile = reinterpret_cast<int*>(s_sort + (size_t)kSortWarps * lcap * 3 / 2);  // [m_cap][33]
     constexpr int kPer = kSortAtoms / kSortWarps;  // atoms per warp and tile
     const int tiles = (n + kSortAtoms - 1) / kSortAtoms;
-    // this warp's k-th atom: tile blockIdx.x + (k / kPer) gridDim.x, column warp + kSortWarps (k % kPer)
+    // this warp's k-th atom: tile block + (k / kPer) gridDim.x, column warp + kSortWarps (k % kPer)
     auto atom_of = [&](int k, int& tile, int& a) {
-        tile = blockIdx.x + (k / kPer) * gridDim.x;
+        tile = block + (k / kPer) * gridDim.x;
         a = warp + kSortWarps * (k % kPer);
         return tile * kSortAtoms + a;
     };
@@ -600,10 +606,11 @@ __global__ void __launch_bounds__(32 * kSortWarps) k_sort_tile(int n, int m_cap,
 __global__ void k_rev_perm(int n, int m_cap, const int* __restrict__ count, const int* __restrict__ rows,
                            const int* __restrict__ inv, int* __restrict__ rev, unsigned* err, const unsigned* gate)
 {
+    const int block = block_after();
     if (gated_off(gate)) return;
     const int lane = threadIdx.x & 31;
     const int warps = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int i = (int)(((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); i < n; i += warps) {
+    for (int i = (int)(((size_t)block * blockDim.x + threadIdx.x) >> 5); i < n; i += warps) {
         const int ci = min(count[i], m_cap);
         for (int s = lane; s < ci; s += 32) {
             const int r = inv[(size_t)i * m_cap + s];
@@ -632,12 +639,13 @@ __global__ void __launch_bounds__(kRevThreads) k_rev_tile(int n, int m_cap, cons
                                                           const int* __restrict__ rows, const int* __restrict__ inv,
                                                           int* __restrict__ rev, unsigned* err, const unsigned* gate)
 {
+    const int block = block_after();
     if (gated_off(gate)) return;
     extern __shared__ int s_tile[];  // [m_cap][kRevAtoms + 1]
     __shared__ int s_cnt[kRevAtoms];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles = (n + kRevAtoms - 1) / kRevAtoms;
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    for (int tile = block; tile < tiles; tile += gridDim.x) {
         const int i0 = tile * kRevAtoms;
         if (threadIdx.x < kRevAtoms) {
             const int i = i0 + threadIdx.x;
@@ -690,12 +698,13 @@ __global__ void __launch_bounds__(kDirectThreads) k_list_direct(int n, int m_cap
                                                                int* __restrict__ vala, unsigned* err, Box b,
                                                                const unsigned* gate)
 {
+    const int block = block_after();
     if (gated_off(gate)) return;
     constexpr int AT = kDirectAtoms;
     extern __shared__ unsigned long long s_rows[];  // [AT][m_cap]
     __shared__ int s_cnt[AT];
     constexpr int PER = kDirectThreads / AT;  // threads that sort one row
-    const int i0 = blockIdx.x * AT;
+    const int i0 = block * AT;
     if (threadIdx.x < AT) s_cnt[threadIdx.x] = 0;
     float hi[AT][3];
 #pragma unroll
@@ -788,10 +797,11 @@ __global__ void __launch_bounds__(kDirectThreads) k_list_direct(int n, int m_cap
 __global__ void k_reverse(int n, int m_cap, const int* __restrict__ count, const float* __restrict__ key,
                           const int* __restrict__ vala, int* __restrict__ rev, unsigned* err, const unsigned* gate)
 {
+    const int block = block_after();
     if (gated_off(gate)) return;
     const int lane = threadIdx.x & 31;
     const int warps = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int i = (int)(((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); i < n; i += warps) {
+    for (int i = (int)(((size_t)block * blockDim.x + threadIdx.x) >> 5); i < n; i += warps) {
         const int ci = min(count[i], m_cap);
         for (int k = lane; k < ci; k += 32) {
             const int v = vala[(size_t)i * m_cap + k];
@@ -853,8 +863,9 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
     k_bin<<<blocks_for(n, T), T, 0, st>>>(n, pos, zatom, wrap_in_place ? 1 : 0, x_ref, nl.xr, nl.atom_cell,
                                           nl.cell_count, nl.count, bb, d_gate, d_err);
     if (cells) {
-        k_scan<<<1, kScanThreads, 0, st>>>(ncell, nl.cell_count, nl.cell_start, nl.cell_fill, d_gate);
-        k_scatter<<<blocks_for(n, T), T, 0, st>>>(n, nl.atom_cell, nl.cell_start, nl.cell_fill, nl.xr, nl.xs, d_gate);
+        launch_after(true, k_scan, 1, kScanThreads, 0, st, ncell, nl.cell_count, nl.cell_start, nl.cell_fill, d_gate);
+        launch_after(true, k_scatter, blocks_for(n, T), T, 0, st, n, nl.atom_cell, nl.cell_start, nl.cell_fill, nl.xr,
+                     nl.xs, d_gate);
         // per-warp buffers of the row sort: a power of two >= m_cap entries
         int lcap = 32;
         while (lcap < nl.m_cap) lcap <<= 1;
@@ -863,31 +874,31 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
         // candidates per cell: 14 mean cells and half as many again
         const int cap = std::min(std::max(128, (int)(1.5 * 14.0 * n / ncell) / 32 * 32), 1024);
         const int warps = ncell <= 608 ? 8 : n < 8 * (long long)ncell ? 2 : 4;
-        (warps == 8 ? k_half_cells<8> : warps == 2 ? k_half_cells<2> : k_half_cells<4>)<<<
-            ncell, 32 * warps, (size_t)cap * sizeof(float4), st>>>(nl.m_cap, rv2, cap, nl.xr, nl.xs, nl.cell_start,
-                                                                   nl.count, rows, b, d_gate);
+        launch_after(true, warps == 8 ? k_half_cells<8> : warps == 2 ? k_half_cells<2> : k_half_cells<4>, ncell,
+                     32 * warps, (size_t)cap * sizeof(float4), st, nl.m_cap, rv2, cap, nl.xr, nl.xs, nl.cell_start,
+                     nl.count, rows, b, d_gate);
         const size_t sort_smem = (size_t)kSortWarps * lcap * 12 + (size_t)nl.m_cap * (kSortAtoms + 1) * sizeof(int);
         if (sort_smem <= kSortTileMaxSmem)
-            k_sort_tile<<<std::min(blocks_for(n, kSortAtoms), kSortGridCap), 32 * kSortWarps, sort_smem, st>>>(
-                n, nl.m_cap, lcap, rows, nl.count, nl.nbr, nl.vala, d_err, d_gate);
+            launch_after(true, k_sort_tile, std::min(blocks_for(n, kSortAtoms), kSortGridCap), 32 * kSortWarps,
+                         sort_smem, st, n, nl.m_cap, lcap, rows, nl.count, nl.nbr, nl.vala, d_err, d_gate);
         else
-            k_sort_rows<<<grid, 32 * kVerletWarps, (size_t)kVerletWarps * lcap * 12, st>>>(
-                n, nl.m_cap, lcap, rows, nl.count, nl.nbr, nl.vala, d_err, d_gate);
+            launch_after(true, k_sort_rows, grid, 32 * kVerletWarps, (size_t)kVerletWarps * lcap * 12, st, n, nl.m_cap,
+                         lcap, rows, nl.count, nl.nbr, nl.vala, d_err, d_gate);
         if (nl.m_cap <= kRevTileMaxSlots)
-            k_rev_tile<<<std::min(blocks_for(n, kRevAtoms), kRevGridCap), kRevThreads,
-                         (size_t)nl.m_cap * (kRevAtoms + 1) * sizeof(int), st>>>(n, nl.m_cap, nl.count, rows,
-                                                                                  nl.vala, nl.rev, d_err, d_gate);
+            launch_after(true, k_rev_tile, std::min(blocks_for(n, kRevAtoms), kRevGridCap), kRevThreads,
+                         (size_t)nl.m_cap * (kRevAtoms + 1) * sizeof(int), st, n, nl.m_cap, nl.count, rows, nl.vala,
+                         nl.rev, d_err, d_gate);
         else
-            k_rev_perm<<<std::min(blocks_for(n, 4), kListGridCap), 128, 0, st>>>(n, nl.m_cap, nl.count, rows,
-                                                                                  nl.vala, nl.rev, d_err, d_gate);
+            launch_after(true, k_rev_perm, std::min(blocks_for(n, 4), kListGridCap), 128, 0, st, n, nl.m_cap, nl.count,
+                         rows, nl.vala, nl.rev, d_err, d_gate);
         return cuda_fail(cudaGetLastError(), "neighbour-list kernels");
     }
     const size_t rows_bytes = (size_t)kDirectAtoms * nl.m_cap * sizeof(unsigned long long);
-    (grid_box ? k_list_direct<false> : k_list_direct<true>)<<<blocks_for(n, kDirectAtoms), kDirectThreads, rows_bytes,
-                                                             st>>>(n, nl.m_cap, rv2, nl.xr, nl.count, nl.nbr, nl.pf,
-                                                                   nl.vala, d_err, b, d_gate);
-    k_reverse<<<std::min(blocks_for(n, 4), kListGridCap), 128, 0, st>>>(n, nl.m_cap, nl.count, nl.pf, nl.vala, nl.rev,
-                                                                         d_err, d_gate);
+    launch_after(true, grid_box ? k_list_direct<false> : k_list_direct<true>, blocks_for(n, kDirectAtoms),
+                 kDirectThreads, rows_bytes, st, n, nl.m_cap, rv2, nl.xr, nl.count, nl.nbr, nl.pf, nl.vala, d_err, b,
+                 d_gate);
+    launch_after(true, k_reverse, std::min(blocks_for(n, 4), kListGridCap), 128, 0, st, n, nl.m_cap, nl.count, nl.pf,
+                 nl.vala, nl.rev, d_err, d_gate);
     return cuda_fail(cudaGetLastError(), "neighbour-list kernels");
 }
 

@@ -204,14 +204,14 @@ extern "C" int nep_compute_efv_static(const nep_hyper* hp, const float* z, int n
     double* part_e = partials;
     double* part_v = partials + ((nblocks + 7) / 8) * 8;
     int nb1 = 0, nb2 = 0, nc2 = 0;
-    if ((rc = launch_site_partial_forces(fa, nl, n, e_atom, part_e, err, st, nb1))) return rc;
+    if ((rc = launch_site_partial_forces(fa, nl, n, e_atom, part_e, err, st, nb1, true))) return rc;
     AssembleArgs aa{};
     aa.rc_max = (float)rmax;
     aa.box = box;
     aa.vel = nullptr;
     if ((rc = launch_assemble(aa, nl, n, force, virial_atom, part_v, err, st, nb2, nc2))) return rc;
     const SumSet e{part_e, nb1, 1, 1, 0, e_total}, w{part_v, nb2, 1, nc2, (size_t)nb2, virial_total};
-    if ((e_total || virial_total) && (rc = launch_sum(e, w, st))) return rc;
+    if ((e_total || virial_total) && (rc = launch_sum(e, w, st, true))) return rc;
     return err_out ? cuda_fail(cudaMemcpyAsync(err_out, err, sizeof(unsigned), cudaMemcpyDeviceToDevice, st),
                                "nep_compute_efv_static error word")
                    : NEP_OK;

@@ -200,3 +200,26 @@ def test_cells_path_search(orc, kind):
         near = int(np.sum(np.abs(r - rc) < 1e-5))
         assert abs(int(cnt[i]) - int(np.sum((r < rc) & (r > 0)))) <= near
     model.close()
+
+
+@pytest.mark.parametrize("cells", [(1, 1, 1), (4, 4, 4), (7, 7, 7), (12, 12, 12), (20, 20, 20)])
+def test_calls_back_to_back(cells):
+    """The kernels of a call are set up while their predecessors still run: calls
+    enqueued without a wait between them give the bits of calls that were waited
+    for (the summation orders are fixed, so equality)."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(5)
+    pos, box = inputs.diamond(*cells)
+    states = [soa(inputs.displace(pos, 0.1, rng)) for _ in range(6)]
+    model = nep.NEP(inputs.random_z(1021, rng))
+    waited = []
+    for x in states:
+        waited.append({k: v.clone() for k, v in model.compute(x, box).items()})
+        torch.cuda.synchronize()
+    queued = [{k: v.clone() for k, v in model.compute(x, box).items()} for x in states]
+    torch.cuda.synchronize()
+    for a, b in zip(waited, queued):
+        for k in a:
+            assert torch.equal(a[k], b[k]), k
+    model.close()
