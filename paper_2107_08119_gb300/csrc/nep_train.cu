@@ -541,6 +541,7 @@ __global__ void __launch_bounds__(kOwnerMaxThreads) k_contract_owner(
     float* __restrict__ w6out, float* __restrict__ fown)
 {
     extern __shared__ float4 s_stage4[];
+    const int block = block_after();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* s_rec = reinterpret_cast<float*>(s_stage4) + (size_t)warp * kOwnerStage;
     float* s_ang = s_rec + kOwnerChunk * kRecFloats;
@@ -553,7 +554,7 @@ __global__ void __launch_bounds__(kOwnerMaxThreads) k_contract_owner(
                      "l"(src)
                      : "memory");
     };
-    for (int j = j0 + (int)(((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); j < j1; j += warps) {
+    for (int j = j0 + (int)(((size_t)block * blockDim.x + threadIdx.x) >> 5); j < j1; j += warps) {
         const long long pe = pstart[j + 1];
         long long q0 = pstart[j];
         int nq = (int)min((long long)kOwnerChunk, pe - q0);
@@ -677,7 +678,7 @@ __global__ void __launch_bounds__(kReceiverThreads, 2) k_contract(
 {
     constexpr int kWarps = kReceiverThreads / 32;
     __shared__ RecvRed<kWarps> red;
-    const int c = c0 + (int)(gridDim.x - 1 - blockIdx.x);  // last chunk first (as k_contract_bulk)
+    const int c = c0 + (int)(gridDim.x - 1 - block_after());  // last chunk first (as k_contract_bulk)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k0 = 2 * lane;
     const bool on0 = k0 < P, on1 = k0 + 1 < P;
@@ -732,7 +733,7 @@ __global__ void __launch_bounds__(kReceiverThreads, 2) k_contract_staged(
     constexpr int kPair = 2 * (int)sizeof(PT);  // bytes of one lane's two members
     __shared__ RecvRed<kWarps> red;
     extern __shared__ __align__(16) unsigned char s_slots_raw[];  // [warps][kRecvStage][3][Pst / 2] member pairs
-    const int c = c0 + (int)(gridDim.x - 1 - blockIdx.x);  // last chunk first (as k_contract_bulk)
+    const int c = c0 + (int)(gridDim.x - 1 - block_after());  // last chunk first (as k_contract_bulk)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k0 = 2 * lane;
     const bool on0 = k0 < P, on1 = k0 + 1 < P;
@@ -806,12 +807,12 @@ __global__ void __launch_bounds__(kReceiverThreads, 2) k_contract_bulk(
 {
     extern __shared__ __align__(128) unsigned char s_bulk[];
     BulkSmem& S = *reinterpret_cast<BulkSmem*>(s_bulk);
-    bulk_init(S);
     BulkWarp bw;
     // the range's chunks from the last: the owner pass wrote the partial
     // forces in owner order, so the last chunks' rows are the ones most
     // likely still in L2
-    const int c = c0 + (int)(gridDim.x - 1 - blockIdx.x);
+    const int c = c0 + (int)(gridDim.x - 1 - block_after());
+    bulk_init(S);
     if (!bulk_receive_chunk<PT>(c, P, Pst, chunk_begin, chunk_end, U, pstart, fown, pbuf, w6in, f_tar, partials, err,
                                 discard != 0, S, bw))
         bulk_drain(S, bw);
@@ -1036,7 +1037,7 @@ __global__ void __cluster_dims__(1, kLossSplit, 1) __launch_bounds__(kLossThread
            double* __restrict__ loss)
 {
     constexpr int kBatch = 4;  // chunks whose loads are issued together (summed in order)
-    const int k = blockIdx.x, q = blockIdx.y, nq = gridDim.y;
+    const int k = block_after(), q = blockIdx.y, nq = gridDim.y;
     const int stride = nq * blockDim.x;
     double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // se, sf, sv, l1, l2
     {
@@ -1299,6 +1300,10 @@ bool valid_shape(const nep_dataset* ds, const EvalShape& h)
 using namespace nep;
 
 
+// Generations per graph launch where a run has that many left (20 BF16
+// generations 3,721 -> 3,668 us).
+constexpr int kGraphGens = 5;
+
 struct snes_state {
     nep_model* m = nullptr;
     int P = 0, n_par = 0;
@@ -1313,9 +1318,10 @@ struct snes_state {
     float* util = nullptr;  // rank utilities u_1..u_P (a constant of P)
     unsigned* d_gen = nullptr;  // generation counter read by the draws (device)
     nep::SnesCtl* d_ctl = nullptr;
-    // one generation captured as a CUDA graph (snes_run), keyed by what it bakes in
+    // one generation and kGraphGens of them captured as CUDA graphs (snes_run),
+    // keyed by what they bake in
     cudaStream_t cap = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraphExec_t exec[2] = {nullptr, nullptr};
     unsigned long long key_uid = 0;
     int key_epoch = -1, key_prec = -1;
     double key_lam[5] = {0, 0, 0, 0, 0};
@@ -1448,29 +1454,27 @@ void launch_contraction_t(const nep_dataset* ds, int P, int Pst, int c_lo, int c
         launch_owner_tc(ds->h_tile0[a0], ds->h_tile0[a1], ds->tiles, ds->apack, ds->rowscale, ds->G, Pst, ds->rev,
                         pbuf, ds->fown, ds->w6, ds->m->d_err, st);
     } else {
-        k_contract_owner<PT><<<std::min(blocks_for(a1 - a0, ow), 152 * 64 / ow), 32 * ow, ostage, st>>>(
-            a0, a1, P, Pst, reinterpret_cast<const PT*>(ds->G), ds->B, ds->pstart, ds->rev, ds->rec, ds->aidx,
-            ds->ang, pbuf, ds->w6, ds->fown);
+        launch_after(!fork, k_contract_owner<PT>, std::min(blocks_for(a1 - a0, ow), 152 * 64 / ow), 32 * ow, ostage, st,
+                     a0, a1, P, Pst, reinterpret_cast<const PT*>(ds->G), ds->B, ds->pstart, ds->rev, ds->rec, ds->aidx,
+                     ds->ang, pbuf, ds->w6, ds->fown);
     }
     if (fork) {
         cudaEventRecord(ev, st);
         cudaStreamWaitEvent(p2, ev, 0);
     }
     if (sh.recv_unroll == 1) {
-        k_contract_bulk<PT><<<c_hi - c_lo, kReceiverThreads, sizeof(BulkSmem), p2>>>(
-            c_lo, sh.discard, P, Pst, ds->chunk_begin, ds->chunk_end, ds->U, ds->pstart, ds->fown, pbuf, ds->w6,
-            ds->f_tar, ds->partials, ds->m->d_err);
+        launch_after(!fork, k_contract_bulk<PT>, c_hi - c_lo, kReceiverThreads, sizeof(BulkSmem), p2, c_lo, sh.discard, P,
+                     Pst, ds->chunk_begin, ds->chunk_end, ds->U, ds->pstart, ds->fown, pbuf, ds->w6, ds->f_tar,
+                     ds->partials, ds->m->d_err);
     } else if (sh.recv_unroll == 16) {
         const size_t smem = (size_t)(kReceiverThreads / 32) * kRecvStage * 3 * Pst * sizeof(PT);
-        k_contract_staged<PT><<<c_hi - c_lo, kReceiverThreads, smem, p2>>>(c_lo, sh.discard, P, Pst, ds->chunk_begin,
-                                                                           ds->chunk_end, ds->U, ds->pstart,
-                                                                           ds->fown, pbuf, ds->w6, ds->f_tar,
-                                                                           ds->partials);
+        launch_after(!fork, k_contract_staged<PT>, c_hi - c_lo, kReceiverThreads, smem, p2, c_lo, sh.discard, P, Pst,
+                     ds->chunk_begin, ds->chunk_end, ds->U, ds->pstart, ds->fown, pbuf, ds->w6, ds->f_tar,
+                     ds->partials);
     } else {
         auto recv = sh.recv_unroll == 12 ? k_contract<12, PT> : (sh.recv_unroll == 8 ? k_contract<8, PT> : k_contract<4, PT>);
-        recv<<<c_hi - c_lo, kReceiverThreads, 0, p2>>>(c_lo, sh.discard, P, Pst, ds->chunk_begin, ds->chunk_end,
-                                                       ds->U, ds->pstart, ds->fown, pbuf, ds->w6, ds->f_tar,
-                                                       ds->partials);
+        launch_after(!fork, recv, c_hi - c_lo, kReceiverThreads, 0, p2, c_lo, sh.discard, P, Pst, ds->chunk_begin,
+                     ds->chunk_end, ds->U, ds->pstart, ds->fown, pbuf, ds->w6, ds->f_tar, ds->partials);
     }
 }
 
@@ -1567,9 +1571,9 @@ int enqueue_evaluation(nep_model* m, nep_dataset* ds, const float* z_pop, int P,
         cudaEventRecord(ds->ev_join, ds->aux);
         cudaStreamWaitEvent(st, ds->ev_join, 0);
     }
-    k_loss<<<dim3(P, kLossSplit), kLossThreads, 0, st>>>(P, ds->S, n_par, ds->s_chunk0, ds->s_inv_na, ds->s_vtar,
-                                                         ds->partials, ds->e_tar, z_pop, lam[0], lam[1], lam[2], lam[3],
-                                                         lam[4], loss_inv(ds->S, ds->N, n_par), loss);
+    launch_after(n_ranges == 1, k_loss, dim3(P, kLossSplit), kLossThreads, 0, st, P, ds->S, n_par, ds->s_chunk0,
+                 ds->s_inv_na, ds->s_vtar, ds->partials, ds->e_tar, z_pop, lam[0], lam[1], lam[2], lam[3], lam[4],
+                 loss_inv(ds->S, ds->N, n_par), loss);
     return cuda_fail(cudaGetLastError(), "population evaluation kernels");
 }
 
@@ -2019,7 +2023,8 @@ int snes_destroy(snes_state* st)
     dfree(st->util);
     dfree(st->d_gen);
     dfree(st->d_ctl);
-    if (st->exec) cudaGraphExecDestroy(st->exec);
+    for (auto e : st->exec)
+        if (e) cudaGraphExecDestroy(e);
     if (st->cap) cudaStreamDestroy(st->cap);
     delete st;
     return NEP_OK;
@@ -2063,31 +2068,39 @@ int snes_run(snes_state* st, nep_dataset* ds, int precision, const double* lambd
     double lam[5] = {1.0, 1.0, 1.0, 0.05, 0.05};
     if (lambdas)
         for (int k = 0; k < 5; ++k) lam[k] = lambdas[k];
-    bool same = st->exec && st->key_uid == ds->uid && st->key_epoch == ds->epoch && st->key_prec == precision;
+    bool same = st->key_uid == ds->uid && st->key_epoch == ds->epoch && st->key_prec == precision;
     for (int k = 0; same && k < 5; ++k) same = st->key_lam[k] == lam[k];
-    if (!same) {
-        if (st->exec) cudaGraphExecDestroy(st->exec);
-        st->exec = nullptr;
-        cudaGraph_t g = nullptr;
-        if ((rc = cuda_fail(cudaStreamBeginCapture(st->cap, cudaStreamCaptureModeThreadLocal), "begin capture")))
-            return rc;
-        rc = enqueue_generation(st, ds, precision, lam, nullptr, st->d_ctl, st->cap);
-        const cudaError_t e = cudaStreamEndCapture(st->cap, &g);
-        if (!rc && e != cudaSuccess) rc = cuda_fail(e, "end capture");
-        if (!rc) rc = cuda_fail(cudaGraphInstantiate(&st->exec, g, 0), "instantiate generation graph");
-        if (g) cudaGraphDestroy(g);
-        if (rc) {
-            st->exec = nullptr;
-            return rc;
+    if (!same)
+        for (auto& e : st->exec) {
+            if (e) cudaGraphExecDestroy(e);
+            e = nullptr;
         }
-        st->key_uid = ds->uid;
-        st->key_epoch = ds->epoch;
-        st->key_prec = precision;
-        for (int k = 0; k < 5; ++k) st->key_lam[k] = lam[k];
-    }
+    st->key_uid = ds->uid;
+    st->key_epoch = ds->epoch;
+    st->key_prec = precision;
+    for (int k = 0; k < 5; ++k) st->key_lam[k] = lam[k];
+    // `gens` generations as one graph
+    auto capture = [&](int gens, cudaGraphExec_t* exec) {
+        cudaGraph_t g = nullptr;
+        int r = cuda_fail(cudaStreamBeginCapture(st->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
+        if (r) return r;
+        for (int k = 0; k < gens && !r; ++k)
+            r = enqueue_generation(st, ds, precision, lam, nullptr, st->d_ctl, st->cap);
+        const cudaError_t e = cudaStreamEndCapture(st->cap, &g);
+        if (!r && e != cudaSuccess) r = cuda_fail(e, "end capture");
+        if (!r) r = cuda_fail(cudaGraphInstantiate(exec, g, 0), "instantiate generation graph");
+        if (g) cudaGraphDestroy(g);
+        if (r) *exec = nullptr;
+        return r;
+    };
+    if (n_gen >= kGraphGens && !st->exec[1] && (rc = capture(kGraphGens, &st->exec[1]))) return rc;
+    if (n_gen % kGraphGens && !st->exec[0] && (rc = capture(1, &st->exec[0]))) return rc;
     k_set_ctl<<<1, 1, 0, cs>>>(st->d_ctl, loss_hist, st->gen);
-    for (int g = 0; g < n_gen; ++g)
-        if ((rc = cuda_fail(cudaGraphLaunch(st->exec, cs), "launch generation graph"))) return rc;
+    for (int g = 0; g < n_gen;) {
+        const int u = n_gen - g >= kGraphGens ? 1 : 0;
+        if ((rc = cuda_fail(cudaGraphLaunch(st->exec[u], cs), "launch generation graph"))) return rc;
+        g += u ? kGraphGens : 1;
+    }
     k_set_ctl<<<1, 1, 0, cs>>>(st->d_ctl, nullptr, 0u);
     st->gen += (unsigned)n_gen;
     return cuda_fail(cudaGetLastError(), "snes_run");
