@@ -330,12 +330,13 @@ __device__ __forceinline__ double sum_partials(const double* __restrict__ src, i
 // predecessor is a kernel of the same call on the same stream, not a wait for an
 // event, a copy or a conditional node.  96 atoms 92 -> 81 us per call, 125,000
 // atoms 430 -> 416, MD step of 4,096 atoms 45.0 -> 43.8 us.
-// Returns blockIdx.x: loads whose address comes from it stay behind the wait.
+// Returns blockIdx.x, so that a kernel has no block before the wait (read in the
+// same inline assembly it was no longer known to be uniform: steps of 64,000
+// two-species atoms 2.5 % slower).
 __device__ __forceinline__ int block_after()
 {
-    int b;
-    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, %%ctaid.x;" : "=r"(b)::"memory");
-    return b;
+    cudaGridDependencySynchronize();
+    return (int)blockIdx.x;
 }
 
 // A read-only pointer for loads that must stay behind block_after()
