@@ -5,7 +5,7 @@
 //   k_kick_drift   v += dt/2 F/m; x += dt v (FP64); FP32 hi/lo split of x;
 //                  largest squared displacement since the last list build;
 //                  its last block sets the gate = (max displacement >
-//                  skin/2) or a pending rebuild
+//                  skin/2)
 //   list build     wrap, bin, Verlet list, reverse index (gated: the kernels
 //                  return at once when the gate is zero)
 //   k_site         site energies and partial forces
@@ -45,23 +45,20 @@ static constexpr double kEvPerAFsK_WPerMK = 1.602176634e6;
 namespace nep {
 namespace {
 
-// control words on the device
-enum { kCtlDisp = 0, kCtlGate = 1, kCtlPending = 2, kCtlStep = 3, kCtlFinish = 4, kCtlKick = 5, kCtlWords = 6 };
+// control words on the device; the two from kCtlKick hold one 64-bit count
+enum { kCtlGate = 0, kCtlStep = 1, kCtlKick = 2, kCtlWords = 4 };
 
-// The rebuild decision: gate = a pending rebuild or the largest squared
-// displacement since the last build above thresh2; the displacement and the
-// pending flag are cleared.  use_cond: the step runs from a CUDA graph whose
-// list rebuild sits behind the conditional node `cond`, which this sets.
-__device__ void decide(unsigned* ctl, float thresh2, unsigned long long* rebuilds, cudaGraphConditionalHandle cond,
+// The rebuild decision: gate = `far`, an atom beyond the threshold since the
+// last build; the step is counted (k_md_finish writes row kCtlStep - 1).
+// use_cond: the step runs from a CUDA graph whose list rebuild sits behind the
+// conditional node `cond`, which this sets.
+__device__ void decide(unsigned* ctl, bool far, unsigned long long* rebuilds, cudaGraphConditionalHandle cond,
                        int use_cond)
 {
-    const unsigned disp = __ldcg(ctl + kCtlDisp);
-    const bool go = __ldcg(ctl + kCtlPending) != 0u || __uint_as_float(disp) > thresh2;
-    ctl[kCtlGate] = go ? 1u : 0u;
-    ctl[kCtlDisp] = 0u;
-    ctl[kCtlPending] = 0u;
-    if (go) *rebuilds += 1ull;
-    if (use_cond) cudaGraphSetConditional(cond, go ? 1u : 0u);
+    ctl[kCtlGate] = far ? 1u : 0u;
+    ctl[kCtlStep] += 1u;
+    if (far) *rebuilds += 1ull;
+    if (use_cond) cudaGraphSetConditional(cond, far ? 1u : 0u);
 }
 
 __global__ void k_kick_drift(int n, double* __restrict__ x, double* __restrict__ v, const float* __restrict__ F,
@@ -87,32 +84,17 @@ __global__ void k_kick_drift(int n, double* __restrict__ x, double* __restrict__
         store_pos(xr, i, xn, load_z(xr, i));  // the species number stays
         d2 = (float)dd;
     }
-    // block maximum, then one atomic per block (one per warp serialised
-    // thousands of atomics on a single word)
-    __shared__ float wmax[32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d2 = fmaxf(d2, __shfl_xor_sync(0xffffffffu, d2, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = d2;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        d2 = threadIdx.x < (blockDim.x >> 5) ? wmax[threadIdx.x] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) d2 = fmaxf(d2, __shfl_xor_sync(0xffffffffu, d2, o));
-        // non-negative floats order like their bit patterns
-        if (threadIdx.x == 0 && d2 > 0.f) atomicMax(ctl + kCtlDisp, __float_as_uint(d2));
-    }
-    // the last block to finish (a count in ctl, which it clears) takes the
-    // rebuild decision
-    __shared__ int last;
-    if (threadIdx.x == 0) {
-        __threadfence();  // this block's maximum before the count
-        last = atomicAdd(ctl + kCtlKick, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last || threadIdx.x != 0) return;
-    __threadfence();
-    ctl[kCtlKick] = 0u;
-    decide(ctl, thresh2, rebuilds, cond, use_cond);
+    // the blocks with an atom beyond the threshold (high half) and those that
+    // are done (low half) are counted by one atomic per block; the last one
+    // clears the count and takes the rebuild decision from it
+    const bool far = __syncthreads_or(d2 > thresh2);
+    if (threadIdx.x != 0) return;
+    unsigned long long* count = reinterpret_cast<unsigned long long*>(ctl + kCtlKick);
+    const unsigned long long mine = far ? (1ull << 32) + 1 : 1ull;
+    const unsigned long long all = atomicAdd(count, mine) + mine;
+    if ((unsigned)all != gridDim.x) return;
+    *count = 0ull;
+    decide(ctl, (all >> 32) != 0, rebuilds, cond, use_cond);
 }
 
 // Second half kick with the HNEMD driving force, E_kin and J per block.
@@ -302,12 +284,15 @@ __global__ void k_scale_v(int n, double* __restrict__ vel, const double* __restr
     for (int c = 0; c < 3; ++c) vel[(size_t)c * n + i] *= lam;
 }
 
-// The step's last kernel, one block per sum: block 0 adds the site-energy
-// block partials into red[0], block 1 + c component c of the other block
-// partials into red[off_x + c] (each thread a fixed stride of the partials in
-// order, then a fixed tree: deterministic).  Several SMs share the FP64 adds
-// (slow on this part).  The last block to finish (a count in ctl, which it
-// clears) writes the thermo row and J and the Berendsen factor.
+// The step's last kernel, one block per sum: block 0 the site-energy block
+// partials, block 1 + c component c of the other block partials (each thread a
+// fixed stride of the partials in order, then a fixed tree: deterministic).
+// Several SMs share the FP64 adds (slow on this part).  No sum needs another
+// one, so each block writes its own place of the thermo row or of J, and that
+// of E_kin the Berendsen factor; a last block that collected all sums cost a
+// fence, an atomic and a second round of loads.  This and the one atomic of
+// k_kick_drift: step of 4,096 atoms 45.4 -> 41.9 us, driven step of 13,824 80.1
+// -> 75.7.
 constexpr int kFinishThreads = 512;
 
 __global__ void __launch_bounds__(kFinishThreads) k_md_finish(const double* __restrict__ part_e, int nb_e,
@@ -315,50 +300,38 @@ __global__ void __launch_bounds__(kFinishThreads) k_md_finish(const double* __re
                                                               int bstride_x, size_t cstride_x, int off_x,
                                                               double* __restrict__ red,
                                                               double* __restrict__ thermo, double* __restrict__ heat,
-                                                              unsigned* __restrict__ ctl, double t0, double tau,
+                                                              const unsigned* ctl, double t0, double tau,
                                                               double dt, double dof_kb)
 {
-    // red: [0] E_pot, [1..9] W (row-major), [10] E_kin, [11..13] J, [14] lambda
+    // sums: 0 E_pot, 1..9 W (row-major), 10 E_kin, 11..13 J; red: [1..9] W with
+    // HNEMD (summed before the kick), [14] lambda
     const int w = block_after();
-    const double t = w == 0 ? sum_partials<kFinishThreads>(part_e, nb_e, 1)
-                            : sum_partials<kFinishThreads>(part_x + (w - 1) * cstride_x, nb_x, bstride_x);
-    __shared__ int last;
-    if (threadIdx.x == 0) {
-        red[w == 0 ? 0 : off_x + w - 1] = t;
-        __threadfence();  // this sum before the count
-        last = atomicAdd(ctl + kCtlFinish, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last || threadIdx.x != 0) return;
-    __threadfence();
-    ctl[kCtlFinish] = 0u;
-    // the other blocks' sums, read from L2
-    auto rd = [&](int k) { return __ldcg(red + k); };
-    const unsigned s = ctl[kCtlStep];
-    double ek = rd(10);
-    if (tau > 0.0) {
-        const double T = 2.0 * ek / dof_kb;
+    double t = w == 0 ? sum_partials<kFinishThreads>(part_e, nb_e, 1)
+                      : sum_partials<kFinishThreads>(part_x + (w - 1) * cstride_x, nb_x, bstride_x);
+    if (threadIdx.x != 0) return;
+    const int k = w == 0 ? 0 : off_x + w - 1;
+    const unsigned s = ctl[kCtlStep] - 1u;  // counted by k_kick_drift
+    if (k == 10 && tau > 0.0) {
+        const double T = 2.0 * t / dof_kb;
         const double lam = T > 0.0 ? sqrt(1.0 + dt / tau * (t0 / T - 1.0)) : 1.0;
         red[14] = lam;
-        ek *= lam * lam;
+        t *= lam * lam;
     }
     if (thermo) {
-        double* t = thermo + (size_t)s * NEP_THERMO_COLS;
-        t[0] = rd(0);
-        t[1] = ek;
-        t[2] = rd(1);  // xx
-        t[3] = rd(5);  // yy
-        t[4] = rd(9);  // zz
-        t[5] = rd(2);  // xy
-        t[6] = rd(6);  // yz
-        t[7] = rd(7);  // zx
+        double* row = thermo + (size_t)s * NEP_THERMO_COLS;  // E_pot, E_kin, W xx yy zz xy yz zx
+        const int col = k == 0 ? 0 : k == 10 ? 1 : k == 1 ? 2 : k == 5 ? 3 : k == 9 ? 4 : k == 2 ? 5 : k == 6 ? 6
+                      : k == 7 ? 7 : -1;
+        if (col >= 0) row[col] = t;
+        if (k == 0 && off_x == 10) {
+            row[2] = red[1];
+            row[3] = red[5];
+            row[4] = red[9];
+            row[5] = red[2];
+            row[6] = red[6];
+            row[7] = red[7];
+        }
     }
-    if (heat) {
-        heat[(size_t)s * 3 + 0] = rd(11);
-        heat[(size_t)s * 3 + 1] = rd(12);
-        heat[(size_t)s * 3 + 2] = rd(13);
-    }
-    ctl[kCtlStep] = s + 1u;
+    if (heat && k >= 11) heat[(size_t)s * 3 + k - 11] = t;
 }
 
 inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
