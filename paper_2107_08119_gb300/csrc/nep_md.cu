@@ -73,7 +73,7 @@ __global__ void k_kick_drift(int n, double* __restrict__ x, double* __restrict__
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const size_t o = (size_t)c * n + i;
-            const double vc = v[o] + hdtm * (double)F[o];
+            const double vc = v[o] + hdtm * to_double(F[o]);
             const double xc = x[o] + dt * vc;
             v[o] = vc;
             x[o] = xc;

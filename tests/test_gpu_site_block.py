@@ -223,3 +223,26 @@ def test_calls_back_to_back(cells):
         for k in a:
             assert torch.equal(a[k], b[k]), k
     model.close()
+
+
+@pytest.mark.parametrize("value", [0.0, -0.0, 1e-310, -1e-40, 2.0 ** -101, 2.0 ** -102, 1e-20, 5.5, 1.0 + 2.0 ** -24,
+                                   1.0 + 3 * 2.0 ** -24, np.nextafter(2.0, 0.0), -3.0 + 2.0 ** -40])
+def test_position_split(orc, value):
+    """Positions are split into two FP32 words by integer operations: zeros,
+    denormals, the ends of that range, halves of the last place and carries into
+    the next binade as coordinates of one atom."""
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(11)
+    pos, box = inputs.diamond(3, 3, 3)
+    pos = inputs.displace(pos, 0.1, rng)
+    pos -= pos[5]
+    pos[5] = value  # all other coordinates moved with it
+    pos[:5] += value
+    pos[6:] += value
+    z = inputs.random_z(1021, rng)
+    model = nep.NEP(z)
+    out = model.compute(soa(pos), box)
+    U, F, W = orc.efv(orc.NepHyper(), f32_exact(z), pos, box)
+    assert np.abs(out["e_atom"].cpu().numpy() - U).max() <= 1e-6
+    assert np.abs(aos(out["force"]) - F).max() <= 1e-4
+    model.close()
