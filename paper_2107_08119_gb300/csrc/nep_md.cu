@@ -105,21 +105,26 @@ __global__ void k_hnemd_kick(int n, float* __restrict__ F, const float* __restri
 {
     const int i = block_after() * blockDim.x + threadIdx.x;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    const double fe[3] = {fe0, fe1, fe2};
+    __shared__ double s_fm[3];
+    if (threadIdx.x < 3) {
+        double fm = 0.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) fm += fe[a] * reread(wtot)[3 * a + threadIdx.x];
+        s_fm[threadIdx.x] = fm;
+    }
+    __syncthreads();
     if (i < n) {
-        const double fe[3] = {fe0, fe1, fe2};
-        wtot = reread(wtot);
         float w[9];
 #pragma unroll
         for (int c = 0; c < 9; ++c) w[c] = W[(size_t)c * n + i];
         double v[3];
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            double fx = 0.0, fm = 0.0;
+            const double fm = s_fm[b];
+            double fx = 0.0;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                fx += fe[a] * (double)w[3 * a + b];
-                fm += fe[a] * wtot[3 * a + b];
-            }
+            for (int a = 0; a < 3; ++a) fx += fe[a] * (double)w[3 * a + b];
             const float ft = (float)((double)F[(size_t)b * n + i] + fx - fm * inv_n);
             F[(size_t)b * n + i] = ft;
             v[b] = vel[(size_t)b * n + i] + hdtm * (double)ft;
@@ -345,6 +350,13 @@ using namespace nep;
 // graphs costs more than the one between their kernels (4,096 atoms 49.4 -> 46.1
 // us per step; 10 steps per graph 45.5).
 constexpr int kGraphSteps = 5;
+
+// Threads per block of the per-atom step kernels: two FP64 lanes per SM and
+// clock bound them, so up to one block of 256 per SM the atoms go to more SMs
+// (driven step of 13,824 atoms 73.9 -> 71.4 us, step of 4,096 39.8 -> 39.4; 128
+// threads the same).  The partial sums of k_hnemd_kick, four per block, need the
+// room that 64 leaves: 14 of 16 words per block of the site pass, two more here.
+inline int step_threads(int n) { return n <= 152 * 256 ? 64 : 256; }
 
 struct nep_md {
     nep_model* m = nullptr;
@@ -691,7 +703,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
     double* part_a = md->ws.partials + ((nb + 7) / 8) * 8;
     double* part_h = part_a + 13 * (size_t)nb;  // HNEMD kick partials
     const bool drive = md->drive;
-    const int nbk = blocks_for(n, 256);
+    const int kt = step_threads(n), nbk = blocks_for(n, kt);
     const double kef = 0.5 * md->mass * kAmuA2Fs2InEv;
     ForceArgs fa{m->d_z, m->hp.n_neu, (float)m->hp.rc_R, (float)m->hp.rc_A, md->box};
     fa.nr = m->hp.n_max_R + 1;
@@ -734,7 +746,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         if (drive) {
             // the starting forces include the driving force (no kick: hdt/m = 0)
             if ((rc = launch_sum(SumSet{part_a, b2, 1, c2, (size_t)b2, md->red + 1}, SumSet{}, st))) return rc;
-            k_hnemd_kick<<<nbk, 256, 0, st>>>(n, md->ws.force, md->w_atom, vel, md->fe[0], md->fe[1], md->fe[2],
+            k_hnemd_kick<<<nbk, kt, 0, st>>>(n, md->ws.force, md->w_atom, vel, md->fe[0], md->fe[1], md->fe[2],
                                               md->red + 1, 1.0 / n, 0.0, kef, part_h, m->d_err);
         }
         if ((rc = cuda_fail(cudaMemsetAsync(md->ctl, 0, sizeof(unsigned) * kCtlWords, st), "cudaMemsetAsync")))
@@ -752,7 +764,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
     // (follows: another step comes before it in the stream)
     auto head = [&](cudaStream_t q, bool use_cond, cudaGraphConditionalHandle cond, bool follows) {
         Profiler::Slot* pk = m->prof.begin(NEP_PROFILE_STEP, q);
-        launch_after(follows, k_kick_drift, blocks_for(n, 256), 256, 0, q, n, pos, vel, md->ws.force, hdtm, dt,
+        launch_after(follows, k_kick_drift, nbk, kt, 0, q, n, pos, vel, md->ws.force, hdtm, dt,
                      nl.xr, md->x_ref, md->ctl, thresh * thresh, md->rebuilds, cond, use_cond ? 1 : 0);
         m->prof.end(pk, q);
     };
@@ -785,7 +797,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         if (drive) {
             // the kick needs the total virial first
             if ((r = launch_sum(SumSet{part_a, b2, 1, c2, (size_t)b2, md->red + 1}, SumSet{}, q, true))) return r;
-            launch_after(true, k_hnemd_kick, nbk, 256, 0, q, n, md->ws.force, w_out, vel, md->fe[0], md->fe[1],
+            launch_after(true, k_hnemd_kick, nbk, kt, 0, q, n, md->ws.force, w_out, vel, md->fe[0], md->fe[1],
                          md->fe[2], md->red + 1, 1.0 / n, hdtm, kef, part_h, m->d_err);
             launch_after(true, k_md_finish, 5, kFinishThreads, 0, q, part_e, b1, part_h, nbk, 4, 1, 10, md->red, thermo,
                          heat, md->ctl, md->t0, md->tau, dt, dof_kb);
@@ -803,7 +815,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             ++md->shc_samples;
         }
         if (md->shc_lags > 0) ++md->shc_step;
-        if (md->tau > 0.0 && n > 1) launch_after(!sample, k_scale_v, nbk, 256, 0, q, n, vel, md->red);
+        if (md->tau > 0.0 && n > 1) launch_after(!sample, k_scale_v, nbk, kt, 0, q, n, vel, md->red);
         m->prof.end(pk, q);
         return cuda_fail(cudaGetLastError(), "md step kernels");
     };

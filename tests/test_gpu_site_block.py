@@ -246,3 +246,31 @@ def test_position_split(orc, value):
     assert np.abs(out["e_atom"].cpu().numpy() - U).max() <= 1e-6
     assert np.abs(aos(out["force"]) - F).max() <= 1e-4
     model.close()
+
+
+@pytest.mark.parametrize("n", [63, 65, 38912, 38913])
+def test_driven_step_sums(n):
+    """The per-atom step kernels run in blocks of 64 atoms up to 38,912 and of
+    256 above: E_kin of the last step is that of the velocities (FP64 sums of
+    n terms: 1e-12 relative), and the drive keeps the total momentum (FP32
+    forces: each of n steps of dt F / m rounds at 2^-24 of at most 10 eV/A)."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(n)
+    pos, box = inputs.diamond(17, 17, 17) if n > 1000 else inputs.diamond(2, 2, 3)
+    pos = inputs.displace(pos, 0.1, rng)[:n]
+    vel = rng.normal(0.0, 1e-3, (n, 3))
+    vel -= vel.mean(axis=0)
+    model = nep.NEP(inputs.random_z(1021, rng))
+    mass, dt = 28.085, 1.0
+    md = nep.MD(model, n, box, mass)
+    md.set_hnemd([1e-4, 0.0, -2e-4])
+    x, v = soa(pos), soa(vel)
+    thermo = torch.zeros((3, 8), dtype=torch.float64, device="cuda")
+    md.step(x, v, 3, dt, thermo=thermo)
+    unit = 1.66053906660e-27 * 1.0e10 / 1.602176634e-19  # amu A^2 / fs^2 in eV
+    ekin = 0.5 * mass * unit * (v * v).sum().item()
+    assert abs(thermo[2, 1].item() - ekin) <= 1e-12 * ekin
+    assert v.sum(dim=1).abs().max().item() <= n * 3 * dt * 10 * 2.0 ** -24 / (mass * unit)
+    md.close()
+    model.close()
