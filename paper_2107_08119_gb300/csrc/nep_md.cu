@@ -48,25 +48,100 @@ namespace {
 // control words on the device; the two from kCtlKick hold one 64-bit count
 enum { kCtlGate = 0, kCtlStep = 1, kCtlKick = 2, kCtlWords = 4 };
 
+// A step's sums, one block each: block 0 the site-energy block partials, block
+// 1 + c component c of the other block partials (each thread a fixed stride of
+// the partials in order, then a fixed tree: deterministic).  Several SMs share
+// the FP64 adds (slow on this part).  No sum needs another one, so each block
+// writes its own place of the thermo row or of J, and that of E_kin the
+// Berendsen factor; a last block that collected all sums cost a fence, an atomic
+// and a second round of loads.  This and the one atomic of k_kick_drift: step of
+// 4,096 atoms 45.4 -> 41.9 us, driven step of 13,824 80.1 -> 75.7.
+// Without a thermostat nothing in the next step's kick needs them, so within a
+// graph they are extra blocks of that kernel, not a launch of their own: step of
+// 4,096 atoms 40.1 -> 37.7 us, of 125,000 294.2 -> 288.9.
+struct StepSums {
+    int nsum = 0;  // blocks
+    const double* part_e = nullptr;
+    int nb_e = 0;
+    const double* part_x = nullptr;
+    int nb_x = 0, bstride_x = 0;
+    size_t cstride_x = 0;
+    int off_x = 0;
+    double* red = nullptr;
+    double* thermo = nullptr;
+    double* heat = nullptr;
+    const unsigned* ctl = nullptr;
+    int row = 0;  // row of the step, from the step counter
+    double t0 = 0.0, tau = 0.0, dt = 0.0, dof_kb = 0.0;
+};
+
+template <int THREADS>
+__device__ __forceinline__ void step_sum(const StepSums& S, int w)
+{
+    // sums: 0 E_pot, 1..9 W (row-major), 10 E_kin, 11..13 J; red: [1..9] W with
+    // HNEMD (summed before the kick), [14] lambda
+    double t = sum_partials<THREADS>(w == 0 ? S.part_e : S.part_x + (w - 1) * S.cstride_x, w == 0 ? S.nb_e : S.nb_x,
+                                     w == 0 ? 1 : S.bstride_x);
+    if (threadIdx.x != 0) return;
+    const int k = w == 0 ? 0 : S.off_x + w - 1;
+    const size_t s = (size_t)((int)S.ctl[kCtlStep] + S.row);
+    if (k == 10 && S.tau > 0.0) {
+        const double T = 2.0 * t / S.dof_kb;
+        const double lam = T > 0.0 ? sqrt(1.0 + S.dt / S.tau * (S.t0 / T - 1.0)) : 1.0;
+        S.red[14] = lam;
+        t *= lam * lam;
+    }
+    if (S.thermo) {
+        double* row = S.thermo + s * NEP_THERMO_COLS;  // E_pot, E_kin, W xx yy zz xy yz zx
+        const int col = k == 0 ? 0 : k == 10 ? 1 : k == 1 ? 2 : k == 5 ? 3 : k == 9 ? 4 : k == 2 ? 5 : k == 6 ? 6
+                      : k == 7 ? 7 : -1;
+        if (col >= 0) row[col] = t;
+        if (k == 0 && S.off_x == 10) {
+            row[2] = S.red[1];
+            row[3] = S.red[5];
+            row[4] = S.red[9];
+            row[5] = S.red[2];
+            row[6] = S.red[6];
+            row[7] = S.red[7];
+        }
+    }
+    if (S.heat && k >= 11) S.heat[s * 3 + k - 11] = t;
+}
+
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_md_finish(StepSums S)
+{
+    step_sum<THREADS>(S, block_after());
+}
+
 // The rebuild decision: gate = `far`, an atom beyond the threshold since the
-// last build; the step is counted (k_md_finish writes row kCtlStep - 1).
+// last build; `count` steps are counted.
 // use_cond: the step runs from a CUDA graph whose list rebuild sits behind the
 // conditional node `cond`, which this sets.
-__device__ void decide(unsigned* ctl, bool far, unsigned long long* rebuilds, cudaGraphConditionalHandle cond,
-                       int use_cond)
+__device__ void decide(unsigned* ctl, bool far, int count, unsigned long long* rebuilds,
+                       cudaGraphConditionalHandle cond, int use_cond)
 {
     ctl[kCtlGate] = far ? 1u : 0u;
-    ctl[kCtlStep] += 1u;
+    if (count) ctl[kCtlStep] += (unsigned)count;
     if (far) *rebuilds += 1ull;
     if (use_cond) cudaGraphSetConditional(cond, far ? 1u : 0u);
 }
 
-__global__ void k_kick_drift(int n, double* __restrict__ x, double* __restrict__ v, const float* __restrict__ F,
-                             double hdtm, double dt, float* __restrict__ xr,
-                             const double* __restrict__ x_ref, unsigned* __restrict__ ctl, float thresh2,
-                             unsigned long long* __restrict__ rebuilds, cudaGraphConditionalHandle cond, int use_cond)
+// The first S.nsum blocks add up the previous step.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, int n, double* __restrict__ x, double* __restrict__ v,
+                                                        const float* __restrict__ F, double hdtm, double dt,
+                                                        float* __restrict__ xr, const double* __restrict__ x_ref,
+                                                        unsigned* __restrict__ ctl, float thresh2, int count,
+                                                        unsigned long long* __restrict__ rebuilds,
+                                                        cudaGraphConditionalHandle cond, int use_cond)
 {
-    const int i = block_after() * blockDim.x + threadIdx.x;
+    const int block = block_after() - S.nsum;
+    if (block < 0) {
+        step_sum<THREADS>(S, blockIdx.x);
+        return;
+    }
+    const int i = block * THREADS + threadIdx.x;
     float d2 = 0.f;
     if (i < n) {
         double dd = 0.0, xn[3];
@@ -89,12 +164,12 @@ __global__ void k_kick_drift(int n, double* __restrict__ x, double* __restrict__
     // clears the count and takes the rebuild decision from it
     const bool far = __syncthreads_or(d2 > thresh2);
     if (threadIdx.x != 0) return;
-    unsigned long long* count = reinterpret_cast<unsigned long long*>(ctl + kCtlKick);
+    unsigned long long* done = reinterpret_cast<unsigned long long*>(ctl + kCtlKick);
     const unsigned long long mine = far ? (1ull << 32) + 1 : 1ull;
-    const unsigned long long all = atomicAdd(count, mine) + mine;
-    if ((unsigned)all != gridDim.x) return;
-    *count = 0ull;
-    decide(ctl, (all >> 32) != 0, rebuilds, cond, use_cond);
+    const unsigned long long all = atomicAdd(done, mine) + mine;
+    if ((unsigned)all != gridDim.x - S.nsum) return;
+    *done = 0ull;
+    decide(ctl, (all >> 32) != 0, count, rebuilds, cond, use_cond);
 }
 
 // Second half kick with the HNEMD driving force, E_kin and J per block.
@@ -287,56 +362,6 @@ __global__ void k_scale_v(int n, double* __restrict__ vel, const double* __restr
     const double lam = reread(red)[14];
 #pragma unroll
     for (int c = 0; c < 3; ++c) vel[(size_t)c * n + i] *= lam;
-}
-
-// The step's last kernel, one block per sum: block 0 the site-energy block
-// partials, block 1 + c component c of the other block partials (each thread a
-// fixed stride of the partials in order, then a fixed tree: deterministic).
-// Several SMs share the FP64 adds (slow on this part).  No sum needs another
-// one, so each block writes its own place of the thermo row or of J, and that
-// of E_kin the Berendsen factor; a last block that collected all sums cost a
-// fence, an atomic and a second round of loads.  This and the one atomic of
-// k_kick_drift: step of 4,096 atoms 45.4 -> 41.9 us, driven step of 13,824 80.1
-// -> 75.7.
-constexpr int kFinishThreads = 512;
-
-__global__ void __launch_bounds__(kFinishThreads) k_md_finish(const double* __restrict__ part_e, int nb_e,
-                                                              const double* __restrict__ part_x, int nb_x,
-                                                              int bstride_x, size_t cstride_x, int off_x,
-                                                              double* __restrict__ red,
-                                                              double* __restrict__ thermo, double* __restrict__ heat,
-                                                              const unsigned* ctl, double t0, double tau,
-                                                              double dt, double dof_kb)
-{
-    // sums: 0 E_pot, 1..9 W (row-major), 10 E_kin, 11..13 J; red: [1..9] W with
-    // HNEMD (summed before the kick), [14] lambda
-    const int w = block_after();
-    double t = w == 0 ? sum_partials<kFinishThreads>(part_e, nb_e, 1)
-                      : sum_partials<kFinishThreads>(part_x + (w - 1) * cstride_x, nb_x, bstride_x);
-    if (threadIdx.x != 0) return;
-    const int k = w == 0 ? 0 : off_x + w - 1;
-    const unsigned s = ctl[kCtlStep] - 1u;  // counted by k_kick_drift
-    if (k == 10 && tau > 0.0) {
-        const double T = 2.0 * t / dof_kb;
-        const double lam = T > 0.0 ? sqrt(1.0 + dt / tau * (t0 / T - 1.0)) : 1.0;
-        red[14] = lam;
-        t *= lam * lam;
-    }
-    if (thermo) {
-        double* row = thermo + (size_t)s * NEP_THERMO_COLS;  // E_pot, E_kin, W xx yy zz xy yz zx
-        const int col = k == 0 ? 0 : k == 10 ? 1 : k == 1 ? 2 : k == 5 ? 3 : k == 9 ? 4 : k == 2 ? 5 : k == 6 ? 6
-                      : k == 7 ? 7 : -1;
-        if (col >= 0) row[col] = t;
-        if (k == 0 && off_x == 10) {
-            row[2] = red[1];
-            row[3] = red[5];
-            row[4] = red[9];
-            row[5] = red[2];
-            row[6] = red[6];
-            row[7] = red[7];
-        }
-    }
-    if (heat && k >= 11) heat[(size_t)s * 3 + k - 11] = t;
 }
 
 inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
@@ -761,11 +786,18 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
 
     // one step in three parts: kick-drift and the rebuild decision, the list
     // rebuild, then forces, second half kick and the step's sums
-    // (follows: another step comes before it in the stream)
-    auto head = [&](cudaStream_t q, bool use_cond, cudaGraphConditionalHandle cond, bool follows) {
+    // (count: steps to count; follows: another step comes before it in the stream,
+    // whose sums are `prev` if it has left them)
+    StepSums prev;
+    // threads per sum: with a thermostat always sums of their own, else as in the
+    // kick, so that a step's sums have the same bits wherever a graph ends
+    const int ft = md->tau > 0.0 ? 512 : kt;
+    auto head = [&](cudaStream_t q, bool use_cond, cudaGraphConditionalHandle cond, int count, bool follows) {
         Profiler::Slot* pk = m->prof.begin(NEP_PROFILE_STEP, q);
-        launch_after(follows, k_kick_drift, nbk, kt, 0, q, n, pos, vel, md->ws.force, hdtm, dt,
-                     nl.xr, md->x_ref, md->ctl, thresh * thresh, md->rebuilds, cond, use_cond ? 1 : 0);
+        launch_after(follows, kt == 64 ? k_kick_drift<64> : k_kick_drift<256>, nbk + prev.nsum, kt, 0, q, prev, n, pos,
+                     vel, md->ws.force, hdtm, dt, nl.xr, md->x_ref, md->ctl, thresh * thresh, count, md->rebuilds, cond,
+                     use_cond ? 1 : 0);
+        prev.nsum = 0;
         m->prof.end(pk, q);
     };
     auto rebuild = [&](cudaStream_t q, const unsigned* g) {
@@ -774,7 +806,8 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         m->prof.end(pk, q);
         return r;
     };
-    auto tail = [&](cudaStream_t q) {
+    // row: the step's row from the step counter; leave: the next head() takes the sums
+    auto tail = [&](cudaStream_t q, int row, bool leave) {
         int b1 = 0, b2 = 0, c2 = 0, r;
         // spectral heat current: this step's W_i goes to the ring when sampled
         const bool sample = md->shc_lags > 0 && md->shc_step % md->shc_every == 0;
@@ -799,12 +832,15 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             if ((r = launch_sum(SumSet{part_a, b2, 1, c2, (size_t)b2, md->red + 1}, SumSet{}, q, true))) return r;
             launch_after(true, k_hnemd_kick, nbk, kt, 0, q, n, md->ws.force, w_out, vel, md->fe[0], md->fe[1],
                          md->fe[2], md->red + 1, 1.0 / n, hdtm, kef, part_h, m->d_err);
-            launch_after(true, k_md_finish, 5, kFinishThreads, 0, q, part_e, b1, part_h, nbk, 4, 1, 10, md->red, thermo,
-                         heat, md->ctl, md->t0, md->tau, dt, dof_kb);
-        } else {
-            launch_after(true, k_md_finish, 1 + c2, kFinishThreads, 0, q, part_e, b1, part_a, b2, 1, (size_t)b2, 1,
-                         md->red, thermo, heat, md->ctl, md->t0, md->tau, dt, dof_kb);
         }
+        StepSums S{drive ? 5 : 1 + c2, part_e, b1, drive ? part_h : part_a, drive ? nbk : b2, drive ? 4 : 1,
+                   drive ? 1 : (size_t)b2, drive ? 10 : 1, md->red, thermo, heat, md->ctl, row, md->t0, md->tau, dt,
+                   dof_kb};
+        if (leave)
+            prev = S;
+        else
+            launch_after(true, ft == 64 ? k_md_finish<64> : ft == 256 ? k_md_finish<256> : k_md_finish<512>, S.nsum, ft,
+                         0, q, S);
         if (sample) {  // v is that of J: after the second half kick, before the thermostat
             const int avail = (int)(md->shc_samples + 1 < md->shc_lags ? md->shc_samples + 1 : md->shc_lags);
             const int chunks = (n + kShcChunk - 1) / kShcChunk;
@@ -846,7 +882,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
                 cudaGraphConditionalHandle cond;
                 r = cuda_fail(cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault), "handle");
                 if (r) break;
-                head(md->gcap, true, cond, s > 0);
+                head(md->gcap, true, cond, s == 0 ? steps : 0, s > 0);
                 cudaStreamCaptureStatus cs;
                 const cudaGraphNode_t* deps = nullptr;
                 size_t nd = 0;
@@ -874,7 +910,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
                         if (!r && e != cudaSuccess) r = cuda_fail(e, "end body capture");
                     }
                 }
-                if (!r) r = tail(md->gcap);
+                if (!r) r = tail(md->gcap, s - steps, md->tau <= 0.0 && s < steps - 1);
             }
             cudaGraph_t g2 = nullptr;
             const cudaError_t e = cudaStreamEndCapture(md->gcap, &g2);
@@ -907,9 +943,9 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
 
     const unsigned* gate = md->ctl + kCtlGate;
     for (int s = 0; s < n_steps; ++s) {
-        head(st, false, cudaGraphConditionalHandle{}, s > 0);
+        head(st, false, cudaGraphConditionalHandle{}, 1, s > 0);
         if ((rc = rebuild(st, gate))) return rc;
-        if ((rc = tail(st))) return rc;
+        if ((rc = tail(st, -1, false))) return rc;
     }
     return NEP_OK;
 }

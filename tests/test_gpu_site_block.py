@@ -274,3 +274,35 @@ def test_driven_step_sums(n):
     assert v.sum(dim=1).abs().max().item() <= n * 3 * dt * 10 * 2.0 ** -24 / (mass * unit)
     md.close()
     model.close()
+
+
+@pytest.mark.parametrize("n,drive", [(512, False), (512, True), (38913, False)])
+def test_step_sums_inside_the_next_kick(n, drive):
+    """The sums of a step are added up by the next step's first kernel where one
+    follows in the same graph and by a kernel of their own where none does: the
+    rows, J and states of one run of 12 steps (graphs of five, five, one and one)
+    have the bits of twelve runs of one step (the same order of sums)."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(n)
+    pos, box = inputs.diamond(17, 17, 17) if n > 1000 else inputs.diamond(4, 4, 4)
+    pos = inputs.displace(pos, 0.1, rng)[:n]
+    vel = rng.normal(0.0, 1e-3, (n, 3))
+    model = nep.NEP(inputs.random_z(1021, rng))
+    got = []
+    for chunk in (12, 1):
+        md = nep.MD(model, n, box, 28.085)
+        if drive:
+            md.set_hnemd([1e-4, 0.0, -2e-4])
+        x, v = soa(pos), soa(vel)
+        thermo = torch.zeros((12, 8), dtype=torch.float64, device="cuda")
+        heat = torch.zeros((12, 3), dtype=torch.float64, device="cuda")
+        for s in range(0, 12, chunk):
+            md.step(x, v, chunk, 1.0, thermo=thermo[s:s + chunk], heat=heat[s:s + chunk])
+        torch.cuda.synchronize()
+        got.append((x, v, thermo, heat))
+        md.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    assert got[0][2][:, 1].min().item() > 0.0 and got[0][3].abs().min().item() > 0.0
+    model.close()
