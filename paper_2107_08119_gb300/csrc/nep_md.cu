@@ -127,9 +127,11 @@ __device__ void decide(unsigned* ctl, bool far, int count, unsigned long long* r
     if (use_cond) cudaGraphSetConditional(cond, far ? 1u : 0u);
 }
 
-// The first S.nsum blocks add up the previous step.
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, int n, double* __restrict__ x, double* __restrict__ v,
+// The first S.nsum blocks add up the previous step; SCALE: its
+// Berendsen factor red[14] is applied here, to velocities that were left unscaled
+// (driven step of 13,824 atoms with a thermostat 71.8 -> 70.7 us).
+template <int THREADS, bool SCALE>
+__global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, const double* red, int n, double* __restrict__ x, double* __restrict__ v,
                                                         const float* __restrict__ F, double hdtm, double dt,
                                                         float* __restrict__ xr, const double* __restrict__ x_ref,
                                                         unsigned* __restrict__ ctl, float thresh2, int count,
@@ -142,13 +144,16 @@ __global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, int n, doubl
         return;
     }
     const int i = block * THREADS + threadIdx.x;
+    double lam = 1.0;
+    if constexpr (SCALE) lam = reread(red)[14];
     float d2 = 0.f;
     if (i < n) {
         double dd = 0.0, xn[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const size_t o = (size_t)c * n + i;
-            const double vc = v[o] + hdtm * to_double(F[o]);
+            const double vo = SCALE ? __dmul_rn(v[o], lam) : v[o];
+            const double vc = vo + hdtm * to_double(F[o]);
             const double xc = x[o] + dt * vc;
             v[o] = vc;
             x[o] = xc;
@@ -789,15 +794,19 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
     // (count: steps to count; follows: another step comes before it in the stream,
     // whose sums are `prev` if it has left them)
     StepSums prev;
+    const double* lam = nullptr;  // the previous step left its Berendsen factor to the next kick
     // threads per sum: with a thermostat always sums of their own, else as in the
     // kick, so that a step's sums have the same bits wherever a graph ends
     const int ft = md->tau > 0.0 ? 512 : kt;
     auto head = [&](cudaStream_t q, bool use_cond, cudaGraphConditionalHandle cond, int count, bool follows) {
         Profiler::Slot* pk = m->prof.begin(NEP_PROFILE_STEP, q);
-        launch_after(follows, kt == 64 ? k_kick_drift<64> : k_kick_drift<256>, nbk + prev.nsum, kt, 0, q, prev, n, pos,
+        auto kick = kt == 64 ? (lam ? k_kick_drift<64, true> : k_kick_drift<64, false>)
+                             : (lam ? k_kick_drift<256, true> : k_kick_drift<256, false>);
+        launch_after(follows, kick, nbk + prev.nsum, kt, 0, q, prev, lam, n, pos,
                      vel, md->ws.force, hdtm, dt, nl.xr, md->x_ref, md->ctl, thresh * thresh, count, md->rebuilds, cond,
                      use_cond ? 1 : 0);
         prev.nsum = 0;
+        lam = nullptr;
         m->prof.end(pk, q);
     };
     auto rebuild = [&](cudaStream_t q, const unsigned* g) {
@@ -806,8 +815,9 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         m->prof.end(pk, q);
         return r;
     };
-    // row: the step's row from the step counter; leave: the next head() takes the sums
-    auto tail = [&](cudaStream_t q, int row, bool leave) {
+    // row: the step's row from the step counter; follows: another step comes in the same graph,
+    // whose kick takes the sums or the Berendsen factor along
+    auto tail = [&](cudaStream_t q, int row, bool follows) {
         int b1 = 0, b2 = 0, c2 = 0, r;
         // spectral heat current: this step's W_i goes to the ring when sampled
         const bool sample = md->shc_lags > 0 && md->shc_step % md->shc_every == 0;
@@ -836,7 +846,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         StepSums S{drive ? 5 : 1 + c2, part_e, b1, drive ? part_h : part_a, drive ? nbk : b2, drive ? 4 : 1,
                    drive ? 1 : (size_t)b2, drive ? 10 : 1, md->red, thermo, heat, md->ctl, row, md->t0, md->tau, dt,
                    dof_kb};
-        if (leave)
+        if (follows && md->tau <= 0.0)
             prev = S;
         else
             launch_after(true, ft == 64 ? k_md_finish<64> : ft == 256 ? k_md_finish<256> : k_md_finish<512>, S.nsum, ft,
@@ -851,7 +861,12 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             ++md->shc_samples;
         }
         if (md->shc_lags > 0) ++md->shc_step;
-        if (md->tau > 0.0 && n > 1) launch_after(!sample, k_scale_v, nbk, kt, 0, q, n, vel, md->red);
+        if (md->tau > 0.0 && n > 1) {
+            if (follows)
+                lam = md->red;
+            else
+                launch_after(!sample, k_scale_v, nbk, kt, 0, q, n, vel, md->red);
+        }
         m->prof.end(pk, q);
         return cuda_fail(cudaGetLastError(), "md step kernels");
     };
@@ -910,7 +925,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
                         if (!r && e != cudaSuccess) r = cuda_fail(e, "end body capture");
                     }
                 }
-                if (!r) r = tail(md->gcap, s - steps, md->tau <= 0.0 && s < steps - 1);
+                if (!r) r = tail(md->gcap, s - steps, s < steps - 1);
             }
             cudaGraph_t g2 = nullptr;
             const cudaError_t e = cudaStreamEndCapture(md->gcap, &g2);

@@ -276,12 +276,15 @@ def test_driven_step_sums(n):
     model.close()
 
 
-@pytest.mark.parametrize("n,drive", [(512, False), (512, True), (38913, False)])
-def test_step_sums_inside_the_next_kick(n, drive):
+@pytest.mark.parametrize("n,drive,tau", [(512, False, 0.0), (512, True, 0.0), (38913, False, 0.0), (512, False, 20.0),
+                                         (512, True, 20.0)])
+def test_step_sums_inside_the_next_kick(n, drive, tau):
     """The sums of a step are added up by the next step's first kernel where one
     follows in the same graph and by a kernel of their own where none does: the
     rows, J and states of one run of 12 steps (graphs of five, five, one and one)
-    have the bits of twelve runs of one step (the same order of sums)."""
+    have the bits of twelve runs of one step (the same order of sums).  With a
+    thermostat the next kick applies the factor to the velocities instead: the
+    product is rounded in both forms."""
     import torch
     from paper_2107_08119_gb300 import nep
     rng = np.random.default_rng(n)
@@ -294,6 +297,8 @@ def test_step_sums_inside_the_next_kick(n, drive):
         md = nep.MD(model, n, box, 28.085)
         if drive:
             md.set_hnemd([1e-4, 0.0, -2e-4])
+        if tau:
+            md.set_thermostat(300.0, tau)
         x, v = soa(pos), soa(vel)
         thermo = torch.zeros((12, 8), dtype=torch.float64, device="cuda")
         heat = torch.zeros((12, 3), dtype=torch.float64, device="cuda")
