@@ -187,16 +187,12 @@ int ensure_workspace(Workspace& ws, int n, int m_cap, int ncell, int nblocks_par
     if (ncell + 1 > nl.ncell_cap) {
         dev_free(nl.cell_count);
         dev_free(nl.cell_start);
-        dev_free(nl.cell_fill);
         nl.ncell_cap = 0;
         const size_t C = (size_t)ncell + 1;
-        if ((rc = dev_alloc(&nl.cell_count, C, "cell counts")) || (rc = dev_alloc(&nl.cell_start, C, "cell offsets")) ||
-            (rc = dev_alloc(&nl.cell_fill, C, "cell fill")))
+        if ((rc = dev_alloc(&nl.cell_count, C, "cell counts")) || (rc = dev_alloc(&nl.cell_start, C, "cell offsets")))
             return rc;
-        // the builder keeps both arrays zero between builds
-        if ((rc = cuda_fail(cudaMemset(nl.cell_count, 0, C * sizeof(int)), "cudaMemset")) ||
-            (rc = cuda_fail(cudaMemset(nl.cell_fill, 0, C * sizeof(int)), "cudaMemset")))
-            return rc;
+        // the builder keeps the counts zero between builds
+        if ((rc = cuda_fail(cudaMemset(nl.cell_count, 0, C * sizeof(int)), "cudaMemset"))) return rc;
         nl.ncell_cap = (int)C;
     }
     const int need_partials = 16 * (nblocks_partials + 8);
@@ -221,7 +217,6 @@ void free_workspace(Workspace& ws)
     dev_free(nl.atom_cell);
     dev_free(nl.cell_count);
     dev_free(nl.cell_start);
-    dev_free(nl.cell_fill);
     dev_free(nl.xs);
     dev_free(nl.mask);
     dev_free(ws.partials);

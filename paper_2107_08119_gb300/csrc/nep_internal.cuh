@@ -413,7 +413,6 @@ struct NeighborList {
     int* atom_cell = nullptr;
     int* cell_count = nullptr;
     int* cell_start = nullptr;
-    int* cell_fill = nullptr;
     float4* xs = nullptr;    // hi parts and indices in cell order [n]
     // [3][n] words: bit k of atom i set when slot k lies within the cutoff,
     // written by the site pass from its cutoff tests; `mask_set`

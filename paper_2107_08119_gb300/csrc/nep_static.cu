@@ -42,8 +42,7 @@ constexpr size_t kOffAtomCell = kOffXr + align256(sizeof(float) * kStaticAtoms *
 constexpr size_t kOffCellAtoms = kOffAtomCell + align256(sizeof(int) * kStaticAtoms);
 constexpr size_t kOffCellCount = kOffCellAtoms + align256(sizeof(float4) * kStaticAtoms);
 constexpr size_t kOffCellStart = kOffCellCount + align256(sizeof(int) * (kStaticCells + 1));
-constexpr size_t kOffCellFill = kOffCellStart + align256(sizeof(int) * (kStaticCells + 1));
-constexpr size_t kOffMask = kOffCellFill + align256(sizeof(int) * (kStaticCells + 1));
+constexpr size_t kOffMask = kOffCellStart + align256(sizeof(int) * (kStaticCells + 1));
 constexpr size_t kOffPartials = kOffMask + align256(sizeof(unsigned) * 3 * kStaticAtoms);
 constexpr size_t kOffErr = kOffPartials + align256(sizeof(double) * 16 * (kStaticBlocks + 8));
 constexpr size_t kStaticBytes = kOffErr + align256(sizeof(unsigned));
@@ -183,7 +182,6 @@ extern "C" int nep_compute_efv_static(const nep_hyper* hp, const float* z, int n
     nl.xs = reinterpret_cast<float4*>(base + kOffCellAtoms);
     nl.cell_count = reinterpret_cast<int*>(base + kOffCellCount);
     nl.cell_start = reinterpret_cast<int*>(base + kOffCellStart);
-    nl.cell_fill = reinterpret_cast<int*>(base + kOffCellFill);
     nl.mask = reinterpret_cast<unsigned*>(base + kOffMask);
     double* partials = reinterpret_cast<double*>(base + kOffPartials);
     unsigned* err = reinterpret_cast<unsigned*>(base + kOffErr);
@@ -192,8 +190,7 @@ extern "C" int nep_compute_efv_static(const nep_hyper* hp, const float* z, int n
     // (the build leaves them zero, but not when a call failed between launches)
     if ((rc = cuda_fail(cudaMemsetAsync(err, 0, sizeof(unsigned), st), "cudaMemsetAsync"))) return rc;
     if (ncell > 0 && !list_is_direct(n) &&
-        ((rc = cuda_fail(cudaMemsetAsync(nl.cell_count, 0, sizeof(int) * (ncell + 1), st), "cudaMemsetAsync")) ||
-         (rc = cuda_fail(cudaMemsetAsync(nl.cell_fill, 0, sizeof(int) * (ncell + 1), st), "cudaMemsetAsync"))))
+        (rc = cuda_fail(cudaMemsetAsync(nl.cell_count, 0, sizeof(int) * (ncell + 1), st), "cudaMemsetAsync")))
         return rc;
 
     if ((rc = build_neighbor_list(nl, box, n, const_cast<double*>(pos), nullptr, false, nullptr, (float)rmax, err, nullptr,

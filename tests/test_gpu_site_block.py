@@ -311,3 +311,30 @@ def test_step_sums_inside_the_next_kick(n, drive, tau):
         assert torch.equal(a, b)
     assert got[0][2][:, 1].min().item() > 0.0 and got[0][3].abs().min().item() > 0.0
     model.close()
+
+
+@pytest.mark.parametrize("nc", [(32, 16, 16), (33, 16, 16), (48, 32, 16), (110, 110, 110)])
+def test_cell_offsets_by_slices(orc, nc):
+    """Cell offsets scanned in slices of 8192 cells (one, one and a rest, three,
+    and with 1.3 million cells two rounds per slice): 1500 pairs of atoms spread
+    over the box find their partners, twice (the counts are zero after a build)."""
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(sum(nc))
+    L = 5.0 * np.array(nc) + 0.5
+    m = np.array([20, 10, 10])
+    g = np.stack(np.meshgrid(*[np.arange(k) for k in m], indexing="ij"), -1).reshape(-1, 3)
+    a = (g[rng.permutation(len(g))[:1500]] + 0.5) * (L / m)  # centres at least 8 A apart
+    d = rng.normal(size=(1500, 3))
+    d *= (rng.uniform(1.0, 1.25, 1500) / np.linalg.norm(d, axis=1))[:, None]
+    pos, box = np.concatenate([a - d, a + d]), np.diag(L)
+    z = inputs.random_z(1021, rng)
+    model = nep.NEP(z)
+    idx = np.unique(rng.integers(0, 3000, 100))
+    U, F, _ = orc.efv_sample(orc.NepHyper(), f32_exact(z), pos, box, idx)
+    for _ in range(2):
+        out = model.compute(soa(pos), box)
+        cnt, _ = model.neighbors(3000)
+        assert int(cnt.min()) >= 1
+        assert np.abs(out["e_atom"].cpu().numpy()[idx] - U).max() <= 1e-6
+        assert np.abs(aos(out["force"])[idx] - F).max() <= 1e-4
+    model.close()
