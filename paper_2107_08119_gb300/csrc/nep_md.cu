@@ -12,7 +12,9 @@
 //   k_assemble     forces, second half kick, E_kin, virial and heat current
 //                  J = sum_i W_i . v_i (Eq. 7), per-block FP64 sums
 //   k_md_finish    block sums in a fixed order (one block per sum), thermo
-//                  row and J of this step, Berendsen factor
+//                  row and J of this step, Berendsen factor; where another
+//                  step of the same graph follows, its k_kick_drift does the
+//                  sums instead, or with a thermostat the scaling
 // Optional extensions (nep_md_set_thermostat, nep_md_set_hnemd):
 //   HNEMD          the assembly writes F and W_i; after the virial sum,
 //                  k_hnemd_kick adds F_i^ext = F_e . W_i - F_e . W / N
