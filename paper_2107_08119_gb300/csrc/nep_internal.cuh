@@ -4,7 +4,8 @@
 //   positions        FP64 [3][n] (caller) + FP32 hi/lo records xr [n][8]
 //   neighbour list   int32 nbr[M][n] = j | image_code << 24, count[n]
 //                    int32 rev[M][n] = slot of i in j's list (reverse pair)
-//                    int32 vala[n][M]: direct list, the list values atom-major; cells path, the rank of each unsorted slot
+//                    int32 vala[n][M]: direct list, the list values atom-major;
+//                    cells path, the rank of each unsorted slot
 //   partial forces   FP32 pf[M][n] float4 (x, y, z, unused) = dU_i/dr_ij
 //                    (Eq. 23), slot-major: one 16-byte gather per reverse pair
 //   forces           FP32 [3][n], per-atom virials FP32 [9][n]
@@ -213,7 +214,7 @@ __host__ __device__ __forceinline__ void split_hilo(double x, float& h, float& l
 // (float)x and its value as a double by integer operations (round to nearest
 // even): conversions from and to FP64 run at the rate of the FP64 pipe, two
 // lanes per clock and SM, and bounded the kernels that split positions
-// (k_kick_drift at 829,440 atoms 51.9 -> 45.6 us, k_bin 35.1 -> 29.2).  In the
+// (k_kick_drift at 921,600 atoms 51.9 -> 45.6 us, k_bin 35.1 -> 29.2).  In the
 // assembly, which waits for gathers, the same changed nothing.
 __device__ __forceinline__ float to_float(double x, double& back)
 {
