@@ -27,13 +27,13 @@ constexpr int kMaskSlots = 96;  // slots per atom covered by the in-cutoff mask 
 // D: descriptor sizes of the model (DescSi: 32 descriptors, DescPbTe: 41).
 // AT: atoms per block.  WORDS: 32-bit words of own-slot bits per thread.
 template <class D, int AT, int WORDS>
-__global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, const int* __restrict__ count,
-                                                          const int* __restrict__ nbr, const float* __restrict__ xr,
-                                                          Box box, const float* __restrict__ z, int n_par,
-                                                          SiteParams P, float* __restrict__ pf,
-                                                          double* __restrict__ e_atom,
-                                                          double* __restrict__ e_partials, unsigned* err,
-                                                          unsigned* __restrict__ mask)
+__global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, const int* count,
+                                                          const int* nbr, const float* xr,
+                                                          Box box, const float* z, int n_par,
+                                                          SiteParams P, float* pf,
+                                                          double* e_atom,
+                                                          double* e_partials, unsigned* err,
+                                                          unsigned* mask)
 {
     const int block = block_after();
     const int lane = threadIdx.x & 31;
@@ -70,14 +70,14 @@ __global__ void __launch_bounds__(kSiteThreads, 5) k_site(int n, int m_cap, cons
 // Four entries per thread (16 warps per SM): 66 us at 125000, 89 at 64000 of
 // the split model; one entry: 50 and 78.
 template <bool MD, int AT>
-__global__ void __launch_bounds__(kAsmThreads, 8) k_assemble(int n, int m_cap, float rc2max, const int* __restrict__ count,
-                                                          const int* __restrict__ nbr, const int* __restrict__ rev,
-                                                          const float* __restrict__ xr, Box box,
-                                                          const float* __restrict__ pf, float* __restrict__ force,
-                                                          float* __restrict__ virial_atom,
-                                                          double* __restrict__ partials, unsigned* err,
-                                                          double* __restrict__ vel, double hdtm, double kef,
-                                                          const unsigned* __restrict__ mask)
+__global__ void __launch_bounds__(kAsmThreads, 8) k_assemble(int n, int m_cap, float rc2max, const int* count,
+                                                          const int* nbr, const int* rev,
+                                                          const float* xr, Box box,
+                                                          const float* pf, float* force,
+                                                          float* virial_atom,
+                                                          double* partials, unsigned* err,
+                                                          double* vel, double hdtm, double kef,
+                                                          const unsigned* mask)
 {
     constexpr int WAYS = kAsmThreads / AT;       // threads per atom
     constexpr int CH = WAYS * kAsmPer;           // slots per tile
@@ -137,8 +137,8 @@ __global__ void __launch_bounds__(kAsmThreads, 8) k_assemble(int n, int m_cap, f
             if (v[u] >= 0) {
                 const int j = v[u] & 0xFFFFFF;
                 load_pos(xr, j, hj[u], lj[u]);
-                pq[u] = NEP_LDG(pf4 + (size_t)kr[u] * n + j);
-                po[u] = NEP_LDG(pf4 + (size_t)(k0 + WAYS * u + way) * n + ia);
+                pq[u] = pf4[(size_t)kr[u] * n + j];
+                po[u] = pf4[(size_t)(k0 + WAYS * u + way) * n + ia];
             }
         }
         load_idx(k0 + CH);
@@ -243,14 +243,14 @@ __global__ void __launch_bounds__(kAsmThreads, 8) k_assemble(int n, int m_cap, f
 // The same with one thread per atom: no tile and no barriers, so it wins once
 // the atoms fill the GPU and their lists are short (asm_by_atoms below).
 template <bool MD>
-__global__ void __launch_bounds__(kAsmThreads) k_assemble_atoms(int n, int m_cap, float rc2max, const int* __restrict__ count,
-                                                          const int* __restrict__ nbr, const int* __restrict__ rev,
-                                                          const float* __restrict__ xr,
-                                                          Box box, const float* __restrict__ pf,
-                                                          float* __restrict__ force, float* __restrict__ virial_atom,
-                                                          double* __restrict__ partials, unsigned* err,
-                                                          double* __restrict__ vel, double hdtm, double kef,
-                                                          const unsigned* __restrict__ mask)
+__global__ void __launch_bounds__(kAsmThreads) k_assemble_atoms(int n, int m_cap, float rc2max, const int* count,
+                                                          const int* nbr, const int* rev,
+                                                          const float* xr,
+                                                          Box box, const float* pf,
+                                                          float* force, float* virial_atom,
+                                                          double* partials, unsigned* err,
+                                                          double* vel, double hdtm, double kef,
+                                                          const unsigned* mask)
 {
     constexpr int K = MD ? 13 : 9;
     const int block = block_after();
@@ -264,6 +264,10 @@ __global__ void __launch_bounds__(kAsmThreads) k_assemble_atoms(int n, int m_cap
         const SlotTable T{nbr, n, i};
         float F[3], W[9];
         assemble_atom(i, n, m_cap, rc2max, count, T, rev, xr, box, pf, F, W, mask);
+        double v[3];  // loaded ahead of the stores
+        if constexpr (MD)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[c] = vel[(size_t)c * n + i];
         if (!(isfinite(F[0]) && isfinite(F[1]) && isfinite(F[2]))) atomicOr(err, kErrNonFinite);
         if (force) {
             force[i] = F[0];
@@ -276,10 +280,9 @@ __global__ void __launch_bounds__(kAsmThreads) k_assemble_atoms(int n, int m_cap
 #pragma unroll
         for (int c = 0; c < 9; ++c) acc[c] = (double)W[c];
         if constexpr (MD) {
-            double v[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                v[c] = vel[(size_t)c * n + i] + hdtm * (double)F[c];
+                v[c] += hdtm * (double)F[c];
                 vel[(size_t)c * n + i] = v[c];
             }
             acc[9] = kef * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);

@@ -18,12 +18,6 @@
 
 #include "nep.h"
 
-#ifdef __CUDA_ARCH__
-#define NEP_LDG(p) __ldg(p)
-#else
-#define NEP_LDG(p) (*(p))
-#endif
-
 namespace nep {
 
 __host__ __device__ __forceinline__ int imin(int a, int b) { return a < b ? a : b; }
@@ -170,13 +164,14 @@ __host__ __device__ __forceinline__ void pair_vector_lo(int code, const float (&
 // x, y, z, 0) per atom, so that a neighbour's coordinates are one sector and
 // one 32-byte load (two 16-byte arrays before: two sectors; an MD step of the
 // 125,000-atom crystal 315 -> 309 us together with the site pass loading its
-// records a slot ahead).
+// records a slot ahead).  An ordinary load in volatile assembly: it stays behind
+// the wait of a dependent kernel (block_after), as the read-only path would not.
 __host__ __device__ __forceinline__ void load_pos(const float* __restrict__ xr, int i, float (&h)[3], float (&l)[3],
                                                   float& zi)
 {
 #ifdef __CUDA_ARCH__
     float u, pad;
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(h[0]), "=f"(h[1]), "=f"(h[2]), "=f"(u), "=f"(l[0]), "=f"(l[1]), "=f"(l[2]), "=f"(pad)
         : "l"(xr + 8 * (size_t)i));
     zi = u;
@@ -201,7 +196,7 @@ __host__ __device__ __forceinline__ void load_pos(const float* __restrict__ xr, 
 // the hi part of the record (x, y, z, species number)
 __host__ __device__ __forceinline__ float4 load_hi(const float* __restrict__ xr, int i)
 {
-    return NEP_LDG(reinterpret_cast<const float4*>(xr) + 2 * (size_t)i);
+    return reinterpret_cast<const float4*>(xr)[2 * (size_t)i];
 }
 
 // Split an FP64 value into FP32 hi + lo.
@@ -366,16 +361,21 @@ __device__ __forceinline__ double sum_partials(const double* __restrict__ src, i
 // predecessor is a kernel of the same call on the same stream, not a wait for an
 // event, a copy or a conditional node.  96 atoms 92 -> 81 us per call, 125,000
 // atoms 430 -> 416, MD step of 4,096 atoms 45.0 -> 43.8 us.
-// Returns blockIdx.x, so that a kernel has no block before the wait (read in the
-// same inline assembly it was no longer known to be uniform: steps of 64,000
-// two-species atoms 2.5 % slower).
+// What orders the loads: the wait clobbers memory, so ordinary loads and stores
+// stay behind it, but a load that the compiler may take for invariant does not
+// have to.  So a kernel that calls block_after() has no __restrict__ parameter,
+// uses no read-only load (__ldg, ld.global.nc), and reaches global memory in
+// inline assembly only where that is volatile, or through a pointer that
+// reread() has passed on behind the wait.
+// Returns blockIdx.x (read in the assembly of the wait it was no longer known to
+// be uniform: steps of 64,000 two-species atoms 2.5 % slower).
 __device__ __forceinline__ int block_after()
 {
     cudaGridDependencySynchronize();
     return (int)blockIdx.x;
 }
 
-// A read-only pointer for loads that must stay behind block_after()
+// The same pointer, known only behind block_after()
 template <class T>
 __device__ __forceinline__ T* reread(T* p)
 {

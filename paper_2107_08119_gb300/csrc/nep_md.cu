@@ -133,11 +133,11 @@ __device__ void decide(unsigned* ctl, bool far, int count, unsigned long long* r
 // Berendsen factor red[14] is applied here, to velocities that were left unscaled
 // (driven step of 13,824 atoms with a thermostat 71.8 -> 70.7 us).
 template <int THREADS, bool SCALE>
-__global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, const double* red, int n, double* __restrict__ x, double* __restrict__ v,
-                                                        const float* __restrict__ F, double hdtm, double dt,
-                                                        float* __restrict__ xr, const double* __restrict__ x_ref,
-                                                        unsigned* __restrict__ ctl, float thresh2, int count,
-                                                        unsigned long long* __restrict__ rebuilds,
+__global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, const double* red, int n, double* x, double* v,
+                                                        const float* F, double hdtm, double dt,
+                                                        float* xr, const double* x_ref,
+                                                        unsigned* ctl, float thresh2, int count,
+                                                        unsigned long long* rebuilds,
                                                         cudaGraphConditionalHandle cond, int use_cond)
 {
     const int block = block_after() - S.nsum;
@@ -147,23 +147,33 @@ __global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, const double
     }
     const int i = block * THREADS + threadIdx.x;
     double lam = 1.0;
-    if constexpr (SCALE) lam = reread(red)[14];
+    if constexpr (SCALE) lam = red[14];
     float d2 = 0.f;
     if (i < n) {
-        double dd = 0.0, xn[3];
+        // all loads ahead of the stores
+        double dd = 0.0, xn[3], xo[3], vo[3], xf[3];
+        float f[3];
+        const float z = load_z(xr, i);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const size_t o = (size_t)c * n + i;
-            const double vo = SCALE ? __dmul_rn(v[o], lam) : v[o];
-            const double vc = vo + hdtm * to_double(F[o]);
-            const double xc = x[o] + dt * vc;
+            vo[c] = v[o];
+            f[c] = F[o];
+            xo[c] = x[o];
+            xf[c] = x_ref[o];
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const size_t o = (size_t)c * n + i;
+            const double vc = (SCALE ? __dmul_rn(vo[c], lam) : vo[c]) + hdtm * to_double(f[c]);
+            const double xc = xo[c] + dt * vc;
             v[o] = vc;
             x[o] = xc;
             xn[c] = xc;
-            const double d = xc - x_ref[o];
+            const double d = xc - xf[c];
             dd += d * d;
         }
-        store_pos(xr, i, xn, load_z(xr, i));  // the species number stays
+        store_pos(xr, i, xn, z);  // the species number stays
         d2 = (float)dd;
     }
     // the blocks with an atom beyond the threshold (high half) and those that
@@ -181,9 +191,9 @@ __global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, const double
 
 // Second half kick with the HNEMD driving force, E_kin and J per block.
 // W is the per-atom virial [9][n]; wtot the total virial (row-major).
-__global__ void k_hnemd_kick(int n, float* __restrict__ F, const float* __restrict__ W, double* __restrict__ vel,
-                             double fe0, double fe1, double fe2, const double* __restrict__ wtot, double inv_n,
-                             double hdtm, double kef, double* __restrict__ partials, unsigned* err)
+__global__ void k_hnemd_kick(int n, float* F, const float* W, double* vel,
+                             double fe0, double fe1, double fe2, const double* wtot, double inv_n,
+                             double hdtm, double kef, double* partials, unsigned* err)
 {
     const int i = block_after() * blockDim.x + threadIdx.x;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -192,7 +202,7 @@ __global__ void k_hnemd_kick(int n, float* __restrict__ F, const float* __restri
     if (threadIdx.x < 3) {
         double fm = 0.0;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) fm += fe[a] * reread(wtot)[3 * a + threadIdx.x];
+        for (int a = 0; a < 3; ++a) fm += fe[a] * wtot[3 * a + threadIdx.x];
         s_fm[threadIdx.x] = fm;
     }
     __syncthreads();
@@ -201,15 +211,21 @@ __global__ void k_hnemd_kick(int n, float* __restrict__ F, const float* __restri
 #pragma unroll
         for (int c = 0; c < 9; ++c) w[c] = W[(size_t)c * n + i];
         double v[3];
+        float f[3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {  // loaded ahead of the stores
+            f[b] = F[(size_t)b * n + i];
+            v[b] = vel[(size_t)b * n + i];
+        }
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
             const double fm = s_fm[b];
             double fx = 0.0;
 #pragma unroll
             for (int a = 0; a < 3; ++a) fx += fe[a] * (double)w[3 * a + b];
-            const float ft = (float)((double)F[(size_t)b * n + i] + fx - fm * inv_n);
+            const float ft = (float)((double)f[b] + fx - fm * inv_n);
             F[(size_t)b * n + i] = ft;
-            v[b] = vel[(size_t)b * n + i] + hdtm * (double)ft;
+            v[b] += hdtm * (double)ft;
             vel[(size_t)b * n + i] = v[b];
         }
         if (!isfinite(v[0] + v[1] + v[2])) atomicOr(err, kErrNonFinite);
@@ -362,13 +378,16 @@ __global__ void __launch_bounds__(kKappaThreads) k_hnemd_kappa(int n, const doub
 }
 
 // v *= lambda (the Berendsen factor k_md_finish left in red[14])
-__global__ void k_scale_v(int n, double* __restrict__ vel, const double* __restrict__ red)
+__global__ void k_scale_v(int n, double* vel, const double* red)
 {
     const int i = block_after() * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double lam = reread(red)[14];
+    const double lam = red[14];
+    double v[3];  // loaded ahead of the stores
 #pragma unroll
-    for (int c = 0; c < 3; ++c) vel[(size_t)c * n + i] *= lam;
+    for (int c = 0; c < 3; ++c) v[c] = vel[(size_t)c * n + i];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) vel[(size_t)c * n + i] = v[c] * lam;
 }
 
 inline int blocks_for(int n, int t) { return (n + t - 1) / t; }

@@ -102,11 +102,10 @@ constexpr int kScanRound = kScanThreads * kScanPer;
 
 __device__ __forceinline__ int scan_pad(int x) { return x + (x >> 5); }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan(int ncell, int slice, const int* __restrict__ count,
-                                                       int* __restrict__ start, const unsigned* gate)
+__global__ void __launch_bounds__(kScanThreads) k_scan(int ncell, int slice, const int* count,
+                                                       int* start, const unsigned* gate)
 {
     const int c0 = block_after() * slice, c1 = min(ncell, c0 + slice);
-    count = reread(count);
     if (gated_off(gate)) return;
     __shared__ int sc[kScanRound + kScanRound / 32];
     __shared__ int wsum[kScanThreads / 32];
@@ -180,8 +179,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(int ncell, int slice, con
 // Atoms in cell order: their hi parts with the index in the fourth word, so
 // that a cell's candidates are contiguous 16-byte reads.  Counts down the cells'
 // counters, which are zero again after it.
-__global__ void k_scatter(int n, const int* __restrict__ atom_cell, const int* __restrict__ cell_start,
-                          int* __restrict__ cell_count, const float* __restrict__ xr, float4* __restrict__ xs,
+__global__ void k_scatter(int n, const int* atom_cell, const int* cell_start,
+                          int* cell_count, const float* xr, float4* xs,
                           const unsigned* gate)
 {
     const int block = block_after();
@@ -326,13 +325,13 @@ __device__ __forceinline__ void half_cell(int cell, int m_cap, float rv2, int ca
         for (int e = threadIdx.x; e < m; e += 32 * WARPS) {
             int r = 0;
             while (s_at[r + 1] <= f0 + e) ++r;
-            const float4 h = NEP_LDG(xs + s_r0[r] + f0 + e);
+            const float4 h = xs[s_r0[r] + f0 + e];
             s_cand[e] = make_float4((h.x - ox) + s_shift[r][0], (h.y - oy) + s_shift[r][1], (h.z - oz) + s_shift[r][2],
                                     __int_as_float(__float_as_int(h.w) | s_code[r]));
         }
         __syncthreads();
         for (int c = c0 + warp; c < c1; c += WARPS) {
-            const float4 me = NEP_LDG(xs + c);
+            const float4 me = xs[c];
             const int i = __float_as_int(me.w);
             const float hx = me.x - ox, hy = me.y - oy, hz = me.z - oz;
             float hi[3], li[3];
@@ -408,10 +407,10 @@ __device__ __forceinline__ void half_cell(int cell, int m_cap, float rv2, int ca
 // (One form for both spilled registers.)
 template <int WARPS, bool GATED>
 __global__ void __launch_bounds__(32 * WARPS) k_half_cells(int ncell, int m_cap, float rv2, int cap,
-                                                          const float* __restrict__ xr,
-                                                          const float4* __restrict__ xs,
-                                                          const int* __restrict__ cell_start,
-                                                          int* __restrict__ count, int* __restrict__ rows, Box b,
+                                                          const float* xr,
+                                                          const float4* xs,
+                                                          const int* cell_start,
+                                                          int* count, int* rows, Box b,
                                                           const unsigned* gate)
 {
     const int block = block_after();
@@ -478,9 +477,9 @@ __device__ __forceinline__ void rank_rows_write(int c0, int ns, int m, int lane,
     }
 }
 
-__global__ void __launch_bounds__(32 * kVerletWarps) k_sort_rows(int n, int m_cap, int lcap, int* __restrict__ rows,
-                                                                const int* __restrict__ count, int* __restrict__ nbr,
-                                                                int* __restrict__ inv, unsigned* err,
+__global__ void __launch_bounds__(32 * kVerletWarps) k_sort_rows(int n, int m_cap, int lcap, int* rows,
+                                                                const int* count, int* nbr,
+                                                                int* inv, unsigned* err,
                                                                 const unsigned* gate)
 {
     const int block = block_after();
@@ -549,9 +548,9 @@ constexpr int kSortAtoms = 32;
 constexpr int kSortGridCap = 152 * 8;
 constexpr size_t kSortTileMaxSmem = 48 * 1024;  // up to 128 slots per atom (the warp-per-atom sort beyond)
 
-__global__ void __launch_bounds__(32 * kSortWarps) k_sort_tile(int n, int m_cap, int lcap, int* __restrict__ rows,
-                                                              const int* __restrict__ count, int* __restrict__ nbr,
-                                                              int* __restrict__ inv, unsigned* err,
+__global__ void __launch_bounds__(32 * kSortWarps) k_sort_tile(int n, int m_cap, int lcap, int* rows,
+                                                              const int* count, int* nbr,
+                                                              int* inv, unsigned* err,
                                                               const unsigned* gate)
 {
     const int block = block_after();
@@ -635,8 +634,8 @@ __global__ void __launch_bounds__(32 * kSortWarps) k_sort_tile(int n, int m_cap,
 // unsorted slot s by the partner's sort; one warp per atom.  A value outside
 // the partner's kept entries (only after an overflow, already latched) is
 // latched again and replaced by the slot's own rank.
-__global__ void k_rev_perm(int n, int m_cap, const int* __restrict__ count, const int* __restrict__ rows,
-                           const int* __restrict__ inv, int* __restrict__ rev, unsigned* err, const unsigned* gate)
+__global__ void k_rev_perm(int n, int m_cap, const int* count, const int* rows,
+                           const int* inv, int* rev, unsigned* err, const unsigned* gate)
 {
     const int block = block_after();
     if (gated_off(gate)) return;
@@ -667,9 +666,9 @@ constexpr int kRevThreads = 256;
 constexpr int kRevTileMaxSlots = 352;  // 352 x 33 x 4 bytes stay under 48 KB
 constexpr int kRevGridCap = 152 * 8;   // blocks walk the 32-atom tiles; a gated-off launch retires fast
 
-__global__ void __launch_bounds__(kRevThreads) k_rev_tile(int n, int m_cap, const int* __restrict__ count,
-                                                          const int* __restrict__ rows, const int* __restrict__ inv,
-                                                          int* __restrict__ rev, unsigned* err, const unsigned* gate)
+__global__ void __launch_bounds__(kRevThreads) k_rev_tile(int n, int m_cap, const int* count,
+                                                          const int* rows, const int* inv,
+                                                          int* rev, unsigned* err, const unsigned* gate)
 {
     const int block = block_after();
     if (gated_off(gate)) return;
@@ -725,9 +724,9 @@ constexpr int kDirectAtoms = 2;
 
 template <bool IMAGES>
 __global__ void __launch_bounds__(kDirectThreads) k_list_direct(int n, int m_cap, float rv2,
-                                                               const float* __restrict__ xr, int* __restrict__ count,
-                                                               int* __restrict__ nbr, float* __restrict__ key,
-                                                               int* __restrict__ vala, unsigned* err, Box b,
+                                                               const float* xr, int* count,
+                                                               int* nbr, float* key,
+                                                               int* vala, unsigned* err, Box b,
                                                                const unsigned* gate)
 {
     const int block = block_after();
@@ -826,8 +825,8 @@ __global__ void __launch_bounds__(kDirectThreads) k_list_direct(int n, int m_cap
 // overflow) is latched as an error.  One warp per atom, a lane per slot; the
 // keys and values are read from their atom-major copies, so every search
 // stays inside one atom's contiguous row.
-__global__ void k_reverse(int n, int m_cap, const int* __restrict__ count, const float* __restrict__ key,
-                          const int* __restrict__ vala, int* __restrict__ rev, unsigned* err, const unsigned* gate)
+__global__ void k_reverse(int n, int m_cap, const int* count, const float* key,
+                          const int* vala, int* rev, unsigned* err, const unsigned* gate)
 {
     const int block = block_after();
     if (gated_off(gate)) return;

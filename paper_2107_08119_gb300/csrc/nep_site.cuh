@@ -528,7 +528,7 @@ __host__ __device__ __forceinline__ void assemble_atom(int i, int n, int m_cap, 
     auto load_idx = [&](int k, int& v, int& kr) {
         if (k < cnt && kept(k)) {
             v = nbr.slots[(size_t)k * nbr.stride + nbr.idx];
-            kr = NEP_LDG(rev + (size_t)k * n + i);
+            kr = rev[(size_t)k * n + i];
         }
     };
     // the gathers of slot k, given its list value and reverse slot
@@ -537,8 +537,8 @@ __host__ __device__ __forceinline__ void assemble_atom(int i, int n, int m_cap, 
             const int j = v & 0xFFFFFF;
             d.v = v;
             load_pos(xr, j, d.h, d.l);
-            d.po = NEP_LDG(pf4 + (size_t)k * n + i);
-            d.pq = NEP_LDG(pf4 + (size_t)kr * n + j);
+            d.po = pf4[(size_t)k * n + i];
+            d.pq = pf4[(size_t)kr * n + j];
         }
     };
     int v1 = 0, kr1 = 0, v2 = 0, kr2 = 0;

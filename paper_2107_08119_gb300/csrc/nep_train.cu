@@ -535,10 +535,10 @@ constexpr int kOwnerStage = kOwnerChunk * (kRecFloats + kAngFloats);  // floats 
 
 template <class PT>
 __global__ void __launch_bounds__(kOwnerMaxThreads) k_contract_owner(
-    int j0, int j1, int P, int Pst, const PT* __restrict__ G, const float* __restrict__ B,
-    const long long* __restrict__ pstart, const long long* __restrict__ rev, const PairRec* __restrict__ rec,
-    const long long* __restrict__ aidx, const float* __restrict__ ang, PT* __restrict__ pbuf,
-    float* __restrict__ w6out, float* __restrict__ fown)
+    int j0, int j1, int P, int Pst, const PT* G, const float* B,
+    const long long* pstart, const long long* rev, const PairRec* rec,
+    const long long* aidx, const float* ang, PT* pbuf,
+    float* w6out, float* fown)
 {
     extern __shared__ float4 s_stage4[];
     const int block = block_after();
@@ -671,14 +671,16 @@ __global__ void __launch_bounds__(kOwnerMaxThreads) k_contract_owner(
 // with a neighbouring atom's slots are left alone.
 template <int UNROLL, class PT>
 __global__ void __launch_bounds__(kReceiverThreads, 2) k_contract(
-    int c0, int discard, int P, int Pst, const int* __restrict__ chunk_begin, const int* __restrict__ chunk_end,
-    const double* __restrict__ U, const long long* __restrict__ pstart, const float* __restrict__ fown,
-    const PT* __restrict__ pbuf, const float* __restrict__ w6in, const float* __restrict__ f_tar,
-    double* __restrict__ partials)
+    int c0, int discard, int P, int Pst, const int* chunk_begin, const int* chunk_end,
+    const double* U, const long long* pstart, const float* fown,
+    const PT* pbuf, const float* w6in, const float* f_tar,
+    double* partials)
 {
     constexpr int kWarps = kReceiverThreads / 32;
     __shared__ RecvRed<kWarps> red;
     const int c = c0 + (int)(gridDim.x - 1 - block_after());  // last chunk first (as k_contract_bulk)
+    fown = reread(fown);  // read by recv_load
+    w6in = reread(w6in);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k0 = 2 * lane;
     const bool on0 = k0 < P, on1 = k0 + 1 < P;
@@ -724,16 +726,18 @@ constexpr int kRecvStage = 16;
 
 template <class PT>
 __global__ void __launch_bounds__(kReceiverThreads, 2) k_contract_staged(
-    int c0, int discard, int P, int Pst, const int* __restrict__ chunk_begin, const int* __restrict__ chunk_end,
-    const double* __restrict__ U, const long long* __restrict__ pstart, const float* __restrict__ fown,
-    const PT* __restrict__ pbuf, const float* __restrict__ w6in, const float* __restrict__ f_tar,
-    double* __restrict__ partials)
+    int c0, int discard, int P, int Pst, const int* chunk_begin, const int* chunk_end,
+    const double* U, const long long* pstart, const float* fown,
+    const PT* pbuf, const float* w6in, const float* f_tar,
+    double* partials)
 {
     constexpr int kWarps = kReceiverThreads / 32;
     constexpr int kPair = 2 * (int)sizeof(PT);  // bytes of one lane's two members
     __shared__ RecvRed<kWarps> red;
     extern __shared__ __align__(16) unsigned char s_slots_raw[];  // [warps][kRecvStage][3][Pst / 2] member pairs
     const int c = c0 + (int)(gridDim.x - 1 - block_after());  // last chunk first (as k_contract_bulk)
+    fown = reread(fown);  // read by recv_load
+    w6in = reread(w6in);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k0 = 2 * lane;
     const bool on0 = k0 < P, on1 = k0 + 1 < P;
@@ -800,10 +804,10 @@ __global__ void __launch_bounds__(kReceiverThreads, 2) k_contract_staged(
 
 template <class PT>
 __global__ void __launch_bounds__(kReceiverThreads, 2) k_contract_bulk(
-    int c0, int discard, int P, int Pst, const int* __restrict__ chunk_begin, const int* __restrict__ chunk_end,
-    const double* __restrict__ U, const long long* __restrict__ pstart, const float* __restrict__ fown,
-    const PT* __restrict__ pbuf, const float* __restrict__ w6in, const float* __restrict__ f_tar,
-    double* __restrict__ partials, unsigned* __restrict__ err)
+    int c0, int discard, int P, int Pst, const int* chunk_begin, const int* chunk_end,
+    const double* U, const long long* pstart, const float* fown,
+    const PT* pbuf, const float* w6in, const float* f_tar,
+    double* partials, unsigned* err)
 {
     extern __shared__ __align__(128) unsigned char s_bulk[];
     BulkSmem& S = *reinterpret_cast<BulkSmem*>(s_bulk);
@@ -812,6 +816,8 @@ __global__ void __launch_bounds__(kReceiverThreads, 2) k_contract_bulk(
     // forces in owner order, so the last chunks' rows are the ones most
     // likely still in L2
     const int c = c0 + (int)(gridDim.x - 1 - block_after());
+    fown = reread(fown);  // read by recv_load
+    w6in = reread(w6in);
     bulk_init(S);
     if (!bulk_receive_chunk<PT>(c, P, Pst, chunk_begin, chunk_end, U, pstart, fown, pbuf, w6in, f_tar, partials, err,
                                 discard != 0, S, bw))
@@ -1031,10 +1037,10 @@ __device__ __forceinline__ double sqrt_refined(double x)
 }
 
 __global__ void __cluster_dims__(1, kLossSplit, 1) __launch_bounds__(kLossThreads)
-    k_loss(int P, int S, int n_par, const int* __restrict__ s_chunk0, const double* __restrict__ s_inv_na,
-           const float* __restrict__ s_vtar, const double* __restrict__ partials, const double* __restrict__ e_tar,
-           const float* __restrict__ z, double l_e, double l_f, double l_v, double l_1, double l_2, LossInv inv,
-           double* __restrict__ loss)
+    k_loss(int P, int S, int n_par, const int* s_chunk0, const double* s_inv_na,
+           const float* s_vtar, const double* partials, const double* e_tar,
+           const float* z, double l_e, double l_f, double l_v, double l_1, double l_2, LossInv inv,
+           double* loss)
 {
     constexpr int kBatch = 4;  // chunks whose loads are issued together (summed in order)
     const int k = block_after(), q = blockIdx.y, nq = gridDim.y;
