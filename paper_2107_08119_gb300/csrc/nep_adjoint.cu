@@ -393,12 +393,12 @@ int ensure_adjoint(nep_model* m, nep_dataset* ds)
     return NEP_OK;
 }
 
-// more than the default 48 KB of shared memory, where needed (an attribute
-// call costs as much host time as a launch)
+// more than the default shared memory, where needed (an attribute call costs as
+// much host time as a launch)
 template <class K>
 int allow_shared(K kern, size_t bytes)
 {
-    if (bytes <= 48 * 1024) return NEP_OK;
+    if (bytes <= kDefaultShared) return NEP_OK;
     return cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
                      "adjoint kernel shared memory");
 }

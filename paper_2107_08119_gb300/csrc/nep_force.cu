@@ -331,9 +331,9 @@ int launch_site(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, dou
     const size_t smem = site_block_smem<D, AT>(n_par, a.n_neu);
     constexpr int kWide = (384 / SiteSplit<AT>::WAYS + 31) / 32;  // words that hold any capacity
     auto kern = nl.m_cap <= 32 * SiteSplit<AT>::WAYS ? k_site<D, AT, 1> : k_site<D, AT, kWide>;
-    // only large networks of the split model need more than the default 48 KB:
-    // an attribute call costs as much host time as a launch
-    if (smem > 48 * 1024) {
+    // only large networks of the split model need more than the default: an
+    // attribute call costs as much host time as a launch
+    if (smem > kDefaultShared) {
         const int rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                                  "site kernel shared memory");
         if (rc) return rc;

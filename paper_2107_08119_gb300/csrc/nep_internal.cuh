@@ -400,6 +400,10 @@ cudaError_t launch_after(bool after, void (*kern)(Par...), dim3 grid, int block,
     return cudaLaunchKernelEx(&cfg, kern, Par(arg)...);
 }
 
+// Dynamic shared memory that a kernel gets without asking: 48 KB hold its static
+// part too, here taken as at most 1 KB (the site pass has 576 bytes).
+constexpr size_t kDefaultShared = 47 * 1024;
+
 // ---------------------------------------------------------------- workspace
 struct NeighborList {
     int n_cap = 0;       // atoms the buffers hold
