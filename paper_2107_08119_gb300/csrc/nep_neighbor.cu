@@ -221,7 +221,7 @@ __device__ __forceinline__ unsigned long long sort_key(float d2, int v)
 //                 slot (vala), and into the fourth word of each partner
 //                 entry the rank it got here: the partner's reverse index
 //                 (k_sort_rows, a warp per atom storing nbr directly, above
-//                 128 slots).
+//                 185 slots).
 //   k_rev_tile    rev[rank of slot s][i] = the fourth word of i's slot s,
 //                 within each row, 32 atoms per block transposed through
 //                 shared memory into whole-row stores (k_rev_perm, a warp
@@ -541,12 +541,13 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_sort_rows(int n, int m_ca
 // registers while the current one sorts); the sorted values go to a shared
 // tile (atom a's column), stored after the block barrier as rows of 32
 // consecutive atoms (one 128-byte store each).  inv and the partner words are
-// written as in k_sort_rows.  Shared memory: the warps' key buffers (lcap x
+// written as in k_sort_rows, which takes longer rows.  Shared memory: the warps' key buffers (lcap x
 // 12 bytes each), then the m_cap x 33-int tile.
 constexpr int kSortWarps = 8;
 constexpr int kSortAtoms = 32;
 constexpr int kSortGridCap = 152 * 8;
-constexpr size_t kSortTileMaxSmem = 48 * 1024;  // up to 128 slots per atom (the warp-per-atom sort beyond)
+// the default 48 KB hold the kernel's counts too: up to 185 slots per atom
+constexpr size_t kSortTileMaxSmem = 48 * 1024 - sizeof(int) * kSortAtoms;
 
 __global__ void __launch_bounds__(32 * kSortWarps) k_sort_tile(int n, int m_cap, int lcap, int* rows,
                                                               const int* count, int* nbr,

@@ -43,3 +43,33 @@ def test_split_model_widths(orc, n, n_neu):
     assert np.abs(out["e_atom"].cpu().numpy()[idx] - U).max() <= 1e-6 * n_neu / 30
     assert np.abs(aos(out["force"])[idx] - F).max() <= 1e-4
     model.close()
+
+
+@pytest.mark.parametrize("capacity,edge", [(128, 3.3), (129, 3.3), (185, 3.0), (186, 3.0), (187, 3.0), (384, 3.0)])
+def test_list_capacities(orc, capacity, edge):
+    """The row sort of the cells path around the capacity at which its shared tile
+    no longer fits (116 and 155 neighbours per atom): the rows are the atoms within
+    the cutoff, distances ascending, and the forces those of the oracle (1e-4 eV/A
+    at forces of 10 eV/A; here they are larger, and FP32 is relative)."""
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(capacity)
+    pos, box = inputs.diamond(6, 8, 7, edge)
+    pos = inputs.displace(pos, 0.05, rng)
+    n = len(pos)
+    hyper = nep.Hyper(max_neighbors=capacity)
+    z = inputs.random_z(hyper.n_par, rng)
+    model = nep.NEP(z, hyper)
+    out = model.compute(soa(pos), box)
+    cnt, nbr = (t.cpu().numpy() for t in model.neighbors(n))
+    idx = np.unique(rng.integers(0, n, 40))
+    _, F, _ = orc.efv_sample(orc.NepHyper(), f32_exact(z), pos, box, idx)
+    assert np.abs(aos(out["force"])[idx] - F).max() <= 1e-4 * max(1.0, np.abs(F).max() / 10)
+    L = np.diag(box)
+    for i in idx:
+        d = pos - pos[i]
+        r = np.linalg.norm(d - L * np.round(d / L), axis=1)
+        row = r[nbr[:cnt[i], i] & 0xFFFFFF]
+        assert abs(int(cnt[i]) - int(np.sum((r < 5.0) & (r > 0)))) <= int(np.sum(np.abs(r - 5.0) < 1e-5))
+        assert row.max() < 5.0 + 1e-5 and np.all(np.diff(row) >= -1e-5)
+        assert len(set((nbr[:cnt[i], i] & 0xFFFFFF).tolist())) == cnt[i]
+    model.close()
