@@ -518,7 +518,10 @@ __host__ __device__ __forceinline__ void assemble_atom(int i, int n, int m_cap, 
         // the loop ends after the last kept slot
         cnt = mb[2] ? 96 - clz32(mb[2]) : mb[1] ? 64 - clz32(mb[1]) : mb[0] ? 32 - clz32(mb[0]) : 0;
     }
-    auto kept = [&](int k) { return ((k < 32 ? mb[0] >> k : k < 64 ? mb[1] >> (k - 32) : mb[2] >> (k - 64)) & 1u) != 0u; };
+    // (without masks every slot is kept, also those past the 96 that the words cover)
+    auto kept = [&](int k) {
+        return !mask || ((k < 32 ? mb[0] >> k : k < 64 ? mb[1] >> (k - 32) : mb[2] >> (k - 64)) & 1u) != 0u;
+    };
 #pragma unroll
     for (int a = 0; a < 3; ++a) F[a] = 0.f;
 #pragma unroll

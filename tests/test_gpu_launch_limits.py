@@ -1,5 +1,5 @@
-"""Launches at the limits of what a kernel gets by default: shared memory (48 KB,
-of which a kernel's static part counts too)."""
+"""Calls at the limits of what a kernel takes: the default shared memory (48 KB, of
+which a kernel's static part counts too), and the 96 slots of the in-cutoff masks."""
 import numpy as np
 import pytest
 
@@ -72,4 +72,31 @@ def test_list_capacities(orc, capacity, edge):
         assert abs(int(cnt[i]) - int(np.sum((r < 5.0) & (r > 0)))) <= int(np.sum(np.abs(r - 5.0) < 1e-5))
         assert row.max() < 5.0 + 1e-5 and np.all(np.diff(row) >= -1e-5)
         assert len(set((nbr[:cnt[i], i] & 0xFFFFFF).tolist())) == cnt[i]
+    model.close()
+
+
+def test_more_than_96_slots_in_a_large_box(orc):
+    """The assembly by atoms (above 60,000 of them) without slot masks: a cluster
+    whose atoms have more than 96 neighbours beside a sparse crystal, net force
+    and a sample of the cluster against the oracle (1e-4 eV/A at forces of
+    10 eV/A)."""
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(3)
+    pos, box = inputs.diamond(20, 20, 20)
+    pos = inputs.displace(pos, 0.1, rng)
+    far = np.linalg.norm(pos - np.diag(box) / 2, axis=1) > 12.0
+    spot, edges = inputs.diamond(5, 5, 5, 3.2)
+    spot = inputs.displace(spot, 0.05, rng) - np.diag(edges) / 2 + np.diag(box) / 2
+    pos = np.concatenate([pos[far], spot])
+    n = len(pos)
+    assert n > 60000
+    hyper = nep.Hyper(max_neighbors=256)
+    z = inputs.random_z(hyper.n_par, rng)
+    model = nep.NEP(z, hyper)
+    out = model.compute(soa(pos), box)
+    cnt, _ = model.neighbors(n)
+    assert int(cnt.max()) > 96 and float(cnt.double().mean()) < 45
+    idx = np.argsort(cnt.cpu().numpy())[-40:]
+    U, F, _ = orc.efv_sample(orc.NepHyper(), f32_exact(z), pos, box, idx)
+    assert np.abs(aos(out["force"])[idx] - F).max() <= 1e-4 * max(1.0, np.abs(F).max() / 10)
     model.close()
