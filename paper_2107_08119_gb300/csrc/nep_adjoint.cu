@@ -42,6 +42,7 @@
 namespace nep {
 namespace {
 
+constexpr int kMostPar = (kNdes + 2) * kMaxNeu + 1;  // parameters of the largest network
 constexpr int kAdjWords = 2;  // own-slot words per thread: 256 pairs per atom at 32 atoms per block
 static_assert(kDsCap <= 32 * kAdjWords * kSiteWarps, "a training set's pairs of an atom have own-slot bits");
 
@@ -394,12 +395,13 @@ int ensure_adjoint(nep_model* m, nep_dataset* ds)
 }
 
 // more than the default shared memory, where needed (an attribute call costs as
-// much host time as a launch)
+// much host time as a launch): `most` bytes, what the largest network takes, as
+// the limit is the kernel's and not the model's
 template <class K>
-int allow_shared(K kern, size_t bytes)
+int allow_shared(K kern, size_t bytes, size_t most)
 {
     if (bytes <= kDefaultShared) return NEP_OK;
-    return cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
+    return cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most),
                      "adjoint kernel shared memory");
 }
 
@@ -464,7 +466,7 @@ int nep_force_loss(nep_model* m, nep_dataset* ds, const float* z, double* loss_f
     rc = by_atoms_per_block(N, [&](auto tag) {
         constexpr int AT = decltype(tag)::value;
         const size_t smem = site_block_smem<DescSi, AT>(n_par, m->hp.n_neu);
-        const int r = allow_shared(k_adj_site<AT>, smem);
+        const int r = allow_shared(k_adj_site<AT>, smem, site_block_smem<DescSi, AT>(kMostPar, kMaxNeu));
         if (r) return r;
         k_adj_site<AT><<<nb, kSiteThreads, smem, st>>>(N, ds->sid, ds->boxes, ds->xr, ds->pstart, ds->pj, a.z, n_par,
                                                        site_params(m, ds->typed), a.pf, m->d_err);
@@ -496,7 +498,7 @@ int nep_force_loss_backward(nep_model* m, nep_dataset* ds, const double* seed, d
     const int rc = by_atoms_per_block(N, [&](auto tag) {
         constexpr int AT = decltype(tag)::value;
         const size_t smem = adj_lambda_smem<AT>(n_par, m->hp.n_neu);
-        const int r = allow_shared(k_adj_lambda<AT>, smem);
+        const int r = allow_shared(k_adj_lambda<AT>, smem, adj_lambda_smem<AT>(kMostPar, kMaxNeu));
         if (r) return r;
         k_adj_lambda<AT><<<nb, kSiteThreads, smem, st>>>(N, ds->sid, ds->boxes, ds->xr, ds->pstart, ds->pj,
                                                          reinterpret_cast<const float4*>(a.res), a.sums, a.z, n_par,

@@ -332,9 +332,11 @@ int launch_site(const ForceArgs& a, NeighborList& nl, int n, double* e_atom, dou
     constexpr int kWide = (384 / SiteSplit<AT>::WAYS + 31) / 32;  // words that hold any capacity
     auto kern = nl.m_cap <= 32 * SiteSplit<AT>::WAYS ? k_site<D, AT, 1> : k_site<D, AT, kWide>;
     // only large networks of the split model need more than the default: an
-    // attribute call costs as much host time as a launch
+    // attribute call costs as much host time as a launch.  The limit is the
+    // kernel's, whatever model is launched: always that of the largest network
     if (smem > kDefaultShared) {
-        const int rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+        constexpr int kMost = (int)site_block_smem<D, AT>((D::Ndes + 2) * kMaxNeu + 1, kMaxNeu);
+        const int rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost),
                                  "site kernel shared memory");
         if (rc) return rc;
     }

@@ -66,7 +66,7 @@ __host__ __device__ constexpr int site_block_at(int n, int lm)
 
 // shared memory: weights | tile / S / A | q / G | radial tile / neuron states and slopes | mask words
 template <class D, int AT>
-__host__ __device__ inline size_t site_block_smem(int n_par, int n_neu)
+__host__ __device__ constexpr size_t site_block_smem(int n_par, int n_neu)
 {
     const size_t x_rows = 2 * (n_neu > kSiteChunk ? n_neu : kSiteChunk);
     return sizeof(float) * (((size_t)n_par + 31) / 32 * 32 +

@@ -499,13 +499,14 @@ size_t mlp_f32_smem(int M, int n_par, int n_neu)
            (kMlpAtoms * kNdes + M * (2 * ((size_t)(n_par + 3) / 4 * 4) + mlp_f32_d_floats(n_neu)));
 }
 
+constexpr size_t kMlpSmemMax = 220 * 1024;  // the largest network takes 212 KB with four members per block
+
 // members per block: mlp_threads / 32, or four where the slopes of eight do
 // not fit in shared memory
 int mlp_f32_members(int threads, int n_par, int n_neu)
 {
-    return threads == 256 && mlp_f32_smem(8, n_par, n_neu) <= 220 * 1024 ? 8 : 4;
+    return threads == 256 && mlp_f32_smem(8, n_par, n_neu) <= kMlpSmemMax ? 8 : 4;
 }
-
 
 // Contraction, pass 1 (owner side): one warp per atom j, lane l holding
 // members 2l and 2l + 1.  The lane loads its members' G_j once (registers).
@@ -1390,7 +1391,8 @@ int ensure_pop(nep_dataset* ds, int P)
 
 // Everything an evaluation with P members needs that must not happen inside a
 // stream capture: scratch allocation, kernel attributes, the second stream
-// and its events.
+// and its events.  The attributes belong to the kernels, which other host threads
+// launch for other training sets: always the most that any set may take.
 int prepare_evaluation(nep_dataset* ds, int P)
 {
     const int cap0 = ds->pop_cap;
@@ -1421,24 +1423,18 @@ int prepare_evaluation(nep_dataset* ds, int P)
         (rc = cuda_fail(cudaFuncSetAttribute(k_contract_bulk<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)sizeof(BulkSmem)), "contraction shared memory")))
         return rc;
-    for (int t = 128; t <= 256; t += 128) {
-        const int n_neu = ds->m->hp.n_neu, M = mlp_f32_members(t, ds->m->n_par, n_neu);
-        auto kern = M == 4 ? k_mlp_f32<4> : k_mlp_f32<8>;
-        if ((rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)mlp_f32_smem(M, ds->m->n_par, n_neu)), "network shared memory")) ||
+    for (auto kern : {k_mlp_f32<4>, k_mlp_f32<8>})
+        if ((rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmemMax),
+                            "network shared memory")) ||
             (rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                  cudaSharedmemCarveoutMaxShared), "network shared memory")))
             return rc;
-    }
-    for (int gm = 4; gm <= 16; gm *= 2) {
-        if (!fused_fits(ds, gm)) continue;
-        const int smem = (int)fused_smem_bytes(ds->amax, gm);
+    for (int gm = 4; gm <= 16; gm *= 2)
         for (int h = 0; h < 2; ++h)
             if ((rc = cuda_fail(cudaFuncSetAttribute(fused_kernel(gm, h != 0),
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemMax),
                                 "fused contraction shared memory")))
                 return rc;
-    }
     if ((rc = prepare_owner_tc())) return rc;
     return prepare_pop_tc();
 }

@@ -100,3 +100,57 @@ def test_more_than_96_slots_in_a_large_box(orc):
     U, F, _ = orc.efv_sample(orc.NepHyper(), f32_exact(z), pos, box, idx)
     assert np.abs(aos(out["force"])[idx] - F).max() <= 1e-4 * max(1.0, np.abs(F).max() / 10)
     model.close()
+
+
+def _training(n_neu, cells, seed):
+    """A training set of two cells and a model of n_neu neurons, and a population."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(seed)
+    hyper = nep.Hyper(n_neu=n_neu)
+    pos, box = inputs.diamond(*cells)
+    structures = [{"pos": inputs.displace(pos, 0.1, rng), "box": box} for _ in range(2)]
+    n = 2 * len(pos)
+    model = nep.NEP(inputs.random_z(hyper.n_par, rng), hyper)
+    ds = nep.Dataset(model, structures, np.zeros(2), rng.normal(0.0, 1.0, (n, 3)), np.zeros((2, 6)))
+    pop = torch.tensor(rng.normal(0.0, 0.1, (16, hyper.n_par)).astype(np.float32), device="cuda")
+    return model, ds, pop
+
+
+@pytest.mark.parametrize("fused", [0, 8])
+def test_training_sets_of_two_widths_in_two_threads(fused):
+    """Kernels' shared-memory limits belong to the kernels, not to a training set:
+    two host threads that evaluate sets of networks of 4 and 64 neurons, with 32
+    and 256 atoms per structure, do not lower them for one another.  Every loss has
+    the bits of the same evaluation alone."""
+    import threading
+
+    import torch
+    sets = [_training(4, (1, 2, 2), 1), _training(64, (4, 4, 2), 2)]
+    want = []
+    for _, ds, pop in sets:
+        ds.set_shape(fused=fused, mlp_threads=256)
+        want.append(ds.evaluate(pop).clone())
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(k):
+        try:
+            _, ds, pop = sets[k]
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(400):
+                    got = ds.evaluate(pop)
+                torch.cuda.current_stream().synchronize()
+                assert torch.equal(got, want[k])
+        except Exception as e:  # reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for model, ds, _ in sets:
+        ds.close()
+        model.close()
