@@ -1389,27 +1389,14 @@ int ensure_pop(nep_dataset* ds, int P)
     return NEP_OK;
 }
 
-// Everything an evaluation with P members needs that must not happen inside a
-// stream capture: scratch allocation, kernel attributes, the second stream
-// and its events.  The attributes belong to the kernels, which other host threads
-// launch for other training sets: always the most that any set may take.
-int prepare_evaluation(nep_dataset* ds, int P)
+// Shared-memory limits of the evaluation's kernels.  They belong to the kernels,
+// which other host threads launch for other training sets: always the most that
+// any set may take.
+int set_kernel_limits()
 {
-    const int cap0 = ds->pop_cap;
-    int rc = ensure_pop(ds, P);
-    if (rc) return rc;
-    if (ds->pop_cap != cap0) ++ds->epoch;
-    if (!ds->aux) {
-        if ((rc = cuda_fail(cudaStreamCreateWithFlags(&ds->aux, cudaStreamNonBlocking), "evaluation stream")))
-            return rc;
-        for (int w = 0; w < kMaxWaves; ++w)
-            if ((rc = cuda_fail(cudaEventCreateWithFlags(&ds->ev_wave[w], cudaEventDisableTiming), "evaluation event")))
-                return rc;
-        if ((rc = cuda_fail(cudaEventCreateWithFlags(&ds->ev_join, cudaEventDisableTiming), "evaluation event")))
-            return rc;
-    }
     const int ostage = (kOwnerMaxThreads / 32) * kOwnerStage * (int)sizeof(float);
     const int rstage = (kReceiverThreads / 32) * kRecvStage * 3 * member_stride(kMaxPop) * (int)sizeof(float);
+    int rc;
     if ((rc = cuda_fail(cudaFuncSetAttribute(k_contract_owner<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              ostage), "contraction shared memory")) ||
         (rc = cuda_fail(cudaFuncSetAttribute(k_contract_owner<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1437,6 +1424,29 @@ int prepare_evaluation(nep_dataset* ds, int P)
                 return rc;
     if ((rc = prepare_owner_tc())) return rc;
     return prepare_pop_tc();
+}
+
+// Everything an evaluation with P members needs that must not happen inside a
+// stream capture: scratch allocation; and once per training set the kernels'
+// limits (twenty calls that each cost about as much host time as a launch), the
+// second stream and its events.
+int prepare_evaluation(nep_dataset* ds, int P)
+{
+    const int cap0 = ds->pop_cap;
+    int rc = ensure_pop(ds, P);
+    if (rc) return rc;
+    if (ds->pop_cap != cap0) ++ds->epoch;
+    if (!ds->aux) {
+        if ((rc = set_kernel_limits())) return rc;
+        if ((rc = cuda_fail(cudaStreamCreateWithFlags(&ds->aux, cudaStreamNonBlocking), "evaluation stream")))
+            return rc;
+        for (int w = 0; w < kMaxWaves; ++w)
+            if ((rc = cuda_fail(cudaEventCreateWithFlags(&ds->ev_wave[w], cudaEventDisableTiming), "evaluation event")))
+                return rc;
+        if ((rc = cuda_fail(cudaEventCreateWithFlags(&ds->ev_join, cudaEventDisableTiming), "evaluation event")))
+            return rc;
+    }
+    return NEP_OK;
 }
 
 // The two contraction passes over the chunk range [c_lo, c_hi) (whole
