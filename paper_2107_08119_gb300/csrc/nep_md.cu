@@ -47,8 +47,31 @@ static constexpr double kEvPerAFsK_WPerMK = 1.602176634e6;
 namespace nep {
 namespace {
 
-// control words on the device; the two from kCtlKick hold one 64-bit count
-enum { kCtlGate = 0, kCtlStep = 1, kCtlKick = 2, kCtlWords = 4 };
+// Control words on the device.  Where a call's rows go and its thermostat's
+// numbers stand here and not in the launches, so that the step graphs outlive
+// them: a block of five steps of 512 atoms with rows of its own took 355 us with
+// new graphs, the same block again 178.
+struct StepCtl {
+    unsigned gate;            // 1: the list is rebuilt in this step
+    unsigned step;            // steps of the call so far
+    unsigned long long kick;  // blocks of k_kick_drift (see there)
+    double *thermo, *heat;    // the call's rows, or NULL
+    double t0, tau;           // thermostat
+};
+
+// The start of a call; `init`: of the first one on a new state too
+__global__ void k_md_begin(StepCtl* ctl, int init, double* thermo, double* heat, double t0, double tau)
+{
+    if (init) {
+        ctl->gate = 0u;
+        ctl->kick = 0ull;
+    }
+    ctl->step = 0u;
+    ctl->thermo = thermo;
+    ctl->heat = heat;
+    ctl->t0 = t0;
+    ctl->tau = tau;
+}
 
 // A step's sums, one block each: block 0 the site-energy block partials, block
 // 1 + c component c of the other block partials (each thread a fixed stride of
@@ -70,11 +93,10 @@ struct StepSums {
     size_t cstride_x = 0;
     int off_x = 0;
     double* red = nullptr;
-    double* thermo = nullptr;
-    double* heat = nullptr;
-    const unsigned* ctl = nullptr;
+    const StepCtl* ctl = nullptr;
     int row = 0;  // row of the step, from the step counter
-    double t0 = 0.0, tau = 0.0, dt = 0.0, dof_kb = 0.0;
+    bool thermostat = false;
+    double dt = 0.0, dof_kb = 0.0;
 };
 
 template <int THREADS>
@@ -82,19 +104,21 @@ __device__ __forceinline__ void step_sum(const StepSums& S, int w)
 {
     // sums: 0 E_pot, 1..9 W (row-major), 10 E_kin, 11..13 J; red: [1..9] W with
     // HNEMD (summed before the kick), [14] lambda
+    StepCtl C = {};
+    if (threadIdx.x == 0) C = *S.ctl;  // ahead of the sum
     double t = sum_partials<THREADS>(w == 0 ? S.part_e : S.part_x + (w - 1) * S.cstride_x, w == 0 ? S.nb_e : S.nb_x,
                                      w == 0 ? 1 : S.bstride_x);
     if (threadIdx.x != 0) return;
     const int k = w == 0 ? 0 : S.off_x + w - 1;
-    const size_t s = (size_t)((int)S.ctl[kCtlStep] + S.row);
-    if (k == 10 && S.tau > 0.0) {
+    const size_t s = (size_t)((int)C.step + S.row);
+    if (k == 10 && S.thermostat) {
         const double T = 2.0 * t / S.dof_kb;
-        const double lam = T > 0.0 ? sqrt(1.0 + S.dt / S.tau * (S.t0 / T - 1.0)) : 1.0;
+        const double lam = T > 0.0 ? sqrt(1.0 + S.dt / C.tau * (C.t0 / T - 1.0)) : 1.0;
         S.red[14] = lam;
         t *= lam * lam;
     }
-    if (S.thermo) {
-        double* row = S.thermo + s * NEP_THERMO_COLS;  // E_pot, E_kin, W xx yy zz xy yz zx
+    if (C.thermo) {
+        double* row = C.thermo + s * NEP_THERMO_COLS;  // E_pot, E_kin, W xx yy zz xy yz zx
         const int col = k == 0 ? 0 : k == 10 ? 1 : k == 1 ? 2 : k == 5 ? 3 : k == 9 ? 4 : k == 2 ? 5 : k == 6 ? 6
                       : k == 7 ? 7 : -1;
         if (col >= 0) row[col] = t;
@@ -107,7 +131,7 @@ __device__ __forceinline__ void step_sum(const StepSums& S, int w)
             row[7] = S.red[7];
         }
     }
-    if (S.heat && k >= 11) S.heat[s * 3 + k - 11] = t;
+    if (C.heat && k >= 11) C.heat[s * 3 + k - 11] = t;
 }
 
 template <int THREADS>
@@ -120,11 +144,11 @@ __global__ void __launch_bounds__(THREADS) k_md_finish(StepSums S)
 // last build; `count` steps are counted.
 // use_cond: the step runs from a CUDA graph whose list rebuild sits behind the
 // conditional node `cond`, which this sets.
-__device__ void decide(unsigned* ctl, bool far, int count, unsigned long long* rebuilds,
+__device__ void decide(StepCtl* ctl, bool far, int count, unsigned long long* rebuilds,
                        cudaGraphConditionalHandle cond, int use_cond)
 {
-    ctl[kCtlGate] = far ? 1u : 0u;
-    if (count) ctl[kCtlStep] += (unsigned)count;
+    ctl->gate = far ? 1u : 0u;
+    if (count) ctl->step += (unsigned)count;
     if (far) *rebuilds += 1ull;
     if (use_cond) cudaGraphSetConditional(cond, far ? 1u : 0u);
 }
@@ -136,7 +160,7 @@ template <int THREADS, bool SCALE>
 __global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, const double* red, int n, double* x, double* v,
                                                         const float* F, double hdtm, double dt,
                                                         float* xr, const double* x_ref,
-                                                        unsigned* ctl, float thresh2, int count,
+                                                        StepCtl* ctl, float thresh2, int count,
                                                         unsigned long long* rebuilds,
                                                         cudaGraphConditionalHandle cond, int use_cond)
 {
@@ -181,11 +205,10 @@ __global__ void __launch_bounds__(THREADS) k_kick_drift(StepSums S, const double
     // clears the count and takes the rebuild decision from it
     const bool far = __syncthreads_or(d2 > thresh2);
     if (threadIdx.x != 0) return;
-    unsigned long long* done = reinterpret_cast<unsigned long long*>(ctl + kCtlKick);
     const unsigned long long mine = far ? (1ull << 32) + 1 : 1ull;
-    const unsigned long long all = atomicAdd(done, mine) + mine;
+    const unsigned long long all = atomicAdd(&ctl->kick, mine) + mine;
     if ((unsigned)all != gridDim.x - S.nsum) return;
-    *done = 0ull;
+    ctl->kick = 0ull;
     decide(ctl, (all >> 32) != 0, count, rebuilds, cond, use_cond);
 }
 
@@ -418,7 +441,7 @@ struct nep_md {
     float skin = 0.f;
     Workspace ws;
     double* x_ref = nullptr;
-    unsigned* ctl = nullptr;
+    StepCtl* ctl = nullptr;
     unsigned long long* rebuilds = nullptr;
     double* red = nullptr;
     bool need_init = true;
@@ -440,16 +463,14 @@ struct nep_md {
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // one step, kGraphSteps steps
     struct GraphKey {
         const double *pos, *vel;
-        double *thermo, *heat;
-        double dt, t0, tau, fe[3];
-        bool drive;
+        double dt, fe[3];
+        bool thermostat, drive;
         const float* zatom;
         bool plain;
         bool operator==(const GraphKey& o) const
         {
-            return pos == o.pos && vel == o.vel && thermo == o.thermo && heat == o.heat && dt == o.dt &&
-                   t0 == o.t0 && tau == o.tau && fe[0] == o.fe[0] && fe[1] == o.fe[1] && fe[2] == o.fe[2] &&
-                   drive == o.drive && zatom == o.zatom && plain == o.plain;
+            return pos == o.pos && vel == o.vel && dt == o.dt && fe[0] == o.fe[0] && fe[1] == o.fe[1] &&
+                   fe[2] == o.fe[2] && thermostat == o.thermostat && drive == o.drive && zatom == o.zatom && plain == o.plain;
         }
     } gkey{};
 };
@@ -506,10 +527,10 @@ int nep_md_create(nep_model* m, int n, const double* box9, double mass, nep_md**
         return rc;
     }
     cudaError_t e = cudaMalloc((void**)&md->x_ref, sizeof(double) * 3 * (size_t)n);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&md->ctl, sizeof(unsigned) * kCtlWords);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&md->ctl, sizeof(StepCtl));
     if (e == cudaSuccess) e = cudaMalloc((void**)&md->rebuilds, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc((void**)&md->red, sizeof(double) * 32);
-    if (e == cudaSuccess) e = cudaMemset(md->ctl, 0, sizeof(unsigned) * kCtlWords);
+    if (e == cudaSuccess) e = cudaMemset(md->ctl, 0, sizeof(StepCtl));
     if (e == cudaSuccess) e = cudaMemset(md->rebuilds, 0, sizeof(unsigned long long));
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -800,11 +821,10 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             k_hnemd_kick<<<nbk, kt, 0, st>>>(n, md->ws.force, md->w_atom, vel, md->fe[0], md->fe[1], md->fe[2],
                                               md->red + 1, 1.0 / n, 0.0, kef, part_h, m->d_err);
         }
-        if ((rc = cuda_fail(cudaMemsetAsync(md->ctl, 0, sizeof(unsigned) * kCtlWords, st), "cudaMemsetAsync")))
-            return rc;
-        md->need_init = false;
     }
-    if ((rc = cuda_fail(cudaMemsetAsync(md->ctl + kCtlStep, 0, sizeof(unsigned), st), "cudaMemsetAsync"))) return rc;
+    k_md_begin<<<1, 1, 0, st>>>(md->ctl, md->need_init ? 1 : 0, thermo, heat, md->t0, md->tau);
+    if ((rc = cuda_fail(cudaGetLastError(), "md step kernels"))) return rc;
+    md->need_init = false;
 
     const double hdtm = 0.5 * dt / (md->mass * conv);
     const float thresh = 0.5f * md->skin;
@@ -865,7 +885,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
                          md->fe[2], md->red + 1, 1.0 / n, hdtm, kef, part_h, m->d_err);
         }
         StepSums S{drive ? 5 : 1 + c2, part_e, b1, drive ? part_h : part_a, drive ? nbk : b2, drive ? 4 : 1,
-                   drive ? 1 : (size_t)b2, drive ? 10 : 1, md->red, thermo, heat, md->ctl, row, md->t0, md->tau, dt,
+                   drive ? 1 : (size_t)b2, drive ? 10 : 1, md->red, md->ctl, row, md->tau > 0.0, dt,
                    dof_kb};
         if (follows && md->tau <= 0.0)
             prev = S;
@@ -955,8 +975,8 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             cudaGraphDestroy(g);
             return r;
         };
-        nep_md::GraphKey key{pos, vel, thermo, heat, dt, md->t0, md->tau, {md->fe[0], md->fe[1], md->fe[2]}, drive,
-                             md_zatom(md), md->plain};
+        nep_md::GraphKey key{pos, vel, dt, {md->fe[0], md->fe[1], md->fe[2]}, md->tau > 0.0, drive, md_zatom(md),
+                             md->plain};
         if (!(key == md->gkey) || !(md->gexec[0] || md->gexec[1])) {
             drop();
             if (!md->gcap && (rc = cuda_fail(cudaStreamCreateWithFlags(&md->gcap, cudaStreamNonBlocking), "stream")))
@@ -977,7 +997,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         return NEP_OK;
     }
 
-    const unsigned* gate = md->ctl + kCtlGate;
+    const unsigned* gate = &md->ctl->gate;
     for (int s = 0; s < n_steps; ++s) {
         head(st, false, cudaGraphConditionalHandle{}, 1, s > 0);
         if ((rc = rebuild(st, gate))) return rc;

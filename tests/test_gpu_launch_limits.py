@@ -154,3 +154,56 @@ def test_training_sets_of_two_widths_in_two_threads(fused):
     for model, ds, _ in sets:
         ds.close()
         model.close()
+
+
+@pytest.mark.parametrize("change", ["rows", "target temperature"])
+def test_step_graphs_outlive_their_rows(change):
+    """A block of steps that writes its rows elsewhere, or has another target
+    temperature, runs from the graphs of the block before: the states and rows of
+    the same run by single steps, and no time for new graphs (twice the block's own
+    time when they were captured again; a factor of 1.5 leaves room for noise)."""
+    import statistics
+    import time
+
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(8)
+    pos, box = inputs.diamond(4, 4, 4)
+    pos = inputs.displace(pos, 0.05, rng)
+    n, steps, blocks = len(pos), 5, 40
+    vel = rng.normal(0.0, 1e-3, (n, 3))
+    model = nep.NEP(inputs.random_z(1021, rng))
+
+    def run(fresh, ramp, chunk):
+        """Blocks with rows of their own (fresh) or in one buffer, in calls of `chunk` steps."""
+        md = nep.MD(model, n, box, 28.085)
+        x, v = soa(pos), soa(vel)
+        thermo = torch.zeros((blocks * steps, 8), dtype=torch.float64, device="cuda")
+        heat = torch.zeros((blocks * steps, 3), dtype=torch.float64, device="cuda")
+        one, two = thermo[:chunk].clone(), heat[:chunk].clone()
+        times = []
+        for s in range(0, blocks * steps, chunk):
+            md.set_thermostat(300.0 + (5.0 * (s // steps) if ramp else 0.0), 100.0)
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            if fresh:
+                md.step(x, v, chunk, 1.0, thermo=thermo[s:s + chunk], heat=heat[s:s + chunk])
+            else:
+                md.step(x, v, chunk, 1.0, thermo=one, heat=two)
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t)
+            if not fresh:
+                thermo[s:s + chunk].copy_(one)
+                heat[s:s + chunk].copy_(two)
+        md.close()
+        return statistics.median(times[len(times) // 2:]), x, v, thermo, heat
+
+    ramp = change != "rows"
+    base, *same = run(False, False, steps)
+    other, *got = run(not ramp, ramp, steps)
+    _, *want = run(False, ramp, 1)
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    assert torch.equal(got[2], same[2]) != ramp
+    assert other <= 1.5 * base, (other, base)
+    model.close()
