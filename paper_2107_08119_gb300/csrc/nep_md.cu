@@ -425,6 +425,13 @@ using namespace nep;
 // us per step; 10 steps per graph 45.5).
 constexpr int kGraphSteps = 5;
 
+// Steps from one capture key at which the graph of kGraphSteps steps pays for its
+// capture (about 200 us against 75 for one step, and 4 us saved per step).  Calls
+// with a new time step each, from one-step graphs -> from graphs of five: 512
+// atoms, 5 steps 256 -> 334 us, 10 steps 455 -> 505, 20 steps 844 -> 832, 40 steps
+// 1636 -> 1518; driven 13,824 atoms, 5 steps 439 -> 580, 40 steps 3237 -> 3225.
+constexpr int kGraphPays = 20;
+
 // Threads per block of the per-atom step kernels: two FP64 lanes per SM and
 // clock bound them, so up to one block of 256 per SM the atoms go to more SMs
 // (driven step of 13,824 atoms 73.9 -> 71.4 us, step of 4,096 39.8 -> 39.4; 128
@@ -457,10 +464,11 @@ struct nep_md {
     float* shc_ring = nullptr;   // [n_lags][9][n]
     double* shc_sum = nullptr;   // [n_lags][3]
     double* shc_part = nullptr;  // [chunks][n_lags][3]
-    // one step captured as a CUDA graph (the list rebuild behind a conditional
-    // node), kept while everything it bakes in is unchanged
+    // steps captured as CUDA graphs (the list rebuild behind conditional nodes),
+    // kept while everything they bake in is unchanged
     cudaStream_t gcap = nullptr, gcap2 = nullptr;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // one step, kGraphSteps steps
+    int gsteps = 0;                                 // steps run with this key, up to kGraphPays
     struct GraphKey {
         const double *pos, *vel;
         double dt, fe[3];
@@ -913,8 +921,8 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
     };
 
     // Without phase timing and without the per-step host logic of the
-    // spectral heat current, the steps run from CUDA graphs of one and of
-    // kGraphSteps steps, captured when first needed: the list rebuild is the
+    // spectral heat current, the steps run from CUDA graphs of one and, where it
+    // pays, of kGraphSteps steps, captured when first needed: the list rebuild is the
     // body of a conditional node that the last block of k_kick_drift switches,
     // so a step without a rebuild launches none of the list kernels.
     if (!m->prof.on && md->shc_lags == 0) {
@@ -984,9 +992,12 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             if (!md->gcap2 && (rc = cuda_fail(cudaStreamCreateWithFlags(&md->gcap2, cudaStreamNonBlocking), "stream")))
                 return rc;
             md->gkey = key;
+            md->gsteps = 0;
         }
+        const bool pays = md->gexec[1] || md->gsteps + (long long)n_steps >= kGraphPays;
+        md->gsteps = pays ? kGraphPays : md->gsteps + n_steps;
         for (int s = 0; s < n_steps;) {
-            const int u = n_steps - s >= kGraphSteps ? 1 : 0;
+            const int u = pays && n_steps - s >= kGraphSteps ? 1 : 0;
             if (!md->gexec[u] && (rc = capture(u ? kGraphSteps : 1, &md->gexec[u]))) {
                 md->gexec[u] = nullptr;
                 return rc;
