@@ -1307,9 +1307,17 @@ bool valid_shape(const nep_dataset* ds, const EvalShape& h)
 using namespace nep;
 
 
-// Generations per graph launch where a run has that many left (20 BF16
-// generations 3,721 -> 3,668 us).
+// Generations per graph launch where a run has that many left.  20 generations of
+// 50 members, one per graph -> five, each the median of 41 runs, equal to 2 us in
+// three repeats: BF16, 200 structures 3764 -> 3707 us, 50 structures 1395 -> 1340,
+// 3 structures 754 -> 721; FP32 7800 -> 7749, 2475 -> 2424, 1082 -> 1040.
 constexpr int kGraphGens = 5;
+
+// Generations with one key at which that graph pays for its capture (2 to 3 us
+// saved per generation).  Runs with new weights of the loss terms, one per graph ->
+// five, 3 structures in BF16: 5 generations 243 -> 292 us, 6 (both graphs) 277 ->
+// 360, 20 generations 795 -> 823.
+constexpr int kGraphGensPay = 30;
 
 struct snes_state {
     nep_model* m = nullptr;
@@ -1329,6 +1337,7 @@ struct snes_state {
     // keyed by what they bake in
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
+    int key_gens = 0;  // generations run with this key, up to kGraphGensPay
     unsigned long long key_uid = 0;
     int key_epoch = -1, key_prec = -1;
     double key_lam[5] = {0, 0, 0, 0, 0};
@@ -2082,11 +2091,13 @@ int snes_run(snes_state* st, nep_dataset* ds, int precision, const double* lambd
         for (int k = 0; k < 5; ++k) lam[k] = lambdas[k];
     bool same = st->key_uid == ds->uid && st->key_epoch == ds->epoch && st->key_prec == precision;
     for (int k = 0; same && k < 5; ++k) same = st->key_lam[k] == lam[k];
-    if (!same)
+    if (!same) {
         for (auto& e : st->exec) {
             if (e) cudaGraphExecDestroy(e);
             e = nullptr;
         }
+        st->key_gens = 0;
+    }
     st->key_uid = ds->uid;
     st->key_epoch = ds->epoch;
     st->key_prec = precision;
@@ -2105,11 +2116,14 @@ int snes_run(snes_state* st, nep_dataset* ds, int precision, const double* lambd
         if (r) *exec = nullptr;
         return r;
     };
-    if (n_gen >= kGraphGens && !st->exec[1] && (rc = capture(kGraphGens, &st->exec[1]))) return rc;
-    if (n_gen % kGraphGens && !st->exec[0] && (rc = capture(1, &st->exec[0]))) return rc;
+    const bool pays = st->exec[1] || st->key_gens + (long long)n_gen >= kGraphGensPay;
+    st->key_gens = pays ? kGraphGensPay : st->key_gens + n_gen;
+    const bool five = pays && n_gen >= kGraphGens, one = !five || n_gen % kGraphGens;
+    if (five && !st->exec[1] && (rc = capture(kGraphGens, &st->exec[1]))) return rc;
+    if (one && !st->exec[0] && (rc = capture(1, &st->exec[0]))) return rc;
     k_set_ctl<<<1, 1, 0, cs>>>(st->d_ctl, loss_hist, st->gen);
     for (int g = 0; g < n_gen;) {
-        const int u = n_gen - g >= kGraphGens ? 1 : 0;
+        const int u = five && n_gen - g >= kGraphGens ? 1 : 0;
         if ((rc = cuda_fail(cudaGraphLaunch(st->exec[u], cs), "launch generation graph"))) return rc;
         g += u ? kGraphGens : 1;
     }

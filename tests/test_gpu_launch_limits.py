@@ -236,3 +236,46 @@ def test_short_blocks_with_a_new_time_step():
     assert new <= 1.6 * again, (new, again)
     md.close()
     model.close()
+
+
+def test_short_runs_with_new_loss_weights():
+    """Few generations with new weights of the loss terms do not pay for a graph of
+    several generations: six take at most 1.45 times as long as the same six again
+    (1.25 times with the capture of one generation, 1.6 with both graphs); and runs
+    of 6, 40 and 14 generations, through both graphs, have the states of one run of
+    60."""
+    import time
+
+    import torch
+    from paper_2107_08119_gb300 import nep
+    model, ds, _ = _training(30, (1, 2, 2), 6)
+    mean = np.random.default_rng(6).uniform(-0.5, 0.5, model.hyper.n_par)
+    ds.set_shape(fused=0, mlp_threads=256, owner_tc=1, pop_pipe=1)
+
+    def fresh():
+        return nep.SNES(model, 16, mean, np.full(len(mean), 0.1), 3)
+
+    snes = fresh()
+
+    def run(weight):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        snes.run(ds, 6, nep.PREC_BF16, lambdas=[weight, 1.0, 1.0, 0.05, 0.05])
+        torch.cuda.synchronize()
+        return time.perf_counter() - t
+
+    times = np.array([[run(1.0 + 1e-4 * k), run(1.0 + 1e-4 * k)] for k in range(80)])
+    new, again = np.median(times[40:], axis=0)
+    assert new <= 1.45 * again, (new, again)
+    snes.close()
+    states = []
+    for blocks in ((60,), (6, 40, 14)):
+        snes = fresh()
+        for g in blocks:
+            snes.run(ds, g, nep.PREC_BF16)
+        states.append([t.clone() for t in snes.state()[:2]])
+        snes.close()
+    for a, b in zip(*states):
+        assert torch.equal(a, b)
+    ds.close()
+    model.close()
