@@ -378,6 +378,8 @@ def run_gpu(args, rank, world, local):
         pass
 
     if rank == 0:
+        # steps that run singly while the graph of five is captured: those of the warm-up, if it has them
+        lone = 0 if W >= 5 else min(K, 5)
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
             "ms_per_step": t_max / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -403,12 +405,12 @@ def run_gpu(args, rank, world, local):
                     "h2d_bytes_per_step": int(state.numel() * 8),
                     "d2h_bytes_per_step": int(state.numel() * 8 + N.THERMO_COLS * 8),
                     "steps": Ke},
-            # per replayed step: kick-drift (with the rebuild decision and the
-            # previous step's sums), site, assembly; per graph (five steps, or
-            # one) the sums of its last step; per rebuild the six list kernels
-            # of the conditional body (bin, scan, scatter, half-shell search,
-            # row sort, reverse index)
-            "gpu_launches": 3 * K + K // 5 + K % 5 + 6 * rebuilds,
+            # the control words of the call; per replayed step: kick-drift (with
+            # the rebuild decision and the previous step's sums), site,
+            # assembly; per graph (five steps, or one) the sums of its last
+            # step; per rebuild the six list kernels of the conditional body
+            # (bin, scan, scatter, half-shell search, row sort, reverse index)
+            "gpu_launches": 1 + 3 * K + lone + (K - lone) // 5 + (K - lone) % 5 + 6 * rebuilds,
             "measured_peaks": {k: peaks.get(k) for k in ("hbm_gbs", "bf16_tflops")} if peaks else None,
         }
         line["force_eval_vs_plain_fp32"] = force_eval_comparison(N, model, p0, box)

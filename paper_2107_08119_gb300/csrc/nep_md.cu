@@ -28,6 +28,7 @@
 //                  next to J, k_shc_corr / k_shc_reduce add
 //                  sum_i W_i(s - tau) . v_i(s) to K[tau] for every lag tau
 //                  already in the ring (Sec. II.B)
+#include <algorithm>
 #include <cmath>
 #include <new>
 
@@ -425,12 +426,16 @@ using namespace nep;
 // us per step; 10 steps per graph 45.5).
 constexpr int kGraphSteps = 5;
 
-// Steps from one capture key at which the graph of kGraphSteps steps pays for its
-// capture (about 200 us against 75 for one step, and 4 us saved per step).  Calls
-// with a new time step each, from one-step graphs -> from graphs of five: 512
-// atoms, 5 steps 256 -> 334 us, 10 steps 455 -> 505, 20 steps 844 -> 832, 40 steps
-// 1636 -> 1518; driven 13,824 atoms, 5 steps 439 -> 580, 40 steps 3237 -> 3225.
-constexpr int kGraphPays = 20;
+// Steps with one capture key at which the graph of kGraphSteps steps pays for its
+// capture: about 200 us of the host against 75 for one step (in part behind the
+// five single steps that run meanwhile), and 4 us saved per step.  Calls with a new
+// time step each, graphs of one step only -> of five whenever they fit: 512 atoms,
+// 5 steps 256 -> 308 us, 10 steps 455 -> 480, 20 steps 844 -> 815; driven 13,824
+// atoms 439 -> 500, 847 -> 896, 1615 -> 1647, 40 steps 3237 -> 3187.  In a large box
+// five steps outlast the capture, which then is nearly free: 125,000 atoms, 5 steps
+// 2020 -> 2080 us, 10 steps 4335 -> 4355, 15 steps 6710 -> 6690, and 20 steps
+// that follow a call of 5 steps 5240 -> 5192.
+constexpr int graph_pays(int n) { return n < 60000 ? 20 : kGraphSteps; }
 
 // Threads per block of the per-atom step kernels: two FP64 lanes per SM and
 // clock bound them, so up to one block of 256 per SM the atoms go to more SMs
@@ -468,7 +473,7 @@ struct nep_md {
     // kept while everything they bake in is unchanged
     cudaStream_t gcap = nullptr, gcap2 = nullptr;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // one step, kGraphSteps steps
-    int gsteps = 0;                                 // steps run with this key, up to kGraphPays
+    int gsteps = 0;                                 // steps run with this key, up to graph_pays
     struct GraphKey {
         const double *pos, *vel;
         double dt, fe[3];
@@ -994,16 +999,24 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             md->gkey = key;
             md->gsteps = 0;
         }
-        const bool pays = md->gexec[1] || md->gsteps + (long long)n_steps >= kGraphPays;
-        md->gsteps = pays ? kGraphPays : md->gsteps + n_steps;
+        const bool several =
+            n_steps >= kGraphSteps && (md->gexec[1] || md->gsteps + (long long)n_steps >= graph_pays(n));
+        if (md->gsteps < graph_pays(n)) md->gsteps += std::min(n_steps, graph_pays(n));
+        auto ensure = [&](int u) {
+            if (md->gexec[u]) return (int)NEP_OK;
+            const int r = capture(u ? kGraphSteps : 1, &md->gexec[u]);
+            if (r) md->gexec[u] = nullptr;
+            return r;
+        };
+        // the first steps singly where the graph of several is missing: the host
+        // captures it while the GPU works on them
+        const int single = several && !md->gexec[1] ? kGraphSteps : 0;
         for (int s = 0; s < n_steps;) {
-            const int u = pays && n_steps - s >= kGraphSteps ? 1 : 0;
-            if (!md->gexec[u] && (rc = capture(u ? kGraphSteps : 1, &md->gexec[u]))) {
-                md->gexec[u] = nullptr;
-                return rc;
-            }
+            const int u = several && s >= single && n_steps - s >= kGraphSteps ? 1 : 0;
+            if ((rc = ensure(u))) return rc;
             if ((rc = cuda_fail(cudaGraphLaunch(md->gexec[u], st), "launch step graph"))) return rc;
             s += u ? kGraphSteps : 1;
+            if (s == single && (rc = ensure(1))) return rc;
         }
         return NEP_OK;
     }
