@@ -405,22 +405,36 @@ __device__ __forceinline__ void half_cell(int cell, int m_cap, float rv2, int ca
 // A block per cell, or with a gate a few blocks per SM that walk the cells: a
 // launch whose gate is off then retires in 5 us instead of 13 (125,000 atoms).
 // (One form for both spilled registers.)
-template <int WARPS, bool GATED>
-__global__ void __launch_bounds__(32 * WARPS) k_half_cells(int ncell, int m_cap, float rv2, int cap,
+// ATOMS: a block (or a turn of the walk) per atom in cell order, of which the
+// first of a cell takes the cell: for sparse grids, where nearly every block of the
+// other form found an empty cell.  50,000 atoms, whole call, by cells -> by atoms:
+// 1.5 atoms per cell 159 -> 169 us, 0.91 157 -> 162, 0.59 159 -> 158, 0.23 204 ->
+// 153, 0.03 995 -> 175; 1,000,000 atoms, 0.75 per cell 2467 -> 2503.  The line lies
+// at half an atom per cell.
+template <int WARPS, bool GATED, bool ATOMS>
+__global__ void __launch_bounds__(32 * WARPS) k_half_cells(int items, int m_cap, float rv2, int cap,
                                                           const float* xr,
-                                                          const float4* xs,
+                                                          const float4* xs, const int* atom_cell,
                                                           const int* cell_start,
                                                           int* count, int* rows, Box b,
                                                           const unsigned* gate)
 {
     const int block = block_after();
+    auto take = [&](int t) {
+        int cell = t;
+        if constexpr (ATOMS) {
+            cell = atom_cell[__float_as_int(xs[t].w)];
+            if (cell_start[cell] != t) return;
+        }
+        half_cell<WARPS>(cell, m_cap, rv2, cap, xr, xs, cell_start, count, rows, b);
+    };
     if constexpr (!GATED) {
-        half_cell<WARPS>(block, m_cap, rv2, cap, xr, xs, cell_start, count, rows, b);
+        take(block);
     } else {
         if (gated_off(gate)) return;
-        for (int cell = block; cell < ncell; cell += gridDim.x) {
-            if (cell != block) __syncthreads();  // the previous cell's tables are read
-            half_cell<WARPS>(cell, m_cap, rv2, cap, xr, xs, cell_start, count, rows, b);
+        for (int t = block; t < items; t += gridDim.x) {
+            if (t != block) __syncthreads();  // the previous cell's tables are read
+            take(t);
         }
     }
 }
@@ -908,12 +922,15 @@ int build_neighbor_list(NeighborList& nl, const Box& b, int n, double* pos, cons
         // candidates per cell: 14 mean cells and half as many again
         const int cap = std::min(std::max(128, (int)(1.5 * 14.0 * n / ncell) / 32 * 32), 1024);
         const int warps = ncell <= 608 ? 8 : n < 8 * (long long)ncell ? 2 : 4;
-        auto half = warps == 8   ? (d_gate ? k_half_cells<8, true> : k_half_cells<8, false>)
-                    : warps == 2 ? (d_gate ? k_half_cells<2, true> : k_half_cells<2, false>)
-                                 : (d_gate ? k_half_cells<4, true> : k_half_cells<4, false>);
-        launch_after(true, half, d_gate ? std::min(ncell, kListGridCap) : ncell, 32 * warps,
-                     (size_t)cap * sizeof(float4), st, ncell, nl.m_cap, rv2, cap, nl.xr, nl.xs, nl.cell_start,
-                     nl.count, rows, b, d_gate);
+        const bool sparse = 2LL * n < ncell;
+        const int items = sparse ? n : ncell;
+        auto half = sparse       ? (d_gate ? k_half_cells<2, true, true> : k_half_cells<2, false, true>)
+                    : warps == 8 ? (d_gate ? k_half_cells<8, true, false> : k_half_cells<8, false, false>)
+                    : warps == 2 ? (d_gate ? k_half_cells<2, true, false> : k_half_cells<2, false, false>)
+                                 : (d_gate ? k_half_cells<4, true, false> : k_half_cells<4, false, false>);
+        launch_after(true, half, d_gate ? std::min(items, kListGridCap) : items, 32 * warps,
+                     (size_t)cap * sizeof(float4), st, items, nl.m_cap, rv2, cap, nl.xr, nl.xs, nl.atom_cell,
+                     nl.cell_start, nl.count, rows, b, d_gate);
         const size_t sort_smem = (size_t)kSortWarps * lcap * 12 + (size_t)nl.m_cap * (kSortAtoms + 1) * sizeof(int);
         if (sort_smem <= kSortTileMaxSmem)
             launch_after(true, k_sort_tile, std::min(blocks_for(n, kSortAtoms), kSortGridCap), 32 * kSortWarps,

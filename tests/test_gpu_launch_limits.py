@@ -279,3 +279,75 @@ def test_short_runs_with_new_loss_weights():
         assert torch.equal(a, b)
     ds.close()
     model.close()
+
+
+@pytest.mark.parametrize("nc", [(17, 17, 17), (18, 18, 18), (60, 9, 10), (100, 100, 100)])
+def test_sparse_boxes(orc, nc):
+    """The cells path below and above two cells per atom, where the search goes by
+    atoms: 2600 atoms in close pairs and triples, one cell with forty of them, all
+    counts against brute force and a sample against the oracle; and MD with the
+    list built behind a gate (spectral heat current) and without, same bits."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(sum(nc))
+    L = 6.0 * np.array(nc) + 0.5  # cells of the list radius of MD
+    a = rng.uniform(0.0, L, (1300, 3))
+    d = rng.normal(size=(1300, 3))
+    pos = np.concatenate([a, a + d * (rng.uniform(1.5, 4.0, 1300) / np.linalg.norm(d, axis=1))[:, None]])
+    g = np.stack(np.meshgrid(*[np.arange(4)] * 3, indexing="ij"), -1).reshape(-1, 3)[:40]
+    pos[:40] = 6.2 + 1.3 * g + rng.normal(0.0, 0.05, (40, 3))
+    box, n = np.diag(L), len(pos)
+    z = inputs.random_z(1021, rng)
+    model = nep.NEP(z)
+    out = model.compute(soa(pos), box)
+    cnt = model.neighbors(n)[0].cpu().numpy()
+    for i in range(n):
+        r = pos - pos[i]
+        r = np.linalg.norm(r - L * np.round(r / L), axis=1)
+        near = int(np.sum(np.abs(r - 5.0) < 1e-5))
+        assert abs(int(cnt[i]) - int(np.sum((r < 5.0) & (r > 0)))) <= near
+    idx = np.unique(np.concatenate([np.arange(40), rng.integers(0, n, 100)]))
+    U, F, _ = orc.efv_sample(orc.NepHyper(), f32_exact(z), pos, box, idx)
+    assert np.abs(out["e_atom"].cpu().numpy()[idx] - U).max() <= 1e-6
+    assert np.abs(aos(out["force"])[idx] - F).max() <= 1e-4
+    got = []
+    for shc in (False, True):
+        md = nep.MD(model, n, box, 28.085)
+        if shc:
+            md.set_shc(4, 2)
+        x, v = soa(pos), soa(np.full((n, 3), 0.05))
+        md.step(x, v, 12, 1.0)
+        torch.cuda.synchronize()
+        assert md.rebuild_count() > 0
+        got.append((x, v))
+        md.close()
+    for s, t in zip(*got):
+        assert torch.equal(s, t)
+    model.close()
+
+
+def test_empty_cells_cost_little():
+    """3,000 atoms in a box of 512,000 cells take at most twice as long as in one of
+    8,000 (five times as long when every empty cell had a block)."""
+    import time
+
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(2)
+    model = nep.NEP(inputs.random_z(1021, rng))
+
+    def call(edge):
+        x, box = soa(rng.uniform(0.0, edge, (3000, 3))), np.diag([edge] * 3)
+        times = []
+        for _ in range(30):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            for _ in range(5):
+                model.compute(x, box, sync=False)
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t)
+        return np.median(times[10:])
+
+    small, large = call(100.0), call(400.0)
+    assert large <= 2.0 * small, (large, small)
+    model.close()
