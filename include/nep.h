@@ -608,7 +608,7 @@ int nep_profile_read(nep_model* m, double* ms, long long* launches);
  *               as for nep_compute_efv.
  *   err_out     dev, 1 unsigned or NULL: device-side error bits of this call
  *               (0 = none; 1 = neighbour overflow, 2 = non-finite value,
- *               4 = asymmetric list), written by the call's last kernel.
+ *               4 = asymmetric list), written by the call's last operation.
  */
 #define NEP_STATIC_MAX_ATOMS 4096
 #define NEP_STATIC_MAX_NEIGHBORS 96

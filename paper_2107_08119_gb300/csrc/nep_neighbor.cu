@@ -54,7 +54,8 @@ __global__ void k_bin(int n, double* __restrict__ pos, const float* __restrict__
         // FP64 operations are slow here (comparisons and division among them):
         // 0 <= x < L, nearly every atom, is one integer comparison of the bits
         // (a negative or non-finite x compares above), and atoms within one box
-        // length of the box wrap by one exact subtraction
+        // length of the box wrap without a division: exactly from above, with one
+        // rounding from below (a tiny negative x gives L, then 0)
         double w = x;
         if ((unsigned long long)__double_as_longlong(x) >= (unsigned long long)__double_as_longlong(L)) {
             if (!isfinite(x)) atomicOr(err, kErrNonFinite);
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_half_cells(int items, int m_cap,
 // to inv[i][unsorted slot] and to the fourth word of the partner entry (the
 // partner's reverse index; j's slot sp[e] of the atom in the value).
 template <int EPL>
-__device__ __forceinline__ void rank_rows_write(int c0, int ns, int m, int lane, const unsigned long long* sk,
+__device__ __forceinline__ void rank_rows_write(int c0, int ns, int lane, const unsigned long long* sk,
                                                 const int* sp, int i, int out_stride, int m_cap, int* out,
                                                 int* __restrict__ rows, int* __restrict__ inv)
 {
@@ -539,12 +540,12 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_sort_rows(int n, int m_ca
         __syncwarp();
         fetch(i + stride);
         if (ns <= 32)
-            rank_rows_write<1>(0, ns, m, lane, sk, sp, i, n, m_cap, nbr + i, rows, inv);
+            rank_rows_write<1>(0, ns, lane, sk, sp, i, n, m_cap, nbr + i, rows, inv);
         else if (ns <= 64)
-            rank_rows_write<2>(0, ns, m, lane, sk, sp, i, n, m_cap, nbr + i, rows, inv);
+            rank_rows_write<2>(0, ns, lane, sk, sp, i, n, m_cap, nbr + i, rows, inv);
         else
             for (int c0 = 0; c0 < ns; c0 += 128)
-                rank_rows_write<4>(c0, ns, m, lane, sk, sp, i, n, m_cap, nbr + i, rows, inv);
+                rank_rows_write<4>(c0, ns, lane, sk, sp, i, n, m_cap, nbr + i, rows, inv);
         __syncwarp();
     }
 }
@@ -626,12 +627,12 @@ __global__ void __launch_bounds__(32 * kSortWarps) k_sort_tile(int n, int m_cap,
         int* col = s_tile + a;
         if (ns == 0) {
         } else if (ns <= 32)
-            rank_rows_write<1>(0, ns, m, lane, sk, sp, i, kSortAtoms + 1, m_cap, col, rows, inv);
+            rank_rows_write<1>(0, ns, lane, sk, sp, i, kSortAtoms + 1, m_cap, col, rows, inv);
         else if (ns <= 64)
-            rank_rows_write<2>(0, ns, m, lane, sk, sp, i, kSortAtoms + 1, m_cap, col, rows, inv);
+            rank_rows_write<2>(0, ns, lane, sk, sp, i, kSortAtoms + 1, m_cap, col, rows, inv);
         else
             for (int c0 = 0; c0 < ns; c0 += 128)
-                rank_rows_write<4>(c0, ns, m, lane, sk, sp, i, kSortAtoms + 1, m_cap, col, rows, inv);
+                rank_rows_write<4>(c0, ns, lane, sk, sp, i, kSortAtoms + 1, m_cap, col, rows, inv);
         __syncwarp();
         if (k % kPer == kPer - 1) {
             // the tile is complete: its rows to nbr, 32 consecutive atoms each
