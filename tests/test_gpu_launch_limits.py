@@ -351,3 +351,49 @@ def test_empty_cells_cost_little():
     small, large = call(100.0), call(400.0)
     assert large <= 2.0 * small, (large, small)
     model.close()
+
+
+@pytest.mark.parametrize("profile", [False, True])
+def test_rows_and_targets_in_turn(profile):
+    """One-step calls whose rows and target temperature stay or change, and with no
+    rows between: every row and state of the same steps with rows of their own, and
+    no row written that its call did not name."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(4)
+    pos, box = inputs.diamond(3, 3, 3)
+    pos = inputs.displace(pos, 0.05, rng)
+    n = len(pos)
+    vel = rng.normal(0.0, 1e-3, (n, 3))
+    model = nep.NEP(inputs.random_z(1021, rng))
+    model.profile(profile)
+    # (buffer of the rows or None, target temperature or None)
+    calls = [(0, None), (0, None), (1, None), (0, None), (None, None), (0, None), (0, 300.0), (0, 300.0), (0, 500.0),
+             (1, 500.0), (1, 300.0), (None, 300.0), (1, None), (1, None), (0, None)]
+
+    def run(shared):
+        md = nep.MD(model, n, box, 28.085)
+        x, v = soa(pos), soa(vel)
+        rows = [torch.zeros(11, dtype=torch.float64, device="cuda") for _ in range(2)]
+        out = []
+        for b, target in calls:
+            md.set_thermostat(target or 0.0, 100.0 if target else 0.0)
+            if not shared:
+                rows = [torch.zeros(11, dtype=torch.float64, device="cuda") for _ in range(2)]
+            for r in rows:
+                r.fill_(-1.0)
+            if b is None:
+                md.step(x, v, 1, 1.0)
+            else:
+                md.step(x, v, 1, 1.0, thermo=rows[b][:8], heat=rows[b][8:])
+            out.append(torch.stack(rows + [torch.cat([x.sum(1), v.sum(1), x[:, 0], v[:, 0]])[:11]]))
+        md.close()
+        return torch.stack(out)
+
+    got, want = run(True), run(False)
+    assert torch.equal(got, want)
+    for (b, _), g in zip(calls, got):
+        for k in range(2):
+            assert bool((g[k] == -1.0).all()) != (k == b)
+    model.profile(False)
+    model.close()
