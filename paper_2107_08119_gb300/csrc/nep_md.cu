@@ -436,6 +436,12 @@ constexpr int kGraphSteps = 5;
 // that follow a call of 5 steps 5240 -> 5192.
 constexpr int graph_pays(int n) { return n < 60000 ? 20 : kGraphSteps; }
 
+// Atoms from which the starting forces of a new state hide the capture of that
+// graph.  20 steps of a new state, the graph behind five single steps -> at once:
+// 13,824 atoms 1213 -> 1260 us, 21,952 1535 -> 1550, 27,000 1828 -> 1821, 32,768 1966
+// -> 1938, 39,304 2384 -> 2339, 125,000 5810 -> 5763.
+constexpr int kHiddenCapture = 30000;
+
 // Threads per block of the per-atom step kernels: two FP64 lanes per SM and
 // clock bound them, so up to one block of 256 per SM the atoms go to more SMs
 // (driven step of 13,824 atoms 73.9 -> 71.4 us, step of 4,096 39.8 -> 39.4; 128
@@ -1023,8 +1029,10 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
             md->gkey = key;
             md->gsteps = 0;
         }
+        // behind the starting forces of a large box the capture costs nothing
+        const bool hidden = init && n >= kHiddenCapture;
         const bool several =
-            n_steps >= kGraphSteps && (md->gexec[1] || md->gsteps + (long long)n_steps >= graph_pays(n));
+            n_steps >= kGraphSteps && (md->gexec[1] || hidden || md->gsteps + (long long)n_steps >= graph_pays(n));
         if (md->gsteps < graph_pays(n)) md->gsteps += std::min(n_steps, graph_pays(n));
         auto ensure = [&](int u) {
             if (md->gexec[u]) return (int)NEP_OK;
@@ -1034,7 +1042,7 @@ int nep_md_step(nep_md* md, double* pos, double* vel, int n_steps, double dt, do
         };
         // the first steps singly where the graph of several is missing: the host
         // captures it while the GPU works on them
-        const int single = several && !md->gexec[1] ? kGraphSteps : 0;
+        const int single = several && !md->gexec[1] && !hidden ? kGraphSteps : 0;
         for (int s = 0; s < n_steps;) {
             const int u = several && s >= single && n_steps - s >= kGraphSteps ? 1 : 0;
             if ((rc = ensure(u))) return rc;

@@ -397,3 +397,31 @@ def test_rows_and_targets_in_turn(profile):
             assert bool((g[k] == -1.0).all()) != (k == b)
     model.profile(False)
     model.close()
+
+
+@pytest.mark.parametrize("cells,steps", [((15, 15, 16), 12), ((15, 16, 16), 5), ((15, 16, 16), 12)])
+def test_first_steps_of_a_new_state(cells, steps):
+    """The first call on a new state below and above 30,000 atoms, where its graph of
+    five steps is captured behind the starting forces: states and rows of the same
+    steps one by one."""
+    import torch
+    from paper_2107_08119_gb300 import nep
+    rng = np.random.default_rng(6)
+    pos, box = inputs.diamond(*cells)
+    pos = inputs.displace(pos, 0.05, rng)
+    n = len(pos)
+    vel = rng.normal(0.0, 1e-3, (n, 3))
+    model = nep.NEP(inputs.random_z(1021, rng))
+    got = []
+    for chunk in (steps, 1):
+        md = nep.MD(model, n, box, 28.085)
+        x, v = soa(pos), soa(vel)
+        rows = torch.zeros((steps, 8), dtype=torch.float64, device="cuda")
+        for s in range(0, steps, chunk):
+            md.step(x, v, chunk, 1.0, thermo=rows[s:s + chunk])
+        torch.cuda.synchronize()
+        got.append((x, v, rows))
+        md.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    model.close()

@@ -1,7 +1,10 @@
-"""The site pass works on 32 atoms per block, 16 list slots per shared tile
-and 32 own slots per word and thread: atom counts around the block, slot
-counts around the tile and every capacity class against the oracle, at the
-bars of the force path (1e-6 eV, 1e-4 eV/A)."""
+"""Kernels at the edges of their tiles, blocks and variants: the site pass (32
+atoms per block, 16 list slots per shared tile and 32 own slots per word and
+thread: atom counts around the block, slot counts around the tile and every
+capacity class against the oracle, at the bars of the force path: 1e-6 eV,
+1e-4 eV/A), the list by direct tests and by cells, the cell offsets, the FP32
+population network, the adjoint, dependent launches back to back, the split of
+the positions, and the step sums of driven and plain MD."""
 import numpy as np
 import pytest
 
