@@ -11,15 +11,19 @@
 //                    tests, unit vector and radial functions, into a shared
 //                    tile of 16 slots (lane-minor: no bank conflicts);
 //   descriptor sums  from the tile, slots in descending order: warps 0-2
-//                    eight of the 24 harmonics each, warp 3 the radial sums (each sum in one thread, in the order of
-//                    site_descriptors, so the same bits);
+//                    eight of the 24 harmonics each, warp 3 the radial sums
+//                    (each sum in one thread);
 //   network          warp w takes the neurons mu = w mod 4, then a quarter of
 //                    the input gradient G;
 //   partial forces   warp w takes its slots again, each angular pair against
 //                    the coefficients A in shared memory.
 // Measured on a GB300, one thread per atom -> this form: 248 -> 186 us for the
-// 125,000-atom crystal (1190 -> 1122 warp instructions per atom, 7.6 -> 18.6
-// warps per SM), 104 -> 71 us for the whole MD step of 4,096 atoms.
+// 125,000-atom crystal (7.6 -> 18.6 warps per SM), 104 -> 71 us for the whole MD
+// step of 4,096 atoms.  Warp instructions per atom there, on the list without a
+// skin: 1190 one thread per atom, 1122 this form at first, 1215 with each record
+// loaded a slot ahead (the moves between the two records; no change of time
+// here, and MD steps 2 % shorter), 1219 with the block sizes below.  On a list
+// with 1 A of skin 1291: 46 instead of 28 slots per atom are tested.
 #pragma once
 
 #include "nep_site.cuh"
